@@ -205,7 +205,7 @@ struct TcWork {
   // that row (as a column) is non-empty; only those lists have a record written
   unsigned int* col_mask;
   int mask_words;
-  long long part_ints;      // entries of each row-side list array (likewise)
+  long long part_lists;     // row-side lists (likewise)
   unsigned int* thr;        // [stacked rows] bit patterns of an upper bound of each row's k-th distance
   int* counter;             // next unit to hand out (zero before the launch)
   int write_lists;          // 0: only publish row bounds (band pre-pass)
@@ -216,6 +216,16 @@ struct TcWork {
   int part_lo, part_hi;
 };
 
+// Capacity of a row-side list: a chunk of 32 columns can append 32 entries, and a list
+// without room for them is cut to between k and cap - 32 of its smallest entries first
+// (list_load reads at most 128). 128 entries are rarely filled (a unit of 2,044 columns
+// takes about 60 at k = 20); where the lists of a call would take more than 4 GB they get
+// the least that leaves a cut some effect.
+constexpr int kListCap = 128;
+__host__ __device__ inline int list_cap(int kstride, long long lists) {
+  return lists * kListCap * 8 <= (4LL << 30) ? kListCap : kstride + 44;
+}
+
 // Ints per column-list record for list pitch kstride (a multiple of 4).
 __host__ __device__ inline int col_pitch(int kstride) { return 4 + 2 * kstride; }
 
@@ -225,8 +235,11 @@ struct TcArgs {
   int out_rows;        // stacked trajectory rows
   int Lmax, kmax;      // largest L and k of the call (shared-memory sizing)
   const float* W;      // [out_rows] window sums of day norms
-  float* part_d;       // [lists][kstride] row-side partial lists
-  int32_t* part_i;
+  // Row-side candidate lists: cap entries (index, distance bits) reserved per list, the
+  // first part_n[list] of them in use, in increasing index order.
+  int2* part;          // [lists][cap]
+  int* part_n;         // [lists]
+  int cap;
   int* err;
   long long wait_limit_ns;
   int debug_withhold;
@@ -243,7 +256,16 @@ struct TcArgs {
   // for every other launch.
   int corr_neg;
   float band_margin;
+  // Main pass: the rows' shared minima, [min_slots(kmax)][out_rows] bit patterns, and the
+  // tiles of a unit after which a row's bound is refreshed from them (a unit's last tile
+  // always does).
+  unsigned int* shared_min;
+  int bound_tiles;
 };
+
+// Slots of the rows' shared minima (a multiple of 32): with k of 64 slots the bound is
+// that of about the 1.2 k-th nearest column at k = 20 and the 1.6 k-th at k = 40.
+__host__ __device__ inline int min_slots(int kmax) { return kmax <= 40 ? 64 : 128; }
 
 // Bytes of TcArgs::scratch for a launch of `num_ctas` CTAs.
 inline size_t tc_scratch_bytes(int num_ctas) {

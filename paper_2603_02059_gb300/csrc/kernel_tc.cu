@@ -27,13 +27,14 @@
 //            from TMEM while scanning: the tensor cores never accumulate more than
 //            one segment of products per output, which bounds the error of their
 //            accumulation however large D is;
-//   warps 2-5 epilogue: each thread owns one accumulator row (TMEM lane), pulls
-//            32 columns at a time with tcgen05.ld, stages them beside the L-1
-//            columns carried from the previous chunk, sums each output's window
-//            down the diagonal, masks the exclusion zone, and keeps the row's k
-//            best in registers (row side). Beyond the strip's own block the same
-//            distances are offered, transposed by warp ballots, to the columns'
-//            lists (column side), so each unordered pair is evaluated once.
+//   warps 2-  epilogue, in one or two groups of four warps (two split a tile's columns):
+//            each thread owns one accumulator row (TMEM lane), pulls 32 columns at a
+//            time with tcgen05.ld, stages them beside the L-1 columns carried from the
+//            previous chunk, sums each output's window down the diagonal, masks the
+//            exclusion zone, and appends the distances within the row's bound to the
+//            row's candidate list (row side) and, beyond the strip's own block, those
+//            within a column's bound to the column's list (column side), so each
+//            unordered pair is evaluated once (epilogue.cuh).
 // Work units (a strip and a range of columns, or a band unit that only seeds the
 // per-row bounds) are handed out dynamically; a unit may serve several series that
 // share its Gram tiles (several trajectory lengths of one record).
@@ -44,6 +45,7 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "epilogue.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
 
@@ -55,14 +57,16 @@ constexpr int BN = kTileCols;  // accumulator columns per tile (256)
 constexpr int KC = 32;         // K elements per stage (64 B rows, 64-B swizzle)
 constexpr int kEpiThreads = 128;  // one epilogue group: one thread per accumulator row
 // Threads of a CTA: warp 0 producer, warp 1 MMA issuer, G epilogue groups of four
-// warps. With G = 2 (L = 1 only: no window, no carry) group g reads the columns
-// [g 128, (g+1) 128) of every tile, so that twice as many warps hide the epilogue's
-// latencies when it, not the contraction, sets the pace (small grids).
+// warps. With G = 2 group g reads the columns [g 128, (g+1) 128) of every tile, so that
+// twice as many warps hide the epilogue's latencies when it, not the contraction, sets
+// the pace.
 __host__ __device__ constexpr int kThreadsG(int G) { return 64 + kEpiThreads * G; }
 // Pitch of the Gram chunk buffer: 32 columns plus the L-1 carried ones, made odd
-// so that the diagonal reads of 32 consecutive rows hit 32 different banks.
-__host__ __device__ constexpr int chunk_pitch(int L) {
-  return 32 + (L - 1) + (((L - 1) % 2 == 0) ? 1 : 0);
+// so that the diagonal reads of 32 consecutive rows hit 32 different banks. Without
+// windows (every L = 1) a row only holds its own distances: 16-byte aligned rows whose 16-byte
+// accesses by eight consecutive lanes hit different banks.
+__host__ __device__ constexpr int chunk_pitch(int L, bool win) {
+  return !win ? 36 : 32 + (L - 1) + (((L - 1) % 2 == 0) ? 1 : 0);
 }
 constexpr uint32_t kTileA = BM * KC * 2;  // bytes of one A operand tile
 constexpr uint32_t kTileB = BN * KC * 2;  // bytes of one B operand tile
@@ -70,53 +74,10 @@ constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(BM, BN);
 constexpr int kMaxStages = 8;
 constexpr size_t kSmemLimit = 232448;  // 227 KB opt-in per block
 
-// Sorted (ascending distance) list of the K best candidates of one row, held in
-// registers. Candidates arrive in increasing index order, so the strict compare
-// keeps an earlier (smaller) index ahead of an equal distance: the order is
-// (distance, index) (Algorithm 1, kNN step). K may exceed k; the first k entries
-// are then the row's k best.
-template <int K>
-struct RegList {
-  float d[K];
-  int32_t i[K];
-
-  __device__ __forceinline__ void reset() {
-#pragma unroll
-    for (int p = 0; p < K; ++p) {
-      d[p] = CUDART_INF_F;
-      i[p] = -1;
-    }
-  }
-  __device__ __forceinline__ float threshold() const { return d[K - 1]; }
-  // Branch-free bubble: the list stays in registers (an early-exit form makes the
-  // compiler move it to local memory).
-  __device__ __forceinline__ void insert(float x, int32_t xi) {
-#pragma unroll
-    for (int p = 0; p < K; ++p) {
-      const bool sw = x < d[p];
-      const float td = d[p];
-      const int32_t ti = i[p];
-      d[p] = sw ? x : td;
-      i[p] = sw ? xi : ti;
-      x = sw ? td : x;
-      xi = sw ? ti : xi;
-    }
-  }
-};
-
-// Shared memory of one epilogue group: Gram chunk with carried columns, W, row
-// bounds and correction values of a tile, column-side row masks, column lists.
-__host__ __device__ constexpr size_t group_bytes(int k, int L) {
-  return (size_t)BM * chunk_pitch(L) * 4 + 3 * BN * 4 + 128 * 4 + (size_t)32 * k * 8;
-}
-
-// Bits [lo, hi) of a 32-bit word (empty when hi <= lo).
-__device__ __forceinline__ uint32_t bit_range(int lo, int hi) {
-  lo = max(lo, 0);
-  hi = min(hi, 32);
-  if (hi <= lo) return 0u;
-  const uint32_t w = (hi - lo >= 32) ? 0xffffffffu : ((1u << (hi - lo)) - 1u);
-  return w << lo;
+// Shared memory of one epilogue group: Gram chunk with carried columns, W, row bounds
+// and correction values of a tile, column-side counters (two chunks).
+__host__ __device__ constexpr size_t group_bytes(int L) {
+  return (size_t)BM * chunk_pitch(L, L > 1) * 4 + 3 * BN * 4 + 64 * 4;
 }
 
 struct TcParams {
@@ -162,11 +123,10 @@ struct UnitSpan {
   long long part_base, col_base;
 };
 
-// Unit u for the sj-th of the series that share its Gram tiles (sj = 0: the one
+// Unit wu for the sj-th of the series that share its Gram tiles (sj = 0: the one
 // with the most trajectories, whose tiles cover the others').
-__device__ __forceinline__ bool unit_span(const TcWork& w, const SeriesInfo* sr, int u, int sj,
+__device__ __forceinline__ bool unit_span(const WorkUnit& wu, const SeriesInfo* sr, int sj,
                                           UnitSpan& us) {
-  const WorkUnit wu = w.units[u];
   const SeriesInfo& si = sr[wu.series + sj];
   us.nser = wu.pad[0] > 1 ? wu.pad[0] : 1;
   us.M = si.M;
@@ -200,30 +160,12 @@ __device__ __forceinline__ bool unit_span(const TcWork& w, const SeriesInfo* sr,
   return true;
 }
 
-// Publish an upper bound of a row's k-th distance. The same pair distance can be
-// evaluated more than once (band pre-pass and main pass; a pair and its transpose)
-// with results a few ulp apart, so a bound taken from one evaluation is widened by
-// a relative 2^-12 (far above those differences) before it prunes another; a wider
-// bound only admits more candidates to the exact final selection.
-__device__ __forceinline__ void publish_bound(unsigned int* thr, float d) {
-  atomicMin(thr, __float_as_uint(__fmul_ru(d, 1.0f + 0x1p-12f)));
-}
-
-// The k-th entry of a sorted register list (k is a run-time value, K a compile-time
-// bound): the minimum of entries k-1 .. K-1, written as a reduction so that the
-// list stays in registers.
-template <int K>
-__device__ __forceinline__ float kth_of(const RegList<K>& l, int k) {
-  float v = CUDART_INF_F;
-#pragma unroll
-  for (int p = 0; p < K; ++p) v = fminf(v, p >= k - 1 ? l.d[p] : CUDART_INF_F);
-  return v;
-}
-
 constexpr int kQueue = 4;  // depth of the per-CTA unit queue
-constexpr size_t kGroupBoundBytes = 2 * BM * 8;  // two groups' tagged row bounds
 
-template <int K, int G>
+// G: epilogue groups; kWin: some series of the call has L > 1 (windows are summed); kBand:
+// the band pre-pass (bounds only, no lists); kLarge: k > 32 in the band pass (two minima
+// per group), k > 40 in the main pass (128 shared minima); one epilogue group only.
+template <int G, bool kWin, bool kBand, bool kLarge>
 __global__ void __launch_bounds__(kThreadsG(G), 1)
     fused_tc_kernel(const __grid_constant__ CUtensorMap tmA_hi,
                     const __grid_constant__ CUtensorMap tmA_lo,
@@ -242,13 +184,8 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   const uint32_t ring = (raw + 1023u) & ~1023u;
   unsigned char* gptr = smem_raw + (ring - raw) + (size_t)NS * p.stage_bytes;
   // epilogue regions (one per group), sized for the largest L and k of the call
-  const size_t gbytes = group_bytes(a.kmax, a.Lmax);
-  // two groups: each row's current list bound in each group, tagged with the unit
-  // (the other group's bound also bounds the row's k-th distance; see the scan)
-  volatile unsigned long long* gbound =
-      reinterpret_cast<volatile unsigned long long*>(gptr + G * gbytes);
-  uint64_t* bars =
-      reinterpret_cast<uint64_t*>(gptr + G * gbytes + (G == 2 ? kGroupBoundBytes : 0));
+  const size_t gbytes = group_bytes(a.Lmax);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(gptr + G * gbytes);
   const uint32_t full0 = ptx::smem_u32(bars);
   const uint32_t empty0 = full0 + 8u * NS;
   const uint32_t tfull0 = empty0 + 8u * NS;
@@ -256,9 +193,14 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   const uint32_t drain = tempty0 + 16u;
   const uint32_t qfull0 = drain + 8u;
   const uint32_t qempty0 = qfull0 + 8u * kQueue;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * NS + 5 + 2 * kQueue);
+  const uint32_t xfull = qempty0 + 8u * kQueue;  // second group's minima are in (band)
+  const uint32_t xempty = xfull + 8u;            // ... and have been read
+  // units handed out, read by the MMA issuer and the epilogue (16-byte aligned; a
+  // negative strip ends the list)
+  WorkUnit* qunit = reinterpret_cast<WorkUnit*>(
+      (reinterpret_cast<uintptr_t>(bars + 2 * NS + 7 + 2 * kQueue) + 15) & ~uintptr_t(15));
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(qunit + kQueue);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* qval = reinterpret_cast<volatile int*>(tmem_slot + 2);  // [kQueue]
 
   Ctl ctl;
   ctl.abort = abort_flag;
@@ -279,7 +221,8 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
       ptx::mbar_init(qfull0 + 8u * i, 1);
       ptx::mbar_init(qempty0 + 8u * i, 1 + G);  // the MMA thread and each group's leader
     }
-
+    ptx::mbar_init(xfull, kEpiThreads);
+    ptx::mbar_init(xempty, kEpiThreads);
     *abort_flag = 0;
     ptx::fence_mbar_init();
     ptx::fence_proxy_async();
@@ -289,8 +232,6 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     ptx::tmem_relinquish();
     ptx::tc_fence_before();
   }
-  if (G == 2)  // no unit has tag 0xFFFFFFFF: every entry starts unused
-    for (int i = threadIdx.x; i < 2 * BM; i += blockDim.x) gbound[i] = ~0ull;
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
@@ -298,6 +239,15 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   const int seg_kb = p.seg_kb;                    // K blocks per accumulation segment
   // segments per tile (the two-group form runs with one segment: checked on the host)
   const int nseg = G == 2 ? 1 : (nkb + seg_kb - 1) / seg_kb;
+  auto read_unit = [&](int slot) {  // a queue slot, by 16-byte reads
+    union {
+      int4 v[2];
+      WorkUnit u;
+    } x;
+    x.v[0] = reinterpret_cast<const int4*>(qunit + slot)[0];
+    x.v[1] = reinterpret_cast<const int4*>(qunit + slot)[1];
+    return x.u;
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
@@ -318,14 +268,17 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
       while (ok) {
         if (!wait_bounded(qempty0 + 8u * qs, qphase ^ 1u, ctl)) break;
         const int u = atomicAdd(w.counter, 1);
-        qval[qs] = u;
+        WorkUnit wu;
+        if (u < w.nunits) wu = w.units[u];
+        else wu.strip = -1;
+        qunit[qs] = wu;
         ptx::mbar_arrive(qfull0 + 8u * qs);
         if (++qs == kQueue) {
           qs = 0;
           qphase ^= 1u;
         }
         if (u >= w.nunits) break;
-        if (!unit_span(w, p.sr.s, u, 0, us)) continue;
+        if (!unit_span(wu, p.sr.s, 0, us)) continue;
         for (int it = 0; ok && it < us.ntiles; ++it) {
           const int c0 = us.row_base + us.jlo + it * us.adv;
           const int a0 = us.row_base + us.T0;
@@ -384,14 +337,14 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           ok = false;
           break;
         }
-        const int u = qval[qs];
+        const WorkUnit wu = read_unit(qs);
         ptx::mbar_arrive(qempty0 + 8u * qs);
         if (++qs == kQueue) {
           qs = 0;
           qphase ^= 1u;
         }
-        if (u >= w.nunits) break;
-        if (!unit_span(w, p.sr.s, u, 0, us)) continue;
+        if (wu.strip < 0) break;
+        if (!unit_span(wu, p.sr.s, 0, us)) continue;
         for (int it = 0; ok && it < us.ntiles; ++it, ++gt) {
           for (int kb = 0; kb < nkb; ++kb) {
             if (kb % seg_kb == 0) {
@@ -467,20 +420,20 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
     const int et = threadIdx.x - 64 - kEpiThreads * gid;  // 0..127 within the group
     const int bar = 1 + gid;          // the group's named barrier
+    constexpr int kSlots = kLarge && !kBand ? 128 : 64;  // shared minima per row (min_slots)
     // the group's chunks of every tile
     const int ch_lo = gid * (BN / 32 / G), ch_hi = ch_lo + BN / 32 / G;
     // the group's shared memory
     float* Gbuf = reinterpret_cast<float*>(gptr + gid * gbytes);
-    float* Wsh = Gbuf + BM * chunk_pitch(a.Lmax);  // window sums of the tile's output columns
+    float* Wsh = Gbuf + BM * chunk_pitch(a.Lmax, kWin);  // window sums of the tile's output columns
     float* Tsh = Wsh + BN;         // row bounds of the tile's output columns (column side)
     float* Csh = Tsh + BN;         // correction values c of the tile's Gram columns
-    uint32_t* Cmask = reinterpret_cast<uint32_t*>(Csh + BN);  // [4][32] column-side row masks
-    float* Cld = reinterpret_cast<float*>(Cmask + 128);  // [kmax][32] column-side lists
-    int32_t* Cli = reinterpret_cast<int32_t*>(Cld + 32 * a.kmax);
-    const long long cpitch = col_pitch(w.kstride);  // ints per column-list record
-    const int cx = ((warp - 2) & 3) * 8 + (lane & 7);      // column-side column of lanes 0..7
-    int qs = 0, gch = 0, gt = 0;
-    uint32_t qphase = 0;
+    ColSide cs;
+    cs.cnt = reinterpret_cast<int*>(Csh + BN);
+    cs.turn = 0;
+    if (et < 64) cs.cnt[et] = 0;  // ordered before their use by a tile's barriers
+    int qs = 0, gt = 0;
+    uint32_t qphase = 0, xphase = 0;
     bool ok = true;
     UnitSpan us;
     // phase timing of the first epilogue thread (diagnostics)
@@ -498,7 +451,6 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         tp = now;
       }
     };
-    RegList<K> list;
     // Segment folding (more than one segment per tile): segment pseg of tile pt is
     // the next to add to the tile's partial total; every segment but a tile's last
     // is folded (segment s of tile t is segment t * nseg + s overall, in accumulator
@@ -564,9 +516,32 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         v[4 * g + 3] = __float_as_uint(r.w);
       }
     };
+    // What a pass over a tile needs from global memory (window sums, bounds and
+    // correction values of two of its 256 columns; the row's own values), fetched while
+    // the pass before it runs.
+    struct Head {
+      float w[2], t[2], c[2], wt, cr, thr;
+    } hd;
+    auto fetch_head = [&](const UnitSpan& s, int it) {
+      const int c0 = s.jlo + it * s.adv, t = s.T0 + l, N = s.M + s.L - 1;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int x = et + kEpiThreads * h, j = c0 - (s.L - 1) + x;
+        const bool in = j >= 0 && j < s.M;
+        hd.w[h] = in ? a.W[s.out_base + j] : 0.f;
+        hd.t[h] = in ? __uint_as_float(__ldcg(w.thr + s.out_base + j)) : 0.f;
+        hd.c[h] = c0 + x < N ? a.cval[s.row_base + c0 + x] : 0.f;  // Gram column day c0 + x
+      }
+      const bool row_ok = l < s.R && t < s.M;
+      hd.wt = row_ok ? a.W[s.out_base + t] : 0.f;
+      hd.thr = row_ok ? __uint_as_float(__ldcg(w.thr + s.out_base + t)) : 0.f;
+      hd.cr = t < N ? a.cval[s.row_base + t] : 0.f;
+    };
     while (ok) {
       bool wok = wait_bounded(qfull0 + 8u * qs, qphase, ctl);
-      const int u = wok ? qval[qs] : 0;
+      WorkUnit wu;
+      wu.strip = -1;
+      if (wok) wu = read_unit(qs);
       wok = ptx::named_bar_and(bar, kEpiThreads, wok);  // everyone has read the slot
       if (!wok) {
         ok = false;
@@ -577,13 +552,18 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         qs = 0;
         qphase ^= 1u;
       }
-      if (u >= w.nunits) break;
-      if (!unit_span(w, p.sr.s, u, 0, us)) continue;
+      if (wu.strip < 0) break;
+      if (!unit_span(wu, p.sr.s, 0, us)) continue;
+      fetch_head(us, 0);
       // Series that share this unit's Gram tiles (several trajectory lengths of one
-      // record) are served one after another from the same accumulator; their units
-      // are one tile long, so their row lists live for one tile.
+      // record) are served one after another from the same accumulator; their row
+      // lists live for one tile (main units are one tile long; band units keep no lists).
       const int nser = us.nser;
       const int ntiles = us.ntiles;
+      RowSide rs;  // this thread's row list in this unit
+      GroupMin<kBand && kLarge> gm;
+      rs.reset();
+      gm.reset();
       for (int it = 0; it < ntiles; ++it, ++gt) {
         lap(6);
         // the earlier segments are folded into the scratch partial total; the last
@@ -600,48 +580,54 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         }
         ptx::tc_fence_after();
         lap(0);
-        bool released = false;
         for (int sj = 0; sj < nser; ++sj) {
-        if (nser > 1 && !unit_span(w, p.sr.s, u, sj, us)) continue;
-        const int L = G == 2 ? 1 : us.L;  // two groups run only at L = 1
-        const int LDG = chunk_pitch(L);
+        const int L = kWin ? us.L : 1;
+        const int LDG = chunk_pitch(L, kWin);
         const int t = us.T0 + l;
         const bool row_ok = l < us.R && t < us.M;
-        const float Wt = row_ok ? a.W[us.out_base + t] : 0.f;
         // the operand layout subtracts groups * c_a * c_b from every Gram entry (see the
-        // operand preparation); it is added back when a chunk is staged, for every
+        // operand preparation); it is added back when a chunk is read, for every
         // accumulator row whose day exists (halo rows feed other rows' windows)
-        const int N = us.M + us.L - 1;
         // (with one product on split operands the correction entries added
         // +groups c_a c_b: subtract it instead)
-        const float crow =
-            t < N ? (a.corr_neg ? -(float)a.groups : (float)a.groups) * a.cval[us.row_base + t]
-                  : 0.f;
+        const float crow = (a.corr_neg ? -(float)a.groups : (float)a.groups) * hd.cr;
+        const float Wt = hd.wt;
+        float thr_row = hd.thr;
         const int jsym = us.T0 + us.R;  // column side from here on (sym)
         const long long cbase = w.sym ? us.col_base + w.col_off[us.strip_base + us.strip] : 0;
-        if (nser > 1 || it == 0) list.reset();
+        if (nser > 1 || it == 0) {
+          rs.reset();
+          gm.reset();
+          if (!kBand)
+            rs.rec = a.part +
+                     (size_t)(us.part_base + (long long)t * us.slots + us.slot * G + gid) * a.cap;
+        }
         const int c0 = us.jlo + it * us.adv;
         // W and row bounds of this tile's output columns j = c0 - (L-1) + x (the
-        // previous tile's readers passed its last barrier)
-        for (int x = et; x < BN; x += kEpiThreads) {
-          const int j = c0 - (L - 1) + x;
-          const bool in = j >= 0 && j < us.M;
-          Wsh[x] = in ? a.W[us.out_base + j] : 0.f;
-          Tsh[x] = in ? __uint_as_float(__ldcg(w.thr + us.out_base + j)) : 0.f;
-          Csh[x] = c0 + x < N ? a.cval[us.row_base + c0 + x] : 0.f;  // Gram column day c0 + x
+        // previous pass's readers passed its last barrier)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          Wsh[et + kEpiThreads * h] = hd.w[h];
+          Tsh[et + kEpiThreads * h] = hd.t[h];
+          Csh[et + kEpiThreads * h] = hd.c[h];
         }
-        const float thr_row = row_ok ? __uint_as_float(__ldcg(w.thr + us.out_base + t)) : 0.f;
-        ptx::named_bar_sync(bar, kEpiThreads);  // Csh is read by every thread when staging
+        ptx::named_bar_sync(bar, kEpiThreads);  // read by every thread of the group
+        const UnitSpan cu = us;  // this pass; `us` moves on to the next one
+        if (sj + 1 < nser) {
+          unit_span(wu, p.sr.s, sj + 1, us);
+          fetch_head(us, it);
+        } else if (it + 1 < ntiles) {
+          if (nser > 1) unit_span(wu, p.sr.s, 0, us);  // (a band unit of several tiles)
+          fetch_head(us, it + 1);
+        }
         lap(1);
         // chunk ch+1 is fetched while chunk ch is scanned: from TMEM with a single
         // segment, else the scratch partial total (the last segment's chunk is
-        // added from TMEM when the chunk is staged)
+        // added from TMEM when the chunk is read)
         const uint32_t tlast = tmem_base + lane_addr + (uint32_t)(acc_l * BN);
-        // with the largest lists, and with two epilogue groups (168 registers a thread;
-        // the other group hides the latency), the chunk is fetched when it is staged
-        // instead (the prefetched registers would otherwise stay live across the scan
-        // and spill)
-        constexpr bool kAhead = K <= 40 && G == 1;
+        // with two epilogue groups (168 registers a thread; the other group hides the
+        // latency) a chunk is fetched when it is read
+        constexpr bool kAhead = G == 1;
         uint32_t vr[32];
         if (kAhead) {
           if (nseg == 1)
@@ -649,266 +635,178 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           else
             load_scr(gt, ch_lo, vr);
         }
+        float* grow = Gbuf + l * LDG;
 #pragma unroll 1
         for (int ch = ch_lo; ch < ch_hi; ++ch) {
-          if (!kAhead) {
-            if (nseg == 1)
-              ptx::tmem_ld32_async(tlast + (uint32_t)(ch * 32), vr);
-            else
-              load_scr(gt, ch, vr);
-          }
-          float* grow = Gbuf + l * LDG;
-          // the diagonal carry: the last L-1 Gram columns of the previous chunk (of
-          // the previous tile of this unit at ch = 0) start this chunk's windows
-          if (ch > 0 || (it > 0 && us.carry))
-            for (int c = 0; c < L - 1; ++c) grow[c] = grow[32 + c];
-          const float* cs = Csh + ch * 32;
+          const float* csh = Csh + ch * 32;
           // Gram values of the chunk (correction added back): staged in shared memory
           // for the diagonal window sums, or, with L = 1 (no window), kept in registers
           float c[32];
+          if (!kAhead) ptx::tmem_ld32_async(tlast + (uint32_t)(ch * 32), vr);
           if (nseg == 1) {
             ptx::tmem_wait();
 #pragma unroll
-            for (int x = 0; x < 32; ++x) c[x] = fmaf(crow, cs[x], __uint_as_float(vr[x]));
+            for (int x = 0; x < 32; ++x) c[x] = fmaf(crow, csh[x], __uint_as_float(vr[x]));
           } else {
             uint32_t tv[32];
             ptx::tmem_ld32_async(tlast + (uint32_t)(ch * 32), tv);
             ptx::tmem_wait();
 #pragma unroll
             for (int x = 0; x < 32; ++x)
-              c[x] = fmaf(crow, cs[x], __uint_as_float(vr[x]) + __uint_as_float(tv[x]));
+              c[x] = fmaf(crow, csh[x], __uint_as_float(vr[x]) + __uint_as_float(tv[x]));
           }
-          if (L > 1) {
+          if (kWin && L > 1) {
+            // the diagonal carry: the L-1 Gram columns before the chunk start its
+            // windows: the last ones of the group's previous chunk (of the previous tile
+            // of this unit at the tile's first chunk), or, for the second group's first
+            // chunk, read from the accumulator
+            if (G == 2 && gid == 1 && ch == ch_lo) {
+              uint32_t pv[16];
+              ptx::tmem_ld16_async(tlast + (uint32_t)(ch_lo * 32 - 16), pv);
+              ptx::tmem_wait();
+#pragma unroll
+              for (int x = 0; x < 16; ++x)
+                if (x >= 17 - L) grow[x - (17 - L)] = fmaf(crow, csh[x - 16], __uint_as_float(pv[x]));
+            } else if (ch > 0 || (it > 0 && cu.carry)) {
+              for (int x = 0; x < L - 1; ++x) grow[x] = grow[32 + x];
+            }
 #pragma unroll
             for (int x = 0; x < 32; ++x) grow[(L - 1) + x] = c[x];
           }
-          if (kAhead && ch + 1 < ch_hi) {
-            if (nseg == 1)
+          if (ch + 1 < ch_hi) {
+            if (!kAhead) {
+            } else if (nseg == 1)
               ptx::tmem_ld32_async(tlast + (uint32_t)((ch + 1) * 32), vr);
             else
               load_scr(gt, ch + 1, vr);
-          }
-          if (ch == ch_hi - 1 && sj == nser - 1) {
-            // the accumulator has been read out: hand it back to the MMA warp
-            ptx::tc_fence_before();
-            ptx::mbar_arrive(tempty0 + 8u * acc_l);
-            released = true;
+          } else {
+            // the first group's next tile starts from this tile's last columns, which the
+            // second group reads: kept in vr until the chunk is done
+            if (kWin && G == 2 && gid == 0 && L > 1 && cu.carry && it + 1 < ntiles) {
+              uint32_t pv[16];
+              ptx::tmem_ld16_async(tlast + (uint32_t)(BN - 16), pv);
+              ptx::tmem_wait();
+#pragma unroll
+              for (int x = 0; x < 16; ++x)
+                vr[x] = __float_as_uint(fmaf(crow, Csh[BN - 16 + x], __uint_as_float(pv[x])));
+            }
+            if (sj == nser - 1) {
+              // the accumulator has been read out: hand it back to the MMA warp
+              ptx::tc_fence_before();
+              ptx::mbar_arrive(tempty0 + 8u * acc_l);
+            }
           }
           lap(2);
           // the window sums read other rows' staged values (nothing to wait for at L = 1)
-          if (L > 1) ptx::named_bar_sync(bar, kEpiThreads);
+          if (kWin && L > 1) ptx::named_bar_sync(bar, kEpiThreads);
           lap(3);
           const int j0 = c0 + ch * 32 - (L - 1);
           // column side of this chunk: output columns j >= jsym inside the unit
           // the first L-1 columns of a unit's first chunk have no carried window
-          const int xfirst = (ch == 0 && (it == 0 || !us.carry)) ? L - 1 : 0;
-          const uint32_t colrange = w.sym ? bit_range(max(jsym, us.jlo) - j0, us.jhi - j0) &
-                                                bit_range(xfirst, 32)
-                                          : 0u;
+          const int xfirst = (ch == 0 && (it == 0 || !cu.carry)) ? L - 1 : 0;
+          const uint32_t unitrange = bit_range(xfirst, 32) & bit_range(cu.jlo - j0, cu.jhi - j0);
+          const uint32_t colrange =
+              w.sym ? bit_range(jsym - j0, 32) & unitrange : 0u;
           uint32_t cand = 0, ccand = 0;
-          float othr = CUDART_INF_F;  // the other group's bound for this row (two groups)
           if (row_ok) {
             // output column x of this chunk is j = j0 + x; its window is the diagonal
             // Gbuf[l+m][x+m], m < L (Eq. 2 as W_t + W_j - 2 sum G)
-            uint32_t valid = bit_range(xfirst, 32) & bit_range(us.jlo - j0, us.jhi - j0);
-            valid &= ~bit_range(t - us.e - j0, t + us.e + 1 - j0);  // exclusion zone
-            const float* g0 = Gbuf + l * LDG;
-            const float* wv = Wsh + ch * 32;
-            const float* tv = Tsh + ch * 32;
-            if (L > 1) {
-#pragma unroll
-              for (int x = 0; x < 32; ++x) c[x] = g0[x];
+            if (kWin && L > 1) {
               for (int m = 1; m < L; ++m) {
-                const float* gm = g0 + m * (LDG + 1);
+                const float* gm = grow + m * (LDG + 1);
+                if (m == 1) {
 #pragma unroll
-                for (int x = 0; x < 32; ++x) c[x] += gm[x];
+                  for (int x = 0; x < 32; ++x) c[x] = grow[x] + gm[x];
+                } else {
+#pragma unroll
+                  for (int x = 0; x < 32; ++x) c[x] += gm[x];
+                }
               }
             }
-            const float lthr = list.threshold();
-            // a row candidate has D < lthr and D <= thr_row, i.e. D <= rthr (the float
-            // below lthr when lthr > 0; none when lthr is 0)
-            // with two groups, the other group's list for this row in this unit holds K
-            // real candidates of other columns: its K-th bounds the row's k-th too
-            if (G == 2) {
-              const unsigned long long ob = gbound[(1 - gid) * BM + l];
-              if ((unsigned)(ob >> 32) == (unsigned)u) othr = __uint_as_float((unsigned)ob);
-            }
-            float rthr =
-                fminf(lthr > 0.f ? __uint_as_float(__float_as_uint(lthr) - 1u) : -1.f, thr_row);
-            if (G == 2) rthr = fminf(rthr, othr);
-            if (G == 1 && a.band_margin != 0.f) {
-              // one-product band pre-pass (long operand rows only, so one epilogue
-              // group): the distance raised by a bound of its error
-#pragma unroll
-              for (int x = 0; x < 32; ++x)
-                c[x] = fmaf(a.band_margin, Wt + wv[x],
-                            fmaxf(fmaf(-2.0f, c[x], Wt + wv[x]), 0.0f)) * (1.0f + 0x1p-20f);
+            distances(c, Wt, Wsh + ch * 32, kBand ? a.band_margin : 0.f);
+            const uint32_t valid = unitrange & ~bit_range(t - cu.e - j0, t + cu.e + 1 - j0);
+            if (kBand) {
+              gm.scan(c, valid);  // (outside the exclusion zone)
             } else {
-#pragma unroll
-              for (int x = 0; x < 32; ++x)
-                c[x] = fmaxf(fmaf(-2.0f, c[x], Wt + wv[x]), 0.0f);  // D(t, j0 + x)
+              candidate_masks(c, rs.limit(thr_row), Tsh + ch * 32, cand, ccand);
+              cand &= valid;
+              ccand &= valid & colrange;
             }
-#pragma unroll
-            for (int x = 0; x < 32; ++x) {
-              cand |= (c[x] <= rthr ? 1u : 0u) << x;
-              ccand |= (c[x] <= tv[x] ? 1u : 0u) << x;
-            }
-            cand &= valid;
-            ccand &= valid & colrange;
           }
-          // column-side candidates, transposed by ballots: lane x of warp quadrant q
-          // holds the rows q*32 + b of column x that pass the column's bound
-          uint32_t cm = 0;
-          if (__any_sync(0xffffffffu, ccand != 0u)) {
-#pragma unroll
-            for (int x = 0; x < 32; ++x) {
-              const uint32_t b = __ballot_sync(0xffffffffu, (ccand >> x) & 1u);
-              cm = lane == x ? b : cm;
-            }
+          // every window sum of the chunk is done before a row overwrites the first 32
+          // entries of its Gram row (the carried columns 32.. stay) by its distances
+          if (kWin && L > 1) ptx::named_bar_sync(bar, kEpiThreads);
+          if (!kBand) {
+            const uint32_t cmask = ccand;
+            if (cand | ccand) store_row<!kWin>(grow, c);
+            lap(4);
+            cnt[0] += __popc(cand);
             cnt[1] += __popc(ccand);
+            const bool over = append<kSlots>(rs, cs, cand, ccand, grow, j0, cu.k, t,
+                                             cbase + (j0 - jsym), a.shared_min + cu.out_base + t,
+                                             a.shared_min + cu.out_base + j0, w, a);
+            if (colrange) {  // the same for the whole group
+              const int ne = cs.finish<!kWin>(over, colrange, cmask, c, Gbuf, LDG, l, et, bar,
+                                              cu.k, cu.T0, cu.strip, cu.out_base, j0,
+                                              cbase + (j0 - jsym), w, a);
+              cnt[3] += ne > 0;
+              cnt[2] += ne > cu.k;
+            }
+            rs.compress(cu.k, a, w.thr + cu.out_base + t);
           }
-          Cmask[q * 32 + lane] = cm;
-          ptx::named_bar_sync(bar, kEpiThreads);
-          // every window sum of the chunk is done: a row with candidates replaces the
-          // first 32 entries of its Gram row by its distances (the carried columns
-          // 32.. stay), so that candidates are read back instead of recomputed
-          if (cand | ccand) {
-            float* drow = Gbuf + l * LDG;
+          if (kWin && G == 2 && gid == 0 && L > 1 && ch == ch_hi - 1) {
 #pragma unroll
-            for (int x = 0; x < 32; ++x) drow[x] = c[x];
+            for (int x = 0; x < 16; ++x)
+              if (x >= 17 - L) grow[32 + x - (17 - L)] = __uint_as_float(vr[x]);
           }
-          if (colrange) ptx::named_bar_sync(bar, kEpiThreads);  // other rows read them
-          lap(4);
-          // row side: the few distances that enter the row's list
-          while (cand) {
-            const int x = __ffs(cand) - 1;
-            cand &= cand - 1;
-            const float dv = Gbuf[l * LDG + x];
-            if (dv < list.threshold() && dv <= thr_row && (G == 1 || dv <= othr)) {
-              list.insert(dv, j0 + x);
-              ++cnt[0];
-            }
-          }
-          if (G == 2 && row_ok)
-            gbound[gid * BM + l] =
-                ((unsigned long long)(unsigned)u << 32) | __float_as_uint(list.threshold());
-          // column side, written by the rows themselves: column x's list holds its
-          // candidate rows in row order (slot = number of candidate rows before
-          // this one), unless more than k rows qualify, in which case the column's
-          // own thread below keeps the k best
-          while (ccand) {
-            const int x = __ffs(ccand) - 1;
-            ccand &= ccand - 1;
-            int before = __popc(Cmask[q * 32 + x] & ((1u << lane) - 1u)), ne = 0;
-#pragma unroll
-            for (int wq = 0; wq < 4; ++wq) {
-              const int cq = __popc(Cmask[wq * 32 + x]);
-              ne += cq;
-              before += wq < q ? cq : 0;
-            }
-            if (ne <= us.k) {
-              const long long li = cbase + (j0 + x - jsym);
-              const long long at = li * cpitch + 2 + 2 * before;
-              if (tk_in(at + 1, w.col_ints, a.err) && tk_in(before, us.k, a.err))
-                *reinterpret_cast<int2*>(w.col_rec + at) =
-                    make_int2(us.T0 + l, __float_as_int(Gbuf[l * LDG + x]));
-            }
-          }
-          if (colrange && lane < 8 && ((colrange >> cx) & 1u)) {
-            const int j = j0 + cx;
-            const long long li = cbase + (j - jsym);
-            int ne = 0;
-#pragma unroll
-            for (int wq = 0; wq < 4; ++wq) ne += __popc(Cmask[wq * 32 + cx]);
-            if (ne == us.k) {
-              // exactly k candidates: the largest is the k-th distance
-              float mx = 0.f;
-              for (int wq = 0; wq < 4; ++wq) {
-                uint32_t mk = Cmask[wq * 32 + cx];
-                while (mk) {
-                  const int r = wq * 32 + __ffs(mk) - 1;
-                  mk &= mk - 1;
-                  mx = fmaxf(mx, Gbuf[r * LDG + cx]);
-                }
-              }
-              if (tk_in(us.out_base + j, a.out_rows, a.err))
-                publish_bound(w.thr + us.out_base + j, mx);
-            } else if (ne > us.k) {
-              // more than k: keep the k best in (distance, row) order; rows arrive in
-              // increasing order, so a strict compare keeps the smaller row first
-              int n = 0;
-              for (int wq = 0; wq < 4; ++wq) {
-                uint32_t mk = Cmask[wq * 32 + cx];
-                while (mk) {
-                  const int r = wq * 32 + __ffs(mk) - 1;
-                  mk &= mk - 1;
-                  const float dv = Gbuf[r * LDG + cx];
-                  int pos;
-                  if (n < us.k) {
-                    pos = n++;
-                  } else if (dv < Cld[(us.k - 1) * 32 + cx]) {
-                    pos = us.k - 1;
-                  } else {
-                    continue;
-                  }
-                  while (pos > 0 && Cld[(pos - 1) * 32 + cx] > dv) {
-                    Cld[pos * 32 + cx] = Cld[(pos - 1) * 32 + cx];
-                    Cli[pos * 32 + cx] = Cli[(pos - 1) * 32 + cx];
-                    --pos;
-                  }
-                  Cld[pos * 32 + cx] = dv;
-                  Cli[pos * 32 + cx] = us.T0 + r;
-                }
-              }
-              for (int pp = 0; pp < us.k; ++pp)
-                if (tk_in(li * cpitch + 3 + 2 * pp, w.col_ints, a.err))
-                  *reinterpret_cast<int2*>(w.col_rec + li * cpitch + 2 + 2 * pp) =
-                      make_int2(Cli[pp * 32 + cx], __float_as_int(Cld[pp * 32 + cx]));
-              if (tk_in(us.out_base + j, a.out_rows, a.err))
-                publish_bound(w.thr + us.out_base + j, Cld[(us.k - 1) * 32 + cx]);
-            }
-            if (ne > 0) {  // an empty list gets no record: its mask bit stays clear
-              if (tk_in(li * cpitch, w.col_ints, a.err)) w.col_rec[li * cpitch] = min(ne, us.k);
-              const long long mi = (long long)(us.out_base + j) * w.mask_words + (us.strip >> 5);
-              if (tk_in(mi, (long long)a.out_rows * w.mask_words, a.err))
-                atomicOr(w.col_mask + mi, 1u << (us.strip & 31));
-            }
-            cnt[3] += ne > 0;
-            cnt[2] += ne > us.k;  // lists kept by this thread's insertion
-          }
-          // the column side read other rows' Gram values: keep them until it is done
-          if (colrange) ptx::named_bar_sync(bar, kEpiThreads);
           cnt[4] += et == 0;
           lap(5);
           fold(false, gt + 1);  // the next tile's finished segments, if any
           lap(2);
-          ++gch;
         }
-        if (row_ok) {
-          const float kth = kth_of(list, us.k);
-          if (kth < thr_row && tk_in(us.out_base + t, a.out_rows, a.err))
-            publish_bound(w.thr + us.out_base + t, kth);
-        }
-        if (row_ok && w.write_lists && (nser > 1 || it == ntiles - 1)) {
-          const size_t base =
-              (size_t)(us.part_base + (long long)t * us.slots + us.slot * G + gid) * w.kstride;
+        const bool last = nser > 1 || it == ntiles - 1;
+        if (last || (!kBand && (it + 1) % a.bound_tiles == 0)) {
+          // a bound of the row's k-th distance: from this unit's columns (band), or from
+          // those of every unit so far (main pass)
+          float bd = CUDART_INF_F;
+          if (!kBand) {
+            bd = row_bound<kSlots>(cu.k, a.shared_min + cu.out_base + t, a.out_rows, row_ok,
+                                   thr_row);
+          } else if (G == 2 && nser == 1) {
+            // the second group hands its minima to the first (the chunk buffer of the
+            // second group, which the band uses only while it sums windows)
+            float* xb = reinterpret_cast<float*>(gptr + gbytes);
+            if (gid == 1) {
+              ptx::named_bar_sync(bar, kEpiThreads);  // the windows of the last chunk are done
 #pragma unroll
-          for (int pp = 0; pp < K; ++pp) {
-            if (pp < us.k) {
-              if (tk_in((long long)base + pp, w.part_ints, a.err)) {
-                a.part_d[base + pp] = list.d[pp];
-                a.part_i[base + pp] = list.i[pp];
-              }
+              for (int x = 0; x < 32; ++x) xb[x * BM + l] = gm.m[x];
+              ptx::mbar_arrive(xfull);
+              wok = wait_bounded(xempty, xphase, ctl);  // read: the buffer is free again
+            } else {
+              wok = wait_bounded(xfull, xphase, ctl);
+              if (wok) bd = gm.bound(cu.k, xb + l);
+              ptx::mbar_arrive(xempty);
             }
+            xphase ^= 1u;
+            wok = ptx::named_bar_and(bar, kEpiThreads, wok);
+            if (!wok) {
+              ok = false;
+              break;
+            }
+          } else {
+            bd = gm.bound(cu.k);
           }
+          if (row_ok && bd < thr_row && tk_in(cu.out_base + t, a.out_rows, a.err))
+            publish_bound(w.thr + cu.out_base + t, bd);
         }
-        // the next series restages the chunk buffer and the tile's W, bounds, masks
-        if (nser > 1) ptx::named_bar_sync(bar, kEpiThreads);
+        if (!kBand && last && row_ok && cu.jlo < cu.jhi) {
+          const long long li = cu.part_base + (long long)t * cu.slots + cu.slot * G + gid;
+          if (tk_in(li, w.part_lists, a.err)) a.part_n[li] = rs.n;
+        }
+        // the next pass rewrites the tile's W, bounds and correction values
+        if (sj + 1 < nser) ptx::named_bar_sync(bar, kEpiThreads);
         }  // series sharing the tile
-        if (!released) {
-          ptx::tc_fence_before();
-          ptx::mbar_arrive(tempty0 + 8u * acc_l);
-        }
+        if (!ok) break;
       }
       if (!ok) break;
     }
@@ -968,8 +866,8 @@ bool make_map(CUtensorMap* m, const void* base, int N, int Dp, int box_rows) {
 }
 
 size_t epilogue_bytes(int k, int L, int G) {
-  return G * group_bytes(k, L) + (G == 2 ? kGroupBoundBytes : 0) +
-         8 * (2 * kMaxStages + 5 + 2 * kQueue) + 8 + 4 * kQueue + 16;
+  return G * group_bytes(L) + 8 * (2 * kMaxStages + 7 + 2 * kQueue) + 16 +
+         kQueue * sizeof(WorkUnit) + 16;
 }
 
 int pick_stages(bool split, int k, int L, int G) {
@@ -979,14 +877,14 @@ int pick_stages(bool split, int k, int L, int G) {
   return ns < kMaxStages ? ns : kMaxStages;
 }
 
-template <int K, int G>
-cudaError_t launch_k(const CUtensorMap& mAh, const CUtensorMap& mAl, const CUtensorMap& mBh,
+template <int G, bool kWin, bool kBand, bool kLarge>
+cudaError_t launch_g(const CUtensorMap& mAh, const CUtensorMap& mAl, const CUtensorMap& mBh,
                      const CUtensorMap& mBl, const TcParams& p, int num_ctas, size_t smem,
                      cudaStream_t st) {
-  cudaError_t err = cudaFuncSetAttribute(fused_tc_kernel<K, G>,
+  cudaError_t err = cudaFuncSetAttribute(fused_tc_kernel<G, kWin, kBand, kLarge>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  fused_tc_kernel<K, G><<<num_ctas, kThreadsG(G), smem, st>>>(mAh, mAl, mBh, mBl, p);
+  fused_tc_kernel<G, kWin, kBand, kLarge><<<num_ctas, kThreadsG(G), smem, st>>>(mAh, mAl, mBh, mBl, p);
   return cudaGetLastError();
 }
 
@@ -1020,33 +918,27 @@ cudaError_t launch_fused_tc(const void* hi, const void* lo, bool split, const Tc
   p.split = split ? 1 : 0;
   p.stage_bytes = split ? 2 * kTileA + 2 * kTileB : kTileA + kTileB;
   const int G = a.egroups;
-  // two epilogue groups: L = 1, one accumulation segment, k <= 32 (host-checked here
-  // too: the kernel's two-group form has no window, carry or segment folding)
-  if (G != 1 && (G != 2 || a.Lmax != 1 || a.kmax > 32 || a.Dp > a.seg_k))
-    return cudaErrorInvalidValue;
+  // two epilogue groups: one accumulation segment (checked on the host: the kernel's
+  // two-group form folds no segments)
+  // and k <= 32
+  if (G != 1 && (G != 2 || a.Dp > a.seg_k || a.kmax > 32)) return cudaErrorInvalidValue;
   p.nstages = pick_stages(split, a.kmax, a.Lmax, G);
   if (p.nstages < 2) return cudaErrorInvalidValue;
   if (a.seg_k < KC || a.seg_k % KC != 0) return cudaErrorInvalidValue;
   p.seg_kb = a.seg_k / KC;
   const size_t smem = fused_tc_smem_bytes(split, a.kmax, a.Lmax, G);
-  const int k = a.kmax;
+  const bool win = a.Lmax > 1, band = !w.write_lists, large = a.kmax > (band ? 32 : 40);
+  auto go = [&](auto fn) { return fn(mAh, mAl, mBh, mBl, p, num_ctas, smem, st); };
   if (G == 2) {
-    if (k <= 4) return launch_k<4, 2>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-    if (k <= 8) return launch_k<8, 2>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-    if (k <= 10) return launch_k<10, 2>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-    if (k <= 16) return launch_k<16, 2>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-    if (k <= 20) return launch_k<20, 2>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-    return launch_k<32, 2>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
+    if (band) return win ? go(launch_g<2, true, true, false>) : go(launch_g<2, false, true, false>);
+    return win ? go(launch_g<2, true, false, false>) : go(launch_g<2, false, false, false>);
   }
-  if (k <= 4) return launch_k<4, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-  if (k <= 8) return launch_k<8, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-  if (k <= 10) return launch_k<10, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-  if (k <= 16) return launch_k<16, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-  if (k <= 20) return launch_k<20, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-  if (k <= 32) return launch_k<32, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-  if (k <= 40) return launch_k<40, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-  if (k <= 48) return launch_k<48, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
-  return launch_k<64, 1>(mAh, mAl, mBh, mBl, p, num_ctas, smem, st);
+  if (large) {
+    if (band) return win ? go(launch_g<1, true, true, true>) : go(launch_g<1, false, true, true>);
+    return win ? go(launch_g<1, true, false, true>) : go(launch_g<1, false, false, true>);
+  }
+  if (band) return win ? go(launch_g<1, true, true, false>) : go(launch_g<1, false, true, false>);
+  return win ? go(launch_g<1, true, false, false>) : go(launch_g<1, false, false, false>);
 }
 
 }  // namespace traknn

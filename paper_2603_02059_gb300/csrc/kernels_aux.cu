@@ -475,7 +475,7 @@ __device__ __forceinline__ bool key_less(float d1, int i1, float d2, int i2) {
 // (distance, index) then give the exact neighbour set in order. If the gathered
 // set overflows the buffer, the rounds scan the lists directly.
 __global__ void __launch_bounds__(32 * kMergeWarps)
-    merge_tc_kernel(const float* __restrict__ part_d, const int32_t* __restrict__ part_i,
+    merge_tc_kernel(const int2* __restrict__ part, const int* __restrict__ part_n, int cap,
                     int out_rows, TcWork w, const __grid_constant__ SeriesTable st, int* err) {
   __shared__ float bd[kMergeWarps][kMergeCap];
   __shared__ int bi[kMergeWarps][kMergeCap];
@@ -608,27 +608,40 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
   for (int pass = 0; pass < 64; ++pass) {
     if (lane == 0) bn[wid] = 0;
     __syncwarp();
-    // lists are read four entries at a time (the list pitch ks is a multiple of 4)
-    for (int c = c_lo + lane; c < c_hi; c += 32) {
-      const size_t b = (size_t)(plist + c) * ks;
-      if (!tk_in((long long)b + ks - 1, w.part_ints, err)) continue;
-      const float4* d4 = reinterpret_cast<const float4*>(part_d + b);
-      const int4* i4 = reinterpret_cast<const int4*>(part_i + b);
-      bool more = true;
-      for (int p = 0; more && p < k; p += 4) {
-        const float4 dv = __ldg(d4 + p / 4);
-        const int4 iv = __ldg(i4 + p / 4);
-        const float dd[4] = {dv.x, dv.y, dv.z, dv.w};
-        const int ii[4] = {iv.x, iv.y, iv.z, iv.w};
+    // row-side lists (not sorted): their counts, one list per lane, then their entries
+    // numbered across the lists (a prefix sum of the counts), one per lane and round,
+    // two rounds of loads in flight
+    for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+      const int c = c0 + lane;
+      int nn = 0;
+      if (c < c_hi && tk_in(plist + c, w.part_lists, err)) nn = __ldg(part_n + plist + c);
+      if (!tk_in(nn, cap + 1, err)) nn = 0;
+      int incl = nn;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (!more || p + u >= k) break;
-          if (ii[u] < 0 || dd[u] > thr) {
-            more = false;  // sorted: nothing further qualifies
-          } else {
-            push(dd[u], ii[u]);
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const int total = __shfl_sync(0xffffffffu, incl, 31);
+      const int excl = incl - nn;
+      for (int e0 = 0; e0 < total; e0 += 64) {
+        int2 en[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int e = e0 + 32 * h + lane;
+          int wl = 0;  // the list of entry e: the last lane whose prefix is <= e
+#pragma unroll
+          for (int step = 16; step > 0; step >>= 1) {
+            const int x = __shfl_sync(0xffffffffu, excl, wl + step);
+            if (x <= e) wl += step;
           }
+          const int pos = e - __shfl_sync(0xffffffffu, excl, wl);
+          en[h] = make_int2(0, 0x7FFFFFFF);
+          if (e < total) en[h] = __ldg(part + (size_t)(plist + c0 + wl) * cap + pos);
         }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (__int_as_float(en[h].y) <= thr) push(__int_as_float(en[h].y), en[h].x);
       }
     }
     if (w.sym) {
@@ -717,12 +730,12 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
       for (int q = lane; q < n; q += 32) consider(bd[wid][q], bi[wid][q]);
     } else {
       for (int c = c_lo + lane; c < c_hi; c += 32) {
-        const size_t b = (size_t)(plist + c) * ks;
-        if (!tk_in((long long)b + ks - 1, w.part_ints, err)) continue;
-        for (int p = 0; p < k; ++p) {
-          const int ii = part_i[b + p];
-          if (ii < 0 || part_d[b + p] > thr) break;
-          consider(part_d[b + p], ii);
+        if (!tk_in(plist + c, w.part_lists, err)) continue;
+        const int2* l2 = part + (size_t)(plist + c) * cap;
+        const int nn = part_n[plist + c];
+        for (int p = 0; p < nn; ++p) {
+          const int2 e = l2[p];
+          if (__int_as_float(e.y) <= thr) consider(__int_as_float(e.y), e.x);
         }
       }
       if (w.sym) {
@@ -766,7 +779,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
 cudaError_t launch_merge_tc(const TcArgs& a, const TcWork& w, const SeriesTable& sr,
                             cudaStream_t st) {
   const int blocks = (a.out_rows + kMergeWarps - 1) / kMergeWarps;
-  merge_tc_kernel<<<blocks, 32 * kMergeWarps, 0, st>>>(a.part_d, a.part_i, a.out_rows, w, sr,
+  merge_tc_kernel<<<blocks, 32 * kMergeWarps, 0, st>>>(a.part, a.part_n, a.cap, a.out_rows, w, sr,
                                                         a.err);
   return cudaGetLastError();
 }

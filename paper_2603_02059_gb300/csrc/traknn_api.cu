@@ -249,7 +249,22 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
       for (int s = std::max(0, part_lo); s < std::min(strips, part_hi); ++s) {
         const int T0 = s * R;
         int jlo = std::max(0, T0 - bw);
-        const int jhi = std::min(M, T0 + R + bw);
+        int jhi = std::min(M, T0 + R + bw);
+        // an exclusion zone that leaves the centred band few candidates: the columns
+        // beside the zone instead (those after it, or before it where they are more)
+        int emax = 0;
+        for (int q = 0; q < nser; ++q) emax = std::max(emax, sd[b + q].e);
+        const int width = 2 * bw + R;
+        if (emax > width / 4) {
+          const int64_t after = (int64_t)T0 + R + emax, before = (int64_t)T0 - emax;
+          if (after + width <= M || M - after >= before) {
+            jlo = (int)std::min<int64_t>(after, M);
+            jhi = (int)std::min<int64_t>(after + width, M);
+          } else {
+            jhi = (int)std::max<int64_t>(before, 0);
+            jlo = std::max(0, jhi - width);
+          }
+        }
         // a phase's band units stay clear of the days still being copied (a band only
         // seeds bounds, from whatever candidates it holds)
         const int q = phase_of(s);
@@ -312,9 +327,10 @@ struct TcBuffers {
   float* W;
   void* hi;
   void* lo;
-  float* part_d;
-  int32_t* part_i;
+  int2* part;
+  int* part_n;
   unsigned int* thr;
+  unsigned int* shared_min;
   int32_t* col_rec;
   unsigned int* col_mask;
   int* counter;
@@ -343,9 +359,13 @@ TcBuffers tc_layout(const TcPlan& p, int64_t D, int num_ctas, char* base) {
   b.W = reinterpret_cast<float*>(take((size_t)p.out_rows * sizeof(float)));
   b.hi = take((size_t)p.rows * b.Dp * 2);
   b.lo = take((size_t)p.rows * b.Dp * 2);
-  b.part_d = reinterpret_cast<float*>(take((size_t)p.part_lists * ks * sizeof(float)));
-  b.part_i = reinterpret_cast<int32_t*>(take((size_t)p.part_lists * ks * sizeof(int32_t)));
-  b.thr = reinterpret_cast<unsigned int*>(take((size_t)p.out_rows * sizeof(unsigned int)));
+  b.part = reinterpret_cast<int2*>(
+      take((size_t)p.part_lists * list_cap((int)ks, p.part_lists) * sizeof(int2)));
+  b.part_n = reinterpret_cast<int*>(take((size_t)p.part_lists * sizeof(int)));
+  // bounds and shared minima: one fill (0x7F) sets both
+  b.thr = reinterpret_cast<unsigned int*>(
+      take((size_t)p.out_rows * (1 + min_slots(p.kmax)) * sizeof(unsigned int)));
+  b.shared_min = b.thr + p.out_rows;
   b.col_rec = reinterpret_cast<int32_t*>(
       take((size_t)p.col_lists * col_pitch((int)ks) * sizeof(int32_t)));
   b.col_mask = reinterpret_cast<unsigned int*>(
@@ -373,24 +393,28 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   key.push_back(part_hi);
   key.push_back((int64_t)pstrip.size());
   key.insert(key.end(), pstrip.begin(), pstrip.end());
-  // two epilogue groups for L = 1 (small grids through embedded operands) when the
-  // tile has one accumulation segment and the lists are short
+  // Two epilogue groups (one accumulation segment, k <= 32) where the epilogue and not the
+  // contraction sets a tile's pace: K entries x products below a line, the more the series
+  // that scan each tile. Measured with one and two groups (N = 10,957, L = 5): split-BF16
+  // D = 1,476 684 / 633 us, 2,116 880 / 855, 2,800 1,020 / 1,056; BF16 D = 2,116 784 / 698,
+  // 2,800 878 / 837, 3,555 (N = 7,301, L = 7) 745 / 746; four lengths of a D = 3,726
+  // record 2,381 / 1,908.
   int Lmax = 1, kmax = 1;
   for (int b = 0; b < B; ++b) {
     Lmax = std::max(Lmax, sd[b].L);
     kmax = std::max(kmax, sd[b].k);
   }
-  const int egroups = (h->epi_groups != 1 && !shared && Lmax == 1 && kmax <= 32 &&
-                       tc_groups((int)D * emb) * 64 <= h->seg_k)
-                          ? 2
-                          : 1;
+  const int Dk = tc_groups((int)D * emb) * 64;
+  const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2304 : 3584) * (shared ? B : 1);
+  const int egroups =
+      (h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k && (Lmax == 1 || Dk <= line)) ? 2 : 1;
   key.push_back(egroups);
   // Band pre-pass width: two tiles per strip when the contraction dominates a tile's
   // cost; with short operand rows (small grids) a tile's contraction is cheap and the
   // epilogue decides, and eight tiles give bounds tight enough to save more list
   // inserts in the main pass than the band costs (D = 32, L = 5: 1.91 -> 1.69 ms; at
   // D = 3,726 four tiles already cost 6 %)
-  const int band_tiles = tc_groups((int)D * emb) * 64 <= 768 ? 8 : 2;
+  const int band_tiles = Dk <= 768 ? 8 : 2;
   key.push_back(band_tiles);
   TcPlan& p = h->plan;
   if (p.key != key) {
@@ -466,8 +490,11 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
   a.Lmax = p.Lmax;
   a.kmax = p.kmax;
   a.W = b.W;
-  a.part_d = b.part_d;
-  a.part_i = b.part_i;
+  a.part = b.part;
+  a.part_n = b.part_n;
+  a.cap = list_cap(list_pitch(p.kmax), p.part_lists);
+  a.shared_min = b.shared_min;
+  a.bound_tiles = b.Dp > 768 ? 1 : 4;
   a.err = h->err;
   a.wait_limit_ns = (long long)h->wait_limit_ms * 1000000LL;
   a.debug_withhold = h->debug_withhold;
@@ -491,7 +518,7 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
   w.col_ints = p.col_lists * col_pitch(w.kstride);
   w.col_mask = b.col_mask;
   w.mask_words = p.mask_words;
-  w.part_ints = p.part_lists * w.kstride;
+  w.part_lists = p.part_lists;
   w.thr = b.thr;
   w.counter = b.counter;
   w.write_lists = 1;
@@ -506,7 +533,8 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
                                     b.hi, b.lo,
                                     b.norms, b.cval, s));
   TRY_CUDA(launch_window_series(sr, p.out_rows, b.norms, b.W, s));
-  TRY_CUDA(cudaMemsetAsync(b.thr, 0x7F, (size_t)p.out_rows * sizeof(unsigned int), s));
+  TRY_CUDA(cudaMemsetAsync(
+      b.thr, 0x7F, (size_t)p.out_rows * (1 + min_slots(p.kmax)) * sizeof(unsigned int), s));
   TRY_CUDA(cudaMemsetAsync(b.col_mask, 0,
                            (size_t)p.out_rows * p.mask_words * sizeof(unsigned int), s));
   TRY_CUDA(cudaMemsetAsync(b.counter, 0, 2 * sizeof(int), s));
@@ -590,8 +618,11 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
   a.Lmax = p.Lmax;
   a.kmax = p.kmax;
   a.W = b.W;
-  a.part_d = b.part_d;
-  a.part_i = b.part_i;
+  a.part = b.part;
+  a.part_n = b.part_n;
+  a.cap = list_cap(list_pitch(p.kmax), p.part_lists);
+  a.shared_min = b.shared_min;
+  a.bound_tiles = b.Dp > 768 ? 1 : 4;
   a.err = h->err;
   a.wait_limit_ns = (long long)h->wait_limit_ms * 1000000LL;
   a.debug_withhold = h->debug_withhold;
@@ -613,7 +644,7 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
   w.col_ints = p.col_lists * col_pitch(w.kstride);
   w.col_mask = b.col_mask;
   w.mask_words = p.mask_words;
-  w.part_ints = p.part_lists * w.kstride;
+  w.part_lists = p.part_lists;
   w.thr = b.thr;
   w.write_lists = 1;
   w.stats = h->stats ? h->stats_dev : nullptr;
@@ -647,7 +678,8 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
     TRY_CUDA(cudaStreamWaitEvent(s, in[q], 0));
     if (q == 0) {
       TRY_CUDA(launch_col_mean_series(sr, (int)D, b.partial, b.mu, h->center != 0, s));
-      TRY_CUDA(cudaMemsetAsync(b.thr, 0x7F, (size_t)p.out_rows * sizeof(unsigned int), s));
+      TRY_CUDA(cudaMemsetAsync(
+      b.thr, 0x7F, (size_t)p.out_rows * (1 + min_slots(p.kmax)) * sizeof(unsigned int), s));
       TRY_CUDA(cudaMemsetAsync(b.col_mask, 0,
                                (size_t)p.out_rows * p.mask_words * sizeof(unsigned int), s));
       TRY_CUDA(cudaMemsetAsync(b.counter, 0, 2 * K * sizeof(int), s));
@@ -742,29 +774,30 @@ traknn_status pick_shape(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
 }
 
 // Work-unit shape when neither the autotuner nor an option sets it: Gram tiles per
-// unit and row strips side by side (0 = the planner's default). Short operand rows
-// (small grids): the epilogue sets the pace, and units of 16 tiles keep fewer partial
-// lists per row, so fewer list inserts (D = 32, L = 5, embedded: 1.70 -> 1.61 ms;
-// longer units lose more at the launch's tail than they save), with 38 strips side by
-// side (1.61 -> 1.58 ms). Otherwise the unit length follows the Gram tiles per SM of
-// an average series of the call (strips [part_lo, part_hi)): eight tiles from 64
-// (the 75-year series has 78), four from 16, two below (L = 5, D = 3,726:
-// N = 10,957 1.31 -> 1.21 ms with two; N = 13,697 1.87 -> 1.83 ms and N = 20,546
-// 3.84 -> 3.72 ms with four; at N = 27,394 the three lengths time alike; 64 series of
-// 3,650 to 27,394 days in one call: four tiles 1.04x faster than eight). Shorter
-// units let the persistent CTAs run out of work together and keep more of a
-// series' operand tiles in L2 while its strips run side by side. Long operand rows
-// make every tile long too, so a unit also holds at most 65,536 K entries x tiles
-// (Dp x tiles), two tiles at least: at the 0.25-degree grid (Dp = 59,072, N = 27,394,
-// L = 5) 8 / 4 / 2 tiles took 106.0-108.8 / 99.8-100.7 / 98.9-99.9 ms, while at
-// Dp = 3,840 eight tiles stay within the cap; between the two the cap is a choice.
+// unit and row strips side by side (0 = the planner's default). Shorter units let the
+// persistent CTAs run out of work together and keep more of a series' operand tiles in
+// L2 while its strips run side by side; longer ones start fewer lists and reload fewer
+// strip operands.
+//
+// Short operand rows (small grids; 38 strips side by side), by the Gram tiles per SM of an
+// average series of the call (strips [part_lo, part_hi)), measured with 1 / 2 / 4 / 8 / 16
+// tiles: D = 32, L = 5, N = 2,500 130 / 142 / 156 / 192 / 216 us, 4,000 150 / 147 / 167 /
+// 212 / 286, 7,000 202 / 198 / 208 / 216 / 277, 10,957 315 / 294 / 292 / 304 / 304, 16,000
+// 497 / 455 / 440 / 451 / 471; D = 640, N = 18,000 915 / 826 / 816 / 843 / 854; N = 27,394
+// times alike from 4 to 16.
+//
+// Otherwise eight tiles from 64 Gram tiles per SM (the 75-year series has 78), four from
+// 16, two below (L = 5, D = 3,726: N = 10,957 1.31 -> 1.21 ms with two; N = 13,697 1.87
+// -> 1.83 ms and N = 20,546 3.84 -> 3.72 ms with four; at N = 27,394 the three lengths
+// time alike; 64 series of 3,650 to 27,394 days in one call: four tiles 1.04x faster than
+// eight), and one where the whole call has fewer than 8 (D = 3,726: N = 1,826 351 ->
+// 300 us, N = 4,500 499 -> 435, N = 6,500 656 -> 589). Long operand rows make every tile
+// long too, so a unit also holds at most 65,536 K entries x tiles (Dp x tiles), two tiles
+// at least: at the 0.25-degree grid (Dp = 59,072, N = 27,394, L = 5) 8 / 4 / 2 tiles took
+// 106.0-108.8 / 99.8-100.7 / 98.9-99.9 ms, while at Dp = 3,840 eight tiles stay within the
+// cap; between the two the cap is a choice.
 void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, int emb,
                    int part_lo, int part_hi, int* tiles, int* group) {
-  if (tc_groups((int)D * emb) * 64 <= 768) {
-    *tiles = 16;
-    if (*group == 0 && h->group_strips == 0) *group = 38;
-    return;
-  }
   double t = 0.0;  // Gram tiles of the call
   for (int b = 0; b < B; ++b) {
     const int64_t M = sd[b].N - sd[b].L + 1;
@@ -773,9 +806,15 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     for (int st = std::max(0, part_lo); st < std::min(strips, part_hi); ++st)
       t += (double)(h->sym ? M - (int64_t)st * R : M) / kTileCols;
   }
-  const double per_sm = t / B / std::max(1, h->sm_count);
-  *tiles = per_sm >= 64.0 ? 8 : per_sm >= 16.0 ? 4 : 2;
+  const double all = t / std::max(1, h->sm_count), per_sm = all / B;
   const int64_t Dp = (int64_t)tc_groups((int)D * emb) * 64;
+  if (Dp <= 768) {
+    *tiles = per_sm >= 64.0 ? 16 : per_sm >= 48.0 ? 8 : per_sm >= 10.0 ? 4 : 2;
+    if (all < 1.5) *tiles = 1;
+    if (*group == 0 && h->group_strips == 0) *group = 38;
+    return;
+  }
+  *tiles = per_sm >= 64.0 ? 8 : per_sm >= 16.0 ? 4 : all >= 8.0 ? 2 : 1;
   while (*tiles > 2 && *tiles * Dp > 65536) *tiles /= 2;
 }
 

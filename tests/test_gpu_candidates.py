@@ -1,0 +1,65 @@
+"""Candidate lists, shared minima and bounds of the tensor-core kernel where they can go
+wrong: few-valued integer fields, whose distances tie by the hundred (lists, column records
+and the merge's buffer overflow, and the order among ties decides), every range of k with its
+own number of shared minima, exclusion zones wider than the band, and two epilogue groups
+with a window. Small integers are exact in BF16 and their sums in FP32, so without centring
+the neighbour sets and distances must equal the oracle's, ties included."""
+import numpy as np
+import pytest
+
+import oracle
+from synth import make_slp_like
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tk():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2603_02059_gb300 as m
+    return m
+
+
+def _integers(N, D, top, seed):
+    return np.random.default_rng(seed).integers(0, top + 1, (N, D)).astype(np.float32)
+
+
+@pytest.mark.parametrize("prec", ["split_bf16", "bf16"])
+@pytest.mark.parametrize("N,D,top,L,k,e", [
+    (700, 3, 1, 1, 1, 0), (700, 3, 1, 2, 5, 1), (700, 4, 2, 1, 20, 0), (1300, 3, 1, 5, 33, 4),
+    (700, 4, 3, 3, 41, 2), (700, 3, 1, 17, 64, 16), (2600, 4, 2, 2, 20, 1),
+    (1500, 4, 3, 2, 10, 400), (1500, 4, 3, 1, 40, 700), (129, 2, 1, 2, 64, 1)])
+def test_ties_and_wide_exclusion_equal_the_oracle(tk, prec, N, D, top, L, k, e):
+    import torch
+    X = _integers(N, D, top, seed=N + k)
+    oidx, odist, _ = oracle.knn_scores(X, L, k, e)
+    for embed in ("never", "always") if L > 1 else ("never",):
+        idx, dist, _ = tk.knn_scores(torch.from_numpy(X).cuda(), L, k, e, precision=prec,
+                                     center=False, embed=embed)
+        assert np.array_equal(dist.cpu().numpy(), odist.astype(np.float32))
+        assert np.array_equal(idx.cpu().numpy(), oidx)
+
+
+@pytest.mark.parametrize("N,h,w,L,k,e", [(1500, 20, 32, 5, 20, 4), (2000, 36, 41, 2, 10, 1),
+                                         (900, 30, 33, 17, 32, 16), (385, 20, 40, 3, 1, 2),
+                                         (3000, 45, 50, 4, 12, 3)])
+def test_two_epilogue_groups_with_a_window_equal_one(tk, N, h, w, L, k, e):
+    """The second group starts its windows from columns it reads itself, the first one a
+    tile's from the columns the second group read: bitwise the same distances."""
+    import torch
+    X = torch.from_numpy(make_slp_like(N, h, w, seed=N + L)[0]).cuda()
+    for prec in ("split_bf16", "bf16"):
+        got = []
+        for groups in (0, 1):
+            hd = tk.Handle()
+            hd.set_option("epi_groups", groups)
+            got.append(tk.knn_scores(X, L, k, e, precision=prec, embed="never", handle=hd))
+            got.append(tk.knn_scores_multi(X, [(L, k, e), (max(1, L - 1), k, e)],
+                                           precision=prec, handle=hd)[0])
+            torch.cuda.synchronize()
+            assert hd.sync_status() == 0
+        for a, b in ((got[0], got[2]), (got[1], got[3])):
+            for x, y in zip(a, b):
+                assert torch.equal(x, y)
