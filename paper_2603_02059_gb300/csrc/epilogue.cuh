@@ -102,6 +102,53 @@ __device__ __forceinline__ void window_topk(const float* g, int ldg, const RowCt
   }
 }
 
+// -------------------------------------------------------------------- work units
+// A unit with its series' parameters.
+struct UnitSpan {
+  int strip, T0, jlo, jhi, ntiles, slot, nser, step;
+  int carry, adv;  // carry: the last L-1 Gram columns pass from tile to tile; adv: tile stride
+  int M, L, k, e, R;      // series: trajectories, length, neighbours, exclusion, rows per strip
+  int row_base, out_base, slots, strip_base;
+  long long part_base, col_base;
+};
+
+// Unit wu for the sj-th of the series that share its Gram tiles (sj = 0: the one
+// with the most trajectories, whose tiles cover the others').
+__device__ __forceinline__ bool unit_span(const WorkUnit& wu, const SeriesInfo* sr, int sj,
+                                          UnitSpan& us) {
+  const SeriesInfo& si = sr[wu.series + sj];
+  us.nser = wu.pad[0] > 1 ? wu.pad[0] : 1;
+  us.M = si.M;
+  us.L = si.L;
+  us.k = si.k;
+  us.e = si.e;
+  us.R = si.rows_out;
+  us.row_base = si.row_base;
+  us.out_base = si.out_base;
+  us.slots = si.slots;
+  us.strip_base = si.strip_base;
+  us.part_base = si.part_base;
+  us.col_base = si.col_base;
+  us.strip = wu.strip;
+  us.T0 = wu.strip * us.R;
+  us.jlo = wu.jlo;
+  us.jhi = min(wu.jhi, si.M);
+  us.slot = wu.slot;
+  us.step = si.step;
+  if (us.jlo >= us.jhi) return false;
+  // A unit of one series: Gram tiles follow each other without overlap, tile it
+  // covering Gram columns [jlo + 256 it, jlo + 256 (it+1)); the epilogue carries the
+  // last L-1 columns of a tile into the next, so the windows of all output columns
+  // [jlo, jhi) are complete once Gram column jhi + L - 2 is in. A unit shared by
+  // several series (each restages the chunk buffer with its own L) has no carry: its
+  // tiles overlap by the largest L - 1 and each yields `step` output columns.
+  us.carry = us.nser == 1;
+  us.adv = us.carry ? kTileCols : us.step;
+  us.ntiles = us.carry ? (us.jhi - us.jlo + us.L - 1 + kTileCols - 1) / kTileCols
+                       : (us.jhi - us.jlo + us.step - 1) / us.step;
+  return true;
+}
+
 // ---------------------------------------------------------------- candidate lists
 // The symmetric kernels do not sort while they scan. A row appends every distance within
 // its current bound to an unsorted list of its own in global memory (one 8-byte store; no

@@ -294,14 +294,16 @@ enum : int {
 };
 
 // ----------------------------------------------------------------- launchers
-cudaError_t launch_col_mean(const float* X, int N, int D, float* partial, float* mu,
-                            bool center, cudaStream_t st);
 // wts: optional [D] grid-point weights (the values are scaled by sqrt(w_p)), or null.
-cudaError_t launch_prep_fp32(const float* X, int N, int D, int Dp, const float* mu,
-                             const float* wts, float* Xc, double* norms, cudaStream_t st);
-cudaError_t launch_window(const double* norms, int M, int L, float* W, cudaStream_t st);
-cudaError_t launch_fused_fp32(const float* Xc, const FusedArgs& a, int num_ctas,
-                              cudaStream_t st);
+cudaError_t launch_prep_fp32_series(const SeriesTable& sr, int rows, int D, int Dp,
+                                    const float* mu, const float* wts, float* Xc, double* norms,
+                                    cudaStream_t st);
+// FP32 CUDA-core path over the work list of the tensor-core path (Xc: the stacked FP32
+// operand copy, pitch a.Dp), and the both-triangles form of traknn_knn_scores_static.
+cudaError_t launch_fused_fp32(const float* Xc, const TcArgs& a, const TcWork& w,
+                              const SeriesTable& sr, int num_ctas, cudaStream_t st);
+cudaError_t launch_fused_fp32_static(const float* Xc, const FusedArgs& a, int num_ctas,
+                                     cudaStream_t st);
 // Tensor-core path; `split` selects the 3-product split-BF16 form.
 cudaError_t launch_fused_tc(const void* hi, const void* lo, bool split, const TcArgs& a,
                             const TcWork& w, const SeriesTable& sr, int num_ctas, cudaStream_t st);
@@ -364,7 +366,6 @@ cudaError_t launch_adjoint(const float* X, int N, int D, int L, int k, const int
 // Levina-Bickel local intrinsic dimension for k_id <= k; either output may be null.
 cudaError_t launch_knn_stats(const float* dist, int M, int k, float* prefix, int k_id,
                              float* local_id, cudaStream_t st);
-size_t fused_fp32_smem_bytes(int k);
 // False until the tensor-core kernel is compiled in.
 bool tc_available();
 

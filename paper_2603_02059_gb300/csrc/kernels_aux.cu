@@ -20,33 +20,6 @@ namespace {
 // the full mean to shrink the Gram values as well, costs a small fraction of a pass
 // over X, and lies in the first part of X a host-buffer call copies in.
 
-// Column sums of the centring days (the last kMeanDays) over fixed slices (fixed
-// summation order: deterministic).
-__global__ void col_partial_kernel(const float* __restrict__ X, int N, int D, float* partial) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= D) return;
-  const int first = mean_first(N), ns = mean_days(N);
-  const int per = (ns + kMeanSlices - 1) / kMeanSlices;
-  const int r0 = blockIdx.y * per, r1 = min(ns, r0 + per);
-  float acc = 0.f;
-  for (int i = r0; i < r1; ++i) acc += X[(size_t)(first + i) * D + p];
-  partial[(size_t)blockIdx.y * D + p] = acc;
-}
-
-// FP32 sums suffice for the offset (see above).
-__global__ void col_final_kernel(const float* __restrict__ partial, int N, int D, float* mu,
-                                 int center) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= D) return;
-  if (!center) {
-    mu[p] = 0.f;
-    return;
-  }
-  float acc = 0.f;
-  for (int s = 0; s < kMeanSlices; ++s) acc += partial[(size_t)s * D + p];
-  mu[p] = acc / (float)mean_days(N);
-}
-
 __device__ __forceinline__ double block_sum(double v, double* red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -57,26 +30,6 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   if (threadIdx.x == 0)
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
   return s;
-}
-
-// One block per day: centred FP32 copy (row pitch Dp, zero padded) and the
-// FP64 squared norm of the centred row.
-__global__ void prep_fp32_kernel(const float* __restrict__ X, int D, int Dp,
-                                 const float* __restrict__ mu, const float* __restrict__ wts,
-                                 float* __restrict__ Xc, double* __restrict__ norms) {
-  __shared__ double red[32];
-  const int a = blockIdx.x;
-  const float* x = X + (size_t)a * D;
-  float* y = Xc + (size_t)a * Dp;
-  double acc = 0.0;
-  for (int p = threadIdx.x; p < Dp; p += blockDim.x) {
-    float v = p < D ? x[p] - mu[p] : 0.f;
-    if (wts && p < D) v *= sqrtf(wts[p]);  // grid-point weight w_p enters as sqrt(w_p)
-    y[p] = v;
-    acc = fma((double)v, (double)v, acc);
-  }
-  const double s = block_sum(acc, red);
-  if (threadIdx.x == 0) norms[a] = s;
 }
 
 // Index of the series whose [base, base + count) range of stacked rows holds r.
@@ -91,7 +44,31 @@ __device__ __forceinline__ int find_series(const SeriesInfo* sr, int ns, int r, 
   return lo;
 }
 
-// Column sums of every series' centring days over fixed slices (grid.z = series).
+// One block per stacked day: centred FP32 copy (row pitch Dp, zero padded) and the
+// FP64 squared norm of the centred row.
+__global__ void prep_fp32_series_kernel(const __grid_constant__ SeriesTable st, int D, int Dp,
+                                        const float* __restrict__ mu,
+                                        const float* __restrict__ wts, float* __restrict__ Xc,
+                                        double* __restrict__ norms) {
+  __shared__ double red[32];
+  const int r = blockIdx.x;
+  const int b = find_series(st.s, st.n, r, false);
+  const float* x = st.s[b].X + (size_t)(r - st.s[b].row_base) * D;
+  const float* m = mu + (size_t)b * D;
+  float* y = Xc + (size_t)r * Dp;
+  double acc = 0.0;
+  for (int p = threadIdx.x; p < Dp; p += blockDim.x) {
+    float v = p < D ? x[p] - m[p] : 0.f;
+    if (wts && p < D) v *= sqrtf(wts[p]);  // grid-point weight w_p enters as sqrt(w_p)
+    y[p] = v;
+    acc = fma((double)v, (double)v, acc);
+  }
+  const double s = block_sum(acc, red);
+  if (threadIdx.x == 0) norms[r] = s;
+}
+
+// Column sums of every series' centring days over fixed slices (fixed summation order:
+// deterministic; grid.z = series).
 __global__ void col_partial_series_kernel(const __grid_constant__ SeriesTable st, int D,
                                           float* partial) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -105,6 +82,7 @@ __global__ void col_partial_series_kernel(const __grid_constant__ SeriesTable st
   partial[((size_t)blockIdx.z * kMeanSlices + blockIdx.y) * D + p] = acc;
 }
 
+// FP32 sums suffice for the offset (see above).
 __global__ void col_final_series_kernel(const __grid_constant__ SeriesTable st,
                                         const float* partial, int D, float* mu, int center) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -346,15 +324,6 @@ __global__ void window_series_kernel(const __grid_constant__ SeriesTable st, int
   double s = 0.0;
   for (int m = 0; m < si.L; ++m) s += norms[si.row_base + t + m];
   W[r] = (float)s;
-}
-
-// W_t = sum_{m<L} n_{t+m}: an explicit L-term FP64 sum per trajectory.
-__global__ void window_kernel(const double* __restrict__ norms, int M, int L, float* W) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= M) return;
-  double s = 0.0;
-  for (int m = 0; m < L; ++m) s += norms[t + m];
-  W[t] = (float)s;
 }
 
 // One warp per trajectory row: a P-way merge of the row's sorted partial lists
@@ -851,22 +820,10 @@ cudaError_t launch_window_series(const SeriesTable& sr, int out_rows, const doub
   return cudaGetLastError();
 }
 
-cudaError_t launch_col_mean(const float* X, int N, int D, float* partial, float* mu, bool center,
-                            cudaStream_t st) {
-  dim3 grid((D + 255) / 256, kMeanSlices);
-  if (center) col_partial_kernel<<<grid, 256, 0, st>>>(X, N, D, partial);
-  col_final_kernel<<<(D + 255) / 256, 256, 0, st>>>(partial, N, D, mu, center ? 1 : 0);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_prep_fp32(const float* X, int N, int D, int Dp, const float* mu,
-                             const float* wts, float* Xc, double* norms, cudaStream_t st) {
-  prep_fp32_kernel<<<N, 256, 0, st>>>(X, D, Dp, mu, wts, Xc, norms);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_window(const double* norms, int M, int L, float* W, cudaStream_t st) {
-  window_kernel<<<(M + 255) / 256, 256, 0, st>>>(norms, M, L, W);
+cudaError_t launch_prep_fp32_series(const SeriesTable& sr, int rows, int D, int Dp,
+                                    const float* mu, const float* wts, float* Xc, double* norms,
+                                    cudaStream_t st) {
+  prep_fp32_series_kernel<<<rows, 256, 0, st>>>(sr, D, Dp, mu, wts, Xc, norms);
   return cudaGetLastError();
 }
 

@@ -6,7 +6,8 @@
 // handle whose workspace grows with cudaMalloc; this entry point needs neither.
 // Its scratch is one file-scope __device__ array of kStaticScratchBytes that every
 // GPU loading the library keeps until the process exits. It runs the FP32
-// CUDA-core path with the same kernels and work split as the handle-based call.
+// CUDA-core path on both triangles (the work lists of the handle-based call's upper
+// triangle do not fit the documented scratch); the distances are the same bit for bit.
 //
 // In host code the array's name is only a host-side stand-in, never a device
 // address. Its device address is looked up with cudaGetSymbolAddress (with the
@@ -106,8 +107,7 @@ extern "C" traknn_status traknn_knn_scores_static(const float* X, int64_t N, int
   }
   if (major != 10 || minor != 3) return TRAKNN_ERR_UNSUPPORTED_DEVICE;
 
-  // work split and scratch layout: those of the handle-based FP32 call with
-  // automatic column chunks, plus the status word after the layout
+  // work split and scratch layout, plus the status word after the layout
   const int M = (int)(N - L + 1);
   const Schedule s = make_schedule(M, L, k, exclusion, sms, 0);
   const Fp32Layout lay = make_layout(N, D, s);
@@ -135,13 +135,23 @@ extern "C" traknn_status traknn_knn_scores_static(const float* X, int64_t N, int
   double* norms = reinterpret_cast<double*>(base + lay.norms);
   float* Xc = reinterpret_cast<float*>(base + lay.ops);
 
+  thread_local SeriesTable sr;  // one series (large: kept off the stack)
+  sr.n = 1;
+  SeriesInfo& si = sr.s[0];
+  si = SeriesInfo{};
+  si.N = (int)N;
+  si.M = M;
+  si.L = L;
+  si.X = X;
+
   // the status word is the only scratch that must start at zero; every other
   // byte a kernel reads is written earlier in this same call
   if (cudaMemsetAsync(a.err, 0, sizeof(int), cs) != cudaSuccess ||
-      launch_col_mean(X, (int)N, (int)D, partial, mu, true, cs) != cudaSuccess ||
-      launch_prep_fp32(X, (int)N, (int)D, lay.Dp, mu, nullptr, Xc, norms, cs) != cudaSuccess ||
-      launch_window(norms, M, L, W, cs) != cudaSuccess ||
-      launch_fused_fp32(Xc, a, sms, cs) != cudaSuccess ||
+      launch_col_mean_series(sr, (int)D, partial, mu, true, cs) != cudaSuccess ||
+      launch_prep_fp32_series(sr, (int)N, (int)D, lay.Dp, mu, nullptr, Xc, norms, cs) !=
+          cudaSuccess ||
+      launch_window_series(sr, M, norms, W, cs) != cudaSuccess ||
+      launch_fused_fp32_static(Xc, a, sms, cs) != cudaSuccess ||
       launch_merge(a, nbr_idx, nbr_dist, score, cs) != cudaSuccess) {
     cudaGetLastError();
     return TRAKNN_ERR_CUDA;

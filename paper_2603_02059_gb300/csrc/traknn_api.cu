@@ -50,6 +50,8 @@ struct TcPlan {
   std::vector<int> pstrip, pu, pb;
   int egroups = 1;  // epilogue groups of the fused kernel; each writes its own row lists
   int mask_words = 1;  // 32-bit words per row of the non-empty column-list masks
+  int sym = 1;         // upper triangle with column lists, or both triangles
+  bool band = true;    // the band units run (see prepare_tc)
 };
 
 constexpr size_t kMaxGraphs = 16;  // captured launch sequences kept per handle
@@ -71,9 +73,7 @@ struct traknn_ctx {
   int wait_limit_ms = 2000;
   int debug_withhold = 0;
   // library-owned buffers, grown on demand
-  void* ws = nullptr;  // FP32 path
-  size_t ws_bytes = 0;
-  void* tcws = nullptr;  // tensor-core path
+  void* tcws = nullptr;  // forward passes
   size_t tcws_bytes = 0;
   void* io = nullptr;  // device staging for the host-buffer entry point
   size_t io_bytes = 0;
@@ -163,7 +163,7 @@ static_assert(sizeof(WorkUnit) == 32, "work unit layout");
 inline int list_pitch(int kmax) { return (kmax + 3) / 4 * 4; }
 
 // Tensor-core work list of a batch. For each series: strips of 128 - (L-1) output
-// rows; units of `tiles` Gram tiles (tiles * kTileCols - (L-1) output columns: the
+// rows; units of `tiles` Gram tiles (tiles * tile_cols - (L-1) output columns: the
 // epilogue carries the last L-1 Gram columns of a tile into the next); with the
 // symmetric split only columns from each strip's own block on. Units
 // are ordered per series in groups of strips that run side by side (sharing A and
@@ -177,7 +177,8 @@ inline int list_pitch(int kmax) { return (kmax + 3) / 4 * 4; }
 // (smallest L, most trajectories) defines the units' column ranges.
 void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, int tiles,
                 int group_opt, bool shared, int part_lo, int part_hi,
-                const std::vector<int>& pstrip, int egroups, int band_tiles, TcPlan& p) {
+                const std::vector<int>& pstrip, int egroups, int band_tiles, TcPlan& p,
+                int tile_cols = kTileCols) {
   p.units.clear();
   p.col_off.clear();
   p.slot_lo.clear();
@@ -201,10 +202,10 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
     const int M = N - L + 1;
     const int Lg = shared ? Lshare : L;  // geometry: strip height and tile step
     const int R = kTileRows - (Lg - 1);
-    const int step = kTileCols - (Lg - 1);
+    const int step = tile_cols - (Lg - 1);
     const int strips = (M + R - 1) / R;
     p.mask_words = std::max(p.mask_words, (strips + 31) / 32);
-    const int cols = shared ? step : cols_opt > 0 ? cols_opt : tiles * kTileCols - (Lg - 1);
+    const int cols = shared ? step : cols_opt > 0 ? cols_opt : tiles * tile_cols - (Lg - 1);
     // row-side list slots per trajectory row: one per column range and epilogue group
     const int slots = (M + cols - 1) / cols * egroups;
     SeriesInfo& si = p.table.s[b];
@@ -281,6 +282,7 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
     p.Lmax = std::max(p.Lmax, L);
   }
   p.pstrip = pstrip;
+  p.sym = sym;
   p.egroups = egroups;
   p.pu.assign(1, 0);
   for (int q = 0; q < K; ++q) {
@@ -308,7 +310,7 @@ traknn_status check_handle(traknn_handle h) {
 
 std::vector<int64_t> shape_key(const HostSeries* sd, int B, int64_t D, const traknn_ctx* h) {
   std::vector<int64_t> key = {D, h->sym, h->unit_cols, (int64_t)h->precision, h->center, B,
-                              h->seg_k, h->group_strips, h->l2_keep_a};
+                              h->seg_k, h->group_strips, h->l2_keep_a, h->col_chunks};
   for (int b = 0; b < B; ++b) {
     key.push_back(sd[b].N);
     key.push_back(sd[b].L);
@@ -325,7 +327,7 @@ struct TcBuffers {
   double* norms;
   float* cval;
   float* W;
-  void* hi;
+  void* hi;  // FP32 path: the FP32 operand copy
   void* lo;
   int2* part;
   int* part_n;
@@ -340,7 +342,7 @@ struct TcBuffers {
   size_t total;
 };
 
-TcBuffers tc_layout(const TcPlan& p, int64_t D, int num_ctas, char* base) {
+TcBuffers tc_layout(const TcPlan& p, int64_t D, bool fp32, int num_ctas, char* base) {
   TcBuffers b;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -349,7 +351,7 @@ TcBuffers tc_layout(const TcPlan& p, int64_t D, int num_ctas, char* base) {
     off += bytes;
     return base + o;
   };
-  b.Dp = tc_groups((int)D * p.emb) * 64;
+  b.Dp = fp32 ? (int)((D + 31) / 32 * 32) : tc_groups((int)D * p.emb) * 64;
   const int B = p.table.n;
   const size_t ks = (size_t)list_pitch(p.kmax);
   b.partial = reinterpret_cast<float*>(take((size_t)B * kMeanSlices * D * sizeof(float)));
@@ -357,8 +359,8 @@ TcBuffers tc_layout(const TcPlan& p, int64_t D, int num_ctas, char* base) {
   b.norms = reinterpret_cast<double*>(take((size_t)p.rows * sizeof(double)));
   b.cval = reinterpret_cast<float*>(take((size_t)p.rows * sizeof(float)));
   b.W = reinterpret_cast<float*>(take((size_t)p.out_rows * sizeof(float)));
-  b.hi = take((size_t)p.rows * b.Dp * 2);
-  b.lo = take((size_t)p.rows * b.Dp * 2);
+  b.hi = take((size_t)p.rows * b.Dp * (fp32 ? 4 : 2));
+  b.lo = take(fp32 ? 0 : (size_t)p.rows * b.Dp * 2);
   b.part = reinterpret_cast<int2*>(
       take((size_t)p.part_lists * list_cap((int)ks, p.part_lists) * sizeof(int2)));
   b.part_n = reinterpret_cast<int*>(take((size_t)p.part_lists * sizeof(int)));
@@ -371,7 +373,7 @@ TcBuffers tc_layout(const TcPlan& p, int64_t D, int num_ctas, char* base) {
   b.col_mask = reinterpret_cast<unsigned int*>(
       take((size_t)p.out_rows * p.mask_words * sizeof(unsigned int)));
   b.counter = reinterpret_cast<int*>(take(256));
-  b.scratch = reinterpret_cast<float*>(take(tc_scratch_bytes(num_ctas)));
+  b.scratch = reinterpret_cast<float*>(take(fp32 ? 0 : tc_scratch_bytes(num_ctas)));
   b.pscore = reinterpret_cast<float*>(take((size_t)p.out_rows * sizeof(float)));
   b.total = off;
   return b;
@@ -406,20 +408,46 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   }
   const int Dk = tc_groups((int)D * emb) * 64;
   const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2304 : 3584) * (shared ? B : 1);
+  const bool fp32 = h->precision == TRAKNN_PREC_FP32;  // (its kernel has two groups)
   const int egroups =
-      (h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k && (Lmax == 1 || Dk <= line)) ? 2 : 1;
+      fp32 || (h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k && (Lmax == 1 || Dk <= line))
+          ? 2
+          : 1;
   key.push_back(egroups);
   // Band pre-pass width: two tiles per strip when the contraction dominates a tile's
   // cost; with short operand rows (small grids) a tile's contraction is cheap and the
   // epilogue decides, and eight tiles give bounds tight enough to save more list
   // inserts in the main pass than the band costs (D = 32, L = 5: 1.91 -> 1.69 ms; at
   // D = 3,726 four tiles already cost 6 %)
-  const int band_tiles = Dk <= 768 ? 8 : 2;
+  // FP32: a band column costs as much as a main one; 1 / 2 / 8 tiles: D = 32, N = 27,394
+  // 2,023 / 1,938 / 1,996 us, N = 4,000 190 / 181 / 233; D = 512, N = 1,826 310 / 410 / 983;
+  // D = 3,726, N = 10,957 11.2 / 12.0 / 16.5 ms
+  const int band_tiles = fp32 ? (D <= 64 ? 2 : 1) : Dk <= 768 ? 8 : 2;
   key.push_back(band_tiles);
   TcPlan& p = h->plan;
   if (p.key != key) {
-    build_plan(sd, B, D, h->sym, h->unit_cols, tiles, group, shared, part_lo, part_hi, pstrip,
-               egroups, band_tiles, p);
+    // the column chunks of the FP32 option: that many units per strip
+    int cols = h->unit_cols, tile_cols = kTileCols;
+    p.band = true;
+    if (fp32) {
+      int64_t M = 1, half_tiles = 0;
+      const int Rmin = kTileRows - (Lmax - 1);
+      for (int b = 0; b < (shared ? 1 : B); ++b) {
+        const int64_t Mb = sd[b].N - sd[b].L + 1;
+        M = std::max(M, Mb);
+        for (int64_t t = 0; t < Mb; t += Rmin) half_tiles += (Mb - t + Rmin - 1) / Rmin;
+      }
+      cols = h->col_chunks > 0 ? (int)((M + h->col_chunks - 1) / h->col_chunks) : 0;
+      // A short FP32 call is as long as its units: half tiles (128 x 128) while they do not
+      // go round the SMs twice, and no band before them where they run all at once and a
+      // half tile's products (128 cycles per grid point) outlast the scan of an unbounded
+      // one (N = 300, D = 16 92 us with it, 137 without; N = 1,500, D = 5,000 about 2 x 0.6
+      // ms with it).
+      if (half_tiles <= 2 * h->sm_count) tile_cols = kTileCols / 2;
+      p.band = half_tiles > h->sm_count || D <= 256;
+    }
+    build_plan(sd, B, D, fp32 ? 1 : h->sym, cols, tile_cols < kTileCols ? 1 : tiles, group,
+               shared, part_lo, part_hi, pstrip, egroups, band_tiles, p, tile_cols);
     p.key = key;
     p.emb = emb;
     p.part_lo = part_lo;
@@ -444,9 +472,9 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     p.table.s[b].dist = sd[b].dist;
     p.table.s[b].score = sd[b].score;
   }
-  const TcBuffers probe = tc_layout(p, D, h->sm_count, nullptr);
+  const TcBuffers probe = tc_layout(p, D, h->precision == TRAKNN_PREC_FP32, h->sm_count, nullptr);
   TRY_ST(ensure_buffer(h, &h->tcws, &h->tcws_bytes, probe.total));
-  *out = tc_layout(p, D, h->sm_count, static_cast<char*>(h->tcws));
+  *out = tc_layout(p, D, h->precision == TRAKNN_PREC_FP32, h->sm_count, static_cast<char*>(h->tcws));
   for (int b = 0; b < B; ++b)  // partial lists: their scores go to the workspace
     if (!p.table.s[b].score) p.table.s[b].score = out->pscore + p.table.s[b].out_base;
   return TRAKNN_OK;
@@ -474,16 +502,14 @@ float band_error_margin(int Dp) {
   return (float)(2.0 * u + u * u + 2.1 * Dp * std::ldexp(1.0, -23) + std::ldexp(1.0, -19));
 }
 
-// The launch sequence of one tensor-core call (also what a graph captures).
-traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
-                         cudaStream_t s, bool record_events) {
+// Kernel arguments of a call on the handle's plan (the whole work list).
+void fused_args(const traknn_ctx* h, const TcBuffers& b, TcArgs* pa, TcWork* pw) {
   const TcPlan& p = h->plan;
-  const SeriesTable& sr = p.table;
   const size_t ub = align_up(p.units.size() * sizeof(WorkUnit), 256);
   const size_t cb = align_up(p.col_off.size() * sizeof(long long), 256);
-  char* pd = static_cast<char*>(h->plan_dev);
+  const char* pd = static_cast<const char*>(h->plan_dev);
 
-  TcArgs a;
+  TcArgs& a = *pa;
   a.Dp = b.Dp;
   a.rows = p.rows;
   a.out_rows = p.out_rows;
@@ -494,6 +520,8 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
   a.part_n = b.part_n;
   a.cap = list_cap(list_pitch(p.kmax), p.part_lists);
   a.shared_min = b.shared_min;
+  // where the contraction sets the pace a refresh after every tile is hidden behind it;
+  // D = 32, 75 years: every 2 / 4 / 8 / 16 tiles 1,045 / 989 / 987 / 1,008 us
   a.bound_tiles = b.Dp > 768 ? 1 : 4;
   a.err = h->err;
   a.wait_limit_ns = (long long)h->wait_limit_ms * 1000000LL;
@@ -507,13 +535,13 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
   a.corr_neg = 0;
   a.band_margin = 0.f;
 
-  TcWork w;
+  TcWork& w = *pw;
   w.units = reinterpret_cast<const WorkUnit*>(pd);
   w.nunits = p.nunits;
   w.kstride = list_pitch(p.kmax);
   w.col_off = reinterpret_cast<const long long*>(pd + ub);
   w.slot_lo = reinterpret_cast<const int*>(pd + ub + cb);
-  w.sym = h->sym;
+  w.sym = p.sym;
   w.col_rec = b.col_rec;
   w.col_ints = p.col_lists * col_pitch(w.kstride);
   w.col_mask = b.col_mask;
@@ -525,45 +553,78 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
   w.stats = h->stats ? h->stats_dev : nullptr;
   w.part_lo = p.part_lo;
   w.part_hi = p.part_hi;
+}
 
-  const bool split = h->precision == TRAKNN_PREC_SPLIT_BF16;
-  TRY_CUDA(launch_col_mean_series(sr, (int)D, b.partial, b.mu, h->center != 0, s));
-  TRY_CUDA(launch_prep_split_series(sr, p.rows, (int)D, p.emb, b.Dp / 64, split, b.mu,
-                                    h->weights,
-                                    b.hi, b.lo,
-                                    b.norms, b.cval, s));
-  TRY_CUDA(launch_window_series(sr, p.out_rows, b.norms, b.W, s));
+// One fused launch: `nu` units from unit u0, unit counter `ctr`; `band`: the pre-pass that
+// only seeds bounds.
+traknn_status launch_units(traknn_ctx* h, const TcBuffers& b, const TcArgs& a, const TcWork& w,
+                           int u0, int nu, int ctr, bool band, cudaStream_t s) {
+  if (nu <= 0) return TRAKNN_OK;
+  TcWork x = w;
+  x.units = w.units + u0;
+  x.nunits = nu;
+  x.counter = b.counter + ctr;
+  TcArgs ax = a;
+  bool split = h->precision == TRAKNN_PREC_SPLIT_BF16;
+  if (band) {
+    x.sym = 0;
+    x.write_lists = 0;
+    if (band_single_product(h, h->plan, b.Dp)) {
+      ax.corr_neg = 1;
+      ax.band_margin = band_error_margin(b.Dp);
+      split = false;
+    }
+  }
+  ++h->launches;
+  const SeriesTable& sr = h->plan.table;
+  if (h->precision == TRAKNN_PREC_FP32)
+    TRY_CUDA(launch_fused_fp32(static_cast<const float*>(b.hi), ax, x, sr, h->sm_count, s));
+  else
+    TRY_CUDA(launch_fused_tc(b.hi, b.lo, split, ax, x, sr, h->sm_count, s));
+  return TRAKNN_OK;
+}
+
+// Everything a main pass accumulates into: bounds and shared minima (0x7F bytes: a large
+// finite value), column-list masks, `counters` unit counters.
+traknn_status clear_lists(const TcPlan& p, const TcBuffers& b, int counters, cudaStream_t s) {
   TRY_CUDA(cudaMemsetAsync(
       b.thr, 0x7F, (size_t)p.out_rows * (1 + min_slots(p.kmax)) * sizeof(unsigned int), s));
   TRY_CUDA(cudaMemsetAsync(b.col_mask, 0,
                            (size_t)p.out_rows * p.mask_words * sizeof(unsigned int), s));
-  TRY_CUDA(cudaMemsetAsync(b.counter, 0, 2 * sizeof(int), s));
+  TRY_CUDA(cudaMemsetAsync(b.counter, 0, counters * sizeof(int), s));
+  return TRAKNN_OK;
+}
+
+// The launch sequence of one call (also what a graph captures).
+traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
+                         cudaStream_t s, bool record_events) {
+  const TcPlan& p = h->plan;
+  const SeriesTable& sr = p.table;
+  TcArgs a;
+  TcWork w;
+  fused_args(h, b, &a, &w);
+  TRY_CUDA(launch_col_mean_series(sr, (int)D, b.partial, b.mu, h->center != 0, s));
+  if (h->precision == TRAKNN_PREC_FP32)
+    TRY_CUDA(launch_prep_fp32_series(sr, p.rows, (int)D, b.Dp, b.mu, h->weights,
+                                     static_cast<float*>(b.hi), b.norms, s));
+  else
+    TRY_CUDA(launch_prep_split_series(sr, p.rows, (int)D, p.emb, b.Dp / 64,
+                                      h->precision == TRAKNN_PREC_SPLIT_BF16, b.mu, h->weights,
+                                      b.hi, b.lo, b.norms, b.cval, s));
+  TRY_CUDA(launch_window_series(sr, p.out_rows, b.norms, b.W, s));
+  TRY_ST(clear_lists(p, b, 2, s));
   const int slot = h->ev_head;
   if (record_events) TRY_CUDA(cudaEventRecord(h->ev_start[slot], s));
-  if (p.nband > 0) {
-    // threshold pre-pass over the band units (stored after the main units)
-    TcWork bw = w;
-    bw.units = w.units + p.nunits;
-    bw.nunits = p.nband;
-    bw.sym = 0;
-    bw.write_lists = 0;
-    bw.counter = w.counter + 1;
-    TcArgs ab = a;
-    const bool one = band_single_product(h, p, b.Dp);
-    if (one) {
-      ab.corr_neg = 1;
-      ab.band_margin = band_error_margin(b.Dp);
-    }
-    TRY_CUDA(launch_fused_tc(b.hi, b.lo, one ? false : split, ab, bw, sr, h->sm_count, s));
-  }
-  TRY_CUDA(launch_fused_tc(b.hi, b.lo, split, a, w, sr, h->sm_count, s));
+  // threshold pre-pass over the band units (stored after the main units), then the rest
+  if (p.band) TRY_ST(launch_units(h, b, a, w, p.nunits, p.nband, 1, true, s));
+  TRY_ST(launch_units(h, b, a, w, 0, p.nunits, 0, false, s));
   if (record_events) {
     TRY_CUDA(cudaEventRecord(h->ev_stop[slot], s));
     h->ev_head = (h->ev_head + 1) % traknn_ctx::kRing;
     h->ev_count = std::min(h->ev_count + 1, traknn_ctx::kRing);
   }
   TRY_CUDA(launch_merge_tc(a, w, sr, s));
-  h->launches += (h->center ? 2 : 1) + 2 + (p.nband > 0 ? 1 : 0) + 2;
+  h->launches += (h->center ? 2 : 1) + 3;
   return TRAKNN_OK;
 }
 
@@ -608,69 +669,10 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
   const SeriesInfo& si = sr.s[0];
   const int R = kTileRows - (si.L - 1);
   const int K = (int)p.pstrip.size() - 1;
-  const size_t ub = align_up(p.units.size() * sizeof(WorkUnit), 256);
-  const size_t cb = align_up(p.col_off.size() * sizeof(long long), 256);
-  char* pd = static_cast<char*>(h->plan_dev);
   TcArgs a;
-  a.Dp = b.Dp;
-  a.rows = p.rows;
-  a.out_rows = p.out_rows;
-  a.Lmax = p.Lmax;
-  a.kmax = p.kmax;
-  a.W = b.W;
-  a.part = b.part;
-  a.part_n = b.part_n;
-  a.cap = list_cap(list_pitch(p.kmax), p.part_lists);
-  a.shared_min = b.shared_min;
-  a.bound_tiles = b.Dp > 768 ? 1 : 4;
-  a.err = h->err;
-  a.wait_limit_ns = (long long)h->wait_limit_ms * 1000000LL;
-  a.debug_withhold = h->debug_withhold;
-  a.seg_k = h->seg_k;
-  a.scratch = b.scratch;
-  a.groups = b.Dp / 64;
-  a.cval = b.cval;
-  a.l2_keep_a = h->l2_keep_a;
-  a.egroups = p.egroups;
-  a.corr_neg = 0;
-  a.band_margin = 0.f;
   TcWork w;
-  w.units = reinterpret_cast<const WorkUnit*>(pd);
-  w.kstride = list_pitch(p.kmax);
-  w.col_off = reinterpret_cast<const long long*>(pd + ub);
-  w.slot_lo = reinterpret_cast<const int*>(pd + ub + cb);
-  w.sym = h->sym;
-  w.col_rec = b.col_rec;
-  w.col_ints = p.col_lists * col_pitch(w.kstride);
-  w.col_mask = b.col_mask;
-  w.mask_words = p.mask_words;
-  w.part_lists = p.part_lists;
-  w.thr = b.thr;
-  w.write_lists = 1;
-  w.stats = h->stats ? h->stats_dev : nullptr;
-  w.part_lo = 0;
-  w.part_hi = INT_MAX;
+  fused_args(h, b, &a, &w);
   const bool split = h->precision == TRAKNN_PREC_SPLIT_BF16;
-  auto fused = [&](int u0, int nu, int ctr, bool band) -> cudaError_t {
-    if (nu <= 0) return cudaSuccess;
-    TcWork x = w;
-    x.units = w.units + u0;
-    x.nunits = nu;
-    x.counter = b.counter + ctr;
-    TcArgs ax = a;
-    bool sp = split;
-    if (band) {
-      x.sym = 0;
-      x.write_lists = 0;
-      if (band_single_product(h, p, b.Dp)) {  // see band_error_margin
-        ax.corr_neg = 1;
-        ax.band_margin = band_error_margin(b.Dp);
-        sp = false;
-      }
-    }
-    ++h->launches;
-    return launch_fused_tc(b.hi, b.lo, sp, ax, x, sr, h->sm_count, s);
-  };
   for (int q = 0; q < K; ++q) {
     const int lo = p.pstrip[q + 1] * R;                      // first day (and row) of phase q
     const int hi = q == 0 ? p.rows : p.pstrip[q] * R;        // rows prepared by phase q
@@ -678,11 +680,7 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
     TRY_CUDA(cudaStreamWaitEvent(s, in[q], 0));
     if (q == 0) {
       TRY_CUDA(launch_col_mean_series(sr, (int)D, b.partial, b.mu, h->center != 0, s));
-      TRY_CUDA(cudaMemsetAsync(
-      b.thr, 0x7F, (size_t)p.out_rows * (1 + min_slots(p.kmax)) * sizeof(unsigned int), s));
-      TRY_CUDA(cudaMemsetAsync(b.col_mask, 0,
-                               (size_t)p.out_rows * p.mask_words * sizeof(unsigned int), s));
-      TRY_CUDA(cudaMemsetAsync(b.counter, 0, 2 * K * sizeof(int), s));
+      TRY_ST(clear_lists(p, b, 2 * K, s));
       h->launches += h->center ? 2 : 1;
     }
     // window sums of rows [lo, ohi) read day norms up to ohi + L - 2: prepared now or
@@ -691,11 +689,9 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
                                       b.hi, b.lo, b.norms, b.cval, s, lo));
     TRY_CUDA(launch_window_series(sr, ohi, b.norms, b.W, s, lo));
     h->launches += (hi > lo ? 1 : 0) + (ohi > lo ? 1 : 0);
-    TRY_CUDA(fused(p.pb[q], p.pb[q + 1] - p.pb[q], 2 * q + 1, true));
-    TRY_CUDA(fused(p.pu[q], p.pu[q + 1] - p.pu[q], 2 * q, false));
+    TRY_ST(launch_units(h, b, a, w, p.pb[q], p.pb[q + 1] - p.pb[q], 2 * q + 1, true, s));
+    TRY_ST(launch_units(h, b, a, w, p.pu[q], p.pu[q + 1] - p.pu[q], 2 * q, false, s));
   }
-  w.nunits = p.nunits;
-  w.counter = b.counter;
   TRY_CUDA(launch_merge_tc(a, w, sr, s));
   h->launches += 1;
   return TRAKNN_OK;
@@ -823,11 +819,16 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
 traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
                      bool graph, bool shared = false, int emb = 1, int part_lo = 0,
                      int part_hi = INT_MAX) {
-  if (!tc_available()) return TRAKNN_ERR_UNSUPPORTED;
+  if (h->precision != TRAKNN_PREC_FP32 && !tc_available()) return TRAKNN_ERR_UNSUPPORTED;
   int tiles = 8, group = 0;
   const bool whole = part_lo == 0 && part_hi == INT_MAX;
   if (!shared && emb == 1 && whole) TRY_ST(pick_shape(h, sd, B, D, s, &tiles, &group));
   if (!h->autotune && !shared) default_shape(h, sd, B, D, emb, part_lo, part_hi, &tiles, &group);
+  // FP32: a tile's contraction takes so long that the units must be short for the CTAs to
+  // end together, except at few grid points. 1 / 2 / 4 / 8 tiles: D = 3,726, N = 27,394 60.5 /
+  // 60.3 / 60.8 / 62.7 ms, N = 10,957 10.8 / 11.2 / 12.0 / 12.8; D = 200, N = 10,957 1,056 /
+  // 1,069 / 1,117 / 1,155 us; D = 32, N = 27,394 2,163 / 2,023 / 1,979 / 1,968
+  if (h->precision == TRAKNN_PREC_FP32 && D > 64) tiles = tiles >= 8 ? 2 : 1;
   TcBuffers buf;
   TRY_ST(prepare_tc(h, sd, B, D, tiles, shared, emb, s, &buf, part_lo, part_hi, {}, group));
   h->last_tiles = tiles;
@@ -848,7 +849,7 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   for (auto& g : h->graphs)
     if (g.key == key) {
       TRY_CUDA(cudaGraphLaunch(g.exec, s));
-      h->launches += (h->center ? 2 : 1) + 2 + (h->plan.nband > 0 ? 1 : 0) + 2;
+      h->launches += (h->center ? 2 : 1) + 4 + (h->plan.band && h->plan.nband > 0 ? 1 : 0);
       return TRAKNN_OK;
     }
   if (!h->cap_stream) TRY_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
@@ -878,7 +879,7 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   }
   h->graphs.push_back(GraphEntry{key, exec});
   TRY_CUDA(cudaGraphLaunch(exec, s));
-  h->launches += (h->center ? 2 : 1) + 2 + (h->plan.nband > 0 ? 1 : 0) + 2;
+  h->launches += (h->center ? 2 : 1) + 4 + (h->plan.band && h->plan.nband > 0 ? 1 : 0);
   return TRAKNN_OK;
 }
 
@@ -949,7 +950,6 @@ traknn_status traknn_destroy(traknn_handle h) {
   if (h->ev_io_free) cudaEventDestroy(h->ev_io_free);
   for (cudaEvent_t ev : h->ev_in)
     if (ev) cudaEventDestroy(ev);
-  if (h->ws) cudaFree(h->ws);
   if (h->tcws) cudaFree(h->tcws);
   if (h->io) cudaFree(h->io);
   if (h->adj) cudaFree(h->adj);
@@ -1046,52 +1046,14 @@ traknn_status traknn_knn_scores(traknn_handle h, const float* X, int64_t N, int6
   TRY_ST(traknn_check_problem(N, D, L, k, e));
   if (h->weights && h->weights_D != D) return TRAKNN_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (h->precision != TRAKNN_PREC_FP32) {
-    if (use_embedding(h, D, L)) {
-      // trajectory-embedded operands: one row per trajectory (L days, contiguous in
-      // X), whose Gram is the window sum itself; the kernels see M rows and L = 1
-      const HostSeries sd{X, N - L + 1, 1, k, e, nbr_idx, nbr_dist, score};
-      return run_tc(h, &sd, 1, D, s, false, false, L);
-    }
-    const HostSeries sd{X, N, L, k, e, nbr_idx, nbr_dist, score};
-    return run_tc(h, &sd, 1, D, s, false);
+  if (h->precision != TRAKNN_PREC_FP32 && use_embedding(h, D, L)) {
+    // trajectory-embedded operands: one row per trajectory (L days, contiguous in
+    // X), whose Gram is the window sum itself; the kernels see M rows and L = 1
+    const HostSeries sd{X, N - L + 1, 1, k, e, nbr_idx, nbr_dist, score};
+    return run_tc(h, &sd, 1, D, s, false, false, L);
   }
-
-  // plain FP32 CUDA-core path
-  const int M = (int)(N - L + 1);
-  const Schedule sch = make_schedule(M, L, k, e, h->sm_count, h->col_chunks);
-  const Fp32Layout lay = make_layout(N, D, sch);
-  TRY_ST(ensure_buffer(h, &h->ws, &h->ws_bytes, lay.total));
-  char* ws = static_cast<char*>(h->ws);
-  float* partial = reinterpret_cast<float*>(ws + lay.partial);
-  float* mu = reinterpret_cast<float*>(ws + lay.mu);
-  double* norms = reinterpret_cast<double*>(ws + lay.norms);
-  float* W = reinterpret_cast<float*>(ws + lay.W);
-  float* Xc = reinterpret_cast<float*>(ws + lay.ops);
-  FusedArgs fa;
-  fa.sch = sch;
-  fa.N = (int)N;
-  fa.Dp = lay.Dp;
-  fa.W = W;
-  fa.part_d = reinterpret_cast<float*>(ws + lay.pd);
-  fa.part_i = reinterpret_cast<int32_t*>(ws + lay.pi);
-  fa.err = h->err;
-  fa.wait_limit_ns = (long long)h->wait_limit_ms * 1000000LL;
-  fa.debug_withhold = h->debug_withhold;
-  TRY_CUDA(launch_col_mean(X, (int)N, (int)D, partial, mu, h->center != 0, s));
-  TRY_CUDA(launch_prep_fp32(X, (int)N, (int)D, lay.Dp, mu, h->weights, Xc, norms, s));
-  TRY_CUDA(launch_window(norms, M, L, W, s));
-  const int slot = h->ev_head;
-  if (h->profile) TRY_CUDA(cudaEventRecord(h->ev_start[slot], s));
-  TRY_CUDA(launch_fused_fp32(Xc, fa, h->sm_count, s));
-  if (h->profile) {
-    TRY_CUDA(cudaEventRecord(h->ev_stop[slot], s));
-    h->ev_head = (h->ev_head + 1) % traknn_ctx::kRing;
-    h->ev_count = std::min(h->ev_count + 1, traknn_ctx::kRing);
-  }
-  TRY_CUDA(launch_merge(fa, nbr_idx, nbr_dist, score, s));
-  h->launches += (h->center ? 2 : 1) + 4;
-  return TRAKNN_OK;
+  const HostSeries sd{X, N, L, k, e, nbr_idx, nbr_dist, score};
+  return run_tc(h, &sd, 1, D, s, false);
 }
 
 traknn_status traknn_knn_scores_batched(traknn_handle h, const traknn_series* series, int B,
@@ -1105,12 +1067,6 @@ traknn_status traknn_knn_scores_batched(traknn_handle h, const traknn_series* se
   TRY_ST(validate_series(sd.data(), B, D));
   if (h->weights && h->weights_D != D) return TRAKNN_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (h->precision == TRAKNN_PREC_FP32) {
-    for (int b = 0; b < B; ++b)
-      TRY_ST(traknn_knn_scores(h, sd[b].X, sd[b].N, D, sd[b].L, sd[b].k, sd[b].e, sd[b].idx,
-                               sd[b].dist, sd[b].score, stream));
-    return TRAKNN_OK;
-  }
   for (int b0 = 0; b0 < B; b0 += kMaxSeries)
     TRY_ST(run_tc(h, sd.data() + b0, std::min(kMaxSeries, B - b0), D, s, true));
   return TRAKNN_OK;
@@ -1130,12 +1086,6 @@ traknn_status traknn_knn_scores_multi(traknn_handle h, const traknn_series* sett
   TRY_ST(validate_series(sd.data(), nset, D));
   if (h->weights && h->weights_D != D) return TRAKNN_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (h->precision == TRAKNN_PREC_FP32) {
-    for (int b = 0; b < nset; ++b)
-      TRY_ST(traknn_knn_scores(h, sd[b].X, sd[b].N, D, sd[b].L, sd[b].k, sd[b].e, sd[b].idx,
-                               sd[b].dist, sd[b].score, stream));
-    return TRAKNN_OK;
-  }
   // the shared geometry takes the smallest L (most trajectories) first
   std::stable_sort(sd.begin(), sd.end(),
                    [](const HostSeries& x, const HostSeries& y) { return x.L < y.L; });

@@ -1,4 +1,4 @@
-"""Candidate lists, shared minima and bounds of the tensor-core kernel where they can go
+"""Candidate lists, shared minima and bounds of the symmetric kernels where they can go
 wrong: few-valued integer fields, whose distances tie by the hundred (lists, column records
 and the merge's buffer overflow, and the order among ties decides), every range of k with its
 own number of shared minima, exclusion zones wider than the band, and two epilogue groups
@@ -40,6 +40,26 @@ def test_ties_and_wide_exclusion_equal_the_oracle(tk, prec, N, D, top, L, k, e):
                                      center=False, embed=embed)
         assert np.array_equal(dist.cpu().numpy(), odist.astype(np.float32))
         assert np.array_equal(idx.cpu().numpy(), oidx)
+
+
+@pytest.mark.parametrize("N,D,top,L,k,e", [
+    (700, 3, 1, 1, 1, 0), (700, 4, 2, 1, 20, 0), (1300, 3, 1, 5, 33, 4), (700, 3, 1, 17, 64, 16),
+    (1500, 4, 3, 2, 10, 400), (129, 70, 3, 2, 64, 1), (384, 600, 1, 4, 5, 3)])
+def test_fp32_upper_triangle_equals_the_oracle(tk, N, D, top, L, k, e):
+    """Small integers again (exact in FP32): single, batched and several-settings calls."""
+    import torch
+    X = _integers(N, D, top, seed=N + k)
+    Xd = torch.from_numpy(X).cuda()
+    L2 = max(1, L - 1)
+    ref = [oracle.knn_scores(X, l, k, e)[:2] for l in (L, L2)]
+    got = [(tk.knn_scores(Xd, L, k, e, precision="fp32", center=False), 0)]
+    got += zip(tk.knn_scores_batched([(Xd, L, k, e), (Xd, L2, k, e)], precision="fp32",
+                                     center=False), (0, 1))
+    got += zip(tk.knn_scores_multi(Xd, [(L, k, e), (L2, k, e)], precision="fp32",
+                                   center=False), (0, 1))
+    for (idx, dist, _), b in got:
+        assert np.array_equal(dist.cpu().numpy(), ref[b][1].astype(np.float32))
+        assert np.array_equal(idx.cpu().numpy(), ref[b][0])
 
 
 @pytest.mark.parametrize("N,h,w,L,k,e", [(1500, 20, 32, 5, 20, 4), (2000, 36, 41, 2, 10, 1),
