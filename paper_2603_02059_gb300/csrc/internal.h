@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 namespace traknn {
 
 // Rows of one Gram tile (the tcgen05 accumulator height and the FP32 SIMT tile).
@@ -25,7 +27,7 @@ constexpr int kMaxK = 64;
 constexpr int kErrTimeout = 5;
 // ... and when an input it reads is out of range (TRAKNN_ERR_INVALID_ARG).
 constexpr int kErrInvalidArg = 1;
-// Column-mean partial sums use this many row slices (fixed order => deterministic).
+// The column mean is summed over this many row slices (fixed order => deterministic).
 constexpr int kMeanSlices = 64;
 // Centring: the per-grid-point mean over the last kMeanDays days (all days when there
 // are fewer): days [mean_first(N), N). A host-buffer call copies those days in first.
@@ -105,7 +107,7 @@ inline Schedule make_schedule(int M, int L, int k, int e, int sm_count, int chun
 }
 
 // Byte offsets of the FP32 path's workspace (each piece starts on a 256-byte
-// boundary): column partial sums, mean, FP64 day norms, window sums, the centred
+// boundary): a reserve of kMeanSlices rows (the documented size counts it), mean, FP64 day norms, window sums, the centred
 // FP32 copy (row pitch Dp = D rounded up to 32) and the partial neighbour lists.
 struct Fp32Layout {
   size_t partial, mu, norms, W, ops, pd, pi, total;
@@ -294,9 +296,35 @@ enum : int {
 };
 
 // ----------------------------------------------------------------- launchers
-// wts: optional [D] grid-point weights (the values are scaled by sqrt(w_p)), or null.
+// The kernels of a call follow one another on one stream, each with the attribute of a
+// programmatic dependent launch: a kernel may be set up while the one before it runs out.
+// Each one therefore waits (launch_wait) before it touches global memory: the wait ends
+// when every kernel before it has finished and its writes are visible, and allows its own
+// successor the same (launch_next) at once. One year of 64 grid points (six launches):
+// see launch_chained.
+__device__ __forceinline__ void launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                                  cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+// sw: optional [D] square roots of the grid-point weights (the values are scaled by them).
 cudaError_t launch_prep_fp32_series(const SeriesTable& sr, int rows, int D, int Dp,
-                                    const float* mu, const float* wts, float* Xc, double* norms,
+                                    const float* mu, const float* sw, float* Xc, double* norms,
                                     cudaStream_t st);
 // FP32 CUDA-core path over the work list of the tensor-core path (Xc: the stacked FP32
 // operand copy, pitch a.Dp), and the both-triangles form of traknn_knn_scores_static.
@@ -312,9 +340,11 @@ cudaError_t launch_fused_tc(const void* hi, const void* lo, bool split, const Tc
 // written to each series' output buffers.
 cudaError_t launch_merge_tc(const TcArgs& a, const TcWork& w, const SeriesTable& sr,
                             cudaStream_t st);
-// Series-aware preparation for the tensor-core path (stacked operands).
-cudaError_t launch_col_mean_series(const SeriesTable& sr, int D, float* partial, float* mu,
-                                   bool center, cudaStream_t st);
+// Means of the series' centring days (zeros without `center`), repeated for the emb days of
+// an operand row: mu[series][emb D]; with wts ([D] grid-point weights, or null) also
+// sw[emb D] = sqrt(w_p), likewise repeated.
+cudaError_t launch_col_mean_series(const SeriesTable& sr, int D, int emb, const float* wts,
+                                   float* mu, float* sw, bool center, cudaStream_t st);
 // Operand layout of the tensor-core path: groups = ceil(D / 63) groups of 64 K
 // entries (63 permuted grid points + 1 correction entry); pitch groups * 64.
 inline int tc_groups(int D) { return (D + 62) / 63; }
@@ -342,12 +372,27 @@ inline void split_strips(long long M, int L, int nparts, int part, int* s_lo, in
 // values, contiguous in X); the series table then describes trajectories (N = M, L = 1).
 // Rows [r_lo, rows) of the stacked operands (all rows with r_lo = 0).
 cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int emb, int groups,
-                                     bool correct, const float* mu, const float* wts, void* hi,
+                                     bool correct, const float* mu, const float* sw, void* hi,
                                      void* lo, double* norms, float* cval, cudaStream_t st,
                                      int r_lo = 0);
-// Window sums of the stacked trajectory rows [r_lo, out_rows).
+// What a main pass accumulates into, cleared by the window kernel row by row: bounds and
+// shared minima (0x7F bytes: a large finite value) and column-list masks of its rows, and
+// (with r_lo = 0 or a series' first launch: `counters` > 0) the unit counters.
+struct ClearArgs {
+  unsigned int* thr;         // [rows], then [slots][rows] shared minima
+  unsigned int* shared_min;
+  long long stride;          // rows in all (distance of a row's shared minima)
+  int slots;
+  unsigned int* col_mask;
+  int mask_words;
+  int* counter;
+  int counters;
+};
+// Window sums of the stacked trajectory rows [r_lo, out_rows); clears what `clear` names
+// for those rows (thr null: nothing).
 cudaError_t launch_window_series(const SeriesTable& sr, int out_rows, const double* norms,
-                                 float* W, cudaStream_t st, int r_lo = 0);
+                                 float* W, const ClearArgs& clear, cudaStream_t st,
+                                 int r_lo = 0);
 cudaError_t launch_merge(const FusedArgs& a, int32_t* idx, float* dist, float* score,
                          cudaStream_t st);
 // Exact top-k of the union of nparts sorted candidate lists per row ([nparts][M][k],

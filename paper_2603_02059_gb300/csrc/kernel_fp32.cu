@@ -174,6 +174,8 @@ __global__ void __launch_bounds__(NT, 1)
   if (l < 64) cs.cnt[l] = 0;
   float* drow = sm.D[gid][l];
   unsigned cnt[5] = {0, 0, 0, 0, 0};
+  launch_wait();
+  launch_next();
   for (;;) {
     __syncthreads();  // the last unit's readers are done
     if (tid == 0) {
@@ -385,8 +387,7 @@ cudaError_t launch_sym(const float* Xc, const TcArgs& a, const TcWork& w, const 
       cudaFuncSetAttribute(fused_fp32_kernel<kBand, S>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
   if (err != cudaSuccess) return err;
-  fused_fp32_kernel<kBand, S><<<num_ctas, NT, sizeof(Smem), st>>>(Xc, a, w, sr);
-  return cudaGetLastError();
+  return launch_chained(fused_fp32_kernel<kBand, S>, num_ctas, NT, sizeof(Smem), st, Xc, a, w, sr);
 }
 
 }  // namespace

@@ -188,6 +188,8 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   }
   __syncthreads();
   ptx::tc_fence_after();
+  launch_wait();  // barriers and tensor memory were set up beside the kernel before
+  launch_next();
   const uint32_t tmem_base = *tmem_slot;
   const int nkb = a.Dp / KC;
   const int seg_kb = p.seg_kb;                    // K blocks per accumulation segment
@@ -838,8 +840,8 @@ cudaError_t launch_g(const CUtensorMap& mAh, const CUtensorMap& mAl, const CUten
   cudaError_t err = cudaFuncSetAttribute(fused_tc_kernel<G, kWin, kBand, kLarge>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  fused_tc_kernel<G, kWin, kBand, kLarge><<<num_ctas, kThreadsG(G), smem, st>>>(mAh, mAl, mBh, mBl, p);
-  return cudaGetLastError();
+  return launch_chained(fused_tc_kernel<G, kWin, kBand, kLarge>, num_ctas, kThreadsG(G), smem, st,
+                        mAh, mAl, mBh, mBl, p);
 }
 
 }  // namespace

@@ -9,6 +9,7 @@
 
 #include <climits>
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -48,9 +49,11 @@ __device__ __forceinline__ int find_series(const SeriesInfo* sr, int ns, int r, 
 // FP64 squared norm of the centred row.
 __global__ void prep_fp32_series_kernel(const __grid_constant__ SeriesTable st, int D, int Dp,
                                         const float* __restrict__ mu,
-                                        const float* __restrict__ wts, float* __restrict__ Xc,
+                                        const float* __restrict__ sw, float* __restrict__ Xc,
                                         double* __restrict__ norms) {
   __shared__ double red[32];
+  launch_wait();
+  launch_next();
   const int r = blockIdx.x;
   const int b = find_series(st.s, st.n, r, false);
   const float* x = st.s[b].X + (size_t)(r - st.s[b].row_base) * D;
@@ -59,7 +62,7 @@ __global__ void prep_fp32_series_kernel(const __grid_constant__ SeriesTable st, 
   double acc = 0.0;
   for (int p = threadIdx.x; p < Dp; p += blockDim.x) {
     float v = p < D ? x[p] - m[p] : 0.f;
-    if (wts && p < D) v *= sqrtf(wts[p]);  // grid-point weight w_p enters as sqrt(w_p)
+    if (sw && p < D) v *= sw[p];  // grid-point weight w_p enters as sqrt(w_p)
     y[p] = v;
     acc = fma((double)v, (double)v, acc);
   }
@@ -67,34 +70,75 @@ __global__ void prep_fp32_series_kernel(const __grid_constant__ SeriesTable st, 
   if (threadIdx.x == 0) norms[r] = s;
 }
 
-// Column sums of every series' centring days over fixed slices (fixed summation order:
-// deterministic; grid.z = series).
-__global__ void col_partial_series_kernel(const __grid_constant__ SeriesTable st, int D,
-                                          float* partial) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= D) return;
-  const SeriesInfo& si = st.s[blockIdx.z];
+// Mean of every series' centring days per grid point (grid.y = series, 32 grid points per
+// CTA): a warp sums slices w and w + 32 of the days, then one warp sums the 64 slices in
+// order (fixed summation order: deterministic; FP32 sums suffice for the offset, see above).
+// The mean, and the square roots of the weights, are written once per day of an operand
+// row, so that the preparation needs neither a division nor a square root per value
+// (7,301 x 3,555 weighted: preparation 193 -> 53 us). Bound by the read of the centring
+// days; one launch instead of two saves about 4 us on every call.
+constexpr int kMeanWarps = 32;
+__global__ void __launch_bounds__(32 * kMeanWarps)
+    col_mean_series_kernel(const __grid_constant__ SeriesTable st, int D, int emb,
+                           const float* __restrict__ wts, float* __restrict__ mu,
+                           float* __restrict__ sw, int center) {
+  __shared__ float part[kMeanSlices][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane, b = blockIdx.y;
+  const SeriesInfo& si = st.s[b];
   const int first = mean_first(si.N), ns = mean_days(si.N);
   const int per = (ns + kMeanSlices - 1) / kMeanSlices;
-  const int r0 = blockIdx.y * per, r1 = min(ns, r0 + per);
-  float acc = 0.f;
-  for (int i = r0; i < r1; ++i) acc += si.X[(size_t)(first + i) * D + p];
-  partial[((size_t)blockIdx.z * kMeanSlices + blockIdx.y) * D + p] = acc;
+  launch_wait();
+  launch_next();
+  if (center && p < D) {
+    // both slices together, 16 days of each at a time (32 loads in flight: a grid of one
+    // CTA has nothing else to hide their latency)
+    const int a0 = min(ns, warp * per), a1 = min(ns, a0 + per);
+    const int b0 = min(ns, (warp + kMeanWarps) * per), b1 = min(ns, b0 + per);
+    const float* xa = si.X + (size_t)(first + a0) * D + p;
+    const float* xb = si.X + (size_t)(first + b0) * D + p;
+    float sa = 0.f, sb = 0.f;
+    for (int i = 0; i < per; i += 16) {
+      float va[16], vb[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        va[u] = a0 + i + u < a1 ? __ldg(xa + (size_t)(i + u) * D) : 0.f;
+        vb[u] = b0 + i + u < b1 ? __ldg(xb + (size_t)(i + u) * D) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        if (a0 + i + u < a1) sa += va[u];
+        if (b0 + i + u < b1) sb += vb[u];
+      }
+    }
+    part[warp][lane] = sa;
+    part[warp + kMeanWarps][lane] = sb;
+  }
+  __syncthreads();
+  if (warp != 0 || p >= D) return;
+  float m = 0.f;
+  if (center) {
+    float acc = 0.f;
+    for (int s = 0; s < kMeanSlices; ++s) acc += part[s][lane];
+    m = acc / (float)ns;
+  }
+  for (int e = 0; e < emb; ++e) mu[((size_t)b * emb + e) * D + p] = m;
+  if (wts && b == 0) {
+    const float q = sqrtf(wts[p]);
+    for (int e = 0; e < emb; ++e) sw[(size_t)e * D + p] = q;
+  }
 }
 
-// FP32 sums suffice for the offset (see above).
-__global__ void col_final_series_kernel(const __grid_constant__ SeriesTable st,
-                                        const float* partial, int D, float* mu, int center) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= D) return;
-  const int b = blockIdx.y;
-  if (!center) {
-    mu[(size_t)b * D + p] = 0.f;
-    return;
-  }
-  float acc = 0.f;
-  for (int s = 0; s < kMeanSlices; ++s) acc += partial[((size_t)b * kMeanSlices + s) * D + p];
-  mu[(size_t)b * D + p] = acc / (float)mean_days(st.s[b].N);
+// The correction value bf16(sqrt(n / groups)) of a row with norm n. FP64 instructions run at
+// 1/64 of the FP32 rate here (a division and a square root of them cost a warp about 300
+// cycles of the SM's FP64 pipe), so the FP32 value decides unless it lies within 16 ulp of
+// a BF16 rounding boundary: its error is below 4 ulp.
+__device__ __forceinline__ float correction(double n, int groups) {
+  float v = sqrtf((float)n / (float)groups);
+  const unsigned low = __float_as_uint(v) & 0xFFFFu;
+  if (!(low < 0x8000u - 16u || low > 0x8000u + 16u) || !(v > 1e-18f && v < 1e18f))
+    v = (float)sqrt(n / groups);
+  return __bfloat162float(__float2bfloat16_rn(v));
 }
 
 // One warp per stacked day: the centred row x - mu(series) as two BF16 copies hi + lo
@@ -117,11 +161,11 @@ __global__ void col_final_series_kernel(const __grid_constant__ SeriesTable st,
 // row-major input are the contiguous values X + a*D .. X + (a+emb)*D. The Gram of
 // such rows is the diagonal window sum of Eq. 2 (sum over m of <x_{a+m}, x_{b+m}>),
 // and the norm of a row is the window sum of the day norms.
-template <bool kCorr, bool kEmb>
+template <bool kCorr>
 __global__ void __launch_bounds__(256)
     prep_split_series_kernel(const __grid_constant__ SeriesTable st, int r_lo, int rows, int D,
                              int emb, int groups, const float* __restrict__ mu,
-                             const float* __restrict__ wts, __nv_bfloat16* __restrict__ hi,
+                             const float* __restrict__ sw, __nv_bfloat16* __restrict__ hi,
                              __nv_bfloat16* __restrict__ lo, double* __restrict__ norms,
                              float* __restrict__ cval) {
   // per warp: 32 finished groups of one copy (36-word rows: 16-byte aligned)
@@ -129,6 +173,8 @@ __global__ void __launch_bounds__(256)
   const int r = r_lo + blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
+  launch_wait();
+  launch_next();
   uint32_t* sh = stage[threadIdx.x >> 5];
   const int b = find_series(st.s, st.n, r, false);
   const SeriesInfo& si = st.s[b];
@@ -149,13 +195,10 @@ __global__ void __launch_bounds__(256)
     return;
   }
   const float* x = si.X + (size_t)a * D;
-  const float* m = mu + (size_t)b * D;
   const int Dlen = emb * D;  // values of one operand row
+  const float* m = mu + (size_t)b * Dlen;
   // grid-point weights w_p enter the distance as sqrt(w_p) scalings of the values
-  auto val = [&](int i) {
-    const int pnt = kEmb ? i % D : i;  // grid point of value i
-    return wts ? (x[i] - m[pnt]) * sqrtf(wts[pnt]) : x[i] - m[pnt];
-  };
+  auto val = [&](int i) { return sw ? (x[i] - m[i]) * sw[i] : x[i] - m[i]; };
   // One read of the row. Lane g0 + lane builds group g0 + lane: its entry pos is grid
   // point pos * groups + g, so for each pos the warp reads 32 consecutive grid points
   // (coalesced). The warp's 32 groups, contiguous in the output row, are staged in
@@ -204,7 +247,7 @@ __global__ void __launch_bounds__(256)
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  const float c = kCorr ? __bfloat162float(__float2bfloat16_rn((float)sqrt(acc / groups))) : 0.f;
+  const float c = kCorr ? correction(acc, groups) : 0.f;
   // the correction entries of this lane's groups (same thread as the stores above)
   __nv_bfloat16* hrow = hi + (size_t)r * Dp;
   __nv_bfloat16* lrow = lo + (size_t)r * Dp;
@@ -221,15 +264,16 @@ __global__ void __launch_bounds__(256)
 // The same operand preparation for rows of few groups (groups <= 16, e.g. the
 // trajectory-embedded rows of a small grid): a warp takes 32 / groups rows at once,
 // lane (r, g) = (lane / groups, lane % groups) building group g of row r, so that no
-// lane idles; the row's FP64 norm is summed over its lanes in a fixed order. The grid
-// point of value i (i mod D) is stepped along with i instead of divided.
+// lane idles; the row's FP64 norm is summed over its lanes in a fixed order.
 template <bool kCorr>
 __global__ void __launch_bounds__(256)
     prep_split_small_kernel(const __grid_constant__ SeriesTable st, int r_lo, int rows, int D,
                             int emb, int groups, const float* __restrict__ mu,
-                            const float* __restrict__ wts, __nv_bfloat16* __restrict__ hi,
+                            const float* __restrict__ sw, __nv_bfloat16* __restrict__ hi,
                             __nv_bfloat16* __restrict__ lo, double* __restrict__ norms,
                             float* __restrict__ cval) {
+  launch_wait();
+  launch_next();
   const int lane = threadIdx.x & 31;
   const int per_warp = 32 / groups;
   const int rl = lane / groups, g = lane - rl * groups;  // row of the warp, group of the row
@@ -250,34 +294,37 @@ __global__ void __launch_bounds__(256)
     float fp = 0.f;
     if (!pad) {
       const float* x = si.X + (size_t)a * D;
-      const float* m = mu + (size_t)b * D;
       const int Dlen = emb * D;
-      int pnt = g % D;  // grid point of value i = pos * groups + g, stepped with pos
+      const float* m = mu + (size_t)b * Dlen;
+      // 16 entries at a time, all their loads before the arithmetic: few rows in flight
+      // (365 days: 6 CTAs) leave nothing else to hide a load's latency
 #pragma unroll
-      for (int pp = 0; pp < 32; ++pp) {
-        float v[2];
+      for (int q = 0; q < 4; ++q) {
+        float xv[16], mv[16], wv[16];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int pos = 2 * pp + h, i = pos * groups + g;
-          float val = 0.f;
-          if (i < Dlen && pos < 63) {
-            val = x[i] - m[pnt];
-            if (wts) val *= sqrtf(wts[pnt]);
-          }
-          v[h] = val;
-          pnt += groups;  // groups <= D (emb <= 17 < 63), so one subtraction suffices
-          if (pnt >= D) pnt -= D;
+        for (int u = 0; u < 16; ++u) {
+          const int pos = 16 * q + u, i = pos * groups + g;
+          const bool in = i < Dlen && pos < 63;  // entry 63 filled later
+          xv[u] = in ? x[i] : 0.f;
+          mv[u] = in ? m[i] : 0.f;
+          wv[u] = in && sw ? sw[i] : 1.f;
         }
-        fp = fmaf(v[0], v[0], fp);
-        fp = fmaf(v[1], v[1], fp);
-        const __nv_bfloat16 h0 = __float2bfloat16_rn(v[0]);
-        const __nv_bfloat16 q0 = __float2bfloat16_rn(v[0] - __bfloat162float(h0));
-        const __nv_bfloat16 h1 = __float2bfloat16_rn(v[1]);
-        const __nv_bfloat16 q1 = __float2bfloat16_rn(v[1] - __bfloat162float(h1));
-        const __nv_bfloat162 hp = __halves2bfloat162(h0, h1);
-        const __nv_bfloat162 lp = __halves2bfloat162(q0, q1);
-        hv[pp] = *reinterpret_cast<const uint32_t*>(&hp);
-        lv[pp] = *reinterpret_cast<const uint32_t*>(&lp);
+#pragma unroll
+        for (int u = 0; u < 16; u += 2) {
+          const int pp = 8 * q + u / 2;
+          const float d0 = xv[u] - mv[u], d1 = xv[u + 1] - mv[u + 1];
+          const float v0 = sw ? d0 * wv[u] : d0, v1 = sw ? d1 * wv[u + 1] : d1;
+          fp = fmaf(v0, v0, fp);
+          fp = fmaf(v1, v1, fp);
+          const __nv_bfloat16 h0 = __float2bfloat16_rn(v0);
+          const __nv_bfloat16 q0 = __float2bfloat16_rn(v0 - __bfloat162float(h0));
+          const __nv_bfloat16 h1 = __float2bfloat16_rn(v1);
+          const __nv_bfloat16 q1 = __float2bfloat16_rn(v1 - __bfloat162float(h1));
+          const __nv_bfloat162 hp = __halves2bfloat162(h0, h1);
+          const __nv_bfloat162 lp = __halves2bfloat162(q0, q1);
+          hv[pp] = *reinterpret_cast<const uint32_t*>(&hp);
+          lv[pp] = *reinterpret_cast<const uint32_t*>(&lp);
+        }
       }
     } else {
 #pragma unroll
@@ -298,9 +345,7 @@ __global__ void __launch_bounds__(256)
     acc += pj;
   }
   if (!act) return;
-  const float c = (kCorr && !pad)
-                      ? __bfloat162float(__float2bfloat16_rn((float)sqrt(acc / groups)))
-                      : 0.f;
+  const float c = kCorr && !pad ? correction(acc, groups) : 0.f;
   hi[(size_t)r * Dp + g * 64 + 63] = __float2bfloat16_rn(c);
   lo[(size_t)r * Dp + g * 64 + 63] = __float2bfloat16_rn(-c);
   if (g == 0) {
@@ -309,11 +354,22 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// W of every stacked trajectory row: an explicit L-term FP64 sum of its series' norms.
+// W of every stacked trajectory row: an explicit L-term FP64 sum of its series' norms. The
+// row's bound, shared minima and column-list mask are cleared here too (three fills fewer
+// on the stream).
 __global__ void window_series_kernel(const __grid_constant__ SeriesTable st, int r_lo,
-                                     int out_rows, const double* __restrict__ norms, float* W) {
+                                     int out_rows, const double* __restrict__ norms, float* W,
+                                     const ClearArgs c) {
   const int r = r_lo + blockIdx.x * blockDim.x + threadIdx.x;
+  launch_wait();
+  launch_next();
+  if (blockIdx.x == 0 && (int)threadIdx.x < c.counters) c.counter[threadIdx.x] = 0;
   if (r >= out_rows) return;
+  if (c.thr) {
+    c.thr[r] = 0x7F7F7F7Fu;
+    for (int i = 0; i < c.slots; ++i) c.shared_min[i * c.stride + r] = 0x7F7F7F7Fu;
+    for (int i = 0; i < c.mask_words; ++i) c.col_mask[(size_t)r * c.mask_words + i] = 0u;
+  }
   const int b = find_series(st.s, st.n, r, true);
   const SeriesInfo& si = st.s[b];
   const int t = r - si.out_base;
@@ -443,15 +499,13 @@ __device__ __forceinline__ bool key_less(float d1, int i1, float d2, int i2) {
 // from the column lists of the strips above; k rounds of a warp arg-min on
 // (distance, index) then give the exact neighbour set in order. If the gathered
 // set overflows the buffer, the rounds scan the lists directly.
-__global__ void __launch_bounds__(32 * kMergeWarps)
-    merge_tc_kernel(const int2* __restrict__ part, const int* __restrict__ part_n, int cap,
-                    int out_rows, TcWork w, const __grid_constant__ SeriesTable st, int* err) {
-  __shared__ float bd[kMergeWarps][kMergeCap];
-  __shared__ int bi[kMergeWarps][kMergeCap];
-  __shared__ int bn[kMergeWarps];
-  __shared__ float sorted_d[kMergeWarps][kMaxK];  // the row's k distances in order
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * kMergeWarps + wid;
+__device__ __forceinline__ void merge_row(const int2* __restrict__ part,
+                                          const int* __restrict__ part_n, int cap, int out_rows,
+                                          const TcWork& w, const SeriesTable& st, int* err,
+                                          float* bd, int* bi, int* bn, float* sorted_d,
+                                          float** score_at, int* score_k) {
+  const int lane = threadIdx.x & 31;
+  const int r = blockIdx.x * kMergeWarps + (threadIdx.x >> 5);
   if (r >= out_rows) return;
   const int sidx = find_series(st.s, st.n, r, true);
   const SeriesInfo& si = st.s[sidx];
@@ -467,10 +521,10 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
     return si.col_base + w.col_off[si.strip_base + s2] + (t - (s2 + 1) * si.rows_out);
   };
   auto push = [&](float d, int i) {
-    const int pos = atomicAdd(&bn[wid], 1);
+    const int pos = atomicAdd(bn, 1);
     if (pos < kMergeCap) {
-      bd[wid][pos] = d;
-      bi[wid][pos] = i;
+      bd[pos] = d;
+      bi[pos] = i;
     }
   };
   // The k smallest (distance, index) keys among the n <= kMergeCap buffered
@@ -481,15 +535,16 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
   // keys are written to the row's outputs in (distance, index) order (index -1,
   // distance +inf for missing ones) with the FP64 mean of the k distances, summed in
   // that order.
-  auto select_k = [&](int n, bool out) -> float {
-    constexpr int kPer = kMergeCap / 32;
+  // kPer of them per lane (n <= 32 kPer): a row usually gathers no more than 64.
+  auto select_n = [&](auto per, int n, bool out) -> float {
+    constexpr int kPer = decltype(per)::value;
     unsigned db[kPer];
     int ib[kPer];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
       const int q = lane + 32 * u;
-      db[u] = q < n ? (__float_as_uint(bd[wid][q]) & 0x7FFFFFFFu) : 0xFFFFFFFFu;
-      ib[u] = q < n ? bi[wid][q] : INT_MAX;
+      db[u] = q < n ? (__float_as_uint(bd[q]) & 0x7FFFFFFFu) : 0xFFFFFFFFu;
+      ib[u] = q < n ? bi[q] : INT_MAX;
     }
     auto count_le = [&](unsigned x) {
       unsigned c = 0;
@@ -502,10 +557,18 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
     unsigned T = kInf;
     int I = INT_MAX;
     if (kk > 0) {
-      unsigned lo = 0, hi = kInf;
+      // from the candidates' own range: the close ones lie within a factor of two or so
+      unsigned mn = 0xFFFFFFFFu, mx = 0u;
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        mn = min(mn, db[u]);
+        mx = max(mx, db[u] <= kInf ? db[u] : 0u);
+      }
+      unsigned lo = __reduce_min_sync(0xffffffffu, mn), hi = __reduce_max_sync(0xffffffffu, mx);
       while (lo < hi) {
         const unsigned mid = lo + ((hi - lo) >> 1);
-        if (count_le(mid) >= kk) hi = mid;
+        const int c = count_le(mid);
+        if (c >= kk) hi = mid;
         else lo = mid + 1;
       }
       T = lo;
@@ -531,7 +594,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
     // compact the selected keys to the front of the buffer, then place each by rank
     float dv[kPer];
 #pragma unroll
-    for (int u = 0; u < kPer; ++u) dv[u] = lane + 32 * u < n ? bd[wid][lane + 32 * u] : 0.f;
+    for (int u = 0; u < kPer; ++u) dv[u] = lane + 32 * u < n ? bd[lane + 32 * u] : 0.f;
     __syncwarp();
     int base = 0;
 #pragma unroll
@@ -540,34 +603,37 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
       const unsigned m = __ballot_sync(0xffffffffu, sel);
       if (sel) {
         const int q = base + __popc(m & ((1u << lane) - 1u));
-        bd[wid][q] = dv[u];
-        bi[wid][q] = ib[u];
+        bd[q] = dv[u];
+        bi[q] = ib[u];
       }
       base += __popc(m);
     }
     __syncwarp();
     for (int e = lane; e < k; e += 32) {
       if (e < kk) {
-        const float de = bd[wid][e];
-        const int ie = bi[wid][e];
+        const float de = bd[e];
+        const int ie = bi[e];
         int rank = 0;
-        for (int j = 0; j < kk; ++j) rank += key_less(bd[wid][j], bi[wid][j], de, ie) ? 1 : 0;
+        for (int j = 0; j < kk; ++j) rank += key_less(bd[j], bi[j], de, ie) ? 1 : 0;
         si.idx[(size_t)t * k + rank] = ie;
         si.dist[(size_t)t * k + rank] = de;
-        sorted_d[wid][rank] = de;
+        sorted_d[rank] = de;
       } else {
         si.idx[(size_t)t * k + e] = -1;
         si.dist[(size_t)t * k + e] = CUDART_INF_F;
-        sorted_d[wid][e] = CUDART_INF_F;
+        sorted_d[e] = CUDART_INF_F;
       }
     }
-    __syncwarp();
     if (lane == 0) {
-      double sum = 0.0;
-      for (int e = 0; e < k; ++e) sum += (double)sorted_d[wid][e];
-      si.score[t] = (float)(sum / (double)k);
+      *score_at = si.score + t;
+      *score_k = k;
     }
     return __uint_as_float(T);
+  };
+  auto select_k = [&](int n, bool out) -> float {
+    if (n <= 64) return select_n(std::integral_constant<int, 2>(), n, out);
+    if (n <= 128) return select_n(std::integral_constant<int, 4>(), n, out);
+    return select_n(std::integral_constant<int, kMergeCap / 32>(), n, out);
   };
   // with a split series only the lists of this call's strips exist
   const bool own = strip >= w.part_lo && strip < w.part_hi;
@@ -575,7 +641,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
   const int c_hi = own ? si.slots : c_lo;
   int n = 0;
   for (int pass = 0; pass < 64; ++pass) {
-    if (lane == 0) bn[wid] = 0;
+    if (lane == 0) *bn = 0;
     __syncwarp();
     // row-side lists (not sorted): their counts, one list per lane, then their entries
     // numbered across the lists (a prefix sum of the counts), one per lane and round,
@@ -669,7 +735,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
       }
     }
     __syncwarp();
-    n = bn[wid];
+    n = *bn;
     __syncwarp();
     if (n <= kMergeCap) break;
     // overflow: the k-th smallest of the buffered (valid, distinct) candidates is a
@@ -696,7 +762,7 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
       }
     };
     if (!direct) {
-      for (int q = lane; q < n; q += 32) consider(bd[wid][q], bi[wid][q]);
+      for (int q = lane; q < n; q += 32) consider(bd[q], bi[q]);
     } else {
       for (int c = c_lo + lane; c < c_hi; c += 32) {
         if (!tk_in(plist + c, w.part_lists, err)) continue;
@@ -743,14 +809,39 @@ __global__ void __launch_bounds__(32 * kMergeWarps)
   if (lane == 0) si.score[t] = (float)(sum / (double)k);
 }
 
+__global__ void __launch_bounds__(32 * kMergeWarps)
+    merge_tc_kernel(const int2* __restrict__ part, const int* __restrict__ part_n, int cap,
+                    int out_rows, TcWork w, const __grid_constant__ SeriesTable st, int* err) {
+  __shared__ float bd[kMergeWarps][kMergeCap];
+  __shared__ int bi[kMergeWarps][kMergeCap];
+  __shared__ int bn[kMergeWarps];
+  __shared__ float sorted_d[kMergeWarps][kMaxK];  // the row's k distances in order
+  __shared__ float* score_at[kMergeWarps];        // where the row's score goes (null: nowhere)
+  __shared__ int score_k[kMergeWarps];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) score_at[wid] = nullptr;
+  launch_wait();
+  launch_next();
+  merge_row(part, part_n, cap, out_rows, w, st, err, bd[wid], bi[wid], &bn[wid], sorted_d[wid],
+            &score_at[wid], &score_k[wid]);
+  // the rows' scores, one lane per row: an FP64 instruction takes as long for one lane as
+  // for 32, and with each warp summing its own row the FP64 pipe was two thirds busy
+  __syncthreads();
+  if (threadIdx.x < kMergeWarps && score_at[threadIdx.x]) {
+    const int k = score_k[threadIdx.x];
+    double sum = 0.0;
+    for (int e = 0; e < k; ++e) sum += (double)sorted_d[threadIdx.x][e];
+    *score_at[threadIdx.x] = (float)(sum / (double)k);
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_merge_tc(const TcArgs& a, const TcWork& w, const SeriesTable& sr,
                             cudaStream_t st) {
   const int blocks = (a.out_rows + kMergeWarps - 1) / kMergeWarps;
-  merge_tc_kernel<<<blocks, 32 * kMergeWarps, 0, st>>>(a.part, a.part_n, a.cap, a.out_rows, w, sr,
-                                                        a.err);
-  return cudaGetLastError();
+  return launch_chained(merge_tc_kernel, blocks, 32 * kMergeWarps, 0, st, a.part, a.part_n, a.cap,
+                        a.out_rows, w, sr, a.err);
 }
 
 cudaError_t launch_merge_parts(const int32_t* idx_parts, const float* dist_parts, int nparts,
@@ -763,68 +854,41 @@ cudaError_t launch_merge_parts(const int32_t* idx_parts, const float* dist_parts
   return cudaGetLastError();
 }
 
-cudaError_t launch_col_mean_series(const SeriesTable& sr, int D, float* partial, float* mu,
-                                   bool center, cudaStream_t st) {
-  if (center) {
-    dim3 grid((D + 255) / 256, kMeanSlices, sr.n);
-    col_partial_series_kernel<<<grid, 256, 0, st>>>(sr, D, partial);
-  }
-  dim3 g2((D + 255) / 256, sr.n);
-  col_final_series_kernel<<<g2, 256, 0, st>>>(sr, partial, D, mu, center ? 1 : 0);
-  return cudaGetLastError();
+cudaError_t launch_col_mean_series(const SeriesTable& sr, int D, int emb, const float* wts,
+                                   float* mu, float* sw, bool center, cudaStream_t st) {
+  return launch_chained(col_mean_series_kernel, dim3((D + 31) / 32, sr.n), 32 * kMeanWarps, 0, st,
+                        sr, D, emb, wts, mu, sw, center ? 1 : 0);
 }
 
 cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int emb, int groups,
-                                     bool correct, const float* mu, const float* wts, void* hi,
+                                     bool correct, const float* mu, const float* sw, void* hi,
                                      void* lo, double* norms, float* cval, cudaStream_t st,
                                      int r_lo) {
   if (rows <= r_lo) return cudaSuccess;
   __nv_bfloat16* h = static_cast<__nv_bfloat16*>(hi);
   __nv_bfloat16* l = static_cast<__nv_bfloat16*>(lo);
-  if (groups <= 16) {
-    // few groups per row: several rows per warp
-    const int per_block = 8 * (32 / groups);
-    const int nb = (rows - r_lo + per_block - 1) / per_block;
-    if (correct)
-      prep_split_small_kernel<true><<<nb, 256, 0, st>>>(sr, r_lo, rows, D, emb, groups, mu, wts,
-                                                        h, l, norms, cval);
-    else
-      prep_split_small_kernel<false><<<nb, 256, 0, st>>>(sr, r_lo, rows, D, emb, groups, mu, wts,
-                                                         h, l, norms, cval);
-    return cudaGetLastError();
-  }
-  const int blocks = (rows - r_lo + 7) / 8;
-  // the embedded form (values of several days per row) maps a value to its grid point
-  // by a division; the plain form needs none
-  if (correct && emb > 1)
-    prep_split_series_kernel<true, true><<<blocks, 256, 0, st>>>(sr, r_lo, rows, D, emb, groups,
-                                                                 mu, wts, h, l, norms, cval);
-  else if (correct)
-    prep_split_series_kernel<true, false><<<blocks, 256, 0, st>>>(sr, r_lo, rows, D, emb, groups,
-                                                                  mu, wts, h, l, norms, cval);
-  else if (emb > 1)
-    prep_split_series_kernel<false, true><<<blocks, 256, 0, st>>>(sr, r_lo, rows, D, emb, groups,
-                                                                  mu, wts, h, l, norms, cval);
-  else
-    prep_split_series_kernel<false, false><<<blocks, 256, 0, st>>>(sr, r_lo, rows, D, emb,
-                                                                   groups, mu, wts, h, l, norms,
-                                                                   cval);
-  return cudaGetLastError();
+  // few groups per row: several rows per warp
+  const bool small = groups <= 16;
+  const int per_block = small ? 8 * (32 / groups) : 8;
+  const int blocks = (rows - r_lo + per_block - 1) / per_block;
+  const auto kernel = small ? (correct ? prep_split_small_kernel<true> : prep_split_small_kernel<false>)
+                            : (correct ? prep_split_series_kernel<true>
+                                       : prep_split_series_kernel<false>);
+  return launch_chained(kernel, blocks, 256, 0, st, sr, r_lo, rows, D, emb, groups, mu, sw, h, l,
+                        norms, cval);
 }
 
 cudaError_t launch_window_series(const SeriesTable& sr, int out_rows, const double* norms,
-                                 float* W, cudaStream_t st, int r_lo) {
+                                 float* W, const ClearArgs& clear, cudaStream_t st, int r_lo) {
   if (out_rows <= r_lo) return cudaSuccess;
-  window_series_kernel<<<(out_rows - r_lo + 255) / 256, 256, 0, st>>>(sr, r_lo, out_rows, norms,
-                                                                     W);
-  return cudaGetLastError();
+  return launch_chained(window_series_kernel, (out_rows - r_lo + 255) / 256, 256, 0, st, sr, r_lo,
+                        out_rows, norms, W, clear);
 }
 
 cudaError_t launch_prep_fp32_series(const SeriesTable& sr, int rows, int D, int Dp,
-                                    const float* mu, const float* wts, float* Xc, double* norms,
+                                    const float* mu, const float* sw, float* Xc, double* norms,
                                     cudaStream_t st) {
-  prep_fp32_series_kernel<<<rows, 256, 0, st>>>(sr, D, Dp, mu, wts, Xc, norms);
-  return cudaGetLastError();
+  return launch_chained(prep_fp32_series_kernel, rows, 256, 0, st, sr, D, Dp, mu, sw, Xc, norms);
 }
 
 cudaError_t launch_merge(const FusedArgs& a, int32_t* idx, float* dist, float* score,

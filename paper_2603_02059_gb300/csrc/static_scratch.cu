@@ -130,7 +130,6 @@ extern "C" traknn_status traknn_knn_scores_static(const float* X, int64_t N, int
   a.err = reinterpret_cast<int*>(base + o_err);
   a.wait_limit_ns = 2000000000LL;
   a.debug_withhold = 0;
-  float* partial = reinterpret_cast<float*>(base + lay.partial);
   float* mu = reinterpret_cast<float*>(base + lay.mu);
   double* norms = reinterpret_cast<double*>(base + lay.norms);
   float* Xc = reinterpret_cast<float*>(base + lay.ops);
@@ -147,10 +146,10 @@ extern "C" traknn_status traknn_knn_scores_static(const float* X, int64_t N, int
   // the status word is the only scratch that must start at zero; every other
   // byte a kernel reads is written earlier in this same call
   if (cudaMemsetAsync(a.err, 0, sizeof(int), cs) != cudaSuccess ||
-      launch_col_mean_series(sr, (int)D, partial, mu, true, cs) != cudaSuccess ||
+      launch_col_mean_series(sr, (int)D, 1, nullptr, mu, nullptr, true, cs) != cudaSuccess ||
       launch_prep_fp32_series(sr, (int)N, (int)D, lay.Dp, mu, nullptr, Xc, norms, cs) !=
           cudaSuccess ||
-      launch_window_series(sr, M, norms, W, cs) != cudaSuccess ||
+      launch_window_series(sr, M, norms, W, ClearArgs{}, cs) != cudaSuccess ||
       launch_fused_fp32_static(Xc, a, sms, cs) != cudaSuccess ||
       launch_merge(a, nbr_idx, nbr_dist, score, cs) != cudaSuccess) {
     cudaGetLastError();

@@ -322,8 +322,8 @@ std::vector<int64_t> shape_key(const HostSeries* sd, int B, int64_t D, const tra
 
 // Device pointers of the tensor-core workspace for plan `p`.
 struct TcBuffers {
-  float* partial;
   float* mu;
+  float* sw;  // square roots of the grid-point weights
   double* norms;
   float* cval;
   float* W;
@@ -354,8 +354,8 @@ TcBuffers tc_layout(const TcPlan& p, int64_t D, bool fp32, int num_ctas, char* b
   b.Dp = fp32 ? (int)((D + 31) / 32 * 32) : tc_groups((int)D * p.emb) * 64;
   const int B = p.table.n;
   const size_t ks = (size_t)list_pitch(p.kmax);
-  b.partial = reinterpret_cast<float*>(take((size_t)B * kMeanSlices * D * sizeof(float)));
-  b.mu = reinterpret_cast<float*>(take((size_t)B * D * sizeof(float)));
+  b.mu = reinterpret_cast<float*>(take((size_t)B * p.emb * D * sizeof(float)));
+  b.sw = reinterpret_cast<float*>(take((size_t)p.emb * D * sizeof(float)));
   b.norms = reinterpret_cast<double*>(take((size_t)p.rows * sizeof(double)));
   b.cval = reinterpret_cast<float*>(take((size_t)p.rows * sizeof(float)));
   b.W = reinterpret_cast<float*>(take((size_t)p.out_rows * sizeof(float)));
@@ -364,7 +364,6 @@ TcBuffers tc_layout(const TcPlan& p, int64_t D, bool fp32, int num_ctas, char* b
   b.part = reinterpret_cast<int2*>(
       take((size_t)p.part_lists * list_cap((int)ks, p.part_lists) * sizeof(int2)));
   b.part_n = reinterpret_cast<int*>(take((size_t)p.part_lists * sizeof(int)));
-  // bounds and shared minima: one fill (0x7F) sets both
   b.thr = reinterpret_cast<unsigned int*>(
       take((size_t)p.out_rows * (1 + min_slots(p.kmax)) * sizeof(unsigned int)));
   b.shared_min = b.thr + p.out_rows;
@@ -414,15 +413,16 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
           ? 2
           : 1;
   key.push_back(egroups);
-  // Band pre-pass width: two tiles per strip when the contraction dominates a tile's
-  // cost; with short operand rows (small grids) a tile's contraction is cheap and the
-  // epilogue decides, and eight tiles give bounds tight enough to save more list
-  // inserts in the main pass than the band costs (D = 32, L = 5: 1.91 -> 1.69 ms; at
-  // D = 3,726 four tiles already cost 6 %)
+  // Band pre-pass width in tiles per strip. Short operand rows: a tile's contraction is cheap
+  // and eight tiles save more list entries in the main pass than the band costs (D = 32, L =
+  // 5, N = 4,000 1 / 2 / 4 / 8 tiles 171 / 152 / 131 / 133 us). Otherwise one tile while its
+  // 64 groups of columns still resolve k (k <= 20; N = 10,957, D = 3,726, k = 10 1 / 2 / 4
+  // tiles 1,180 / 1,209 / 1,293 us, four lengths 1,865 / 1,952; D = 512, N = 1,826 139 / 155
+  // / 199), two for larger k (the last case with k = 40: 220 / 203 / 234).
   // FP32: a band column costs as much as a main one; 1 / 2 / 8 tiles: D = 32, N = 27,394
   // 2,023 / 1,938 / 1,996 us, N = 4,000 190 / 181 / 233; D = 512, N = 1,826 310 / 410 / 983;
   // D = 3,726, N = 10,957 11.2 / 12.0 / 16.5 ms
-  const int band_tiles = fp32 ? (D <= 64 ? 2 : 1) : Dk <= 768 ? 8 : 2;
+  const int band_tiles = fp32 ? (D <= 64 ? 2 : 1) : Dk <= 768 ? 8 : kmax <= 20 ? 1 : 2;
   key.push_back(band_tiles);
   TcPlan& p = h->plan;
   if (p.key != key) {
@@ -584,14 +584,27 @@ traknn_status launch_units(traknn_ctx* h, const TcBuffers& b, const TcArgs& a, c
   return TRAKNN_OK;
 }
 
-// Everything a main pass accumulates into: bounds and shared minima (0x7F bytes: a large
-// finite value), column-list masks, `counters` unit counters.
-traknn_status clear_lists(const TcPlan& p, const TcBuffers& b, int counters, cudaStream_t s) {
-  TRY_CUDA(cudaMemsetAsync(
-      b.thr, 0x7F, (size_t)p.out_rows * (1 + min_slots(p.kmax)) * sizeof(unsigned int), s));
-  TRY_CUDA(cudaMemsetAsync(b.col_mask, 0,
-                           (size_t)p.out_rows * p.mask_words * sizeof(unsigned int), s));
-  TRY_CUDA(cudaMemsetAsync(b.counter, 0, counters * sizeof(int), s));
+// Means, operand rows [lo, hi) and window sums of the trajectory rows [lo, ohi), whose bounds
+// and masks are cleared; `counters` > 0 also clears that many unit counters, and computes
+// the means first.
+traknn_status enqueue_prep(traknn_ctx* h, const TcBuffers& b, int64_t D, int lo, int hi, int ohi,
+                           int counters, cudaStream_t s) {
+  const TcPlan& p = h->plan;
+  const SeriesTable& sr = p.table;
+  const float* sw = h->weights ? b.sw : nullptr;
+  if (counters > 0)
+    TRY_CUDA(launch_col_mean_series(sr, (int)D, p.emb, h->weights, b.mu, b.sw, h->center != 0, s));
+  if (h->precision == TRAKNN_PREC_FP32)
+    TRY_CUDA(launch_prep_fp32_series(sr, p.rows, (int)D, b.Dp, b.mu, sw,
+                                     static_cast<float*>(b.hi), b.norms, s));
+  else
+    TRY_CUDA(launch_prep_split_series(sr, hi, (int)D, p.emb, b.Dp / 64,
+                                      h->precision == TRAKNN_PREC_SPLIT_BF16, b.mu, sw, b.hi, b.lo,
+                                      b.norms, b.cval, s, lo));
+  const ClearArgs clear{b.thr,      b.shared_min, p.out_rows, min_slots(p.kmax),
+                        b.col_mask, p.mask_words, b.counter,  counters};
+  TRY_CUDA(launch_window_series(sr, ohi, b.norms, b.W, clear, s, lo));
+  h->launches += (counters > 0 ? 1 : 0) + (hi > lo ? 1 : 0) + (ohi > lo ? 1 : 0);
   return TRAKNN_OK;
 }
 
@@ -603,16 +616,7 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
   TcArgs a;
   TcWork w;
   fused_args(h, b, &a, &w);
-  TRY_CUDA(launch_col_mean_series(sr, (int)D, b.partial, b.mu, h->center != 0, s));
-  if (h->precision == TRAKNN_PREC_FP32)
-    TRY_CUDA(launch_prep_fp32_series(sr, p.rows, (int)D, b.Dp, b.mu, h->weights,
-                                     static_cast<float*>(b.hi), b.norms, s));
-  else
-    TRY_CUDA(launch_prep_split_series(sr, p.rows, (int)D, p.emb, b.Dp / 64,
-                                      h->precision == TRAKNN_PREC_SPLIT_BF16, b.mu, h->weights,
-                                      b.hi, b.lo, b.norms, b.cval, s));
-  TRY_CUDA(launch_window_series(sr, p.out_rows, b.norms, b.W, s));
-  TRY_ST(clear_lists(p, b, 2, s));
+  TRY_ST(enqueue_prep(h, b, D, 0, p.rows, p.out_rows, 2, s));
   const int slot = h->ev_head;
   if (record_events) TRY_CUDA(cudaEventRecord(h->ev_start[slot], s));
   // threshold pre-pass over the band units (stored after the main units), then the rest
@@ -624,7 +628,7 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
     h->ev_count = std::min(h->ev_count + 1, traknn_ctx::kRing);
   }
   TRY_CUDA(launch_merge_tc(a, w, sr, s));
-  h->launches += (h->center ? 2 : 1) + 3;
+  h->launches += 1;
   return TRAKNN_OK;
 }
 
@@ -672,23 +676,14 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
   TcArgs a;
   TcWork w;
   fused_args(h, b, &a, &w);
-  const bool split = h->precision == TRAKNN_PREC_SPLIT_BF16;
   for (int q = 0; q < K; ++q) {
     const int lo = p.pstrip[q + 1] * R;                      // first day (and row) of phase q
     const int hi = q == 0 ? p.rows : p.pstrip[q] * R;        // rows prepared by phase q
     const int ohi = q == 0 ? p.out_rows : std::min(hi, p.out_rows);
     TRY_CUDA(cudaStreamWaitEvent(s, in[q], 0));
-    if (q == 0) {
-      TRY_CUDA(launch_col_mean_series(sr, (int)D, b.partial, b.mu, h->center != 0, s));
-      TRY_ST(clear_lists(p, b, 2 * K, s));
-      h->launches += h->center ? 2 : 1;
-    }
     // window sums of rows [lo, ohi) read day norms up to ohi + L - 2: prepared now or
     // by an earlier phase
-    TRY_CUDA(launch_prep_split_series(sr, hi, (int)D, 1, b.Dp / 64, split, b.mu, h->weights,
-                                      b.hi, b.lo, b.norms, b.cval, s, lo));
-    TRY_CUDA(launch_window_series(sr, ohi, b.norms, b.W, s, lo));
-    h->launches += (hi > lo ? 1 : 0) + (ohi > lo ? 1 : 0);
+    TRY_ST(enqueue_prep(h, b, D, lo, hi, ohi, q == 0 ? 2 * K : 0, s));
     TRY_ST(launch_units(h, b, a, w, p.pb[q], p.pb[q + 1] - p.pb[q], 2 * q + 1, true, s));
     TRY_ST(launch_units(h, b, a, w, p.pu[q], p.pu[q + 1] - p.pu[q], 2 * q, false, s));
   }
@@ -849,7 +844,7 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   for (auto& g : h->graphs)
     if (g.key == key) {
       TRY_CUDA(cudaGraphLaunch(g.exec, s));
-      h->launches += (h->center ? 2 : 1) + 4 + (h->plan.band && h->plan.nband > 0 ? 1 : 0);
+      h->launches += 5 + (h->plan.band && h->plan.nband > 0 ? 1 : 0);
       return TRAKNN_OK;
     }
   if (!h->cap_stream) TRY_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
@@ -879,7 +874,7 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   }
   h->graphs.push_back(GraphEntry{key, exec});
   TRY_CUDA(cudaGraphLaunch(exec, s));
-  h->launches += (h->center ? 2 : 1) + 4 + (h->plan.band && h->plan.nband > 0 ? 1 : 0);
+  h->launches += 5 + (h->plan.band && h->plan.nband > 0 ? 1 : 0);
   return TRAKNN_OK;
 }
 
