@@ -105,7 +105,7 @@ __device__ __forceinline__ void window_topk(const float* g, int ldg, const RowCt
 // -------------------------------------------------------------------- work units
 // A unit with its series' parameters.
 struct UnitSpan {
-  int strip, T0, jlo, jhi, ntiles, slot, nser, step;
+  int strip, T0, jt0, jlo, jhi, ntiles, slot, nser, step;  // jt0: first Gram column
   int carry, adv;  // carry: the last L-1 Gram columns pass from tile to tile; adv: tile stride
   int M, L, k, e, R;      // series: trajectories, length, neighbours, exclusion, rows per strip
   int row_base, out_base, slots, strip_base;
@@ -114,8 +114,10 @@ struct UnitSpan {
 
 // Unit wu for the sj-th of the series that share its Gram tiles (sj = 0: the one
 // with the most trajectories, whose tiles cover the others').
+// A unit of a pair of CTAs covers two strips with the Gram tiles of the first; `rank` 1 is
+// the second one, whose own output columns start later (sym).
 __device__ __forceinline__ bool unit_span(const WorkUnit& wu, const SeriesInfo* sr, int sj,
-                                          UnitSpan& us) {
+                                          UnitSpan& us, int rank = 0, int sym = 0) {
   const SeriesInfo& si = sr[wu.series + sj];
   us.nser = wu.pad[0] > 1 ? wu.pad[0] : 1;
   us.M = si.M;
@@ -129,13 +131,15 @@ __device__ __forceinline__ bool unit_span(const WorkUnit& wu, const SeriesInfo* 
   us.strip_base = si.strip_base;
   us.part_base = si.part_base;
   us.col_base = si.col_base;
-  us.strip = wu.strip;
-  us.T0 = wu.strip * us.R;
-  us.jlo = wu.jlo;
+  us.strip = wu.strip + rank;
+  us.T0 = us.strip * us.R;
+  us.jt0 = wu.jlo;
+  us.jlo = rank && sym ? max(wu.jlo, us.T0) : wu.jlo;
   us.jhi = min(wu.jhi, si.M);
   us.slot = wu.slot;
   us.step = si.step;
-  if (us.jlo >= us.jhi) return false;
+  if (rank && wu.pad[1] == 0) us.R = 0;  // the pair's second strip is not of this launch
+  if (us.jt0 >= us.jhi) return false;
   // A unit of one series: Gram tiles follow each other without overlap, tile it
   // covering Gram columns [jlo + 256 it, jlo + 256 (it+1)); the epilogue carries the
   // last L-1 columns of a tile into the next, so the windows of all output columns
@@ -144,8 +148,8 @@ __device__ __forceinline__ bool unit_span(const WorkUnit& wu, const SeriesInfo* 
   // tiles overlap by the largest L - 1 and each yields `step` output columns.
   us.carry = us.nser == 1;
   us.adv = us.carry ? kTileCols : us.step;
-  us.ntiles = us.carry ? (us.jhi - us.jlo + us.L - 1 + kTileCols - 1) / kTileCols
-                       : (us.jhi - us.jlo + us.step - 1) / us.step;
+  us.ntiles = us.carry ? (us.jhi - us.jt0 + us.L - 1 + kTileCols - 1) / kTileCols
+                       : (us.jhi - us.jt0 + us.step - 1) / us.step;
   return true;
 }
 

@@ -187,7 +187,8 @@ struct WorkUnit {
   int jlo;     // first output column
   int jhi;     // one past the last output column (clipped to each series' M)
   int slot;    // slot of the row-side partial lists written by this unit
-  int pad[3];  // pad[0]: number of consecutive series sharing the unit's Gram tiles
+  int pad[3];  // pad[0]: number of consecutive series sharing the unit's Gram tiles; pad[1]
+               // (units of CTA pairs): 1 if strip + 1 belongs to the unit too
 };
 
 struct TcWork {
@@ -250,7 +251,8 @@ struct TcArgs {
   const float* cval;   // [rows] correction value c of every stacked operand row
   int l2_keep_a;       // 1: load the strip operand with an L2 evict-last policy
   float* scratch;      // [CTAs][2][128 x 256] running tile totals (more than one segment)
-  int egroups;         // epilogue groups of the tensor-core kernel (1, or 2 at L = 1)
+  int egroups;         // epilogue groups of the tensor-core kernel (1 or 2)
+  int pair;            // 1: the units are those of CTA pairs (main pass, one epilogue group)
   // Band pre-pass in one BF16 product (hi only) on split operands: the correction
   // entries then add +groups c_a c_b, which the epilogue subtracts (corr_neg = 1), and
   // every distance is raised by band_margin (W_t + W_j), a bound of its error, before
@@ -307,19 +309,29 @@ __device__ __forceinline__ void launch_next() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <class... P, class... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
-                                  cudaStream_t st, A&&... args) {
+inline cudaError_t launch_chained_clusters(void (*kernel)(P...), int cluster, dim3 grid,
+                                           int threads, size_t smem, cudaStream_t st,
+                                           A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                                  cudaStream_t st, A&&... args) {
+  return launch_chained_clusters(kernel, 1, grid, threads, smem, st, std::forward<A>(args)...);
 }
 
 // sw: optional [D] square roots of the grid-point weights (the values are scaled by them).
@@ -414,6 +426,6 @@ cudaError_t launch_knn_stats(const float* dist, int M, int k, float* prefix, int
 // False until the tensor-core kernel is compiled in.
 bool tc_available();
 
-size_t fused_tc_smem_bytes(bool split, int kmax, int Lmax, int G);
+size_t fused_tc_smem_bytes(bool split, bool pair, int kmax, int Lmax, int G);
 
 }  // namespace traknn

@@ -71,6 +71,7 @@ __host__ __device__ constexpr int chunk_pitch(int L, bool win) {
 constexpr uint32_t kTileA = BM * KC * 2;  // bytes of one A operand tile
 constexpr uint32_t kTileB = BN * KC * 2;  // bytes of one B operand tile
 constexpr uint32_t kIdesc = ptx::idesc_bf16_f32(BM, BN);
+constexpr uint32_t kIdescPair = ptx::idesc_bf16_f32(2 * BM, BN);
 constexpr int kMaxStages = 8;
 constexpr size_t kSmemLimit = 232448;  // 227 KB opt-in per block
 
@@ -99,12 +100,17 @@ struct Ctl {
 
 // Bounded wait on an mbarrier phase. Records a timeout and raises the CTA's abort
 // flag when the limit runs out; gives up early when another role aborted.
+// kCluster: what the other CTA of a pair wrote before it arrived is visible afterwards.
+template <bool kCluster = false>
 __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, const Ctl& c,
                                              bool honor_abort = true) {
-  if (ptx::mbar_try_wait(bar, parity)) return true;
+  auto ready = [&]() {
+    return kCluster ? ptx::mbar_try_wait_cluster(bar, parity) : ptx::mbar_try_wait(bar, parity);
+  };
+  if (ready()) return true;
   const uint64_t t0 = ptx::globaltimer();
   for (;;) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
+    if (ready()) return true;
     if (honor_abort && *c.abort) return false;
     if (ptx::globaltimer() - t0 > c.limit_ns) {
       atomicCAS(c.err, 0, kErrTimeout);
@@ -119,7 +125,17 @@ constexpr int kQueue = 4;  // depth of the per-CTA unit queue
 // G: epilogue groups; kWin: some series of the call has L > 1 (windows are summed); kBand:
 // the band pre-pass (bounds only, no lists); kLarge: k > 32 in the band pass (two minima
 // per group), k > 40 in the main pass (128 shared minima); one epilogue group only.
-template <int G, bool kWin, bool kBand, bool kLarge>
+//
+// kPair (main pass, one epilogue group): clusters of two CTAs work as one on units of two
+// neighbouring strips. Each CTA loads its own strip's rows and half of a tile's columns
+// (128) and computes its strip's 128 x 256 outputs with both halves (cta_group::2), so a
+// stage is 32 KB per CTA instead of 48 KB: a third less operand traffic from L2 and into
+// shared memory (96 bytes a cycle of operand reads and 62 of TMA writes against the 128
+// that it takes, at the full MMA rate), and six stages instead of four. 75 years, D =
+// 3,726, L = 5, k = 20: 6,016 -> 4,949 us; 30 years 1,147 -> 997. The first CTA hands out
+// the units and issues the MMAs for both; every role's waits, its own CTA's and the
+// other's, are bounded as in a single CTA.
+template <int G, bool kWin, bool kBand, bool kLarge, bool kPair>
 __global__ void __launch_bounds__(kThreadsG(G), 1)
     fused_tc_kernel(const __grid_constant__ CUtensorMap tmA_hi,
                     const __grid_constant__ CUtensorMap tmA_lo,
@@ -132,6 +148,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int NS = p.nstages;
+  const int rank = kPair ? (int)ptx::cluster_rank() : 0;
 
   // ---- shared memory carve-up (ring base aligned to 1 KB for the swizzle pattern)
   const uint32_t raw = ptx::smem_u32(smem_raw);
@@ -168,12 +185,14 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     }
     for (int b = 0; b < 2; ++b) {
       ptx::mbar_init(tfull0 + 8u * b, 1);
-      ptx::mbar_init(tempty0 + 8u * b, kEpiThreads * G);  // every epilogue thread
+      // every epilogue thread; in a pair one lane of each of the eight warps
+      ptx::mbar_init(tempty0 + 8u * b, kPair ? 8 : kEpiThreads * G);
     }
     ptx::mbar_init(drain, 1);
     for (int i = 0; i < kQueue; ++i) {
       ptx::mbar_init(qfull0 + 8u * i, 1);
-      ptx::mbar_init(qempty0 + 8u * i, 1 + G);  // the MMA thread and each group's leader
+      // the MMA thread and each group's leader; in a pair also the second CTA's producer
+      ptx::mbar_init(qempty0 + 8u * i, kPair ? 4 : 1 + G);
     }
     ptx::mbar_init(xfull, kEpiThreads);
     ptx::mbar_init(xempty, kEpiThreads);
@@ -182,10 +201,16 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     ptx::fence_proxy_async();
   }
   if (warp == 1) {
-    ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
-    ptx::tmem_relinquish();
+    if (kPair) {
+      ptx::tmem_alloc_pair(ptx::smem_u32(tmem_slot), 512);
+      ptx::tmem_relinquish_pair();
+    } else {
+      ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
+      ptx::tmem_relinquish();
+    }
     ptx::tc_fence_before();
   }
+  if (kPair) ptx::cluster_sync();  // the other CTA's barriers are initialised
   __syncthreads();
   ptx::tc_fence_after();
   launch_wait();  // barriers and tensor memory were set up beside the kernel before
@@ -208,162 +233,209 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     // Hands out units in list order (global counter) through a small queue, so the
-    // units in flight across the GPU stay a contiguous window of the list.
-    if (lane == 0) {
+    // units in flight across the GPU stay a contiguous window of the list. The whole warp
+    // walks the units and waits; an elected lane issues the copies (see the MMA issuer).
+    if (ptx::elect_one()) {
       ptx::prefetch_tensormap(&tmA_hi);
-      ptx::prefetch_tensormap(&tmB_hi);
+      if (!kPair) ptx::prefetch_tensormap(&tmB_hi);
       if (p.split) {
         ptx::prefetch_tensormap(&tmA_lo);
-        ptx::prefetch_tensormap(&tmB_lo);
+        if (!kPair) ptx::prefetch_tensormap(&tmB_lo);
       }
-      const uint64_t pol_a = ptx::l2_policy_evict_last();
-      int stage = 0, qs = 0;
-      uint32_t phase = 0, qphase = 0, issued = 0, issued_par = 0;
-      bool ok = true, withheld = false;
-      UnitSpan us;
-      while (ok) {
-        if (!wait_bounded(qempty0 + 8u * qs, qphase ^ 1u, ctl)) break;
-        const int u = atomicAdd(w.counter, 1);
-        WorkUnit wu;
-        if (u < w.nunits) wu = w.units[u];
-        else wu.strip = -1;
-        qunit[qs] = wu;
-        ptx::mbar_arrive(qfull0 + 8u * qs);
-        if (++qs == kQueue) {
-          qs = 0;
-          qphase ^= 1u;
+    }
+    const uint64_t pol_a = ptx::l2_policy_evict_last();
+    int stage = 0, qs = 0;
+    uint32_t phase = 0, qphase = 0, issued = 0, issued_par = 0;
+    bool ok = true, withheld = false, first_unit = false;
+    UnitSpan us;
+    while (ok) {
+      if (rank == 0) {
+        ok = __all_sync(0xffffffffu, wait_bounded(qempty0 + 8u * qs, qphase ^ 1u, ctl));
+        if (!ok) break;
+        if (lane == 0) {
+          const int u = atomicAdd(w.counter, 1);
+          WorkUnit wu;
+          if (u < w.nunits) wu = w.units[u];
+          else wu.strip = -1;
+          if (u == 0) first_unit = true;
+          qunit[qs] = wu;
+          if (kPair) {
+            const uint32_t at = ptx::mapa(ptx::smem_u32(qunit + qs), 1);
+            const int4* v = reinterpret_cast<const int4*>(qunit + qs);
+            ptx::st_remote(at, v[0]);
+            ptx::st_remote(at + 16u, v[1]);
+            ptx::mbar_arrive_remote(ptx::mapa(qfull0 + 8u * qs, 1));
+          }
+          ptx::mbar_arrive(qfull0 + 8u * qs);
         }
-        if (u >= w.nunits) break;
-        if (!unit_span(wu, p.sr.s, 0, us)) continue;
-        for (int it = 0; ok && it < us.ntiles; ++it) {
-          const int c0 = us.row_base + us.jlo + it * us.adv;
-          const int a0 = us.row_base + us.T0;
-          for (int kb = 0; kb < nkb; ++kb) {
-            if (!wait_bounded(empty0 + 8u * stage, phase ^ 1u, ctl)) {
-              ok = false;
-              break;
-            }
-            if (a.debug_withhold && u == 0 && !withheld) {
-              withheld = true;  // test hook: unit 0's first stage is never filled
-            } else {
-              const uint32_t fb = full0 + 8u * stage;
-              const uint32_t sb = ring + (uint32_t)stage * p.stage_bytes;
-              ptx::mbar_arrive_expect_tx(fb, p.stage_bytes);
-              // the strip operand (A) is read again for every tile of the unit: keep it
-              // in L2 ahead of the column tiles when asked to
-              if (a.l2_keep_a) {
-                ptx::tma_load_2d_hint(sb, &tmA_hi, fb, kb * KC, a0, pol_a);
-                if (p.split) ptx::tma_load_2d_hint(sb + kTileA, &tmA_lo, fb, kb * KC, a0, pol_a);
+        first_unit = __shfl_sync(0xffffffffu, first_unit, 0);
+        __syncwarp();
+      } else {
+        ok = __all_sync(0xffffffffu, wait_bounded<kPair>(qfull0 + 8u * qs, qphase, ctl));
+        if (!ok) break;
+      }
+      const WorkUnit wu = read_unit(qs);
+      __syncwarp();
+      if (rank && lane == 0) ptx::mbar_arrive_remote(ptx::mapa(qempty0 + 8u * qs, 0));
+      if (++qs == kQueue) {
+        qs = 0;
+        qphase ^= 1u;
+      }
+      if (wu.strip < 0) break;
+      if (!unit_span(wu, p.sr.s, 0, us, rank, w.sym)) continue;
+      const int ntiles = us.ntiles, a0 = us.row_base + us.T0;
+      for (int it = 0; ok && it < ntiles; ++it) {
+        const int c0 = us.row_base + us.jt0 + it * us.adv + (kPair ? rank * BM : 0);
+        for (int kb = 0; kb < nkb; ++kb) {
+          ok = __all_sync(0xffffffffu, wait_bounded(empty0 + 8u * stage, phase ^ 1u, ctl));
+          if (!ok) break;
+          if (a.debug_withhold && first_unit && !withheld) {
+            withheld = true;  // test hook: unit 0's first stage is never filled
+          } else {
+            const uint32_t fb = full0 + 8u * stage;
+            const uint32_t sb = ring + (uint32_t)stage * p.stage_bytes;
+            if (ptx::elect_one()) {
+              if (kPair) {
+                // both CTAs' copies complete on the first one's barrier
+                const uint32_t lb = ptx::mapa(fb, 0);
+                if (rank == 0) ptx::mbar_arrive_expect_tx(fb, 2 * p.stage_bytes);
+                const uint32_t sB = sb + (p.split ? 2 * kTileA : kTileA);
+                ptx::tma_load_2d_pair(sb, &tmA_hi, lb, kb * KC, a0);
+                ptx::tma_load_2d_pair(sB, &tmA_hi, lb, kb * KC, c0);
+                if (p.split) {
+                  ptx::tma_load_2d_pair(sb + kTileA, &tmA_lo, lb, kb * KC, a0);
+                  ptx::tma_load_2d_pair(sB + kTileA, &tmA_lo, lb, kb * KC, c0);
+                }
               } else {
-                ptx::tma_load_2d(sb, &tmA_hi, fb, kb * KC, a0);
-                if (p.split) ptx::tma_load_2d(sb + kTileA, &tmA_lo, fb, kb * KC, a0);
+                ptx::mbar_arrive_expect_tx(fb, p.stage_bytes);
+                // the strip operand (A) is read again for every tile of the unit: keep it
+                // in L2 ahead of the column tiles when asked to
+                if (a.l2_keep_a) {
+                  ptx::tma_load_2d_hint(sb, &tmA_hi, fb, kb * KC, a0, pol_a);
+                  if (p.split)
+                    ptx::tma_load_2d_hint(sb + kTileA, &tmA_lo, fb, kb * KC, a0, pol_a);
+                } else {
+                  ptx::tma_load_2d(sb, &tmA_hi, fb, kb * KC, a0);
+                  if (p.split) ptx::tma_load_2d(sb + kTileA, &tmA_lo, fb, kb * KC, a0);
+                }
+                if (p.split) {
+                  ptx::tma_load_2d(sb + 2 * kTileA, &tmB_hi, fb, kb * KC, c0);
+                  ptx::tma_load_2d(sb + 2 * kTileA + kTileB, &tmB_lo, fb, kb * KC, c0);
+                } else {
+                  ptx::tma_load_2d(sb + kTileA, &tmB_hi, fb, kb * KC, c0);
+                }
               }
-              if (p.split) {
-                ptx::tma_load_2d(sb + 2 * kTileA, &tmB_hi, fb, kb * KC, c0);
-                ptx::tma_load_2d(sb + 2 * kTileA + kTileB, &tmB_lo, fb, kb * KC, c0);
-              } else {
-                ptx::tma_load_2d(sb + kTileA, &tmB_hi, fb, kb * KC, c0);
-              }
-              issued |= 1u << stage;
-              issued_par = (issued_par & ~(1u << stage)) | (phase << stage);
             }
-            if (++stage == NS) {
-              stage = 0;
-              phase ^= 1u;
-            }
+            issued |= 1u << stage;
+            issued_par = (issued_par & ~(1u << stage)) | (phase << stage);
+          }
+          if (++stage == NS) {
+            stage = 0;
+            phase ^= 1u;
           }
         }
       }
-      // every copy issued into this CTA's shared memory must land before exit
-      for (int i = 0; i < NS; ++i)
-        if ((issued >> i) & 1u) wait_bounded(full0 + 8u * i, (issued_par >> i) & 1u, ctl, false);
     }
+    // every copy issued into this CTA's shared memory must land before exit (in a pair the
+    // first CTA waits for both: its barriers count the other's copies too)
+    for (int i = 0; rank == 0 && i < NS; ++i)
+      if ((issued >> i) & 1u) wait_bounded(full0 + 8u * i, (issued_par >> i) & 1u, ctl, false);
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // The whole warp walks the units and waits; an elected lane issues. Everything an MMA
+    // needs is then uniform over the warp, and the instruction takes its descriptors from
+    // uniform registers directly: issued by a lane of a divergent branch, each MMA waited
+    // for its operands to be moved there and took 172 cycles instead of 128, whatever the
+    // data, the clock or the operand traffic.
+    if (rank == 0) {
       int stage = 0, qs = 0, gt = 0, gs = 0, acc = 0;  // gs: segments issued so far
       uint32_t phase = 0, qphase = 0;
       bool ok = true, issued_any = false;
       long long wait_tmem = 0, wait_full = 0;
       const long long t_start = clock64();
       UnitSpan us;
+      auto commit = [&](uint32_t b) {
+        if (kPair) ptx::mma_commit_pair(b);
+        else ptx::mma_commit(b);
+      };
+      auto mma = [&](uint32_t d, uint64_t da, uint64_t db, uint32_t accumulate) {
+        if (kPair) ptx::mma_f16_pair(d, da, db, kIdescPair, accumulate);
+        else ptx::mma_f16(d, da, db, kIdesc, accumulate);
+      };
+      // descriptors of stage 0's operands (a stage or 16 K entries further: a plain offset)
+      const uint64_t desc_a = ptx::sdesc_kmajor_sw64(ring);
+      const uint64_t desc_b = ptx::sdesc_kmajor_sw64(ring + (p.split ? 2 * kTileA : kTileA));
+      constexpr uint32_t kLoA = kTileA >> 4;                         // hi to lo copy
+      constexpr uint32_t kLoB = (kPair ? kTileA : kTileB) >> 4;      // (a pair: 128 rows each)
       while (ok) {
-        if (!wait_bounded(qfull0 + 8u * qs, qphase, ctl)) {
-          ok = false;
-          break;
-        }
+        ok = __all_sync(0xffffffffu, wait_bounded(qfull0 + 8u * qs, qphase, ctl));
+        if (!ok) break;
         const WorkUnit wu = read_unit(qs);
-        ptx::mbar_arrive(qempty0 + 8u * qs);
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(qempty0 + 8u * qs);
         if (++qs == kQueue) {
           qs = 0;
           qphase ^= 1u;
         }
         if (wu.strip < 0) break;
-        if (!unit_span(wu, p.sr.s, 0, us)) continue;
-        for (int it = 0; ok && it < us.ntiles; ++it, ++gt) {
+        if (!unit_span(wu, p.sr.s, 0, us, 0, w.sym)) continue;
+        const int ntiles = us.ntiles;
+        for (int it = 0; ok && it < ntiles; ++it, ++gt) {
           for (int kb = 0; kb < nkb; ++kb) {
             if (kb % seg_kb == 0) {
               // a new segment: segment gs uses accumulator gs & 1 for the (gs >> 1)-th time
               if (kb > 0) {
-                ptx::mma_commit(tfull0 + 8u * acc);  // the finished segment to the epilogue
+                if (ptx::elect_one()) commit(tfull0 + 8u * acc);  // the finished segment
                 ++gs;
               }
               acc = gs & 1;
               const long long tw0 = w.stats ? clock64() : 0;
-              if (!wait_bounded(tempty0 + 8u * acc, ((gs >> 1) & 1) ^ 1u, ctl)) {
-                ok = false;
-                break;
-              }
+              ok = __all_sync(0xffffffffu, wait_bounded<kPair>(tempty0 + 8u * acc,
+                                                               ((gs >> 1) & 1) ^ 1u, ctl));
+              if (!ok) break;
               if (w.stats) wait_tmem += clock64() - tw0;
               ptx::tc_fence_after();
             }
             const uint32_t d = tmem_base + (uint32_t)(acc * BN);
             const long long tf0 = w.stats ? clock64() : 0;
-            if (!wait_bounded(full0 + 8u * stage, phase, ctl)) {
-              ok = false;
-              break;
-            }
+            ok = __all_sync(0xffffffffu, wait_bounded(full0 + 8u * stage, phase, ctl));
+            if (!ok) break;
             if (w.stats) wait_full += clock64() - tf0;
             ptx::tc_fence_after();
-            const uint32_t sb = ring + (uint32_t)stage * p.stage_bytes;
-            const uint32_t a_hi = sb;
-            const uint32_t a_lo = sb + kTileA;
-            const uint32_t b_hi = p.split ? sb + 2 * kTileA : sb + kTileA;
-            const uint32_t b_lo = b_hi + kTileB;
+            const uint32_t off = ((uint32_t)stage * p.stage_bytes) >> 4;
             const uint32_t first = kb % seg_kb == 0 ? 1u : 0u;
+            if (ptx::elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < KC / 16; ++kk) {
-              const uint64_t dah = ptx::sdesc_kmajor_sw64(a_hi + kk * 32);
-              const uint64_t dbh = ptx::sdesc_kmajor_sw64(b_hi + kk * 32);
-              ptx::mma_f16(d, dah, dbh, kIdesc, (first && kk == 0) ? 0u : 1u);
-              if (p.split) {
-                const uint64_t dal = ptx::sdesc_kmajor_sw64(a_lo + kk * 32);
-                const uint64_t dbl = ptx::sdesc_kmajor_sw64(b_lo + kk * 32);
-                ptx::mma_f16(d, dah, dbl, kIdesc, 1u);
-                ptx::mma_f16(d, dal, dbh, kIdesc, 1u);
+              for (int kk = 0; kk < KC / 16; ++kk) {
+                const uint64_t dah = desc_a + (off + 2 * kk), dbh = desc_b + (off + 2 * kk);
+                mma(d, dah, dbh, (first && kk == 0) ? 0u : 1u);
+                if (p.split) {
+                  mma(d, dah, dbh + kLoB, 1u);
+                  mma(d, dah + kLoA, dbh, 1u);
+                }
               }
+              commit(empty0 + 8u * stage);  // frees the stage once these MMAs finish
             }
             issued_any = true;
-            ptx::mma_commit(empty0 + 8u * stage);  // frees the stage once these MMAs finish
             if (++stage == NS) {
               stage = 0;
               phase ^= 1u;
             }
           }
           if (!ok) break;
-          ptx::mma_commit(tfull0 + 8u * acc);  // the tile's last segment
+          if (ptx::elect_one()) commit(tfull0 + 8u * acc);  // the tile's last segment
           ++gs;
         }
       }
-      if (w.stats) {
+      if (w.stats && lane == 0) {
         atomicAdd(w.stats + kStatMmaWaitTmem, (unsigned long long)wait_tmem);
         atomicAdd(w.stats + kStatMmaWaitFull, (unsigned long long)wait_full);
         atomicAdd(w.stats + kStatMmaCycles, (unsigned long long)(clock64() - t_start));
       }
       if (!ok && issued_any) {
-        // all MMAs of this thread must finish before TMEM is released
-        ptx::mma_commit(drain);
+        // all MMAs of the elected lane must finish before TMEM is released
+        if (ptx::elect_one()) commit(drain);
         wait_bounded(drain, 0, ctl, false);
       }
     }
@@ -416,6 +488,17 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     // reads only its own row, so warps fold independently.
     int pt = 0, pseg = 0;
     long long fold_cycles = 0;
+    // this thread has read accumulator b out (in a pair the first CTA's barrier counts the
+    // warps of both)
+    auto release = [&](int b) {
+      ptx::tc_fence_before();
+      if (kPair) {
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive_remote(ptx::mapa(tempty0 + 8u * b, 0));
+      } else {
+        ptx::mbar_arrive(tempty0 + 8u * b);
+      }
+    };
     float4* const scr = reinterpret_cast<float4*>(a.scratch) + (size_t)blockIdx.x * (2 * BM * BN / 4);
     auto fold = [&](bool block, int upto) -> bool {
       while (nseg > 1 && pt <= upto) {
@@ -450,8 +533,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
               atomicAdd(srow + (c * 8 + g) * BM, r);
           }
         }
-        ptx::tc_fence_before();
-        ptx::mbar_arrive(tempty0 + 8u * b);  // the accumulator is free for the next segment
+        release(b);  // the accumulator is free for the next segment
         if (timed) fold_cycles += clock64() - f0;
         if (++pseg == nseg - 1) {
           pseg = 0;
@@ -479,7 +561,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
       float w[2], t[2], c[2], wt, cr, thr;
     } hd;
     auto fetch_head = [&](const UnitSpan& s, int it) {
-      const int c0 = s.jlo + it * s.adv, t = s.T0 + l, N = s.M + s.L - 1;
+      const int c0 = s.jt0 + it * s.adv, t = s.T0 + l, N = s.M + s.L - 1;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int x = et + kEpiThreads * h, j = c0 - (s.L - 1) + x;
@@ -494,7 +576,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
       hd.cr = t < N ? a.cval[s.row_base + t] : 0.f;
     };
     while (ok) {
-      bool wok = wait_bounded(qfull0 + 8u * qs, qphase, ctl);
+      bool wok = wait_bounded<kPair>(qfull0 + 8u * qs, qphase, ctl);
       WorkUnit wu;
       wu.strip = -1;
       if (wok) wu = read_unit(qs);
@@ -503,13 +585,16 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         ok = false;
         break;
       }
-      if (et == 0) ptx::mbar_arrive(qempty0 + 8u * qs);
+      if (et == 0) {
+        if (rank) ptx::mbar_arrive_remote(ptx::mapa(qempty0 + 8u * qs, 0));
+        else ptx::mbar_arrive(qempty0 + 8u * qs);
+      }
       if (++qs == kQueue) {
         qs = 0;
         qphase ^= 1u;
       }
       if (wu.strip < 0) break;
-      if (!unit_span(wu, p.sr.s, 0, us)) continue;
+      if (!unit_span(wu, p.sr.s, 0, us, rank, w.sym)) continue;
       fetch_head(us, 0);
       // Series that share this unit's Gram tiles (several trajectory lengths of one
       // record) are served one after another from the same accumulator; their row
@@ -558,7 +643,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
             rs.rec = a.part +
                      (size_t)(us.part_base + (long long)t * us.slots + us.slot * G + gid) * a.cap;
         }
-        const int c0 = us.jlo + it * us.adv;
+        const int c0 = us.jt0 + it * us.adv;
         // W and row bounds of this tile's output columns j = c0 - (L-1) + x (the
         // previous pass's readers passed its last barrier)
 #pragma unroll
@@ -570,10 +655,10 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         ptx::named_bar_sync(bar, kEpiThreads);  // read by every thread of the group
         const UnitSpan cu = us;  // this pass; `us` moves on to the next one
         if (sj + 1 < nser) {
-          unit_span(wu, p.sr.s, sj + 1, us);
+          unit_span(wu, p.sr.s, sj + 1, us, rank, w.sym);
           fetch_head(us, it);
         } else if (it + 1 < ntiles) {
-          if (nser > 1) unit_span(wu, p.sr.s, 0, us);  // (a band unit of several tiles)
+          if (nser > 1) unit_span(wu, p.sr.s, 0, us, rank, w.sym);  // (a band unit of several tiles)
           fetch_head(us, it + 1);
         }
         lap(1);
@@ -648,8 +733,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
             }
             if (sj == nser - 1) {
               // the accumulator has been read out: hand it back to the MMA warp
-              ptx::tc_fence_before();
-              ptx::mbar_arrive(tempty0 + 8u * acc_l);
+              release(acc_l);
             }
           }
           lap(2);
@@ -783,9 +867,11 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   }
 
   __syncthreads();
+  if (kPair) ptx::cluster_sync();  // neither CTA leaves while the other may still reach it
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem_base, 512);
+    if (kPair) ptx::tmem_dealloc_pair(tmem_base, 512);
+    else ptx::tmem_dealloc(tmem_base, 512);
   }
 }
 
@@ -826,31 +912,35 @@ size_t epilogue_bytes(int k, int L, int G) {
          kQueue * sizeof(WorkUnit) + 16;
 }
 
-int pick_stages(bool split, int k, int L, int G) {
-  const uint32_t stage = split ? 2 * kTileA + 2 * kTileB : kTileA + kTileB;
+uint32_t stage_bytes(bool split, bool pair) {
+  return (split ? 2 : 1) * (kTileA + (pair ? kTileA : kTileB));
+}
+
+int pick_stages(bool split, bool pair, int k, int L, int G) {
+  const uint32_t stage = stage_bytes(split, pair);
   const size_t avail = kSmemLimit - 1024 - epilogue_bytes(k, L, G);
   int ns = (int)(avail / stage);
   return ns < kMaxStages ? ns : kMaxStages;
 }
 
-template <int G, bool kWin, bool kBand, bool kLarge>
+template <int G, bool kWin, bool kBand, bool kLarge, bool kPair = false>
 cudaError_t launch_g(const CUtensorMap& mAh, const CUtensorMap& mAl, const CUtensorMap& mBh,
                      const CUtensorMap& mBl, const TcParams& p, int num_ctas, size_t smem,
                      cudaStream_t st) {
-  cudaError_t err = cudaFuncSetAttribute(fused_tc_kernel<G, kWin, kBand, kLarge>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const auto kernel = fused_tc_kernel<G, kWin, kBand, kLarge, kPair>;
+  cudaError_t err =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  return launch_chained(fused_tc_kernel<G, kWin, kBand, kLarge>, num_ctas, kThreadsG(G), smem, st,
-                        mAh, mAl, mBh, mBl, p);
+  return launch_chained_clusters(kernel, kPair ? 2 : 1, kPair ? num_ctas / 2 * 2 : num_ctas,
+                                 kThreadsG(G), smem, st, mAh, mAl, mBh, mBl, p);
 }
 
 }  // namespace
 
 bool tc_available() { return encode_fn() != nullptr; }
 
-size_t fused_tc_smem_bytes(bool split, int kmax, int Lmax, int G) {
-  const uint32_t stage = split ? 2 * kTileA + 2 * kTileB : kTileA + kTileB;
-  return 1024 + (size_t)pick_stages(split, kmax, Lmax, G) * stage +
+size_t fused_tc_smem_bytes(bool split, bool pair, int kmax, int Lmax, int G) {
+  return 1024 + (size_t)pick_stages(split, pair, kmax, Lmax, G) * stage_bytes(split, pair) +
          epilogue_bytes(kmax, Lmax, G);
 }
 
@@ -872,22 +962,29 @@ cudaError_t launch_fused_tc(const void* hi, const void* lo, bool split, const Tc
   p.w = w;
   p.sr = sr;
   p.split = split ? 1 : 0;
-  p.stage_bytes = split ? 2 * kTileA + 2 * kTileB : kTileA + kTileB;
+  const bool pair = a.pair != 0 && w.write_lists;
+  p.stage_bytes = stage_bytes(split, pair);
   const int G = a.egroups;
   // two epilogue groups: one accumulation segment (checked on the host: the kernel's
   // two-group form folds no segments)
   // and k <= 32
   if (G != 1 && (G != 2 || a.Dp > a.seg_k || a.kmax > 32)) return cudaErrorInvalidValue;
-  p.nstages = pick_stages(split, a.kmax, a.Lmax, G);
+  p.nstages = pick_stages(split, pair, a.kmax, a.Lmax, G);
+  if (pair && (G != 1 || num_ctas < 2)) return cudaErrorInvalidValue;
   if (p.nstages < 2) return cudaErrorInvalidValue;
   if (a.seg_k < KC || a.seg_k % KC != 0) return cudaErrorInvalidValue;
   p.seg_kb = a.seg_k / KC;
-  const size_t smem = fused_tc_smem_bytes(split, a.kmax, a.Lmax, G);
+  const size_t smem = fused_tc_smem_bytes(split, pair, a.kmax, a.Lmax, G);
   const bool win = a.Lmax > 1, band = !w.write_lists, large = a.kmax > (band ? 32 : 40);
   auto go = [&](auto fn) { return fn(mAh, mAl, mBh, mBl, p, num_ctas, smem, st); };
   if (G == 2) {
     if (band) return win ? go(launch_g<2, true, true, false>) : go(launch_g<2, false, true, false>);
     return win ? go(launch_g<2, true, false, false>) : go(launch_g<2, false, false, false>);
+  }
+  if (pair) {
+    if (large)
+      return win ? go(launch_g<1, true, false, true, true>) : go(launch_g<1, false, false, true, true>);
+    return win ? go(launch_g<1, true, false, false, true>) : go(launch_g<1, false, false, false, true>);
   }
   if (large) {
     if (band) return win ? go(launch_g<1, true, true, true>) : go(launch_g<1, false, true, true>);

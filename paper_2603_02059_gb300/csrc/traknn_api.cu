@@ -48,6 +48,9 @@ struct TcPlan {
   // (stored after every main unit). One phase: pstrip empty, pu = {0, nunits},
   // pb = {nunits, nunits + nband}.
   std::vector<int> pstrip, pu, pb;
+  // Main units of CTA pairs (two neighbouring strips, the Gram tiles of the first), stored
+  // after all others; phase q's are units[pp[q] .. pp[q+1]). Empty: single CTAs.
+  std::vector<int> pp;
   int egroups = 1;  // epilogue groups of the fused kernel; each writes its own row lists
   int mask_words = 1;  // 32-bit words per row of the non-empty column-list masks
   int sym = 1;         // upper triangle with column lists, or both triangles
@@ -302,6 +305,26 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
   p.col_lists = col_base;
 }
 
+// The main units of CTA pairs from those of single CTAs: within a phase's strips (or a
+// part's) every other strip's units, whose columns include those of the strip after it.
+void pair_units(TcPlan& p) {
+  const int K = (int)p.pu.size() - 1;
+  p.pp.assign(1, (int)p.units.size());
+  for (int q = 0; q < K; ++q) {
+    for (int u = p.pu[q]; u < p.pu[q + 1]; ++u) {
+      WorkUnit w = p.units[u];
+      const SeriesInfo& si = p.table.s[w.series];
+      const int strips = (si.M + si.rows_out - 1) / si.rows_out;
+      const int lo = K > 1 ? p.pstrip[q + 1] : std::max(0, p.part_lo);
+      const int hi = K > 1 ? p.pstrip[q] : std::min(strips, p.part_hi);
+      if ((w.strip - lo) % 2 != 0) continue;
+      w.pad[1] = w.strip + 1 < hi ? 1 : 0;
+      p.units.push_back(w);
+    }
+    p.pp.push_back((int)p.units.size());
+  }
+}
+
 traknn_status check_handle(traknn_handle h) {
   if (!h) return TRAKNN_ERR_INVALID_ARG;
   if (cudaSetDevice(h->device) != cudaSuccess) return TRAKNN_ERR_CUDA;
@@ -395,23 +418,29 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   key.push_back((int64_t)pstrip.size());
   key.insert(key.end(), pstrip.begin(), pstrip.end());
   // Two epilogue groups (one accumulation segment, k <= 32) where the epilogue and not the
-  // contraction sets a tile's pace: K entries x products below a line, the more the series
-  // that scan each tile. Measured with one and two groups (N = 10,957, L = 5): split-BF16
-  // D = 1,476 684 / 633 us, 2,116 880 / 855, 2,800 1,020 / 1,056; BF16 D = 2,116 784 / 698,
-  // 2,800 878 / 837, 3,555 (N = 7,301, L = 7) 745 / 746; four lengths of a D = 3,726
-  // record 2,381 / 1,908.
+  // contraction sets a tile's pace: K entries below a line (the more the series that scan
+  // each tile), or hardly more tiles than SMs, so that a call is as long as one tile. Else
+  // one group and pairs of CTAs (kernel_tc.cu). Measured, two groups / pairs (N = 10,957, L =
+  // 5): split-BF16 D = 990 453 / 611 us, 1,476 552 / 639, 2,116 763 / 806, 3,726 1,291 /
+  // 997; BF16 D = 1,476 513 / 614, 3,726 1,009 / 880; D = 3,726, N = 1,826 230 / 240, 3,000
+  // 313 / 342, 4,500 368 / 371, 6,500 538 / 498.
   int Lmax = 1, kmax = 1;
+  double tiles_all = 0.0;  // Gram tiles of the call
   for (int b = 0; b < B; ++b) {
     Lmax = std::max(Lmax, sd[b].L);
     kmax = std::max(kmax, sd[b].k);
+    const double M = (double)(sd[b].N - sd[b].L + 1);
+    tiles_all += M * M / ((h->sym ? 2.0 : 1.0) * kTileRows * kTileCols);
   }
   const int Dk = tc_groups((int)D * emb) * 64;
-  const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2304 : 3584) * (shared ? B : 1);
+  const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2304 : 3072) * (shared ? B : 1);
   const bool fp32 = h->precision == TRAKNN_PREC_FP32;  // (its kernel has two groups)
   const int egroups =
-      fp32 || (h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k && (Lmax == 1 || Dk <= line))
+      fp32 || (h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k &&
+               (Lmax == 1 || Dk <= line || (!shared && tiles_all < 2.0 * h->sm_count)))
           ? 2
           : 1;
+  const bool pair = !fp32 && egroups == 1 && h->sm_count >= 2;
   key.push_back(egroups);
   // Band pre-pass width in tiles per strip. Short operand rows: a tile's contraction is cheap
   // and eight tiles save more list entries in the main pass than the band costs (D = 32, L =
@@ -452,6 +481,8 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     p.emb = emb;
     p.part_lo = part_lo;
     p.part_hi = part_hi;
+    p.pp.clear();
+    if (pair) pair_units(p);
     const size_t ub = align_up(p.units.size() * sizeof(WorkUnit), 256);
     const size_t cb = align_up(p.col_off.size() * sizeof(long long), 256);
     const size_t sb = align_up(p.slot_lo.size() * sizeof(int), 256);
@@ -532,6 +563,7 @@ void fused_args(const traknn_ctx* h, const TcBuffers& b, TcArgs* pa, TcWork* pw)
   a.cval = b.cval;
   a.l2_keep_a = h->l2_keep_a;
   a.egroups = p.egroups;
+  a.pair = p.pp.empty() ? 0 : 1;
   a.corr_neg = 0;
   a.band_margin = 0.f;
 
@@ -621,7 +653,10 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
   if (record_events) TRY_CUDA(cudaEventRecord(h->ev_start[slot], s));
   // threshold pre-pass over the band units (stored after the main units), then the rest
   if (p.band) TRY_ST(launch_units(h, b, a, w, p.nunits, p.nband, 1, true, s));
-  TRY_ST(launch_units(h, b, a, w, 0, p.nunits, 0, false, s));
+  if (a.pair)
+    TRY_ST(launch_units(h, b, a, w, p.pp[0], p.pp[1] - p.pp[0], 0, false, s));
+  else
+    TRY_ST(launch_units(h, b, a, w, 0, p.nunits, 0, false, s));
   if (record_events) {
     TRY_CUDA(cudaEventRecord(h->ev_stop[slot], s));
     h->ev_head = (h->ev_head + 1) % traknn_ctx::kRing;
@@ -685,7 +720,8 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
     // by an earlier phase
     TRY_ST(enqueue_prep(h, b, D, lo, hi, ohi, q == 0 ? 2 * K : 0, s));
     TRY_ST(launch_units(h, b, a, w, p.pb[q], p.pb[q + 1] - p.pb[q], 2 * q + 1, true, s));
-    TRY_ST(launch_units(h, b, a, w, p.pu[q], p.pu[q + 1] - p.pu[q], 2 * q, false, s));
+    const std::vector<int>& m = a.pair ? p.pp : p.pu;
+    TRY_ST(launch_units(h, b, a, w, m[q], m[q + 1] - m[q], 2 * q, false, s));
   }
   TRY_CUDA(launch_merge_tc(a, w, sr, s));
   h->launches += 1;
@@ -809,6 +845,27 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   while (*tiles > 2 && *tiles * Dp > 65536) *tiles /= 2;
 }
 
+// The unit length a forward call takes: one Gram tile for operand rows of more than 768 K
+// entries, whatever default_shape says. Issued at its full rate the contraction no longer
+// hides what the longer units cost at the end of a launch and in L2, and lists and bounds
+// that live for one tile cost little: 1 / 2 / 4 / 8 tiles, N = 27,394, D = 3,726, L = 5, k =
+// 20 4,949 / 5,062 / 5,905 / 5,945 us (the last two before the MMAs were issued by an
+// elected lane), N = 10,957 997 / 1,029, D = 58,101 91.9 / 94.4 ms, D = 990, N = 10,957 452 /
+// 473 us. Longer again while the call's row-side lists (one per row and unit) number more
+// than 4 M (4 GB).
+int unit_tiles(const HostSeries* sd, int B, int64_t D, int emb, int tiles) {
+  if (tc_groups((int)D * emb) * 64 <= 768) return tiles;
+  for (int t = 1; t < tiles; t *= 2) {
+    double lists = 0.0;
+    for (int b = 0; b < B; ++b) {
+      const double M = (double)(sd[b].N - sd[b].L + 1);
+      lists += M * std::ceil(M / (t * kTileCols - (sd[b].L - 1)));
+    }
+    if (lists <= 4e6) return t;
+  }
+  return tiles;
+}
+
 // Forward pass of B series on the tensor cores. With `graph` set the launch
 // sequence is captured once per (shape, pointers, options) and replayed.
 traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
@@ -818,7 +875,10 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   int tiles = 8, group = 0;
   const bool whole = part_lo == 0 && part_hi == INT_MAX;
   if (!shared && emb == 1 && whole) TRY_ST(pick_shape(h, sd, B, D, s, &tiles, &group));
-  if (!h->autotune && !shared) default_shape(h, sd, B, D, emb, part_lo, part_hi, &tiles, &group);
+  if (!h->autotune && !shared) {
+    default_shape(h, sd, B, D, emb, part_lo, part_hi, &tiles, &group);
+    if (h->precision != TRAKNN_PREC_FP32) tiles = unit_tiles(sd, B, D, emb, tiles);
+  }
   // FP32: a tile's contraction takes so long that the units must be short for the CTAs to
   // end together, except at few grid points. 1 / 2 / 4 / 8 tiles: D = 3,726, N = 27,394 60.5 /
   // 60.3 / 60.8 / 62.7 ms, N = 10,957 10.8 / 11.2 / 12.0 / 12.8; D = 200, N = 10,957 1,056 /
@@ -1191,6 +1251,7 @@ traknn_status traknn_knn_scores_host(traknn_handle h, const float* Xh, int64_t N
     const HostSeries sd{Xd, N, L, k, e, idx_d, dist_d, score_d};
     int tiles = 8, group = 0;
     default_shape(h, &sd, 1, D, 1, 0, INT_MAX, &tiles, &group);
+    tiles = unit_tiles(&sd, 1, D, 1, tiles);
     TcBuffers buf;
     TRY_ST(prepare_tc(h, &sd, 1, D, tiles, false, 1, s, &buf, 0, INT_MAX, ps, group));
     const size_t row = (size_t)D * sizeof(float);
