@@ -250,7 +250,6 @@ struct TcArgs {
   int groups;          // K groups of the operand layout (see tc_groups)
   const float* cval;   // [rows] correction value c of every stacked operand row
   int l2_keep_a;       // 1: load the strip operand with an L2 evict-last policy
-  float* scratch;      // [CTAs][2][128 x 256] running tile totals (more than one segment)
   int egroups;         // epilogue groups of the tensor-core kernel (1 or 2)
   int pair;            // 1: the units are those of CTA pairs (main pass, one epilogue group)
   // Band pre-pass in one BF16 product (hi only) on split operands: the correction
@@ -270,11 +269,6 @@ struct TcArgs {
 // Slots of the rows' shared minima (a multiple of 32): with k of 64 slots the bound is
 // that of about the 1.2 k-th nearest column at k = 20 and the 1.6 k-th at k = 40.
 __host__ __device__ inline int min_slots(int kmax) { return kmax <= 40 ? 64 : 128; }
-
-// Bytes of TcArgs::scratch for a launch of `num_ctas` CTAs.
-inline size_t tc_scratch_bytes(int num_ctas) {
-  return (size_t)num_ctas * 2 * kTileRows * kTileCols * sizeof(float);
-}
 
 // Event counters of the tensor-core kernel (diagnostics, TRAKNN_OPT_STATS).
 enum : int {

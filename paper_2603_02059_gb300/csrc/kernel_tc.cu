@@ -19,14 +19,13 @@
 //            32 elements into a ring of shared-memory stages (hi and lo copies);
 //   warp 1   tcgen05.mma issuer into one of two 128 x 256 FP32 accumulators in
 //            TMEM (512 columns). The K range of a tile is cut into segments
-//            (8192 elements by default); every segment accumulates afresh into
-//            the next accumulator, so segment s+1 multiplies while segment s is
-//            read out. With more than one segment per tile the epilogue adds every
-//            segment but the last, in FP32 on the CUDA cores, into a running total
-//            of the tile in a per-CTA scratch array (L2-resident), and adds the last
-//            from TMEM while scanning: the tensor cores never accumulate more than
-//            one segment of products per output, which bounds the error of their
-//            accumulation however large D is;
+//            (8192 elements by default) that accumulate afresh: the tensor cores never
+//            accumulate more than one segment of products per output, which bounds the
+//            error of their accumulation however large D is. A tile's first segment goes
+//            to one accumulator and stays there as its running total; every other one
+//            goes to the other accumulator, from where the epilogue adds it to the total
+//            in FP32 on the CUDA cores. The next tile takes them the other way round, so
+//            its first segment multiplies while the total is scanned;
 //   warps 2-  epilogue, in one or two groups of four warps (two split a tile's columns):
 //            each thread owns one accumulator row (TMEM lane), pulls 32 columns at a
 //            time with tcgen05.ld, stages them beside the L-1 columns carried from the
@@ -218,8 +217,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   const uint32_t tmem_base = *tmem_slot;
   const int nkb = a.Dp / KC;
   const int seg_kb = p.seg_kb;                    // K blocks per accumulation segment
-  // segments per tile (the two-group form runs with one segment: checked on the host)
-  const int nseg = G == 2 ? 1 : (nkb + seg_kb - 1) / seg_kb;
+  const int nseg = (nkb + seg_kb - 1) / seg_kb;  // segments per tile
   auto read_unit = [&](int slot) {  // a queue slot, by 16-byte reads
     union {
       int4 v[2];
@@ -349,7 +347,8 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     // for its operands to be moved there and took 172 cycles instead of 128, whatever the
     // data, the clock or the operand traffic.
     if (rank == 0) {
-      int stage = 0, qs = 0, gt = 0, gs = 0, acc = 0;  // gs: segments issued so far
+      int stage = 0, qs = 0, gt = 0, acc = 0;
+      uint32_t used = 0;  // bit b: parity of the segments that accumulator b has taken
       uint32_t phase = 0, qphase = 0;
       bool ok = true, issued_any = false;
       long long wait_tmem = 0, wait_full = 0;
@@ -384,15 +383,13 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         for (int it = 0; ok && it < ntiles; ++it, ++gt) {
           for (int kb = 0; kb < nkb; ++kb) {
             if (kb % seg_kb == 0) {
-              // a new segment: segment gs uses accumulator gs & 1 for the (gs >> 1)-th time
-              if (kb > 0) {
-                if (ptx::elect_one()) commit(tfull0 + 8u * acc);  // the finished segment
-                ++gs;
-              }
-              acc = gs & 1;
+              // a new segment: the first of a tile to accumulator gt & 1, others to the other
+              if (kb > 0 && ptx::elect_one()) commit(tfull0 + 8u * acc);  // the finished one
+              acc = (gt & 1) ^ (kb > 0 ? 1 : 0);
               const long long tw0 = w.stats ? clock64() : 0;
               ok = __all_sync(0xffffffffu, wait_bounded<kPair>(tempty0 + 8u * acc,
-                                                               ((gs >> 1) & 1) ^ 1u, ctl));
+                                                               ((used >> acc) & 1u) ^ 1u, ctl));
+              used ^= 1u << acc;
               if (!ok) break;
               if (w.stats) wait_tmem += clock64() - tw0;
               ptx::tc_fence_after();
@@ -425,7 +422,6 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           }
           if (!ok) break;
           if (ptx::elect_one()) commit(tfull0 + 8u * acc);  // the tile's last segment
-          ++gs;
         }
       }
       if (w.stats && lane == 0) {
@@ -479,15 +475,6 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         tp = now;
       }
     };
-    // Segment folding (more than one segment per tile): segment pseg of tile pt is
-    // the next to add to the tile's partial total; every segment but a tile's last
-    // is folded (segment s of tile t is segment t * nseg + s overall, in accumulator
-    // (t * nseg + s) & 1), the last is added while the tile is scanned. The partial
-    // totals live in this CTA's scratch array, two tile slots of
-    // [8 chunks][8 float4 groups][128 rows] float4; each thread folds and later
-    // reads only its own row, so warps fold independently.
-    int pt = 0, pseg = 0;
-    long long fold_cycles = 0;
     // this thread has read accumulator b out (in a pair the first CTA's barrier counts the
     // warps of both)
     auto release = [&](int b) {
@@ -499,60 +486,40 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         ptx::mbar_arrive(tempty0 + 8u * b);
       }
     };
-    float4* const scr = reinterpret_cast<float4*>(a.scratch) + (size_t)blockIdx.x * (2 * BM * BN / 4);
-    auto fold = [&](bool block, int upto) -> bool {
-      while (nseg > 1 && pt <= upto) {
-        const long long gsi = (long long)pt * nseg + pseg;
-        const int b = (int)(gsi & 1);
-        const uint32_t par = (uint32_t)((gsi >> 1) & 1);
-        if (!block) {
-          const bool r = ptx::mbar_try_wait(tfull0 + 8u * b, par);
-          if (!__shfl_sync(0xffffffffu, r, 0)) return true;  // not ready: try later
-        }
-        if (!wait_bounded(tfull0 + 8u * b, par, ctl)) return false;
-        const long long f0 = timed ? clock64() : 0;
+    uint32_t seen = 0;  // bit b: parity of the segments read from accumulator b
+    auto wait_acc = [&](int b) {
+      const bool r =
+          __all_sync(0xffffffffu, wait_bounded(tfull0 + 8u * b, (seen >> b) & 1u, ctl));
+      seen ^= 1u << b;
+      return r;
+    };
+    // Waits for tile gt's segments and adds all to the first one's accumulator, each thread
+    // its own row (this group's columns). Formerly the totals were a scratch array in L2,
+    // updated by FP32 reductions: D = 58,101, N = 27,394, where the power limit sets the
+    // clock, 93.9 -> 90.8 ms (86.2 -> 84.1 a call alone).
+    auto collect = [&](int total) -> bool {
+      if (!wait_acc(total)) return false;
+      ptx::tc_fence_after();
+      for (int sg = 1; sg < nseg; ++sg) {
+        if (!wait_acc(total ^ 1)) return false;
         ptx::tc_fence_after();
-        const uint32_t tA = tmem_base + lane_addr + (uint32_t)(b * BN);
-        float4* srow = scr + (size_t)(pt & 1) * (BM * BN / 4) + l;
-        // the first segment is stored, later ones are added by FP32 reductions in L2
-        // (round to nearest); every element has this thread as its only writer, so
-        // the additions happen in segment order and the total is deterministic
+        const uint32_t tT = tmem_base + lane_addr + (uint32_t)(total * BN);
+        const uint32_t tU = tmem_base + lane_addr + (uint32_t)((total ^ 1) * BN);
 #pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
-          uint32_t v[32];
-          ptx::tmem_ld32_async(tA + c * 32, v);
+        for (int c = ch_lo; c < ch_hi; ++c) {
+          uint32_t t[32], u[32];
+          ptx::tmem_ld32_async(tT + c * 32, t);
+          ptx::tmem_ld32_async(tU + c * 32, u);
           ptx::tmem_wait();
 #pragma unroll
-          for (int g = 0; g < 8; ++g) {
-            const float4 r = make_float4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]),
-                                         __uint_as_float(v[4 * g + 2]),
-                                         __uint_as_float(v[4 * g + 3]));
-            if (pseg == 0)
-              __stcg(srow + (c * 8 + g) * BM, r);
-            else
-              atomicAdd(srow + (c * 8 + g) * BM, r);
-          }
+          for (int x = 0; x < 32; ++x)
+            t[x] = __float_as_uint(__uint_as_float(t[x]) + __uint_as_float(u[x]));
+          ptx::tmem_st32(tT + c * 32, t);
         }
-        release(b);  // the accumulator is free for the next segment
-        if (timed) fold_cycles += clock64() - f0;
-        if (++pseg == nseg - 1) {
-          pseg = 0;
-          ++pt;
-        }
+        ptx::tmem_wait_st();
+        release(total ^ 1);
       }
       return true;
-    };
-    // 32 columns (chunk ch) of this thread's row of tile gt's total, from the scratch
-    auto load_scr = [&](int tile, int ch, uint32_t (&v)[32]) {
-      const float4* srow = scr + (size_t)(tile & 1) * (BM * BN / 4) + l;
-#pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        const float4 r = __ldcg(srow + (ch * 8 + g) * BM);
-        v[4 * g] = __float_as_uint(r.x);
-        v[4 * g + 1] = __float_as_uint(r.y);
-        v[4 * g + 2] = __float_as_uint(r.z);
-        v[4 * g + 3] = __float_as_uint(r.w);
-      }
     };
     // What a pass over a tile needs from global memory (window sums, bounds and
     // correction values of two of its 256 columns; the row's own values), fetched while
@@ -607,19 +574,13 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
       gm.reset();
       for (int it = 0; it < ntiles; ++it, ++gt) {
         lap(6);
-        // the earlier segments are folded into the scratch partial total; the last
-        // one is read from its accumulator while the tile is scanned
-        // accumulator holding the tile's last segment (the whole tile if nseg == 1)
-        const long long glast = (long long)gt * nseg + nseg - 1;
-        const int acc_l = (int)(glast & 1);
-        if (nseg > 1) wok = fold(true, gt);
-        if (wok) wok = wait_bounded(tfull0 + 8u * acc_l, (uint32_t)((glast >> 1) & 1), ctl);
+        const int acc_l = gt & 1;  // the accumulator of the tile's total
+        wok = collect(acc_l);
         wok = ptx::named_bar_and(bar, kEpiThreads, wok);  // all four warps agree
         if (!wok) {
           ok = false;
           break;
         }
-        ptx::tc_fence_after();
         lap(0);
         for (int sj = 0; sj < nser; ++sj) {
         const int L = kWin ? us.L : 1;
@@ -662,20 +623,12 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           fetch_head(us, it + 1);
         }
         lap(1);
-        // chunk ch+1 is fetched while chunk ch is scanned: from TMEM with a single
-        // segment, else the scratch partial total (the last segment's chunk is
-        // added from TMEM when the chunk is read)
+        // chunk ch+1 is fetched while chunk ch is scanned; with two epilogue groups (168
+        // registers a thread; the other group hides the latency) when it is read
         const uint32_t tlast = tmem_base + lane_addr + (uint32_t)(acc_l * BN);
-        // with two epilogue groups (168 registers a thread; the other group hides the
-        // latency) a chunk is fetched when it is read
         constexpr bool kAhead = G == 1;
         uint32_t vr[32];
-        if (kAhead) {
-          if (nseg == 1)
-            ptx::tmem_ld32_async(tlast + (uint32_t)(ch_lo * 32), vr);
-          else
-            load_scr(gt, ch_lo, vr);
-        }
+        if (kAhead) ptx::tmem_ld32_async(tlast + (uint32_t)(ch_lo * 32), vr);
         float* grow = Gbuf + l * LDG;
 #pragma unroll 1
         for (int ch = ch_lo; ch < ch_hi; ++ch) {
@@ -684,18 +637,9 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           // for the diagonal window sums, or, with L = 1 (no window), kept in registers
           float c[32];
           if (!kAhead) ptx::tmem_ld32_async(tlast + (uint32_t)(ch * 32), vr);
-          if (nseg == 1) {
-            ptx::tmem_wait();
+          ptx::tmem_wait();
 #pragma unroll
-            for (int x = 0; x < 32; ++x) c[x] = fmaf(crow, csh[x], __uint_as_float(vr[x]));
-          } else {
-            uint32_t tv[32];
-            ptx::tmem_ld32_async(tlast + (uint32_t)(ch * 32), tv);
-            ptx::tmem_wait();
-#pragma unroll
-            for (int x = 0; x < 32; ++x)
-              c[x] = fmaf(crow, csh[x], __uint_as_float(vr[x]) + __uint_as_float(tv[x]));
-          }
+          for (int x = 0; x < 32; ++x) c[x] = fmaf(crow, csh[x], __uint_as_float(vr[x]));
           if (kWin && L > 1) {
             // the diagonal carry: the L-1 Gram columns before the chunk start its
             // windows: the last ones of the group's previous chunk (of the previous tile
@@ -715,11 +659,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
             for (int x = 0; x < 32; ++x) grow[(L - 1) + x] = c[x];
           }
           if (ch + 1 < ch_hi) {
-            if (!kAhead) {
-            } else if (nseg == 1)
-              ptx::tmem_ld32_async(tlast + (uint32_t)((ch + 1) * 32), vr);
-            else
-              load_scr(gt, ch + 1, vr);
+            if (kAhead) ptx::tmem_ld32_async(tlast + (uint32_t)((ch + 1) * 32), vr);
           } else {
             // the first group's next tile starts from this tile's last columns, which the
             // second group reads: kept in vr until the chunk is done
@@ -801,8 +741,6 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           }
           cnt[4] += et == 0;
           lap(5);
-          fold(false, gt + 1);  // the next tile's finished segments, if any
-          lap(2);
         }
         const bool last = nser > 1 || it == ntiles - 1;
         if (last || (!kBand && (it + 1) % a.bound_tiles == 0)) {
@@ -862,7 +800,6 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
       lap(6);
       for (int i = 0; i < 6; ++i) atomicAdd(w.stats + kStatEpiWaitAcc + i, (unsigned long long)ph[i]);
       atomicAdd(w.stats + kStatEpiCycles, (unsigned long long)(clock64() - e_start));
-      atomicAdd(w.stats + kStatEpiStage, (unsigned long long)fold_cycles);
     }
   }
 
@@ -965,10 +902,7 @@ cudaError_t launch_fused_tc(const void* hi, const void* lo, bool split, const Tc
   const bool pair = a.pair != 0 && w.write_lists;
   p.stage_bytes = stage_bytes(split, pair);
   const int G = a.egroups;
-  // two epilogue groups: one accumulation segment (checked on the host: the kernel's
-  // two-group form folds no segments)
-  // and k <= 32
-  if (G != 1 && (G != 2 || a.Dp > a.seg_k || a.kmax > 32)) return cudaErrorInvalidValue;
+  if (G != 1 && (G != 2 || a.kmax > 32)) return cudaErrorInvalidValue;
   p.nstages = pick_stages(split, pair, a.kmax, a.Lmax, G);
   if (pair && (G != 1 || num_ctas < 2)) return cudaErrorInvalidValue;
   if (p.nstages < 2) return cudaErrorInvalidValue;

@@ -359,13 +359,12 @@ struct TcBuffers {
   int32_t* col_rec;
   unsigned int* col_mask;
   int* counter;
-  float* scratch;
   float* pscore;  // [out_rows] scores of partial lists (split series), not returned
   int Dp;
   size_t total;
 };
 
-TcBuffers tc_layout(const TcPlan& p, int64_t D, bool fp32, int num_ctas, char* base) {
+TcBuffers tc_layout(const TcPlan& p, int64_t D, bool fp32, char* base) {
   TcBuffers b;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -395,7 +394,6 @@ TcBuffers tc_layout(const TcPlan& p, int64_t D, bool fp32, int num_ctas, char* b
   b.col_mask = reinterpret_cast<unsigned int*>(
       take((size_t)p.out_rows * p.mask_words * sizeof(unsigned int)));
   b.counter = reinterpret_cast<int*>(take(256));
-  b.scratch = reinterpret_cast<float*>(take(fp32 ? 0 : tc_scratch_bytes(num_ctas)));
   b.pscore = reinterpret_cast<float*>(take((size_t)p.out_rows * sizeof(float)));
   b.total = off;
   return b;
@@ -503,9 +501,9 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     p.table.s[b].dist = sd[b].dist;
     p.table.s[b].score = sd[b].score;
   }
-  const TcBuffers probe = tc_layout(p, D, h->precision == TRAKNN_PREC_FP32, h->sm_count, nullptr);
+  const TcBuffers probe = tc_layout(p, D, h->precision == TRAKNN_PREC_FP32, nullptr);
   TRY_ST(ensure_buffer(h, &h->tcws, &h->tcws_bytes, probe.total));
-  *out = tc_layout(p, D, h->precision == TRAKNN_PREC_FP32, h->sm_count, static_cast<char*>(h->tcws));
+  *out = tc_layout(p, D, h->precision == TRAKNN_PREC_FP32, static_cast<char*>(h->tcws));
   for (int b = 0; b < B; ++b)  // partial lists: their scores go to the workspace
     if (!p.table.s[b].score) p.table.s[b].score = out->pscore + p.table.s[b].out_base;
   return TRAKNN_OK;
@@ -558,7 +556,6 @@ void fused_args(const traknn_ctx* h, const TcBuffers& b, TcArgs* pa, TcWork* pw)
   a.wait_limit_ns = (long long)h->wait_limit_ms * 1000000LL;
   a.debug_withhold = h->debug_withhold;
   a.seg_k = h->seg_k;
-  a.scratch = b.scratch;
   a.groups = b.Dp / 64;
   a.cval = b.cval;
   a.l2_keep_a = h->l2_keep_a;

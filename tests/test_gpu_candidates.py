@@ -83,3 +83,39 @@ def test_two_epilogue_groups_with_a_window_equal_one(tk, N, h, w, L, k, e):
         for a, b in ((got[0], got[2]), (got[1], got[3])):
             for x, y in zip(a, b):
                 assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("N,h,w,L,k,sym,seg", [
+    (1500, 9, 14, 5, 10, True, 0), (700, 9, 14, 2, 41, True, 0), (130, 9, 14, 3, 5, True, 0),
+    (900, 20, 40, 17, 20, False, 0), (1000, 20, 40, 1, 64, True, 0), (1100, 20, 40, 5, 20, True, 256),
+    (9000, 8, 9, 4, 10, True, 64)])
+def test_pairs_of_ctas_equal_two_groups(tk, N, h, w, L, k, sym, seg):
+    """Pairs of CTAs (one epilogue group) on single, split and host-array calls: odd numbers
+    of strips, parts that start on odd strips, both triangles, several segments; against two
+    epilogue groups on single CTAs where k allows them, else against the FP32 path."""
+    import torch
+    X = torch.from_numpy(make_slp_like(N, h, w, seed=N + k)[0])
+    Xd, e = X.cuda(), L - 1
+    one, two = tk.Handle(), tk.Handle()
+    one.set_option("epi_groups", 1)
+    for hd in (one, two):
+        hd.set_option("segment_k", seg)
+    kw = dict(symmetric=sym, embed="never", handle=one)
+    got = [tk.knn_scores(Xd, L, k, e, **kw)]
+    if sym:
+        got.append(tk.knn_scores_host(X, L, k, e, **kw))
+        P = 3
+        parts = [tk.knn_partial(Xd, L, k, e, p, P, handle=one) for p in range(P)]
+        got.append(tk.merge_partials(torch.stack([p[0] for p in parts]),
+                                     torch.stack([p[1] for p in parts]), handle=one))
+    ref = tk.knn_scores(Xd, L, k, e, symmetric=sym, embed="never", handle=two) if k <= 32 else \
+        tk.knn_scores(Xd, L, k, e, precision="fp32", handle=two)
+    torch.cuda.synchronize()
+    assert one.sync_status() == 0 and two.sync_status() == 0
+    for g in got:
+        if k <= 32:
+            assert all(torch.equal(x.cpu(), y.cpu()) for x, y in zip(g, ref))
+        else:
+            rel = (g[1].cpu() - ref[1].cpu()).abs() / ref[1].cpu()
+            assert rel.max().item() <= 2e-4
+            assert all(torch.equal(x.cpu(), y.cpu()) for x, y in zip(g, got[0]))
