@@ -563,35 +563,45 @@ struct ColSide {
 // row's distances; t: the row; first: the column list of the chunk's column 0 (output column
 // j0); rmin, cmin: the shared minima of the row and of column j0. Returns whether a column
 // is overfull.
+//
+// The warp runs as many rounds as its fullest row has candidates (two or three), without
+// divergent branches: a round's latency is what the loop costs, so the next distance is
+// read a round ahead and the column's counter is asked before the row's stores.
 template <int S>
 __device__ __forceinline__ bool append(RowSide& rs, const ColSide& cs, uint32_t cand,
                                        uint32_t ccand, const float* drow, int j0, int k, int t,
                                        long long first, unsigned* rmin, unsigned* cmin,
                                        const TcWork& w, const TcArgs& a) {
-  int* c = cs.counters();
-  const long long cp = col_pitch(w.kstride);
-  bool over = false;
   uint32_t both = cand | ccand;
-  while (both) {
-    const int x = __ffs(both) - 1;
-    both &= both - 1;
-    const int dv = __float_as_int(fmaxf(drow[x], 0.0f));
+  const int rounds = __reduce_max_sync(0xffffffffu, __popc(both));
+  if (rounds == 0) return false;
+  int* c = cs.counters();
+  const int cp = col_pitch(w.kstride) / 2;  // in entries
+  const long long at0 = first * cp + 1;
+  int2* col = reinterpret_cast<int2*>(w.col_rec) + at0;
+  unsigned* cm = cmin + (long long)(t & (S - 1)) * a.out_rows;
+  bool over = false;
+  int x = both ? __ffs(both) - 1 : 0;
+  float v = drow[x];
+  for (int i = 0; i < rounds; ++i) {
+    const bool act = both != 0;
+    const bool row = act && ((cand >> x) & 1u), cl = act && ((ccand >> x) & 1u);
+    const int y = x, dv = __float_as_int(fmaxf(v, 0.0f));
     const unsigned bits = (unsigned)dv & 0x7FFFFFFFu;
-    if ((cand >> x) & 1u) {
-      atomicMin(rmin + (long long)((j0 + x) & (S - 1)) * a.out_rows, bits);
-      if (tk_in(rs.n, a.cap, a.err)) rs.rec[rs.n] = make_int2(j0 + x, dv);
-      ++rs.n;
+    int pos = 0;
+    if (cl) pos = atomicAdd(c + y, 1);
+    both &= both - 1u;
+    x = both ? __ffs(both) - 1 : 0;
+    v = drow[x];
+    if (row) {
+      atomicMin(rmin + (long long)((j0 + y) & (S - 1)) * a.out_rows, bits);
+      if (tk_in(rs.n, a.cap, a.err)) rs.rec[rs.n] = make_int2(j0 + y, dv);
     }
-    if ((ccand >> x) & 1u) {
-      const int pos = atomicAdd(c + x, 1);
-      atomicMin(cmin + (long long)(t & (S - 1)) * a.out_rows + x, bits);
-      const long long at = (first + x) * cp + 2 + 2 * pos;
-      if (pos >= k) {
-        over = true;
-      } else if (tk_in(at + 1, w.col_ints, a.err)) {
-        *reinterpret_cast<int2*>(w.col_rec + at) = make_int2(t, dv);
-      }
-    }
+    rs.n += row ? 1 : 0;
+    if (cl) atomicMin(cm + y, bits);
+    if (cl && pos < k && tk_in(2 * (at0 + y * cp + pos) + 1, w.col_ints, a.err))
+      col[y * cp + pos] = make_int2(t, dv);
+    over |= cl && pos >= k;
   }
   return over;
 }

@@ -673,7 +673,7 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
 // is concentrated in few strips with few units each, so every phase ends with a tail
 // of idle SMs: a few large phases overlap the copy better than many small ones.
 // Empty when the series is too short to split.
-constexpr double kPhaseDays[] = {0.35};
+constexpr double kPhaseDays[] = {0.45};
 std::vector<int> phase_plan(int strips, int R, int64_t N) {
   std::vector<int> ps;
   if (strips < 8) return ps;
