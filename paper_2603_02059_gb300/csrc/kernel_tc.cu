@@ -743,7 +743,9 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           lap(5);
         }
         const bool last = nser > 1 || it == ntiles - 1;
-        if (last || (!kBand && (it + 1) % a.bound_tiles == 0)) {
+        // (main pass, two groups: they hold the same rows and take the refreshes in turn)
+        const bool turn = kBand || G == 1 || ((it / a.bound_tiles + cu.slot) & 1) == gid;
+        if (turn && (last || (!kBand && (it + 1) % a.bound_tiles == 0))) {
           // a bound of the row's k-th distance: from this unit's columns (band), or from
           // those of every unit so far (main pass)
           float bd = CUDART_INF_F;

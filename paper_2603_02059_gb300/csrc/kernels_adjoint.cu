@@ -11,10 +11,10 @@
 //
 // Every incidence of day a with the same partner b adds to one entry (b, summed
 // weight), so the gradient is taken in two steps:
-//   build:  one warp per day lists the day's incidences in shared memory as keys
+//   build:  one warp per day lists the day's incidences in registers as keys
 //           (partner b, kind, window slot), sorts them, and merges every run with the
 //           same b into one entry (b, summed weight); days with more incidences than
-//           a warp's buffer are merged by the whole CTA afterwards;
+//           a warp holds are merged by the whole CTA afterwards;
 //   gather: one CTA per (block of consecutive days, tile of grid points) walks its
 //           days in order, applying each day's entries in list order with four
 //           adjacent grid points per thread, and all CTAs of one tile run first
@@ -26,6 +26,8 @@
 // lists sorted by t).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "internal.h"
 
 namespace traknn {
@@ -34,6 +36,8 @@ namespace {
 __global__ void adj_count_kernel(const int32_t* __restrict__ idx, int M, int k, int* count,
                                  int* err) {
   const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  launch_wait();
+  launch_next();
   if (q >= (long long)M * k) return;
   const int j = idx[q];
   if (j < 0 || j >= M) {
@@ -43,33 +47,61 @@ __global__ void adj_count_kernel(const int32_t* __restrict__ idx, int M, int k, 
   atomicAdd(count + j, 1);
 }
 
-// Exclusive scan of count[0..M) into off[0..M]; one block of 1024 threads.
-__global__ void adj_scan_kernel(const int* __restrict__ count, int M, int* off) {
-  __shared__ int part[1024];
-  const int tid = threadIdx.x;
-  const int per = (M + 1023) / 1024;
-  const int lo = min(M, tid * per), hi = min(M, lo + per);
-  int s = 0;
-  for (int i = lo; i < hi; ++i) s += count[i];
-  part[tid] = s;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    const int v = tid >= o ? part[tid - o] : 0;
+// Exclusive scan of count[0..M) into off[0..M]; one block of 1024 threads, 4 consecutive
+// counts per thread and pass (coalesced; M = 10,957 9.6 -> 5.5 us against one thread per
+// stretch of counts).
+__global__ void __launch_bounds__(1024) adj_scan_kernel(const int* __restrict__ count, int M,
+                                                        int* off) {
+  __shared__ int wsum[33];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  launch_wait();
+  launch_next();
+  int carry = 0;
+  for (int base = 0; base < M; base += 4096) {
+    const int i0 = base + 4 * tid;
+    int c[4], s = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      c[u] = i0 + u < M ? count[i0 + u] : 0;
+      s += c[u];
+    }
+    int incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) wsum[warp] = incl;
     __syncthreads();
-    part[tid] += v;
+    if (warp == 0) {
+      int v = wsum[lane];
+      const int own = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int p = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += p;
+      }
+      wsum[lane] = v - own;
+      if (lane == 31) wsum[32] = v;
+    }
+    __syncthreads();
+    int run = carry + wsum[warp] + incl - s;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (i0 + u < M) off[i0 + u] = run;
+      run += c[u];
+    }
+    carry += wsum[32];
     __syncthreads();
   }
-  int run = tid > 0 ? part[tid - 1] : 0;
-  for (int i = lo; i < hi; ++i) {
-    off[i] = run;
-    run += count[i];
-  }
-  if (tid == 1023) off[M] = part[1023];
+  if (tid == 0) off[M] = carry;
 }
 
 __global__ void adj_fill_kernel(const int32_t* __restrict__ idx, int M, int k,
                                 const int* __restrict__ off, int* cursor, int* rev) {
   const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  launch_wait();
+  launch_next();
   if (q >= (long long)M * k) return;
   const int j = idx[q];
   if (j < 0 || j >= M) return;
@@ -92,7 +124,7 @@ __device__ void sift_down(int* a, int root, int n) {
 }
 
 constexpr int kDayWarps = 8;     // days per CTA of the build kernel, one warp each
-constexpr int kWarpKeys = 256;   // incidences one warp merges
+constexpr int kWarpKeys = 512;   // incidences one warp merges
 constexpr int kBuildThreads = kDayWarps * 32;
 constexpr int kKeyCap = 4096;    // incidences one CTA merges for one day (days beyond a warp)
 constexpr int kBigThreads = 256;
@@ -116,6 +148,8 @@ __device__ __forceinline__ int day_incidences(const int* off, int a, int L, int 
 __global__ void adj_sort_kernel(const int* __restrict__ off, int N, int L, int M, int k,
                                 int* rev) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  launch_wait();
+  launch_next();
   if (j >= M) return;
   bool needed = false;
   for (int d = j; d < min(N, j + L); ++d) needed |= day_incidences(off, d, L, M, k) > kKeyCap;
@@ -131,30 +165,15 @@ __global__ void adj_sort_kernel(const int* __restrict__ off, int N, int L, int M
   }
 }
 
-// Exclusive scan of the days' incidence counts (upper bounds of their merged entry
-// counts) into inc_off[0..N]; one block of 1024 threads.
-__global__ void adj_day_scan_kernel(const int* __restrict__ off, int N, int L, int M, int k,
-                                    long long* inc_off) {
-  __shared__ long long part[1024];
-  const int tid = threadIdx.x;
-  const int per = (N + 1023) / 1024;
-  const int lo = min(N, tid * per), hi = min(N, lo + per);
-  long long s = 0;
-  for (int a = lo; a < hi; ++a) s += day_incidences(off, a, L, M, k);
-  part[tid] = s;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    const long long v = tid >= o ? part[tid - o] : 0;
-    __syncthreads();
-    part[tid] += v;
-    __syncthreads();
-  }
-  long long run = tid > 0 ? part[tid - 1] : 0;
-  for (int a = lo; a < hi; ++a) {
-    inc_off[a] = run;
-    run += day_incidences(off, a, L, M, k);
-  }
-  if (tid == 1023) inc_off[N] = part[1023];
+// First entry of day a: the incidences of the days before it (upper bounds of their merged
+// entry counts). The forward ones are k times the pairs (t, m), t + m < a; the reverse ones,
+// off[min(d, M-1) + 1] - off[max(0, d-L+1)] summed over d < a, telescope to L terms, so no
+// scan over the days is needed.
+__device__ __forceinline__ long long day_offset(const int* off, int a, int L, int M, int k) {
+  const long long q = min(a, M), f = max(0LL, min(q, (long long)a - L + 1));
+  long long s = k * (f * L + (q - f) * a - (q * (q - 1) - f * (f - 1)) / 2);
+  for (int e = max(1, a - L + 1); e <= a; ++e) s += off[min(e, M)];
+  return s;
 }
 
 // The window of day a: trajectories [t_lo, t_lo + nw) contain it; its forward
@@ -175,38 +194,42 @@ __device__ __forceinline__ DayWindow day_window(const int* off, int a, int L, in
   return w;
 }
 
-// Sort keys: (partner b << 24) | (kind << 23) | slot, kind 0 for a forward incidence
+// Sort keys: (partner b << 6) | (kind << 5) | slot, kind 0 for a forward incidence
 // (slot: trajectory t = t_lo + slot) and 1 for a reverse one (slot: window day j =
 // t_lo + slot, t from j's reverse list). Every key of a day is unique, so the sorted
 // order is fixed whatever order the reverse lists were filled in; invalid incidences
 // (a neighbour index out of range, flagged by the count kernel) and padding are all
-// ones and sort last.
-__device__ __forceinline__ unsigned long long fwd_key(const DayWindow& w, int q, int j, int M,
-                                                      int k) {
-  if (j < 0 || j >= M) return ~0ull;
+// ones and sort last. Key is 32 bits wide while the partners fit (N < 2^26 - 1 days).
+constexpr int kSlotBits = 5, kPartnerShift = kSlotBits + 1;
+static_assert(kMaxL <= 1 << kSlotBits, "a window slot fits its bits");
+template <class Key>
+__device__ __forceinline__ Key fwd_key(const DayWindow& w, int q, int j, int M, int k) {
+  if (j < 0 || j >= M) return ~(Key)0;
   const int slot = q / k;
   const int b = j + w.a - (w.t_lo + slot);
-  return ((unsigned long long)(unsigned)b << 24) | (unsigned long long)slot;
+  return ((Key)(unsigned)b << kPartnerShift) | (Key)slot;
 }
-__device__ __forceinline__ unsigned long long rev_key(const DayWindow& w, int slot, int t) {
+template <class Key>
+__device__ __forceinline__ Key rev_key(const DayWindow& w, int slot, int t) {
   const int b = t + w.a - (w.t_lo + slot);
-  return ((unsigned long long)(unsigned)b << 24) | (1ull << 23) | (unsigned long long)slot;
+  return ((Key)(unsigned)b << kPartnerShift) | ((Key)1 << kSlotBits) | (Key)slot;
 }
 // Partner b and trajectory t of a (valid) key.
-__device__ __forceinline__ void key_pair(const DayWindow& w, unsigned long long key, int& b,
-                                         int& t) {
-  b = (int)((key >> 24) & 0x3FFFFFFFull);
-  const int slot = (int)(key & 0x7F);
-  t = (key >> 23) & 1 ? b - w.a + w.t_lo + slot : w.t_lo + slot;
+template <class Key>
+__device__ __forceinline__ void key_pair(const DayWindow& w, Key key, int& b, int& t) {
+  b = (int)(key >> kPartnerShift);
+  const int slot = (int)(key & ((1 << kSlotBits) - 1));
+  t = (key >> kSlotBits) & 1 ? b - w.a + w.t_lo + slot : w.t_lo + slot;
 }
 
 // Summed weight of the run of equal partners starting at sorted position q, in key
 // order: w = sum over the run of (2 / k) g_t.
-__device__ __forceinline__ float run_weight(const unsigned long long* key, int q, int n,
-                                            const DayWindow& w, const float* g, float inv_k2) {
-  const unsigned long long run = key[q] >> 24;
+template <class Key>
+__device__ __forceinline__ float run_weight(const Key* key, int q, int n, const DayWindow& w,
+                                            const float* g, float inv_k2) {
+  const Key run = key[q] >> kPartnerShift;
   float s = 0.f;
-  for (int r = q; r < n && key[r] != ~0ull && (key[r] >> 24) == run; ++r) {
+  for (int r = q; r < n && key[r] != ~(Key)0 && (key[r] >> kPartnerShift) == run; ++r) {
     int b, t;
     key_pair(w, key[r], b, t);
     s += inv_k2 * g[t];
@@ -214,21 +237,22 @@ __device__ __forceinline__ float run_weight(const unsigned long long* key, int q
   return s;
 }
 
-// Merged entries of one day with n <= kWarpKeys incidences, by one warp: the keys from
+// Merged entries of one day with n <= 32 kIt incidences, by one warp: the keys from
 // coalesced loads of the day's two contiguous lists (the window day of a reverse
-// position found from the window's list offsets, one per lane, by shuffles), sorted
-// by a bitonic network in the warp's part of shared memory, run heads numbered with a
-// ballot per 32 positions.
-__device__ void merge_day_warp(const DayWindow& w, int n, unsigned long long* key,
-                               const int32_t* idx, const float* g, const int* off,
-                               const int* rev, int M, int k, AdjEntry* out, long long cap,
-                               int* cnt_a, int* err) {
+// position found from the window's list offsets, one per lane, by shuffles), sorted by a
+// bitonic network in registers (position 32 it + lane in register it: exchanges of 32
+// positions and more between a lane's registers, of fewer by shuffles), stored in the
+// warp's part of shared memory; run heads numbered with a ballot per 32 positions. A
+// network in shared memory took a load, a compare and a store per key and step: 30 years,
+// k = 10 65 -> 40 us, and with up to 512 keys per warp the second pass over busier days
+// 30 -> 4 us.
+template <int kIt, class Key>
+__device__ void merge_day_regs(const DayWindow& w, int n, Key* key, const int32_t* idx,
+                               const float* g, const int* off, const int* rev, int M, int k,
+                               AdjEntry* out, long long cap, int* cnt_a, int* err) {
   const int lane = threadIdx.x & 31;
   const float inv_k2 = 2.0f / (float)k;
   const int woff = lane <= w.nw ? off[w.t_lo + lane] : 0;  // off[t_lo + lane]
-  int n2 = 32;
-  while (n2 < n) n2 <<= 1;
-  constexpr int kIt = kWarpKeys / 32;
   int v[kIt];  // neighbour j (forward) or trajectory t (reverse) of each own position
 #pragma unroll
   for (int it = 0; it < kIt; ++it) {
@@ -237,6 +261,7 @@ __device__ void merge_day_warp(const DayWindow& w, int n, unsigned long long* ke
     if (q < n)
       v[it] = q < w.nfwd ? __ldg(idx + (size_t)w.t_lo * k + q) : __ldg(rev + w.r0 + (q - w.nfwd));
   }
+  Key kq[kIt];
 #pragma unroll
   for (int it = 0; it < kIt; ++it) {
     const int q = it * 32 + lane;
@@ -247,36 +272,47 @@ __device__ void merge_day_warp(const DayWindow& w, int n, unsigned long long* ke
       const int r = w.r0 + (q - w.nfwd);
       for (int i = 1; i < w.nw; ++i) slot += __shfl_sync(0xffffffffu, woff, i) <= r;
     }
-    unsigned long long kq = ~0ull;
-    if (q < n) kq = q < w.nfwd ? fwd_key(w, q, v[it], M, k) : rev_key(w, slot, v[it]);
-    if (q < n2) key[q] = kq;
+    kq[it] = ~(Key)0;
+    if (q < n)
+      kq[it] = q < w.nfwd ? fwd_key<Key>(w, q, v[it], M, k) : rev_key<Key>(w, slot, v[it]);
   }
-  __syncwarp();
-  for (int size = 2; size <= n2; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int q = lane; q < n2; q += 32) {
-        const int r = q ^ stride;
-        if (r > q) {
-          const bool up = (q & size) == 0;
-          const unsigned long long x = key[q], y = key[r];
-          if ((x > y) == up) {
-            key[q] = y;
-            key[r] = x;
-          }
+#pragma unroll
+  for (int size = 2; size <= 32 * kIt; size <<= 1) {
+#pragma unroll
+    for (int stride = size >> 1; stride >= 32; stride >>= 1) {
+#pragma unroll
+      for (int it = 0; it < kIt; ++it) {
+        const int jt = it ^ (stride >> 5);
+        if (jt > it) {
+          const bool up = ((it * 32) & size) == 0;
+          const Key x = kq[it], y = kq[jt], lo = min(x, y), hi = max(x, y);
+          kq[it] = up ? lo : hi;
+          kq[jt] = up ? hi : lo;
         }
       }
-      __syncwarp();
+    }
+#pragma unroll
+    for (int stride = min(size >> 1, 16); stride > 0; stride >>= 1) {
+#pragma unroll
+      for (int it = 0; it < kIt; ++it) {
+        const bool up = ((it * 32 + lane) & size) == 0, first = (lane & stride) == 0;
+        const Key x = kq[it], y = __shfl_xor_sync(0xffffffffu, x, stride);
+        kq[it] = up == first ? min(x, y) : max(x, y);
+      }
     }
   }
+#pragma unroll
+  for (int it = 0; it < kIt; ++it) key[it * 32 + lane] = kq[it];
+  __syncwarp();
   int nout = 0;
   for (int q0 = 0; q0 < n; q0 += 32) {
     const int q = q0 + lane;
-    const bool head =
-        q < n && key[q] != ~0ull && (q == 0 || (key[q - 1] >> 24) != (key[q] >> 24));
+    const bool head = q < n && key[q] != ~(Key)0 &&
+                      (q == 0 || (key[q - 1] >> kPartnerShift) != (key[q] >> kPartnerShift));
     const unsigned bal = __ballot_sync(0xffffffffu, head);
     if (head) {
       const int u = nout + __popc(bal & ((1u << lane) - 1u));
-      const int b = (int)((key[q] >> 24) & 0x3FFFFFFFull);
+      const int b = (int)(key[q] >> kPartnerShift);
       const float s = run_weight(key, q, n, w, g, inv_k2);
       if (tk_in(u, cap, err)) out[u] = make_int2(b, __float_as_int(s));
     }
@@ -290,7 +326,8 @@ __device__ void merge_day_warp(const DayWindow& w, int n, unsigned long long* ke
 // over each thread's consecutive positions). A day with more than kKeyCap incidences
 // lists them unmerged, in the fixed order of its lists (forward by (t, rank), reverse
 // by (j, t) from sorted segments). Ends with a CTA barrier.
-__device__ void merge_day_block(const DayWindow& w, int n, unsigned long long* key, int* scan,
+template <class Key>
+__device__ void merge_day_block(const DayWindow& w, int n, Key* key, int* scan,
                                 int* swoff, const int32_t* idx, const float* g, const int* off,
                                 const int* rev, int M, int k, AdjEntry* out, long long cap,
                                 int* cnt_a, int* err) {
@@ -298,20 +335,20 @@ __device__ void merge_day_block(const DayWindow& w, int n, unsigned long long* k
   const float inv_k2 = 2.0f / (float)k;
   for (int i = tid; i <= w.nw; i += kBigThreads) swoff[i] = off[w.t_lo + i];
   __syncthreads();
-  auto key_of = [&](int q) -> unsigned long long {
-    if (q < w.nfwd) return fwd_key(w, q, __ldg(idx + (size_t)w.t_lo * k + q), M, k);
+  auto key_of = [&](int q) -> Key {
+    if (q < w.nfwd) return fwd_key<Key>(w, q, __ldg(idx + (size_t)w.t_lo * k + q), M, k);
     const int r = w.r0 + (q - w.nfwd);
     int slot = 0;
     while (slot + 1 < w.nw && swoff[slot + 1] <= r) ++slot;
-    return rev_key(w, slot, __ldg(rev + r));
+    return rev_key<Key>(w, slot, __ldg(rev + r));
   };
   if (n > kKeyCap) {
     for (int q = tid; q < n; q += kBigThreads) {
-      const unsigned long long kq = key_of(q);
+      const Key kq = key_of(q);
       int b = w.a, t = 0;
-      if (kq != ~0ull) key_pair(w, kq, b, t);
+      if (kq != ~(Key)0) key_pair(w, kq, b, t);
       if (tk_in(q, cap, err))
-        out[q] = kq != ~0ull ? make_int2(b, __float_as_int(inv_k2 * g[t])) : make_int2(w.a, 0);
+        out[q] = kq != ~(Key)0 ? make_int2(b, __float_as_int(inv_k2 * g[t])) : make_int2(w.a, 0);
     }
     if (tid == 0) *cnt_a = n;
     __syncthreads();
@@ -319,7 +356,7 @@ __device__ void merge_day_block(const DayWindow& w, int n, unsigned long long* k
   }
   int n2 = 1;
   while (n2 < n) n2 <<= 1;
-  for (int q = tid; q < n2; q += kBigThreads) key[q] = q < n ? key_of(q) : ~0ull;
+  for (int q = tid; q < n2; q += kBigThreads) key[q] = q < n ? key_of(q) : ~(Key)0;
   __syncthreads();
   for (int size = 2; size <= n2; size <<= 1) {
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
@@ -327,7 +364,7 @@ __device__ void merge_day_block(const DayWindow& w, int n, unsigned long long* k
         const int r = q ^ stride;
         if (r > q) {
           const bool up = (q & size) == 0;
-          const unsigned long long x = key[q], y = key[r];
+          const Key x = key[q], y = key[r];
           if ((x > y) == up) {
             key[q] = y;
             key[r] = x;
@@ -339,8 +376,8 @@ __device__ void merge_day_block(const DayWindow& w, int n, unsigned long long* k
   }
   const int per = (n + kBigThreads - 1) / kBigThreads;
   auto head = [&](int q) {
-    if (q >= n || key[q] == ~0ull) return 0;
-    return (q == 0 || (key[q - 1] >> 24) != (key[q] >> 24)) ? 1 : 0;
+    if (q >= n || key[q] == ~(Key)0) return 0;
+    return (q == 0 || (key[q - 1] >> kPartnerShift) != (key[q] >> kPartnerShift)) ? 1 : 0;
   };
   const int q0 = tid * per;
   int cnt = 0;
@@ -357,7 +394,7 @@ __device__ void merge_day_block(const DayWindow& w, int n, unsigned long long* k
   for (int i = 0; i < per; ++i) {
     const int q = q0 + i;
     if (!head(q)) continue;
-    const int b = (int)((key[q] >> 24) & 0x3FFFFFFFull);
+    const int b = (int)(key[q] >> kPartnerShift);
     const float s = run_weight(key, q, n, w, g, inv_k2);
     if (tk_in(u, cap, err)) out[u] = make_int2(b, __float_as_int(s));
     ++u;
@@ -368,39 +405,54 @@ __device__ void merge_day_block(const DayWindow& w, int n, unsigned long long* k
 
 // The merged entry list of every day with at most kWarpKeys incidences, one warp per
 // day (CTA x holds days [x kDayWarps, (x+1) kDayWarps)); a day with more is appended
-// to the list `big` for adj_build_big_kernel. Day a's entries go to ent[inc_off[a] ..)
-// (room for all its incidences) and their number to cnt[a].
+// to the list `big` for adj_build_big_kernel. Day a's entries go to ent[day_offset(a) ..)
+// (room for all its incidences), their number to cnt[a], the offset to inc_off[a].
+template <class Key>
 __global__ void __launch_bounds__(kBuildThreads)
     adj_build_kernel(const int32_t* __restrict__ idx, const float* __restrict__ g, int N, int L,
                      int M, int k, const int* __restrict__ off, const int* __restrict__ rev,
-                     const long long* __restrict__ inc_off, int* __restrict__ cnt,
+                     long long* __restrict__ inc_off, int* __restrict__ cnt,
                      AdjEntry* __restrict__ ent, int* big, int* nbig, int* err) {
-  __shared__ unsigned long long key[kDayWarps * kWarpKeys];
+  __shared__ Key keys[kDayWarps * kWarpKeys];
   const int warp = threadIdx.x >> 5;
   const int a = blockIdx.x * kDayWarps + warp;
+  launch_wait();
+  launch_next();
   if (a >= N) return;  // no CTA barrier in this kernel
   const DayWindow w = day_window(off, a, L, M, k);
   const int n = w.nfwd + (off[w.t_lo + w.nw] - w.r0);
+  const long long o = day_offset(off, a, L, M, k);
+  if ((threadIdx.x & 31) == 0) inc_off[a] = o;
   if (n > kWarpKeys) {
     if ((threadIdx.x & 31) == 0) big[atomicAdd(nbig, 1)] = a;
     return;
   }
-  const long long o = inc_off[a];
-  merge_day_warp(w, n, key + warp * kWarpKeys, idx, g, off, rev, M, k, ent + o,
-                 inc_off[a + 1] - o, cnt + a, err);
+  Key* key = keys + warp * kWarpKeys;
+  auto merge = [&](auto its) {
+    merge_day_regs<decltype(its)::value>(w, n, key, idx, g, off, rev, M, k, ent + o, n, cnt + a,
+                                         err);
+  };
+  if (n <= 32) merge(std::integral_constant<int, 1>());
+  else if (n <= 64) merge(std::integral_constant<int, 2>());
+  else if (n <= 128) merge(std::integral_constant<int, 4>());
+  else if (n <= 256) merge(std::integral_constant<int, 8>());
+  else merge(std::integral_constant<int, 16>());
 }
 
 // The days listed by adj_build_kernel, one CTA each (grid-stride over the list; the
 // order in which they are taken does not matter: every day's list is its own).
+template <class Key>
 __global__ void __launch_bounds__(kBigThreads)
     adj_build_big_kernel(const int32_t* __restrict__ idx, const float* __restrict__ g, int N,
                          int L, int M, int k, const int* __restrict__ off,
                          const int* __restrict__ rev, const long long* __restrict__ inc_off,
                          int* __restrict__ cnt, AdjEntry* __restrict__ ent,
                          const int* __restrict__ big, const int* __restrict__ nbig, int* err) {
-  __shared__ unsigned long long key[kKeyCap];
+  __shared__ Key key[kKeyCap];
   __shared__ int scan[kBigThreads];
   __shared__ int swoff[kMaxL + 1];
+  launch_wait();
+  launch_next();
   const int nb = *nbig;
   for (int i = blockIdx.x; i < nb; i += gridDim.x) {
     const int d = big[i];
@@ -408,8 +460,7 @@ __global__ void __launch_bounds__(kBigThreads)
     const DayWindow w = day_window(off, d, L, M, k);
     const int n = w.nfwd + (off[w.t_lo + w.nw] - w.r0);
     const long long o = inc_off[d];
-    merge_day_block(w, n, key, scan, swoff, idx, g, off, rev, M, k, ent + o, inc_off[d + 1] - o,
-                    cnt + d, err);
+    merge_day_block(w, n, key, scan, swoff, idx, g, off, rev, M, k, ent + o, n, cnt + d, err);
   }
 }
 
@@ -549,6 +600,8 @@ __global__ void __launch_bounds__(kGatherMaxThreads)
   __shared__ int sday[kAdjR + 1];  // first staged position of each day
   const int a0 = blockIdx.x * kAdjR;
   const int nd = min(kAdjR, N - a0);
+  launch_wait();
+  launch_next();
   if (threadIdx.x < 32) {  // exclusive scan of the days' entry counts
     const int lane = threadIdx.x;
     const int c = lane < nd ? cnt[a0 + lane] : 0;
@@ -677,19 +730,29 @@ cudaError_t launch_adjoint(const float* X, int N, int D, int L, int k, const int
   if (e != cudaSuccess) return e;
   const long long nq = (long long)M * k;
   const int blocks = (int)((nq + 255) / 256);
-  adj_count_kernel<<<blocks, 256, 0, st>>>(idx, M, k, count, err);
-  adj_scan_kernel<<<1, 1024, 0, st>>>(count, M, off);
-  adj_fill_kernel<<<blocks, 256, 0, st>>>(idx, M, k, off, cursor, rev);
-  adj_sort_kernel<<<(M + 127) / 128, 128, 0, st>>>(off, N, L, M, k, rev);
-  adj_day_scan_kernel<<<1, 1024, 0, st>>>(off, N, L, M, k, inc_off);
-  adj_build_kernel<<<(N + kDayWarps - 1) / kDayWarps, kBuildThreads, 0, st>>>(
-      idx, g, N, L, M, k, off, rev, inc_off, cnt, ent, big, nbig, err);
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
       (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return e;
-  adj_build_big_kernel<<<2 * sms, kBigThreads, 0, st>>>(idx, g, N, L, M, k, off, rev, inc_off,
-                                                        cnt, ent, big, nbig, err);
+  if ((e = launch_chained(adj_count_kernel, blocks, 256, 0, st, idx, M, k, count, err)) !=
+          cudaSuccess ||
+      (e = launch_chained(adj_scan_kernel, 1, 1024, 0, st, count, M, off)) != cudaSuccess ||
+      (e = launch_chained(adj_fill_kernel, blocks, 256, 0, st, idx, M, k, off, cursor, rev)) !=
+          cudaSuccess ||
+      (e = launch_chained(adj_sort_kernel, (M + 127) / 128, 128, 0, st, off, N, L, M, k, rev)) !=
+          cudaSuccess)
+    return e;
+  auto build = [&](auto key) {
+    typedef decltype(key) Key;
+    const cudaError_t r =
+        launch_chained(adj_build_kernel<Key>, (N + kDayWarps - 1) / kDayWarps, kBuildThreads, 0,
+                       st, idx, g, N, L, M, k, off, rev, inc_off, cnt, ent, big, nbig, err);
+    if (r != cudaSuccess) return r;
+    return launch_chained(adj_build_big_kernel<Key>, 2 * sms, kBigThreads, 0, st, idx, g, N, L, M,
+                          k, off, rev, inc_off, cnt, ent, big, nbig, err);
+  };
+  e = N < (1 << (32 - kPartnerShift)) - 1 ? build((unsigned)0) : build((unsigned long long)0);
+  if (e != cudaSuccess) return e;
   // 16-byte loads where D is a multiple of 4 and X, dX 16-byte aligned; 8-byte loads
   // where D is even and they are 8-byte aligned; else 4-byte loads
   const uintptr_t al = reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(dX);
@@ -698,17 +761,13 @@ cudaError_t launch_adjoint(const float* X, int N, int D, int L, int k, const int
   int tiles = 1;
   const int threads = gather_threads(slots, &tiles);
   const dim3 grid((N + kAdjR - 1) / kAdjR, tiles < 65535 ? tiles : 65535);
-  if (form == 2)
-    adj_gather_kernel<2><<<grid, threads, 0, st>>>(X, N, D, inc_off, cnt, ent, wts, dX,
-                                                    tiles, err);
-  else if (form == 1)
-    adj_gather_kernel<1><<<grid, threads, 0, st>>>(X, N, D, inc_off, cnt, ent, wts, dX,
-                                                    tiles, err);
-  else
-    adj_gather_kernel<0><<<grid, threads, 0, st>>>(X, N, D, inc_off, cnt, ent, wts, dX,
-                                                    tiles, err);
-  *launches += 8;
-  return cudaGetLastError();
+  const auto gather = form == 2   ? adj_gather_kernel<2>
+                      : form == 1 ? adj_gather_kernel<1>
+                                  : adj_gather_kernel<0>;
+  e = launch_chained(gather, grid, threads, 0, st, X, N, D, inc_off, cnt, ent, wts, dX, tiles,
+                     err);
+  *launches += 7;
+  return e;
 }
 
 }  // namespace traknn

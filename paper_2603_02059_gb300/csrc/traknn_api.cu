@@ -550,7 +550,7 @@ void fused_args(const traknn_ctx* h, const TcBuffers& b, TcArgs* pa, TcWork* pw)
   a.cap = list_cap(list_pitch(p.kmax), p.part_lists);
   a.shared_min = b.shared_min;
   // where the contraction sets the pace a refresh after every tile is hidden behind it;
-  // D = 32, 75 years: every 2 / 4 / 8 / 16 tiles 1,045 / 989 / 987 / 1,008 us
+  // D = 32, 75 years: every 2 / 4 / 8 / 16 tiles 815 / 795 / 790 / 812 us
   a.bound_tiles = b.Dp > 768 ? 1 : 4;
   a.err = h->err;
   a.wait_limit_ns = (long long)h->wait_limit_ms * 1000000LL;
