@@ -107,7 +107,8 @@ inline Schedule make_schedule(int M, int L, int k, int e, int sm_count, int chun
 }
 
 // Byte offsets of the FP32 path's workspace (each piece starts on a 256-byte
-// boundary): a reserve of kMeanSlices rows (the documented size counts it), mean, FP64 day norms, window sums, the centred
+// boundary): a reserve of kMeanSlices rows (the documented size counts it; it holds the
+// square roots of the grid-point weights, if any), mean, FP64 day norms, window sums, the centred
 // FP32 copy (row pitch Dp = D rounded up to 32) and the partial neighbour lists.
 struct Fp32Layout {
   size_t partial, mu, norms, W, ops, pd, pi, total;
@@ -333,10 +334,11 @@ cudaError_t launch_prep_fp32_series(const SeriesTable& sr, int rows, int D, int 
                                     const float* mu, const float* sw, float* Xc, double* norms,
                                     cudaStream_t st);
 // FP32 CUDA-core path over the work list of the tensor-core path (Xc: the stacked FP32
-// operand copy, pitch a.Dp), and the both-triangles form of traknn_knn_scores_static.
+// operand copy, pitch a.Dp), and the both-triangles form of traknn_knn_scores_static and of
+// the shortest calls.
 cudaError_t launch_fused_fp32(const float* Xc, const TcArgs& a, const TcWork& w,
                               const SeriesTable& sr, int num_ctas, cudaStream_t st);
-cudaError_t launch_fused_fp32_static(const float* Xc, const FusedArgs& a, int num_ctas,
+cudaError_t launch_fused_fp32_both(const float* Xc, const FusedArgs& a, int num_ctas,
                                      cudaStream_t st);
 // Tensor-core path; `split` selects the 3-product split-BF16 form.
 cudaError_t launch_fused_tc(const void* hi, const void* lo, bool split, const TcArgs& a,

@@ -7,8 +7,9 @@
 // tensor-core path (upper triangle only, epilogue.cuh): one persistent CTA per SM computes
 // a unit's 128 x 256 Gram tiles in two halves into shared memory, beside the L-1 columns
 // carried from the previous tile, and two groups of 128 threads, one thread per row, scan
-// 128 columns each. fused_fp32_static_kernel evaluates both triangles in 128 x 128 tiles
-// with sorted lists in shared memory: the form of the entry point whose scratch is fixed.
+// 128 columns each. fused_fp32_both_kernel evaluates both triangles in 128 x 128 tiles
+// with sorted lists in shared memory: the form of the entry point whose scratch is fixed, and
+// of the shortest calls (one tile per CTA and no band before it).
 //
 // What bounds both is the FP32 FMA rate; a Gram entry's products are summed in the same
 // order in either triangle and either kernel, so G(a, b) = G(b, a) bit for bit and the
@@ -27,7 +28,7 @@ constexpr int BN = 128;        // Gram columns per half tile
 constexpr int BK = 16;         // depth of one shared-memory stage
 constexpr int NT = 256;        // threads
 constexpr int LDA = BM + 4;
-constexpr int kPitchStatic = kHalo + BN + 1;   // odd row pitches: conflict-free diagonal reads
+constexpr int kPitchBoth = kHalo + BN + 1;   // odd row pitches: conflict-free diagonal reads
 constexpr int kPitch = kHalo + 2 * BN + 1;
 constexpr int kRowPitch = 36;  // a row of 32 distances (16-byte aligned, conflict-free)
 
@@ -319,25 +320,27 @@ __global__ void __launch_bounds__(NT, 1)
   }
 }
 
-// ------------------------------------------------- both triangles, fixed scratch
-struct SmemStatic {
+// ------------------------------------------------------------- both triangles
+struct SmemBoth {
   Stages st;
-  float G[BM][kPitchStatic];
+  float G[BM][kPitchBoth];
 };
 
 __global__ void __launch_bounds__(NT, 1)
-    fused_fp32_static_kernel(const float* __restrict__ Xc, FusedArgs a) {
+    fused_fp32_both_kernel(const float* __restrict__ Xc, FusedArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SmemStatic& sm = *reinterpret_cast<SmemStatic*>(smem_raw);
+  SmemBoth& sm = *reinterpret_cast<SmemBoth*>(smem_raw);
   const Schedule& s = a.sch;
   SmemList list;
-  list.d = reinterpret_cast<float*>(smem_raw + sizeof(SmemStatic));
+  list.d = reinterpret_cast<float*>(smem_raw + sizeof(SmemBoth));
   list.i = reinterpret_cast<int32_t*>(list.d + BM * s.k);
   list.stride = BM;
   list.k = s.k;
 
   const int tid = threadIdx.x;
   const int L = s.L;
+  launch_wait();
+  launch_next();
   for (int u = blockIdx.x; u < s.units; u += gridDim.x) {
     const UnitCoord uc = unit_coord(s, u);
     if (uc.strip >= s.strips) continue;
@@ -358,11 +361,11 @@ __global__ void __launch_bounds__(NT, 1)
     const int ntiles = (rc.jhi - rc.jlo + L - 1 + BN - 1) / BN;
     for (int it = 0; it < ntiles; ++it) {
       const int c0 = rc.jlo + it * BN;  // first Gram column of the tile
-      gram_tile(sm.st, Xc, a.N, a.Dp, T0, c0, tid, &sm.G[0][kHalo], kPitchStatic);
+      gram_tile(sm.st, Xc, a.N, a.Dp, T0, c0, tid, &sm.G[0][kHalo], kPitchBoth);
       // output column x of this tile is j = c0 - (L-1) + x; its window starts in
       // the carried columns, which sit just left of kHalo
       if (row_ok)
-        window_topk(&sm.G[0][kHalo - (L - 1)], kPitchStatic, rc, it == 0 ? L - 1 : 0, BN,
+        window_topk(&sm.G[0][kHalo - (L - 1)], kPitchBoth, rc, it == 0 ? L - 1 : 0, BN,
                     c0 - (L - 1), a.W, list, tid, thr);
       __syncthreads();
       for (int q = tid; q < BM * (L - 1); q += NT) {
@@ -399,14 +402,13 @@ cudaError_t launch_fused_fp32(const float* Xc, const TcArgs& a, const TcWork& w,
                                  : launch_sym<false, 128>(Xc, a, w, sr, num_ctas, st);
 }
 
-cudaError_t launch_fused_fp32_static(const float* Xc, const FusedArgs& a, int num_ctas,
+cudaError_t launch_fused_fp32_both(const float* Xc, const FusedArgs& a, int num_ctas,
                                      cudaStream_t st) {
-  const size_t smem = sizeof(SmemStatic) + (size_t)BM * a.sch.k * 8;
-  cudaError_t err = cudaFuncSetAttribute(fused_fp32_static_kernel,
+  const size_t smem = sizeof(SmemBoth) + (size_t)BM * a.sch.k * 8;
+  cudaError_t err = cudaFuncSetAttribute(fused_fp32_both_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  fused_fp32_static_kernel<<<num_ctas, NT, smem, st>>>(Xc, a);
-  return cudaGetLastError();
+  return launch_chained(fused_fp32_both_kernel, num_ctas, NT, smem, st, Xc, a);
 }
 
 }  // namespace traknn

@@ -127,7 +127,7 @@ constexpr int kDayWarps = 8;     // days per CTA of the build kernel, one warp e
 constexpr int kWarpKeys = 512;   // incidences one warp merges
 constexpr int kBuildThreads = kDayWarps * 32;
 constexpr int kKeyCap = 4096;    // incidences one CTA merges for one day (days beyond a warp)
-constexpr int kBigThreads = 256;
+constexpr int kBigThreads = 1024;  // (256: the few busy days of 30 years 30 us instead of 17)
 
 // One merged entry of a day's gradient list: partner day b and summed weight w (as
 // FP32 bits). A day's entries are in order of partner.
@@ -244,8 +244,7 @@ __device__ __forceinline__ float run_weight(const Key* key, int q, int n, const 
 // positions and more between a lane's registers, of fewer by shuffles), stored in the
 // warp's part of shared memory; run heads numbered with a ballot per 32 positions. A
 // network in shared memory took a load, a compare and a store per key and step: 30 years,
-// k = 10 65 -> 40 us, and with up to 512 keys per warp the second pass over busier days
-// 30 -> 4 us.
+// k = 10 65 -> 40 us.
 template <int kIt, class Key>
 __device__ void merge_day_regs(const DayWindow& w, int n, Key* key, const int32_t* idx,
                                const float* g, const int* off, const int* rev, int M, int k,

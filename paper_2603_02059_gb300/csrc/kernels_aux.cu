@@ -390,6 +390,8 @@ __global__ void merge_kernel(const float* __restrict__ part_d, const int32_t* __
                              float* __restrict__ dist, float* __restrict__ score) {
   const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  launch_wait();
+  launch_next();
   if (t >= M) return;
   const float* pd = part_d + (size_t)t * P * k;
   const int32_t* pi = part_i + (size_t)t * P * k;
@@ -895,9 +897,8 @@ cudaError_t launch_merge(const FusedArgs& a, int32_t* idx, float* dist, float* s
                          cudaStream_t st) {
   const int warps_per_block = 8;
   const int blocks = (a.sch.M + warps_per_block - 1) / warps_per_block;
-  merge_kernel<<<blocks, 32 * warps_per_block, 0, st>>>(a.part_d, a.part_i, a.sch.M,
-                                                        a.sch.chunks, a.sch.k, idx, dist, score);
-  return cudaGetLastError();
+  return launch_chained(merge_kernel, blocks, 32 * warps_per_block, 0, st, a.part_d, a.part_i,
+                        a.sch.M, a.sch.chunks, a.sch.k, idx, dist, score);
 }
 
 // ----------------------------------------------------------- kNN statistics

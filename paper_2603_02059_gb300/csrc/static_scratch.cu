@@ -150,7 +150,7 @@ extern "C" traknn_status traknn_knn_scores_static(const float* X, int64_t N, int
       launch_prep_fp32_series(sr, (int)N, (int)D, lay.Dp, mu, nullptr, Xc, norms, cs) !=
           cudaSuccess ||
       launch_window_series(sr, M, norms, W, ClearArgs{}, cs) != cudaSuccess ||
-      launch_fused_fp32_static(Xc, a, sms, cs) != cudaSuccess ||
+      launch_fused_fp32_both(Xc, a, sms, cs) != cudaSuccess ||
       launch_merge(a, nbr_idx, nbr_dist, score, cs) != cudaSuccess) {
     cudaGetLastError();
     return TRAKNN_ERR_CUDA;

@@ -935,6 +935,61 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   return TRAKNN_OK;
 }
 
+// The shortest FP32 calls on both triangles: one tile per CTA, no band and no column side,
+// five launches. Its scan inserts into sorted lists in shared memory, about k steps per
+// candidate, so it pays up to a product of rows and neighbours, the more the longer a tile's
+// products take. Both triangles / upper triangle (us, L = 5): D = 16, N = 300 k = 5 48 / 64, k =
+// 20 86 / 70, N = 800 k = 5 74 / 81; D = 256, N = 300 k = 5 70 / 126, k = 20 106 / 133, N = 500
+// k = 20 134 / 143, N = 800 k = 5 95 / 137, k = 20 175 / 149, N = 1,200 k = 5 140 / 143; D =
+// 800, N = 1,200 k = 5 237 / 210.
+bool fp32_short(int64_t M, int64_t D, int k) {
+  return M <= 1024 && M * k <= (D >= 200 ? 10000 : 4500);
+}
+traknn_status run_fp32_short(traknn_ctx* h, const HostSeries& sd, int64_t D, cudaStream_t s) {
+  const int M = (int)(sd.N - sd.L + 1);
+  const Schedule sch = make_schedule(M, sd.L, sd.k, sd.e, h->sm_count, h->col_chunks);
+  const Fp32Layout lay = make_layout(sd.N, D, sch);
+  TRY_ST(ensure_buffer(h, &h->tcws, &h->tcws_bytes, lay.total));
+  char* ws = static_cast<char*>(h->tcws);
+  float* mu = reinterpret_cast<float*>(ws + lay.mu);
+  float* sw = reinterpret_cast<float*>(ws + lay.partial);
+  double* norms = reinterpret_cast<double*>(ws + lay.norms);
+  float* W = reinterpret_cast<float*>(ws + lay.W);
+  float* Xc = reinterpret_cast<float*>(ws + lay.ops);
+  FusedArgs fa;
+  fa.sch = sch;
+  fa.N = (int)sd.N;
+  fa.Dp = lay.Dp;
+  fa.W = W;
+  fa.part_d = reinterpret_cast<float*>(ws + lay.pd);
+  fa.part_i = reinterpret_cast<int32_t*>(ws + lay.pi);
+  fa.err = h->err;
+  fa.wait_limit_ns = (long long)h->wait_limit_ms * 1000000LL;
+  fa.debug_withhold = h->debug_withhold;
+  thread_local SeriesTable sr;  // one series (large: kept off the stack)
+  sr.n = 1;
+  sr.s[0] = SeriesInfo{};
+  sr.s[0].N = (int)sd.N;
+  sr.s[0].M = M;
+  sr.s[0].L = sd.L;
+  sr.s[0].X = sd.X;
+  TRY_CUDA(launch_col_mean_series(sr, (int)D, 1, h->weights, mu, sw, h->center != 0, s));
+  TRY_CUDA(launch_prep_fp32_series(sr, (int)sd.N, (int)D, lay.Dp, mu, h->weights ? sw : nullptr,
+                                   Xc, norms, s));
+  TRY_CUDA(launch_window_series(sr, M, norms, W, ClearArgs{}, s));
+  const int slot = h->ev_head;
+  if (h->profile) TRY_CUDA(cudaEventRecord(h->ev_start[slot], s));
+  TRY_CUDA(launch_fused_fp32_both(Xc, fa, h->sm_count, s));
+  if (h->profile) {
+    TRY_CUDA(cudaEventRecord(h->ev_stop[slot], s));
+    h->ev_head = (h->ev_head + 1) % traknn_ctx::kRing;
+    h->ev_count = std::min(h->ev_count + 1, traknn_ctx::kRing);
+  }
+  TRY_CUDA(launch_merge(fa, sd.idx, sd.dist, sd.score, s));
+  h->launches += 5;
+  return TRAKNN_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1105,6 +1160,8 @@ traknn_status traknn_knn_scores(traknn_handle h, const float* X, int64_t N, int6
     return run_tc(h, &sd, 1, D, s, false, false, L);
   }
   const HostSeries sd{X, N, L, k, e, nbr_idx, nbr_dist, score};
+  if (h->precision == TRAKNN_PREC_FP32 && fp32_short(N - L + 1, D, k))
+    return run_fp32_short(h, sd, D, s);
   return run_tc(h, &sd, 1, D, s, false);
 }
 
