@@ -48,7 +48,7 @@ __global__ void adj_count_kernel(const int32_t* __restrict__ idx, int M, int k, 
 }
 
 // Exclusive scan of count[0..M) into off[0..M]; one block of 1024 threads, 4 consecutive
-// counts per thread and pass (coalesced; M = 10,957 9.6 -> 5.5 us against one thread per
+// counts per thread and pass (coalesced; M = 10,957 9.6 -> 7.0 us against one thread per
 // stretch of counts).
 __global__ void __launch_bounds__(1024) adj_scan_kernel(const int* __restrict__ count, int M,
                                                         int* off) {

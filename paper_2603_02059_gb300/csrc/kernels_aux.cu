@@ -70,21 +70,21 @@ __global__ void prep_fp32_series_kernel(const __grid_constant__ SeriesTable st, 
   if (threadIdx.x == 0) norms[r] = s;
 }
 
-// Mean of every series' centring days per grid point (grid.y = series, 32 grid points per
+// Mean of a series' centring days per grid point (grid.y = series, 32 grid points per
 // CTA): a warp sums slices w and w + 32 of the days, then one warp sums the 64 slices in
 // order (fixed summation order: deterministic; FP32 sums suffice for the offset, see above).
 // The mean, and the square roots of the weights, are written once per day of an operand
 // row, so that the preparation needs neither a division nor a square root per value
-// (7,301 x 3,555 weighted: preparation 193 -> 53 us). Bound by the read of the centring
+// (7,301 x 3,555 weighted: preparation 193 -> 61 us). Bound by the read of the centring
 // days; one launch instead of two saves about 4 us on every call.
 constexpr int kMeanWarps = 32;
 __global__ void __launch_bounds__(32 * kMeanWarps)
-    col_mean_series_kernel(const __grid_constant__ SeriesTable st, int D, int emb,
+    col_mean_series_kernel(const __grid_constant__ SeriesTable st, int first_series, int D, int emb,
                            const float* __restrict__ wts, float* __restrict__ mu,
                            float* __restrict__ sw, int center) {
   __shared__ float part[kMeanSlices][33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int p = blockIdx.x * 32 + lane, b = blockIdx.y;
+  const int p = blockIdx.x * 32 + lane, b = first_series + blockIdx.y;
   const SeriesInfo& si = st.s[b];
   const int first = mean_first(si.N), ns = mean_days(si.N);
   const int per = (ns + kMeanSlices - 1) / kMeanSlices;
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(32 * kMeanWarps)
     m = acc / (float)ns;
   }
   for (int e = 0; e < emb; ++e) mu[((size_t)b * emb + e) * D + p] = m;
-  if (wts && b == 0) {
+  if (wts && blockIdx.y == 0) {
     const float q = sqrtf(wts[p]);
     for (int e = 0; e < emb; ++e) sw[(size_t)e * D + p] = q;
   }
@@ -856,10 +856,10 @@ cudaError_t launch_merge_parts(const int32_t* idx_parts, const float* dist_parts
   return cudaGetLastError();
 }
 
-cudaError_t launch_col_mean_series(const SeriesTable& sr, int D, int emb, const float* wts,
+cudaError_t launch_col_mean_series(const SeriesTable& sr, int n, int D, int emb, const float* wts,
                                    float* mu, float* sw, bool center, cudaStream_t st) {
-  return launch_chained(col_mean_series_kernel, dim3((D + 31) / 32, sr.n), 32 * kMeanWarps, 0, st,
-                        sr, D, emb, wts, mu, sw, center ? 1 : 0);
+  return launch_chained(col_mean_series_kernel, dim3((D + 31) / 32, n), 32 * kMeanWarps, 0, st, sr,
+                        sr.n - n, D, emb, wts, mu, sw, center ? 1 : 0);
 }
 
 cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int emb, int groups,

@@ -146,7 +146,7 @@ extern "C" traknn_status traknn_knn_scores_static(const float* X, int64_t N, int
   // the status word is the only scratch that must start at zero; every other
   // byte a kernel reads is written earlier in this same call
   if (cudaMemsetAsync(a.err, 0, sizeof(int), cs) != cudaSuccess ||
-      launch_col_mean_series(sr, (int)D, 1, nullptr, mu, nullptr, true, cs) != cudaSuccess ||
+      launch_col_mean_series(sr, 1, (int)D, 1, nullptr, mu, nullptr, true, cs) != cudaSuccess ||
       launch_prep_fp32_series(sr, (int)N, (int)D, lay.Dp, mu, nullptr, Xc, norms, cs) !=
           cudaSuccess ||
       launch_window_series(sr, M, norms, W, ClearArgs{}, cs) != cudaSuccess ||

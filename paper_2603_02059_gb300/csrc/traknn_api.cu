@@ -55,6 +55,7 @@ struct TcPlan {
   int mask_words = 1;  // 32-bit words per row of the non-empty column-list masks
   int sym = 1;         // upper triangle with column lists, or both triangles
   bool band = true;    // the band units run (see prepare_tc)
+  bool shared = false; // several settings of one record: one set of operand rows
 };
 
 constexpr size_t kMaxGraphs = 16;  // captured launch sequences kept per handle
@@ -286,6 +287,7 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
   }
   p.pstrip = pstrip;
   p.sym = sym;
+  p.shared = shared;
   p.egroups = egroups;
   p.pu.assign(1, 0);
   for (int q = 0; q < K; ++q) {
@@ -419,9 +421,9 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   // contraction sets a tile's pace: K entries below a line (the more the series that scan
   // each tile), or hardly more tiles than SMs, so that a call is as long as one tile. Else
   // one group and pairs of CTAs (kernel_tc.cu). Measured, two groups / pairs (N = 10,957, L =
-  // 5): split-BF16 D = 990 453 / 611 us, 1,476 552 / 639, 2,116 763 / 806, 3,726 1,291 /
-  // 997; BF16 D = 1,476 513 / 614, 3,726 1,009 / 880; D = 3,726, N = 1,826 230 / 240, 3,000
-  // 313 / 342, 4,500 368 / 371, 6,500 538 / 498.
+  // 5): split-BF16 D = 990 453 / 611 us, 1,476 552 / 639, 2,200 746 / 677 (L = 10, k = 20 829 /
+  // 834), 3,726 1,291 / 997; BF16 D = 1,800 559 / 577, 2,800 787 / 714; D = 3,726, N = 1,826
+  // 230 / 240, 3,000 313 / 342, 4,500 368 / 371, 6,500 538 / 498.
   int Lmax = 1, kmax = 1;
   double tiles_all = 0.0;  // Gram tiles of the call
   for (int b = 0; b < B; ++b) {
@@ -431,7 +433,7 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     tiles_all += M * M / ((h->sym ? 2.0 : 1.0) * kTileRows * kTileCols);
   }
   const int Dk = tc_groups((int)D * emb) * 64;
-  const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2304 : 3072) * (shared ? B : 1);
+  const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2048 : 2304) * (shared ? B : 1);
   const bool fp32 = h->precision == TRAKNN_PREC_FP32;  // (its kernel has two groups)
   const int egroups =
       fp32 || (h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k &&
@@ -440,16 +442,20 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
           : 1;
   const bool pair = !fp32 && egroups == 1 && h->sm_count >= 2;
   key.push_back(egroups);
-  // Band pre-pass width in tiles per strip. Short operand rows: a tile's contraction is cheap
-  // and eight tiles save more list entries in the main pass than the band costs (D = 32, L =
-  // 5, N = 4,000 1 / 2 / 4 / 8 tiles 171 / 152 / 131 / 133 us). Otherwise one tile while its
-  // 64 groups of columns still resolve k (k <= 20; N = 10,957, D = 3,726, k = 10 1 / 2 / 4
-  // tiles 1,180 / 1,209 / 1,293 us, four lengths 1,865 / 1,952; D = 512, N = 1,826 139 / 155
-  // / 199), two for larger k (the last case with k = 40: 220 / 203 / 234).
+  // Band pre-pass width in tiles per strip. Short operand rows: four tiles, two where the
+  // whole call has fewer Gram tiles than the GPU SMs, so that the band lasts as long as its
+  // units (1 / 2 / 4 / 8 tiles, k = 20 or 10: D = 100, N = 27,394 1,169 / 1,065 / 1,046 / 1,087
+  // us; D = 320, N = 10,957 373 / 348 / 342 / 380; D = 600, N = 5,000 242 / 218 / 215 / 246; D =
+  // 750, N = 3,000 145 / 145 / 163 / 209; D = 32, N = 4,000 171 / 152 / 131 / 133). Otherwise
+  // one tile while its 64 groups of columns still resolve k (k <= 20; N = 10,957, D = 3,726, k
+  // = 10 1 / 2 / 4 tiles 1,180 / 1,209 / 1,293 us, four lengths 1,865 / 1,952; D = 512, N =
+  // 1,826 139 / 155 / 199), two for larger k (the last case with k = 40: 220 / 203 / 234).
   // FP32: a band column costs as much as a main one; 1 / 2 / 8 tiles: D = 32, N = 27,394
   // 2,023 / 1,938 / 1,996 us, N = 4,000 190 / 181 / 233; D = 512, N = 1,826 310 / 410 / 983;
   // D = 3,726, N = 10,957 11.2 / 12.0 / 16.5 ms
-  const int band_tiles = fp32 ? (D <= 64 ? 2 : 1) : Dk <= 768 ? 8 : kmax <= 20 ? 1 : 2;
+  const int band_tiles = fp32 ? (D <= 64 ? 2 : 1)
+                         : Dk <= 768 ? (tiles_all < h->sm_count ? 2 : 4)
+                                     : (kmax <= 20 ? 1 : 2);
   key.push_back(band_tiles);
   TcPlan& p = h->plan;
   if (p.key != key) {
@@ -622,7 +628,8 @@ traknn_status enqueue_prep(traknn_ctx* h, const TcBuffers& b, int64_t D, int lo,
   const SeriesTable& sr = p.table;
   const float* sw = h->weights ? b.sw : nullptr;
   if (counters > 0)
-    TRY_CUDA(launch_col_mean_series(sr, (int)D, p.emb, h->weights, b.mu, b.sw, h->center != 0, s));
+    TRY_CUDA(launch_col_mean_series(sr, p.shared ? 1 : sr.n, (int)D, p.emb, h->weights, b.mu, b.sw,
+                                    h->center != 0, s));
   if (h->precision == TRAKNN_PREC_FP32)
     TRY_CUDA(launch_prep_fp32_series(sr, p.rows, (int)D, b.Dp, b.mu, sw,
                                      static_cast<float*>(b.hi), b.norms, s));
@@ -843,7 +850,8 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
 }
 
 // The unit length a forward call takes: one Gram tile for operand rows of more than 768 K
-// entries, whatever default_shape says. Issued at its full rate the contraction no longer
+// entries, or k > 32 (pairs of CTAs: D = 32, N = 27,394, k = 64 1 / 2 / 4 / 16 tiles 2,238 /
+// 2,301 / 2,353 / 2,609 us), whatever default_shape says. Issued at its full rate the contraction no longer
 // hides what the longer units cost at the end of a launch and in L2, and lists and bounds
 // that live for one tile cost little: 1 / 2 / 4 / 8 tiles, N = 27,394, D = 3,726, L = 5, k =
 // 20 4,949 / 5,062 / 5,905 / 5,945 us (the last two before the MMAs were issued by an
@@ -851,15 +859,21 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
 // 473 us. Longer again while the call's row-side lists (one per row and unit) number more
 // than 4 M (4 GB).
 int unit_tiles(const HostSeries* sd, int B, int64_t D, int emb, int tiles) {
-  if (tc_groups((int)D * emb) * 64 <= 768) return tiles;
-  for (int t = 1; t < tiles; t *= 2) {
-    double lists = 0.0;
+  int kmax = 1;
+  for (int b = 0; b < B; ++b) kmax = std::max(kmax, sd[b].k);
+  auto lists = [&](int t) {
+    double n = 0.0;
     for (int b = 0; b < B; ++b) {
       const double M = (double)(sd[b].N - sd[b].L + 1);
-      lists += M * std::ceil(M / (t * kTileCols - (sd[b].L - 1)));
+      n += M * std::ceil(M / (t * kTileCols - (sd[b].L - 1)));
     }
-    if (lists <= 4e6) return t;
-  }
+    return n;
+  };
+  if (tc_groups((int)D * emb) * 64 > 768 || kmax > 32)
+    for (int t = 1; t < tiles; t *= 2)
+      if (lists(t) <= 4e6) return t;
+  // (hundreds of thousands of days: at most 16 GB of lists of the least capacity)
+  while (tiles < 1024 && 2.0 * lists(tiles) * (list_pitch(kmax) + 44) * 8.0 > 16e9) tiles *= 2;
   return tiles;
 }
 
@@ -973,7 +987,7 @@ traknn_status run_fp32_short(traknn_ctx* h, const HostSeries& sd, int64_t D, cud
   sr.s[0].M = M;
   sr.s[0].L = sd.L;
   sr.s[0].X = sd.X;
-  TRY_CUDA(launch_col_mean_series(sr, (int)D, 1, h->weights, mu, sw, h->center != 0, s));
+  TRY_CUDA(launch_col_mean_series(sr, 1, (int)D, 1, h->weights, mu, sw, h->center != 0, s));
   TRY_CUDA(launch_prep_fp32_series(sr, (int)sd.N, (int)D, lay.Dp, mu, h->weights ? sw : nullptr,
                                    Xc, norms, s));
   TRY_CUDA(launch_window_series(sr, M, norms, W, ClearArgs{}, s));
