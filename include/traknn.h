@@ -62,7 +62,9 @@ typedef enum {
  * "Optimized Spatial Distance Computation"). Day norms, window sums and
  * scores are accumulated in FP64 in every mode. */
 typedef enum {
-  TRAKNN_PREC_FP32 = 0,       /* CUDA-core FP32 FMA Gram */
+  TRAKNN_PREC_FP32 = 0,       /* CUDA-core FP32 FMA Gram, upper triangle (both triangles for the
+                                 shortest series and where the column-side lists would exceed
+                                 32 GB or find no memory) */
   TRAKNN_PREC_SPLIT_BF16 = 1, /* tensor cores: x = hi + lo (two BF16), G = hi.hi + hi.lo + lo.hi, FP32 accumulate */
   TRAKNN_PREC_BF16 = 2        /* tensor cores: single BF16 product, FP32 accumulate (lower accuracy) */
 } traknn_precision;
@@ -72,7 +74,8 @@ typedef enum {
   TRAKNN_OPT_CENTER = 1,             /* 1: subtract the per-grid-point mean over days before the
                                         Gram (the last 4,096 days, or all when fewer; exact by the
                                         offset invariance of Eq. 2 whatever the mean; default 1) */
-  TRAKNN_OPT_COL_CHUNKS = 2,         /* column chunks per row strip, 0 = automatic */
+  TRAKNN_OPT_COL_CHUNKS = 2,         /* FP32 path: column chunks of the longest row strip (the
+                                        results are the same); 0 = automatic */
   TRAKNN_OPT_WAIT_LIMIT_MS = 3,      /* limit of every device spin-wait in ms (default 2000) */
   TRAKNN_OPT_DEBUG_WITHHOLD = 4,     /* test hook: 1 makes the tensor-core kernel's producer withhold
                                         the first stage of work unit 0, so that the consumer's bounded
@@ -83,11 +86,11 @@ typedef enum {
   TRAKNN_OPT_SYMMETRIC = 6,          /* tensor-core paths: 1 evaluates each unordered pair once
                                         (upper triangle, Sec. 3.3), 0 both triangles (default 1) */
   TRAKNN_OPT_UNIT_COLS = 7,          /* tensor-core paths: output columns per work unit; 0 = auto:
-                                        units of 2, 4 or 8 Gram tiles of 256 columns, by the Gram
-                                        tiles per SM of an average series of the call (8 from
-                                        64, 4 from 16) and at most 65,536 operand K entries x
-                                        tiles; 16 tiles for operand rows of at most 768 K
-                                        entries (the results are the same) */
+                                        units of one Gram tile of 256 columns for operand rows
+                                        of more than 768 K entries or k > 32, else 1 to 16 tiles
+                                        by the Gram tiles per SM of an average series of the
+                                        call; longer where the call's candidate lists would take
+                                        many GB (the results are the same) */
   TRAKNN_OPT_STATS = 8,              /* 1: count kernel events (read with traknn_stats_read) */
   TRAKNN_OPT_AUTOTUNE = 9,           /* tensor-core paths: 1 times every work-unit shape of
                                         {4, 8, 16} Gram tiles per unit x {10, 19, 38} row strips
@@ -111,11 +114,13 @@ typedef enum {
                                         (L times the contraction, no diagonal sums); 2 never;
                                         0 (default) when L*D <= 1536, the small-grid form (Sec. 5:
                                         fields reduced to a few dozen principal components) */
-  TRAKNN_OPT_EPI_GROUPS = 14         /* tensor-core paths: 1 keeps one epilogue warpgroup; 0
-                                        (default) uses two at L = 1 (embedded operands included)
-                                        when the grid fits one accumulation segment and k <= 32,
-                                        each reading half of every tile's columns (the results
-                                        are the same) */
+  TRAKNN_OPT_EPI_GROUPS = 14         /* tensor-core paths: 1 keeps one epilogue warpgroup, with
+                                        pairs of CTAs sharing their column operands; 0 (default)
+                                        uses two, each reading half of every tile's columns,
+                                        when the grid fits one accumulation segment, k <= 32 and
+                                        the epilogue sets a tile's pace: operand rows of up to
+                                        about 2,000 K entries, or hardly more tiles than SMs
+                                        (the results are the same) */
 } traknn_option;
 
 #define TRAKNN_MAX_L 17  /* longest trajectory (days) supported */
@@ -184,13 +189,12 @@ typedef struct {
  * its own N, L, k and exclusion; the method of Sec. 3.2 applied to each series
  * separately, as when a study scores several regions, variables or ensemble
  * members). Every series' outputs equal those of traknn_knn_scores on it alone.
- * With a tensor-core precision up to 64 series run in one persistent launch
- * sequence, which is captured as a CUDA graph on first use and replayed on later
+ * Up to 64 series run in one persistent launch sequence, which is captured as a CUDA graph on first use and replayed on later
  * calls with the same shapes, pointers and options (the handle keeps one graph
  * per such signature, the 16 most recent; a change of shape or a larger workspace
  * drops them; evicting the oldest synchronises `stream` once).
- * With TRAKNN_PREC_FP32 the series run one after another. Each series is
- * checked as traknn_check_problem would check it; the first failing series'
+ * With TRAKNN_PREC_FP32 series whose column-side lists would together take more
+ * than 32 GB run one after another. Each series is checked as traknn_check_problem would check it; the first failing series'
  * status is returned before anything is enqueued. */
 traknn_status traknn_knn_scores_batched(traknn_handle handle, const traknn_series* series, int B,
                                         int64_t D, void* stream);
@@ -198,14 +202,14 @@ traknn_status traknn_knn_scores_batched(traknn_handle handle, const traknn_serie
 /* Several (L, k, exclusion) settings of ONE record in one Gram sweep (Sec. 6: the
  * "what-if" analyses over trajectory lengths). All nset entries must share X and N
  * (the same device pointer and day count; D as given) and differ in L, k, exclusion
- * and their output buffers (layouts as in traknn_knn_scores). With a tensor-core
- * precision the Gram tiles are computed once (strip height and tile step sized for
+ * and their output buffers (layouts as in traknn_knn_scores). The Gram tiles are computed once (strip height and tile step sized for
  * the largest L) and every tile is scanned once per setting, so the cost is close to
  * that of one setting when the contraction dominates (large D). Each setting's
  * outputs equal those of traknn_knn_scores on it alone except that, as in that call,
  * D(t,j) may be evaluated from either operand order: distances agree to a few ulp
- * and neighbour sets may differ only at near ties. With TRAKNN_PREC_FP32 the settings
- * run one after another. 1 <= nset <= 64; each entry is checked as
+ * and neighbour sets may differ only at near ties. With TRAKNN_PREC_FP32 settings
+ * whose column-side lists would together take more than 32 GB run one after another.
+ * 1 <= nset <= 64; each entry is checked as
  * traknn_check_problem would check it; entries with another X or N are refused
  * (TRAKNN_ERR_INVALID_ARG). */
 traknn_status traknn_knn_scores_multi(traknn_handle handle, const traknn_series* settings,
@@ -326,8 +330,8 @@ traknn_status traknn_sync_status(traknn_handle handle, void* stream);
 traknn_status traknn_profile_read(traknn_handle handle, float* ms, int max_n, int* n_out);
 
 /* Event counters of the tensor-core kernel accumulated while TRAKNN_OPT_STATS was on
- * (diagnostics): [0] row-side list insertions, [1] column-side candidates,
- * [2] column lists with more than k candidates (the column's own thread keeps the
+ * (diagnostics): [0] row-side candidates appended, [1] column-side candidates,
+ * [2] column lists with more candidates than their records hold (a warp keeps the
  * k best), [3] non-empty column lists,
  * [4] 32-column chunks processed, [5] MMA-thread cycles waiting for a free
  * accumulator, [6] MMA-thread cycles waiting for operands, [7] MMA-thread cycles

@@ -481,7 +481,7 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     }
     build_plan(sd, B, D, fp32 ? 1 : h->sym, cols, tile_cols < kTileCols ? 1 : tiles, group,
                shared, part_lo, part_hi, pstrip, egroups, band_tiles, p, tile_cols);
-    p.key = key;
+    p.key.clear();  // until the new list is on the device
     p.emb = emb;
     p.part_lo = part_lo;
     p.part_hi = part_hi;
@@ -499,6 +499,7 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
                         cudaMemcpyHostToDevice));
     TRY_CUDA(cudaMemcpy(pd + ub + cb, p.slot_lo.data(), p.slot_lo.size() * sizeof(int),
                         cudaMemcpyHostToDevice));
+    p.key = key;
     drop_graphs(h);  // graphs captured the previous work list
   }
   for (int b = 0; b < B; ++b) {
@@ -949,7 +950,8 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   return TRAKNN_OK;
 }
 
-// The shortest FP32 calls on both triangles: one tile per CTA, no band and no column side,
+// FP32 calls on both triangles: the shortest ones, and those whose column-side lists would
+// not fit (run_fp32). Short calls: one tile per CTA, no band and no column side,
 // five launches. Its scan inserts into sorted lists in shared memory, about k steps per
 // candidate, so it pays up to a product of rows and neighbours, the more the longer a tile's
 // products take. Both triangles / upper triangle (us, L = 5): D = 16, N = 300 k = 5 48 / 64, k =
@@ -959,7 +961,7 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
 bool fp32_short(int64_t M, int64_t D, int k) {
   return M <= 1024 && M * k <= (D >= 200 ? 10000 : 4500);
 }
-traknn_status run_fp32_short(traknn_ctx* h, const HostSeries& sd, int64_t D, cudaStream_t s) {
+traknn_status run_fp32_both(traknn_ctx* h, const HostSeries& sd, int64_t D, cudaStream_t s) {
   const int M = (int)(sd.N - sd.L + 1);
   const Schedule sch = make_schedule(M, sd.L, sd.k, sd.e, h->sm_count, h->col_chunks);
   const Fp32Layout lay = make_layout(sd.N, D, sch);
@@ -1001,6 +1003,28 @@ traknn_status run_fp32_short(traknn_ctx* h, const HostSeries& sd, int64_t D, cud
   }
   TRY_CUDA(launch_merge(fa, sd.idx, sd.dist, sd.score, s));
   h->launches += 5;
+  return TRAKNN_OK;
+}
+
+// Forward pass on the CUDA cores: the upper triangle over the shared work plan (one launch
+// sequence for all series), or each series on both triangles. The column-side lists grow
+// with M^2 (0.7 KB per row and 1,024 rows at k = 20), both triangles need row lists only:
+// calls whose lists would take more than 32 GB (M > 215,000 at k = 20) or that find no
+// memory for them go series by series and, if it is one series, to both triangles.
+traknn_status run_fp32(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
+                       bool graph, bool shared) {
+  double lists = 0.0;
+  for (int b = 0; b < B; ++b) {
+    const double M = (double)(sd[b].N - sd[b].L + 1);
+    lists += M * M / (2.0 * (kTileRows - (sd[b].L - 1))) * col_pitch(list_pitch(sd[b].k)) * 4.0;
+  }
+  if (B == 1 && fp32_short(sd->N - sd->L + 1, D, sd->k)) return run_fp32_both(h, *sd, D, s);
+  if (lists <= 32e9) {
+    const traknn_status st = run_tc(h, sd, B, D, s, graph, shared);
+    if (st != TRAKNN_ERR_ALLOC) return st;
+  }
+  if (B == 1) return run_fp32_both(h, *sd, D, s);
+  for (int b = 0; b < B; ++b) TRY_ST(run_fp32(h, sd + b, 1, D, s, false, false));
   return TRAKNN_OK;
 }
 
@@ -1174,8 +1198,7 @@ traknn_status traknn_knn_scores(traknn_handle h, const float* X, int64_t N, int6
     return run_tc(h, &sd, 1, D, s, false, false, L);
   }
   const HostSeries sd{X, N, L, k, e, nbr_idx, nbr_dist, score};
-  if (h->precision == TRAKNN_PREC_FP32 && fp32_short(N - L + 1, D, k))
-    return run_fp32_short(h, sd, D, s);
+  if (h->precision == TRAKNN_PREC_FP32) return run_fp32(h, &sd, 1, D, s, false, false);
   return run_tc(h, &sd, 1, D, s, false);
 }
 
@@ -1190,8 +1213,12 @@ traknn_status traknn_knn_scores_batched(traknn_handle h, const traknn_series* se
   TRY_ST(validate_series(sd.data(), B, D));
   if (h->weights && h->weights_D != D) return TRAKNN_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  for (int b0 = 0; b0 < B; b0 += kMaxSeries)
-    TRY_ST(run_tc(h, sd.data() + b0, std::min(kMaxSeries, B - b0), D, s, true));
+  const bool fp32 = h->precision == TRAKNN_PREC_FP32;
+  for (int b0 = 0; b0 < B; b0 += kMaxSeries) {
+    const int n = std::min(kMaxSeries, B - b0);
+    TRY_ST(fp32 ? run_fp32(h, sd.data() + b0, n, D, s, true, false)
+                : run_tc(h, sd.data() + b0, n, D, s, true));
+  }
   return TRAKNN_OK;
 }
 
@@ -1212,6 +1239,7 @@ traknn_status traknn_knn_scores_multi(traknn_handle h, const traknn_series* sett
   // the shared geometry takes the smallest L (most trajectories) first
   std::stable_sort(sd.begin(), sd.end(),
                    [](const HostSeries& x, const HostSeries& y) { return x.L < y.L; });
+  if (h->precision == TRAKNN_PREC_FP32) return run_fp32(h, sd.data(), nset, D, s, false, true);
   return run_tc(h, sd.data(), nset, D, s, false, true);
 }
 

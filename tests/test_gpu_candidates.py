@@ -119,3 +119,22 @@ def test_pairs_of_ctas_equal_two_groups(tk, N, h, w, L, k, sym, seg):
             rel = (g[1].cpu() - ref[1].cpu()).abs() / ref[1].cpu()
             assert rel.max().item() <= 2e-4
             assert all(torch.equal(x.cpu(), y.cpu()) for x, y in zip(g, got[0]))
+
+
+@pytest.mark.parametrize("N,count", [(125000, 1), (90000, 2)])
+def test_fp32_calls_with_too_many_column_lists_equal_exact_rows(tk, N, count):
+    """Column-side lists above 32 GB (k = 64): one series goes to both triangles, two go one
+    after the other. Small integers, so rows compare exactly, ties included."""
+    import torch
+    k, e = 64, 3
+    X = _integers(N, 4, 200, seed=N)
+    Xd = torch.from_numpy(X).cuda()
+    got = tk.knn_scores_batched([(Xd, 1, k, e)] * count, precision="fp32", center=False)
+    Xi = X.astype(np.int64)
+    for t in (0, 1, N // 2, N - 1, 127, 128, 77777):
+        d = ((Xi - Xi[t]) ** 2).sum(axis=1)
+        d[max(0, t - e):t + e + 1] = np.iinfo(np.int64).max
+        order = np.argsort(d, kind="stable")[:k]
+        for idx, dist, _ in got:
+            assert np.array_equal(idx[t].cpu().numpy(), order)
+            assert np.array_equal(dist[t].cpu().numpy(), d[order].astype(np.float32))
