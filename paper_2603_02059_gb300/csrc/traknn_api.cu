@@ -920,9 +920,9 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
       return TRAKNN_OK;
     }
   if (!h->cap_stream) TRY_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
-  // run once outside the capture (kernel attributes, first-use costs), then capture
+  // The first call's results come from plain launches (kernel attributes, first-use costs);
+  // its sequence is captured for later calls while they run.
   TRY_ST(enqueue_tc(h, buf, D, s, false));
-  TRY_CUDA(cudaStreamSynchronize(s));
   const int64_t l0 = h->launches;
   TRY_CUDA(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
   const traknn_status st = enqueue_tc(h, buf, D, h->cap_stream, false);
@@ -945,8 +945,7 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
     h->graphs.erase(h->graphs.begin());
   }
   h->graphs.push_back(GraphEntry{key, exec});
-  TRY_CUDA(cudaGraphLaunch(exec, s));
-  h->launches += 5 + (h->plan.band && h->plan.nband > 0 ? 1 : 0);
+  TRY_CUDA(cudaStreamSynchronize(s));
   return TRAKNN_OK;
 }
 
