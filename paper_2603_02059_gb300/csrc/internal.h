@@ -377,13 +377,6 @@ inline void split_strips(long long M, int L, int nparts, int part, int* s_lo, in
   *s_lo = first(part);
   *s_hi = first(part + 1);
 }
-// emb > 1: each operand row is the emb-day trajectory starting at that day (emb * D
-// values, contiguous in X); the series table then describes trajectories (N = M, L = 1).
-// Rows [r_lo, rows) of the stacked operands (all rows with r_lo = 0).
-cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int emb, int groups,
-                                     bool correct, const float* mu, const float* sw, void* hi,
-                                     void* lo, double* norms, float* cval, cudaStream_t st,
-                                     int r_lo = 0);
 // What a main pass accumulates into, cleared by the window kernel row by row: bounds and
 // shared minima (0x7F bytes: a large finite value) and column-list masks of its rows, and
 // (with r_lo = 0 or a series' first launch: `counters` > 0) the unit counters.
@@ -397,6 +390,14 @@ struct ClearArgs {
   int* counter;
   int counters;
 };
+// emb > 1: each operand row is the emb-day trajectory starting at that day (emb * D
+// values, contiguous in X); the series table then describes trajectories (N = M, L = 1).
+// Rows [r_lo, rows) of the stacked operands (all rows with r_lo = 0). With W (one series,
+// L = 1: a row's norm is its window sum) it also does what launch_window_series does.
+cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int emb, int groups,
+                                     bool correct, const float* mu, const float* sw, void* hi,
+                                     void* lo, double* norms, float* cval, float* W,
+                                     const ClearArgs& clear, cudaStream_t st, int r_lo = 0);
 // Window sums of the stacked trajectory rows [r_lo, out_rows); clears what `clear` names
 // for those rows (thr null: nothing).
 cudaError_t launch_window_series(const SeriesTable& sr, int out_rows, const double* norms,

@@ -141,6 +141,22 @@ __device__ __forceinline__ float correction(double n, int groups) {
   return __bfloat162float(__float2bfloat16_rn(v));
 }
 
+// What the window kernel clears, for the `n` rows of a block that prepares operand rows which
+// are trajectories (one series, L = 1: embedded operands above all). Saves those calls the
+// window kernel: one year of 8 x 8 61.7 -> 59.7 us, five years of 16 x 32 121.6 -> 119.8.
+__device__ __forceinline__ void clear_block(const ClearArgs& c, int r_lo, int rows, int n) {
+  const int r0 = r_lo + blockIdx.x * n;
+  n = min(n, rows - r0);
+  if (blockIdx.x == 0 && (int)threadIdx.x < c.counters) c.counter[threadIdx.x] = 0;
+  for (int q = threadIdx.x; q < n * c.slots; q += blockDim.x) {
+    const int i = q / n, r = r0 + q - i * n;
+    c.shared_min[i * c.stride + r] = 0x7F7F7F7Fu;
+    if (i == 0) c.thr[r] = 0x7F7F7F7Fu;
+  }
+  for (int q = threadIdx.x; q < n * c.mask_words; q += blockDim.x)
+    c.col_mask[(size_t)r0 * c.mask_words + q] = 0u;
+}
+
 // One warp per stacked day: the centred row x - mu(series) as two BF16 copies hi + lo
 // (split form; the BF16 form uses hi alone) in the tensor-core operand layout, its
 // FP64 norm, and its correction value.
@@ -167,14 +183,16 @@ __global__ void __launch_bounds__(256)
                              int emb, int groups, const float* __restrict__ mu,
                              const float* __restrict__ sw, __nv_bfloat16* __restrict__ hi,
                              __nv_bfloat16* __restrict__ lo, double* __restrict__ norms,
-                             float* __restrict__ cval) {
+                             float* __restrict__ cval, float* __restrict__ W,
+                             const ClearArgs ca) {
   // per warp: 32 finished groups of one copy (36-word rows: 16-byte aligned)
   __shared__ __align__(16) uint32_t stage[8][32 * 36];
   const int r = r_lo + blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (r >= rows) return;
   launch_wait();
   launch_next();
+  if (W) clear_block(ca, r_lo, rows, 8);
+  if (r >= rows) return;
   uint32_t* sh = stage[threadIdx.x >> 5];
   const int b = find_series(st.s, st.n, r, false);
   const SeriesInfo& si = st.s[b];
@@ -191,6 +209,7 @@ __global__ void __launch_bounds__(256)
     if (lane == 0) {
       norms[r] = 0.0;
       cval[r] = 0.f;
+      if (W) W[r] = 0.f;
     }
     return;
   }
@@ -258,6 +277,7 @@ __global__ void __launch_bounds__(256)
   if (lane == 0) {
     norms[r] = acc;
     cval[r] = c;
+    if (W) W[r] = (float)acc;
   }
 }
 
@@ -271,9 +291,11 @@ __global__ void __launch_bounds__(256)
                             int emb, int groups, const float* __restrict__ mu,
                             const float* __restrict__ sw, __nv_bfloat16* __restrict__ hi,
                             __nv_bfloat16* __restrict__ lo, double* __restrict__ norms,
-                            float* __restrict__ cval) {
+                            float* __restrict__ cval, float* __restrict__ W,
+                            const ClearArgs ca) {
   launch_wait();
   launch_next();
+  if (W) clear_block(ca, r_lo, rows, 8 * (32 / groups));
   const int lane = threadIdx.x & 31;
   const int per_warp = 32 / groups;
   const int rl = lane / groups, g = lane - rl * groups;  // row of the warp, group of the row
@@ -351,6 +373,7 @@ __global__ void __launch_bounds__(256)
   if (g == 0) {
     norms[r] = pad ? 0.0 : acc;
     cval[r] = c;
+    if (W) W[r] = pad ? 0.f : (float)acc;
   }
 }
 
@@ -864,8 +887,8 @@ cudaError_t launch_col_mean_series(const SeriesTable& sr, int n, int D, int emb,
 
 cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int emb, int groups,
                                      bool correct, const float* mu, const float* sw, void* hi,
-                                     void* lo, double* norms, float* cval, cudaStream_t st,
-                                     int r_lo) {
+                                     void* lo, double* norms, float* cval, float* W,
+                                     const ClearArgs& clear, cudaStream_t st, int r_lo) {
   if (rows <= r_lo) return cudaSuccess;
   __nv_bfloat16* h = static_cast<__nv_bfloat16*>(hi);
   __nv_bfloat16* l = static_cast<__nv_bfloat16*>(lo);
@@ -877,7 +900,7 @@ cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int
                             : (correct ? prep_split_series_kernel<true>
                                        : prep_split_series_kernel<false>);
   return launch_chained(kernel, blocks, 256, 0, st, sr, r_lo, rows, D, emb, groups, mu, sw, h, l,
-                        norms, cval);
+                        norms, cval, W, clear);
 }
 
 cudaError_t launch_window_series(const SeriesTable& sr, int out_rows, const double* norms,

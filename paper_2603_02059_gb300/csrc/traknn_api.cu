@@ -620,6 +620,13 @@ traknn_status launch_units(traknn_ctx* h, const TcBuffers& b, const TcArgs& a, c
   return TRAKNN_OK;
 }
 
+// Whether the operand preparation also writes the window sums: its rows are trajectories.
+bool windows_in_prep(const traknn_ctx* h) {
+  const SeriesTable& sr = h->plan.table;
+  return h->precision != TRAKNN_PREC_FP32 && sr.n == 1 && sr.s[0].L == 1 &&
+         h->plan.rows == h->plan.out_rows;
+}
+
 // Means, operand rows [lo, hi) and window sums of the trajectory rows [lo, ohi), whose bounds
 // and masks are cleared; `counters` > 0 also clears that many unit counters, and computes
 // the means first.
@@ -631,17 +638,20 @@ traknn_status enqueue_prep(traknn_ctx* h, const TcBuffers& b, int64_t D, int lo,
   if (counters > 0)
     TRY_CUDA(launch_col_mean_series(sr, p.shared ? 1 : sr.n, (int)D, p.emb, h->weights, b.mu, b.sw,
                                     h->center != 0, s));
+  const ClearArgs clear{b.thr,      b.shared_min, p.out_rows, min_slots(p.kmax),
+                        b.col_mask, p.mask_words, b.counter,  counters};
+  const bool rows_are_windows = windows_in_prep(h);
   if (h->precision == TRAKNN_PREC_FP32)
     TRY_CUDA(launch_prep_fp32_series(sr, p.rows, (int)D, b.Dp, b.mu, sw,
                                      static_cast<float*>(b.hi), b.norms, s));
   else
     TRY_CUDA(launch_prep_split_series(sr, hi, (int)D, p.emb, b.Dp / 64,
                                       h->precision == TRAKNN_PREC_SPLIT_BF16, b.mu, sw, b.hi, b.lo,
-                                      b.norms, b.cval, s, lo));
-  const ClearArgs clear{b.thr,      b.shared_min, p.out_rows, min_slots(p.kmax),
-                        b.col_mask, p.mask_words, b.counter,  counters};
-  TRY_CUDA(launch_window_series(sr, ohi, b.norms, b.W, clear, s, lo));
-  h->launches += (counters > 0 ? 1 : 0) + (hi > lo ? 1 : 0) + (ohi > lo ? 1 : 0);
+                                      b.norms, b.cval, rows_are_windows ? b.W : nullptr, clear, s,
+                                      lo));
+  if (!rows_are_windows) TRY_CUDA(launch_window_series(sr, ohi, b.norms, b.W, clear, s, lo));
+  h->launches += (counters > 0 ? 1 : 0) + (hi > lo ? 1 : 0) +
+                 (ohi > lo && !rows_are_windows ? 1 : 0);
   return TRAKNN_OK;
 }
 
@@ -916,7 +926,8 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   for (auto& g : h->graphs)
     if (g.key == key) {
       TRY_CUDA(cudaGraphLaunch(g.exec, s));
-      h->launches += 5 + (h->plan.band && h->plan.nband > 0 ? 1 : 0);
+      h->launches += 5 - (windows_in_prep(h) ? 1 : 0) +
+                     (h->plan.band && h->plan.nband > 0 ? 1 : 0);
       return TRAKNN_OK;
     }
   if (!h->cap_stream) TRY_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));

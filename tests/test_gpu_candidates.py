@@ -138,3 +138,22 @@ def test_fp32_calls_with_too_many_column_lists_equal_exact_rows(tk, N, count):
         for idx, dist, _ in got:
             assert np.array_equal(idx[t].cpu().numpy(), order)
             assert np.array_equal(dist[t].cpu().numpy(), d[order].astype(np.float32))
+
+
+@pytest.mark.parametrize("N,D,L", [(301, 1100, 1), (129, 40, 1), (1003, 600, 1), (333, 90, 4),
+                                   (4100, 700, 1)])
+def test_rows_that_are_trajectories_equal_the_oracle(tk, N, D, L):
+    """L = 1 and embedded operands: the operand preparation writes the window sums and clears
+    the bounds, for few and many groups per row and ragged blocks, on used workspaces too."""
+    import torch
+    for seed in (N, N + 1):
+        X = _integers(N, D, 3, seed=seed)
+        oidx, odist, _ = oracle.knn_scores(X, L, 7, 2)
+        Xd = torch.from_numpy(X).cuda()
+        for prec in ("split_bf16", "bf16"):
+            got = [tk.knn_scores(Xd, L, 7, 2, precision=prec, center=False, embed="always")]
+            if L == 1:
+                got += tk.knn_scores_batched([(Xd, L, 7, 2)], precision=prec, center=False)
+            for idx, dist, _ in got:
+                assert np.array_equal(dist.cpu().numpy(), odist.astype(np.float32))
+                assert np.array_equal(idx.cpu().numpy(), oidx)
