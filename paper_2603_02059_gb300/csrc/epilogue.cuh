@@ -264,18 +264,25 @@ __device__ __forceinline__ unsigned list_bound(const unsigned (&db)[kListRegs], 
   }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
+  // Three thresholds a step: their counts (at most 128 each) share a word, and so one
+  // reduction, whose latency is most of a step (against one threshold: four lengths at 30
+  // years 1,661 -> 1,641 us, 20 years BF16 544 -> 539, five years of 16 x 32 122.3 -> 121.0).
   while (lo < hi) {
-    const unsigned mid = lo + ((hi - lo) >> 1);
-    int c = 0;
+    const unsigned d = hi - lo, m1 = lo + (d >> 2), m2 = lo + (d >> 1), m3 = m2 + (d >> 2);
+    unsigned n = 0;
 #pragma unroll
-    for (int u = 0; u < kListRegs; ++u) c += db[u] <= mid ? 1 : 0;
-    c = __reduce_add_sync(0xffffffffu, c);
-    if (c < k) {
-      lo = mid + 1;
-    } else {
-      hi = mid;
-      if (c <= most) break;
+    for (int u = 0; u < kListRegs; ++u)
+      n += (db[u] <= m1 ? 1u : 0u) + (db[u] <= m2 ? 1u << 8 : 0u) + (db[u] <= m3 ? 1u << 16 : 0u);
+    n = __reduce_add_sync(0xffffffffu, n);
+    const int c1 = n & 0xFF, c2 = (n >> 8) & 0xFF, c3 = n >> 16;
+    if (c3 < k) {
+      lo = m3 + 1;
+      continue;
     }
+    const int c = c1 >= k ? c1 : c2 >= k ? c2 : c3;
+    if (c1 < k) lo = (c2 >= k ? m1 : m2) + 1;
+    hi = c1 >= k ? m1 : c2 >= k ? m2 : m3;
+    if (c <= most) break;
   }
   return hi;
 }
