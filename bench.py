@@ -313,14 +313,14 @@ def l2_note(N, D):
 
 
 def fp32_roofline(N, D, kms, peaks):
-    """FP32 CUDA-core path: both triangles of the Gram (N^2 x 2D flops) against the
+    """FP32 CUDA-core path: the Gram's upper triangle (N(N+1)/2 x 2D flops) against the
     FP32 FMA peak of 152 SMs at the maximum SM clock."""
     if not kms:
         return None
     import torch
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
     peak = fp32_alu_peak_tflops(sms, float(peaks.get("sm_max_mhz", 2070.0)))
-    ach = float(N) * N * 2 * D / (statistics.mean(kms) * 1e-3) / 1e12
+    ach = float(N) * (N + 1) * D / (statistics.mean(kms) * 1e-3) / 1e12
     return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
             "peak_source": f"{sms} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 x sm_max_mhz"}
 
