@@ -273,7 +273,7 @@ __host__ __device__ inline int min_slots(int kmax) { return kmax <= 40 ? 64 : 12
 
 // Event counters of the tensor-core kernel (diagnostics, TRAKNN_OPT_STATS).
 enum : int {
-  kStatRowInserts = 0,     // row-side list insertions
+  kStatRowInserts = 0,     // row-side candidates appended
   kStatColEmits = 1,       // column-side candidates handed to a column
   kStatColFull = 2,        // column lists with more than k candidates (k best kept)
   kStatColLists = 3,       // non-empty column lists written

@@ -84,7 +84,8 @@ __device__ __forceinline__ void store_stage(Stages& sm, int buf, int tid, const 
 // both triangles with scalar FMAs, 60.3 ms now (0.63 of the FMA rate). What bounds it: a
 // 16-byte shared-memory load of a warp takes four cycles of the SM's return path, so the
 // four loads per product of eight warps take as long as their FMAs. 8 x 16 outputs per
-// thread would need three quarters of that, but spill (80 ms).
+// thread would need three quarters of that, but their partial sums leave no registers to hold
+// the next operands (running sums in tensor memory, asynchronous copies: 67 to 81 ms).
 __device__ __forceinline__ void gram_tile(Stages& sm, const float* __restrict__ Xc, int end,
                                           int Dp, int r0, int c0, int tid, float* g, int pitch) {
   const int lane = tid & 31, warp = tid >> 5;

@@ -862,8 +862,9 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
 
 // The unit length a forward call takes: one Gram tile for operand rows of more than 768 K
 // entries, or k > 32 (pairs of CTAs: D = 32, N = 27,394, k = 64 1 / 2 / 4 / 16 tiles 2,238 /
-// 2,301 / 2,353 / 2,609 us), whatever default_shape says. Issued at its full rate the contraction no longer
-// hides what the longer units cost at the end of a launch and in L2, and lists and bounds
+// 2,301 / 2,353 / 2,609 us), whatever default_shape says. Issued at its full rate the
+// contraction no longer hides what the longer units cost at the end of a launch and in L2, and
+// lists and bounds
 // that live for one tile cost little: 1 / 2 / 4 / 8 tiles, N = 27,394, D = 3,726, L = 5, k =
 // 20 4,949 / 5,062 / 5,905 / 5,945 us (the last two before the MMAs were issued by an
 // elected lane), N = 10,957 997 / 1,029, D = 58,101 91.9 / 94.4 ms, D = 990, N = 10,957 452 /
