@@ -230,6 +230,13 @@ __host__ __device__ inline int list_cap(int kstride, long long lists) {
   return lists * kListCap * 8 <= (4LL << 30) ? kListCap : kstride + 44;
 }
 
+// Entries to read of a list that records n of them in room for `cap`. A CTA that gives up a
+// bounded wait leaves the counts of its units unwritten: they hold whatever the workspace
+// held before, and such a list counts as empty (the call reports the timeout).
+__host__ __device__ inline int list_entries(int n, int cap) {
+  return (unsigned)n <= (unsigned)cap ? n : 0;
+}
+
 // Ints per column-list record for list pitch kstride (a multiple of 4).
 __host__ __device__ inline int col_pitch(int kstride) { return 4 + 2 * kstride; }
 

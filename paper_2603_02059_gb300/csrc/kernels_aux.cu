@@ -697,7 +697,7 @@ __device__ __forceinline__ void merge_row(const int2* __restrict__ part,
       const int c = c0 + lane;
       int nn = 0;
       if (c < c_hi && tk_in(plist + c, w.part_lists, err)) nn = __ldg(part_n + plist + c);
-      if (!tk_in(nn, cap + 1, err)) nn = 0;
+      nn = tk_in(nn, cap + 1, err) ? list_entries(nn, cap) : 0;
       int incl = nn;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -770,7 +770,7 @@ __device__ __forceinline__ void merge_row(const int2* __restrict__ part,
           if (ri < 0) continue;
           const int4* r4 = reinterpret_cast<const int4*>(w.col_rec + ri);
           const int4 h0 = __ldg(r4), h1 = __ldg(r4 + 1);
-          const int nn = tk_in(h0.x, ks + 1, err) ? h0.x : 0;  // count <= k
+          const int nn = tk_in(h0.x, ks + 1, err) ? list_entries(h0.x, ks) : 0;
           if (nn > 0 && __int_as_float(h0.w) <= thr) push(__int_as_float(h0.w), h0.z);
           if (nn > 1 && __int_as_float(h1.y) <= thr) push(__int_as_float(h1.y), h1.x);
           if (nn > 2 && __int_as_float(h1.w) <= thr) push(__int_as_float(h1.w), h1.z);
@@ -814,7 +814,7 @@ __device__ __forceinline__ void merge_row(const int2* __restrict__ part,
       for (int c = c_lo + lane; c < c_hi; c += 32) {
         if (!tk_in(plist + c, w.part_lists, err)) continue;
         const int2* l2 = part + (size_t)(plist + c) * cap;
-        const int nn = part_n[plist + c];
+        const int nn = list_entries(part_n[plist + c], cap);
         for (int p = 0; p < nn; ++p) {
           const int2 e = l2[p];
           if (__int_as_float(e.y) <= thr) consider(__int_as_float(e.y), e.x);
@@ -828,7 +828,7 @@ __device__ __forceinline__ void merge_row(const int2* __restrict__ part,
             continue;  // an empty list has no record
           if (!tk_in(collist(s2) * cp + cp - 1, w.col_ints, err)) continue;
           const int2* rec = reinterpret_cast<const int2*>(w.col_rec + collist(s2) * cp);
-          const int nn = tk_in(rec[0].x, ks + 1, err) ? rec[0].x : 0;
+          const int nn = tk_in(rec[0].x, ks + 1, err) ? list_entries(rec[0].x, ks) : 0;
           for (int p = 0; p < nn; ++p) {
             const int2 e = rec[1 + p];
             if (__int_as_float(e.y) <= thr) consider(__int_as_float(e.y), e.x);
