@@ -95,10 +95,19 @@ struct Ctl {
   volatile int* abort;
   int* err;
   unsigned long long limit_ns;
+  uint32_t peer_abort;  // the abort flag of the pair's other CTA (0: a single CTA)
 };
 
+// A wait has run out: records the timeout and raises the abort flags.
+__device__ __forceinline__ void give_up(const Ctl& c) {
+  atomicCAS(c.err, 0, kErrTimeout);
+  *c.abort = 1;
+  if (c.peer_abort) ptx::st_remote_u32(c.peer_abort, 1u);
+}
+
 // Bounded wait on an mbarrier phase. Records a timeout and raises the CTA's abort
-// flag when the limit runs out; gives up early when another role aborted.
+// flag (and that of the pair's other CTA, whose roles would wait for this one's) when the
+// limit runs out; gives up early when another role aborted.
 // kCluster: what the other CTA of a pair wrote before it arrived is visible afterwards.
 template <bool kCluster = false>
 __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, const Ctl& c,
@@ -112,8 +121,7 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, cons
     if (ready()) return true;
     if (honor_abort && *c.abort) return false;
     if (ptx::globaltimer() - t0 > c.limit_ns) {
-      atomicCAS(c.err, 0, kErrTimeout);
-      *c.abort = 1;
+      give_up(c);
       return false;
     }
   }
@@ -165,17 +173,21 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
   const uint32_t qempty0 = qfull0 + 8u * kQueue;
   const uint32_t xfull = qempty0 + 8u * kQueue;  // second group's minima are in (band)
   const uint32_t xempty = xfull + 8u;            // ... and have been read
+  const uint32_t pdone = xempty + 8u;            // the pair's second producer has ended
   // units handed out, read by the MMA issuer and the epilogue (16-byte aligned; a
   // negative strip ends the list)
   WorkUnit* qunit = reinterpret_cast<WorkUnit*>(
-      (reinterpret_cast<uintptr_t>(bars + 2 * NS + 7 + 2 * kQueue) + 15) & ~uintptr_t(15));
+      (reinterpret_cast<uintptr_t>(bars + 2 * NS + 8 + 2 * kQueue) + 15) & ~uintptr_t(15));
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(qunit + kQueue);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  // the stages the pair's second CTA issued copies for, and their parities
+  volatile uint32_t* second = tmem_slot + 2;
 
   Ctl ctl;
   ctl.abort = abort_flag;
   ctl.err = a.err;
   ctl.limit_ns = (unsigned long long)a.wait_limit_ns;
+  ctl.peer_abort = kPair ? ptx::mapa(ptx::smem_u32(tmem_slot + 1), rank ^ 1) : 0u;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NS; ++i) {
@@ -195,6 +207,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     }
     ptx::mbar_init(xfull, kEpiThreads);
     ptx::mbar_init(xempty, kEpiThreads);
+    ptx::mbar_init(pdone, 1);
     *abort_flag = 0;
     ptx::fence_mbar_init();
     ptx::fence_proxy_async();
@@ -334,10 +347,54 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         }
       }
     }
-    // every copy issued into this CTA's shared memory must land before exit (in a pair the
-    // first CTA waits for both: its barriers count the other's copies too)
-    for (int i = 0; rank == 0 && i < NS; ++i)
-      if ((issued >> i) & 1u) wait_bounded(full0 + 8u * i, (issued_par >> i) & 1u, ctl, false);
+    // Every copy issued into shared memory must land before a CTA exits. A pair's copies all
+    // complete on the first CTA's barriers, so that one waits for both, and neither leaves
+    // before (cluster barrier at the end). Where a wait runs out the two producers may have
+    // stopped one use of a stage apart: the second says what it issued, and the first, once
+    // the abort flag says that nobody relies on the stage, takes the bytes that will never
+    // come out of a phase that it armed alone, and arms one for the copies of the second
+    // alone. (Neither is ever further ahead: a stage is filled again only once its last
+    // contents, of both, were multiplied.)
+    if (kPair && rank) {
+      __syncwarp();
+      if (lane == 0) {
+        const uint32_t at = ptx::mapa(ptx::smem_u32(tmem_slot + 2), 0);
+        ptx::st_remote_u32(at, issued);
+        ptx::st_remote_u32(at + 4u, issued_par);
+        ptx::mbar_arrive_remote(ptx::mapa(pdone, 0));
+      }
+    } else {
+      uint32_t i2 = issued, p2 = issued_par;
+      if (kPair) {
+        if (wait_bounded<true>(pdone, 0, ctl, false)) {
+          i2 = second[0];
+          p2 = second[1];
+        }
+        __syncwarp();
+      }
+      for (int i = 0; i < NS; ++i) {
+        const uint32_t fb = full0 + 8u * i;
+        const bool own = (issued >> i) & 1u, other = (i2 >> i) & 1u;
+        uint32_t par = (issued_par >> i) & 1u;
+        if (!own && !other) continue;
+        if (kPair && (own != other || ((p2 >> i) & 1u) != par)) {
+          const uint64_t t0 = ptx::globaltimer();
+          while (!*ctl.abort)
+            if (ptx::globaltimer() - t0 > ctl.limit_ns) give_up(ctl);
+          __syncwarp();
+          // the phase this CTA armed is over: the other one's copies are of the next
+          const bool behind =
+              __any_sync(0xffffffffu, !own || (other && ptx::mbar_try_wait(fb, par)));
+          if (behind) par = (p2 >> i) & 1u;
+          if (lane == 0) {
+            if (behind) ptx::mbar_arrive_expect_tx(fb, p.stage_bytes);
+            else ptx::mbar_complete_tx(fb, p.stage_bytes);
+          }
+          __syncwarp();
+        }
+        wait_bounded(fb, par, ctl, false);
+      }
+    }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
@@ -429,9 +486,13 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         atomicAdd(w.stats + kStatMmaWaitFull, (unsigned long long)wait_full);
         atomicAdd(w.stats + kStatMmaCycles, (unsigned long long)(clock64() - t_start));
       }
-      if (!ok && issued_any) {
-        // all MMAs of the elected lane must finish before TMEM is released
-        if (ptx::elect_one()) commit(drain);
+      if (issued_any) {
+        // all MMAs of the elected lane must finish before TMEM is released (the epilogue,
+        // which waits for them otherwise, may have given up)
+        if (ptx::elect_one()) {
+          if (kPair) ptx::mma_commit_pair_own(drain);
+          else ptx::mma_commit(drain);
+        }
         wait_bounded(drain, 0, ctl, false);
       }
     }
@@ -847,7 +908,7 @@ bool make_map(CUtensorMap* m, const void* base, int N, int Dp, int box_rows) {
 }
 
 size_t epilogue_bytes(int k, int L, int G) {
-  return G * group_bytes(L) + 8 * (2 * kMaxStages + 7 + 2 * kQueue) + 16 +
+  return G * group_bytes(L) + 8 * (2 * kMaxStages + 8 + 2 * kQueue) + 16 +
          kQueue * sizeof(WorkUnit) + 16;
 }
 
