@@ -156,7 +156,7 @@ struct Smem {
   Stages st;
   float G[BM][kPitch];          // kHalo carried columns, then the tile's 256
   float D[2][BM][kRowPitch];    // each group's rows of distances
-  float W[2 * BN], T[2 * BN];   // window sums and bounds of the tile's output columns
+  float W[2 * BN], T[2 * BN];   // window sums and (above the) bounds of the tile's columns
   int cnt[2][64];               // column-side counters of each group
   WorkUnit unit;
 };
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(NT, 1)
           const int j = c0 - (L - 1) + tid;
           const bool in = j >= 0 && j < us.M;
           sm.W[tid] = in ? a.W[us.out_base + j] : 0.f;
-          sm.T[tid] = in ? __uint_as_float(__ldcg(w.thr + us.out_base + j)) : 0.f;
+          sm.T[tid] = in ? above_bound(__ldcg(w.thr + us.out_base + j)) : 0.f;
         }
         const int jsym = us.T0 + us.R;  // column side from here on (sym)
         const long long cbase = w.sym ? us.col_base + w.col_off[us.strip_base + us.strip] : 0;

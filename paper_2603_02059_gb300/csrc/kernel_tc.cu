@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     // the group's shared memory
     float* Gbuf = reinterpret_cast<float*>(gptr + gid * gbytes);
     float* Wsh = Gbuf + BM * chunk_pitch(a.Lmax, kWin);  // window sums of the tile's output columns
-    float* Tsh = Wsh + BN;         // row bounds of the tile's output columns (column side)
+    float* Tsh = Wsh + BN;         // above the bounds of the tile's output columns (column side)
     float* Csh = Tsh + BN;         // correction values c of the tile's Gram columns
     ColSide cs;
     cs.cnt = reinterpret_cast<int*>(Csh + BN);
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         const int x = et + kEpiThreads * h, j = c0 - (s.L - 1) + x;
         const bool in = j >= 0 && j < s.M;
         hd.w[h] = in ? a.W[s.out_base + j] : 0.f;
-        hd.t[h] = in ? __uint_as_float(__ldcg(w.thr + s.out_base + j)) : 0.f;
+        hd.t[h] = in ? above_bound(__ldcg(w.thr + s.out_base + j)) : 0.f;
         hd.c[h] = c0 + x < N ? a.cval[s.row_base + c0 + x] : 0.f;  // Gram column day c0 + x
       }
       const bool row_ok = l < s.R && t < s.M;
