@@ -897,8 +897,9 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   if (h->precision != TRAKNN_PREC_FP32 && !tc_available()) return TRAKNN_ERR_UNSUPPORTED;
   int tiles = 8, group = 0;
   const bool whole = part_lo == 0 && part_hi == INT_MAX;
-  if (!shared && emb == 1 && whole) TRY_ST(pick_shape(h, sd, B, D, s, &tiles, &group));
-  if (!h->autotune && !shared) {
+  const bool tune = h->autotune && h->precision != TRAKNN_PREC_FP32;  // (tensor cores only)
+  if (tune && !shared && emb == 1 && whole) TRY_ST(pick_shape(h, sd, B, D, s, &tiles, &group));
+  if (!tune && !shared) {
     default_shape(h, sd, B, D, emb, part_lo, part_hi, &tiles, &group);
     if (h->precision != TRAKNN_PREC_FP32) tiles = unit_tiles(sd, B, D, emb, tiles);
   }
