@@ -189,13 +189,15 @@ typedef struct {
  * its own N, L, k and exclusion; the method of Sec. 3.2 applied to each series
  * separately, as when a study scores several regions, variables or ensemble
  * members). Every series' outputs equal those of traknn_knn_scores on it alone.
- * Up to 64 series run in one persistent launch sequence, which is captured as a CUDA graph on first use and replayed on later
+ * Up to 64 series run in one persistent launch sequence. With a tensor-core
+ * precision it is captured as a CUDA graph on first use and replayed on later
  * calls with the same shapes, pointers and options (the handle keeps one graph
  * per such signature, the 16 most recent; a change of shape or a larger workspace
- * drops them; evicting the oldest synchronises `stream` once).
- * With TRAKNN_PREC_FP32 series whose column-side lists would together take more
- * than 32 GB run one after another. Each series is checked as traknn_check_problem would check it; the first failing series'
- * status is returned before anything is enqueued. */
+ * drops them; evicting the oldest synchronises `stream` once). With
+ * TRAKNN_PREC_FP32 it is a sequence of plain launches, and series whose column-side
+ * lists would together take more than 32 GB run one after another. Each series is
+ * checked as traknn_check_problem would check it; the first failing series' status
+ * is returned before anything is enqueued. */
 traknn_status traknn_knn_scores_batched(traknn_handle handle, const traknn_series* series, int B,
                                         int64_t D, void* stream);
 

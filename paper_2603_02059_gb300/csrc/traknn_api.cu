@@ -1022,9 +1022,11 @@ traknn_status run_fp32_both(traknn_ctx* h, const HostSeries& sd, int64_t D, cuda
 // sequence for all series), or each series on both triangles. The column-side lists grow
 // with M^2 (0.7 KB per row and 1,024 rows at k = 20), both triangles need row lists only:
 // calls whose lists would take more than 32 GB (M > 215,000 at k = 20) or that find no
-// memory for them go series by series and, if it is one series, to both triangles.
+// memory for them go series by series and, if it is one series, to both triangles. Plain
+// launches, batched calls too (no captured graph): they can be captured by the caller, and
+// calls on new buffers cost no more than others.
 traknn_status run_fp32(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
-                       bool graph, bool shared) {
+                       bool shared = false) {
   double lists = 0.0;
   for (int b = 0; b < B; ++b) {
     const double M = (double)(sd[b].N - sd[b].L + 1);
@@ -1032,11 +1034,11 @@ traknn_status run_fp32(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cu
   }
   if (B == 1 && fp32_short(sd->N - sd->L + 1, D, sd->k)) return run_fp32_both(h, *sd, D, s);
   if (lists <= 32e9) {
-    const traknn_status st = run_tc(h, sd, B, D, s, graph, shared);
+    const traknn_status st = run_tc(h, sd, B, D, s, false, shared);
     if (st != TRAKNN_ERR_ALLOC) return st;
   }
   if (B == 1) return run_fp32_both(h, *sd, D, s);
-  for (int b = 0; b < B; ++b) TRY_ST(run_fp32(h, sd + b, 1, D, s, false, false));
+  for (int b = 0; b < B; ++b) TRY_ST(run_fp32(h, sd + b, 1, D, s));
   return TRAKNN_OK;
 }
 
@@ -1210,7 +1212,7 @@ traknn_status traknn_knn_scores(traknn_handle h, const float* X, int64_t N, int6
     return run_tc(h, &sd, 1, D, s, false, false, L);
   }
   const HostSeries sd{X, N, L, k, e, nbr_idx, nbr_dist, score};
-  if (h->precision == TRAKNN_PREC_FP32) return run_fp32(h, &sd, 1, D, s, false, false);
+  if (h->precision == TRAKNN_PREC_FP32) return run_fp32(h, &sd, 1, D, s);
   return run_tc(h, &sd, 1, D, s, false);
 }
 
@@ -1228,7 +1230,7 @@ traknn_status traknn_knn_scores_batched(traknn_handle h, const traknn_series* se
   const bool fp32 = h->precision == TRAKNN_PREC_FP32;
   for (int b0 = 0; b0 < B; b0 += kMaxSeries) {
     const int n = std::min(kMaxSeries, B - b0);
-    TRY_ST(fp32 ? run_fp32(h, sd.data() + b0, n, D, s, true, false)
+    TRY_ST(fp32 ? run_fp32(h, sd.data() + b0, n, D, s)
                 : run_tc(h, sd.data() + b0, n, D, s, true));
   }
   return TRAKNN_OK;
@@ -1251,7 +1253,7 @@ traknn_status traknn_knn_scores_multi(traknn_handle h, const traknn_series* sett
   // the shared geometry takes the smallest L (most trajectories) first
   std::stable_sort(sd.begin(), sd.end(),
                    [](const HostSeries& x, const HostSeries& y) { return x.L < y.L; });
-  if (h->precision == TRAKNN_PREC_FP32) return run_fp32(h, sd.data(), nset, D, s, false, true);
+  if (h->precision == TRAKNN_PREC_FP32) return run_fp32(h, sd.data(), nset, D, s, true);
   return run_tc(h, sd.data(), nset, D, s, false, true);
 }
 

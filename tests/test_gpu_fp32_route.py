@@ -44,3 +44,32 @@ def test_autotune_leaves_fp32_calls_alone(tk):
         counts.append(hd.launch_count())
         hd.close()
     assert counts[0] == counts[1]
+
+
+def _captured(hd, call):
+    import torch
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        call()
+    g.replay()
+    assert hd.sync_status() == 0
+
+
+def test_fp32_batched_calls_can_be_captured(tk):
+    import torch
+    shapes = [(1500, 5, 8), (1301, 3, 20), (1200, 1, 4)]
+    Xs = [_integers(N, 40, 5, seed=N) for N, _, _ in shapes]
+    series = [(X, L, k, L - 1) for X, (_, L, k) in zip(Xs, shapes)]
+    ref = [tk.knn_scores(X, L, k, e, precision="fp32") for X, L, k, e in series]
+    outs = [_outs(N - L + 1, k) for N, L, k in shapes]
+    hd = tk.Handle()
+    kw = dict(precision="fp32", handle=hd, outs=outs)
+    tk.knn_scores_batched(series, **kw)
+    assert hd.sync_status() == 0
+    for o in outs:
+        for t in o:
+            t.zero_()
+    torch.cuda.synchronize()
+    _captured(hd, lambda: tk.knn_scores_batched(series, **kw))
+    assert all(_equal(o, r) for o, r in zip(outs, ref))
+    hd.close()
