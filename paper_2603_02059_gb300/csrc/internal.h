@@ -160,6 +160,8 @@ struct SeriesInfo {
   int out_base;         // first stacked trajectory row
   int slots;            // row-side list slots per trajectory row
   int strip_base;       // index of the series' strip 0 in col_off / slot_lo
+  int cols;             // output columns of a column range (of a unit, but for its clipped ends)
+  int unit_base;        // first main unit of the series (UnitList)
   long long part_base;  // first row-side list of the series
   long long col_base;   // first column list of the series
   const float* X;       // input [N][D]
@@ -190,6 +192,73 @@ struct WorkUnit {
   int slot;    // slot of the row-side partial lists written by this unit
   int pad[3];  // pad[0]: number of consecutive series sharing the unit's Gram tiles; pad[1]
                // (units of CTA pairs): 1 if strip + 1 belongs to the unit too
+};
+
+// The same work list in closed form (upper triangle): the units of strips [g group,
+// (g+1) group) by column range and then by strip, for the groups g from the last to the first.
+struct UnitOrder {
+  int M, R, cols, group;
+  __host__ __device__ int strips() const { return (M + R - 1) / R; }
+  __host__ __device__ int ranges() const { return (M + cols - 1) / cols; }
+  __host__ __device__ int groups() const { return (strips() + group - 1) / group; }
+  // Units of group g in the column ranges before c: in range q those of the strips that
+  // start before its end, up to the range of the group's last strip; all strips after it.
+  __host__ __device__ int before(int g, int c) const {
+    const int lo = g * group, hi = lo + group < strips() ? lo + group : strips();
+    const int q0 = (int)((long long)lo * R / cols), q1 = (int)((long long)(hi - 1) * R / cols);
+    int n = c > q1 ? (c - q1) * (hi - lo) : 0;
+    for (int q = q0; q < (c < q1 ? c : q1); ++q)
+      n += (int)(((long long)(q + 1) * cols + R - 1) / R) - lo;
+    return n;
+  }
+  // Units of the groups g+1+i, g+1+i+step, ... (which come before group g's).
+  __host__ __device__ int after(int g, int i, int step) const {
+    int n = 0;
+    for (int h = g + 1 + i; h < groups(); h += step) n += before(h, ranges());
+    return n;
+  }
+};
+__host__ __device__ inline UnitOrder unit_order(const SeriesInfo& si, int group) {
+  UnitOrder o{si.M, si.rows_out, si.cols, group};
+  if (o.strips() < group) o.group = o.strips();
+  return o;
+}
+// Main unit of strip s in column range c (upper triangle), of series b and the nser - 1 after it.
+__host__ __device__ inline WorkUnit main_unit(const SeriesInfo& si, int b, int s, int c, int nser) {
+  const int lo = c * si.cols, T0 = s * si.rows_out;
+  return WorkUnit{b, s, lo > T0 ? lo : T0, si.M - lo < si.cols ? si.M : lo + si.cols, c,
+                  {nser, 0, 0}};
+}
+// Columns of strip s's band unit: R + 2 bw of them centred on its rows, or, where the
+// exclusion zone leaves those few candidates, the columns beside the zone (those after it,
+// or before it where they are more).
+__host__ __device__ inline void band_columns(int M, int R, int s, int bw, int e, int* jlo,
+                                             int* jhi) {
+  const long long T0 = (long long)s * R, width = 2LL * bw + R;
+  long long lo = T0 - bw, hi = T0 + R + bw;
+  if (e > width / 4) {
+    const long long after = T0 + R + e, before = T0 - e;
+    const bool up = after + width <= M || M - after >= before;
+    lo = up ? after : before - width;
+    hi = up ? after + width : before;
+  }
+  *jlo = (int)(lo < 0 ? 0 : lo > M ? M : lo);
+  *jhi = (int)(hi < 0 ? 0 : hi > M ? M : hi);
+}
+// A work list that the window kernel writes (units null: none). FP32 calls have no list of
+// their own on the host: their launches then depend on nothing but their arguments, so that
+// they are asynchronous whatever the shape, and can be captured.
+struct UnitList {
+  WorkUnit* units = nullptr;
+  long long* col_off = nullptr;
+  int* slot_lo = nullptr;
+  int strips = 0;         // stacked strips
+  int nmain = 0;          // main units; the band units follow, one per strip
+  int group = 1;          // strips side by side
+  int bw = 0;             // columns of a band on either side of a strip's rows
+  int nser = 1;           // > 1: the series share their Gram tiles
+  int emax = 0;           // largest exclusion of those that share
+  int egroups = 2;        // row-side lists per column range
 };
 
 struct TcWork {
@@ -406,10 +475,10 @@ cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int
                                      void* lo, double* norms, float* cval, float* W,
                                      const ClearArgs& clear, cudaStream_t st, int r_lo = 0);
 // Window sums of the stacked trajectory rows [r_lo, out_rows); clears what `clear` names
-// for those rows (thr null: nothing).
+// for those rows (thr null: nothing) and writes the work list `list` (units null: none).
 cudaError_t launch_window_series(const SeriesTable& sr, int out_rows, const double* norms,
                                  float* W, const ClearArgs& clear, cudaStream_t st,
-                                 int r_lo = 0);
+                                 int r_lo = 0, const UnitList& list = UnitList{});
 cudaError_t launch_merge(const FusedArgs& a, int32_t* idx, float* dist, float* score,
                          cudaStream_t st);
 // Exact top-k of the union of nparts sorted candidate lists per row ([nparts][M][k],

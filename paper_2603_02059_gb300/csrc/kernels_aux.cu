@@ -377,15 +377,44 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// The work list's entries of stacked strip gs, by one warp (a lane per column range).
+__device__ __forceinline__ void write_units(const SeriesTable& st, const UnitList& ul, int gs) {
+  const int lane = threadIdx.x & 31;
+  int b = 0;
+  while (b + 1 < st.n && st.s[b + 1].strip_base <= gs) ++b;
+  const SeriesInfo& si = st.s[b];
+  const int s = gs - si.strip_base, R = si.rows_out, q0 = (int)((long long)s * R / si.cols);
+  if (lane == 0) {  // the columns beyond strips 0 .. s-1, each from its next strip on
+    ul.col_off[gs] = (long long)s * si.M - (long long)R * ((long long)s * (s + 1) / 2);
+    ul.slot_lo[gs] = q0 * ul.egroups;
+  }
+  if (ul.nser > 1 && b > 0) return;  // the first series' units are everyone's
+  if (lane == 0) {
+    WorkUnit u{b, s, 0, 0, 0, {ul.nser, 0, 0}};
+    band_columns(si.M, R, s, ul.bw, ul.nser > 1 ? ul.emax : si.e, &u.jlo, &u.jhi);
+    ul.units[ul.nmain + gs] = u;
+  }
+  const UnitOrder o = unit_order(si, ul.group);
+  const int g = s / o.group;
+  const int base = si.unit_base + (int)__reduce_add_sync(0xffffffffu, o.after(g, lane, 32)) + s -
+                   g * o.group;
+  for (int c = q0 + lane; c < o.ranges(); c += 32)
+    ul.units[base + o.before(g, c)] = main_unit(si, b, s, c, ul.nser);
+}
+
 // W of every stacked trajectory row: an explicit L-term FP64 sum of its series' norms. The
 // row's bound, shared minima and column-list mask are cleared here too (three fills fewer
 // on the stream).
 __global__ void window_series_kernel(const __grid_constant__ SeriesTable st, int r_lo,
                                      int out_rows, const double* __restrict__ norms, float* W,
-                                     const ClearArgs c) {
+                                     const ClearArgs c, const UnitList ul) {
   const int r = r_lo + blockIdx.x * blockDim.x + threadIdx.x;
   launch_wait();
   launch_next();
+  if (ul.units)
+    for (int gs = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; gs < ul.strips;
+         gs += (gridDim.x * blockDim.x) >> 5)
+      write_units(st, ul, gs);
   if (blockIdx.x == 0 && (int)threadIdx.x < c.counters) c.counter[threadIdx.x] = 0;
   if (r >= out_rows) return;
   if (c.thr) {
@@ -926,10 +955,11 @@ cudaError_t launch_prep_split_series(const SeriesTable& sr, int rows, int D, int
 }
 
 cudaError_t launch_window_series(const SeriesTable& sr, int out_rows, const double* norms,
-                                 float* W, const ClearArgs& clear, cudaStream_t st, int r_lo) {
+                                 float* W, const ClearArgs& clear, cudaStream_t st, int r_lo,
+                                 const UnitList& list) {
   if (out_rows <= r_lo) return cudaSuccess;
   return launch_chained(window_series_kernel, (out_rows - r_lo + 255) / 256, 256, 0, st, sr, r_lo,
-                        out_rows, norms, W, clear);
+                        out_rows, norms, W, clear, list);
 }
 
 cudaError_t launch_prep_fp32_series(const SeriesTable& sr, int rows, int D, int Dp,

@@ -56,6 +56,9 @@ struct TcPlan {
   int sym = 1;         // upper triangle with column lists, or both triangles
   bool band = true;    // the band units run (see prepare_tc)
   bool shared = false; // several settings of one record: one set of operand rows
+  bool fp32 = false;   // FP32 path: the window kernel writes the work list (list)
+  int strips = 0;      // stacked strips
+  UnitList list;
 };
 
 constexpr size_t kMaxGraphs = 16;  // captured launch sequences kept per handle
@@ -77,8 +80,10 @@ struct traknn_ctx {
   int wait_limit_ms = 2000;
   int debug_withhold = 0;
   // library-owned buffers, grown on demand
-  void* tcws = nullptr;  // forward passes
+  void* tcws = nullptr;  // tensor-core forward passes
   size_t tcws_bytes = 0;
+  void* fpws = nullptr;  // FP32 forward passes
+  size_t fpws_bytes = 0;
   void* io = nullptr;  // device staging for the host-buffer entry point
   size_t io_bytes = 0;
   void* adj = nullptr;  // reverse neighbour index of the adjoint
@@ -104,7 +109,7 @@ struct traknn_ctx {
   int64_t weights_D = 0;
   int stats = 0;
   unsigned long long* stats_dev = nullptr;
-  TcPlan plan;
+  TcPlan plan, fplan;        // tensor-core plan; the FP32 call's (rebuilt by every call)
   void* plan_dev = nullptr;  // units, col_off, slot_lo of `plan`
   size_t plan_dev_bytes = 0;
   // shape key -> (tiles per unit, strips side by side) chosen by the autotuner
@@ -140,10 +145,11 @@ void drop_graphs(traknn_ctx* h) {
   h->graphs.clear();
 }
 
-// Grow a library buffer. Captured graphs refer to the old buffers, so they go too.
+// Grow a library buffer. Captured graphs refer to the old ones of the tensor-core path, so
+// they go too.
 traknn_status ensure_buffer(traknn_ctx* h, void** buf, size_t* have, size_t need) {
   if (*have >= need) return TRAKNN_OK;
-  drop_graphs(h);
+  if (buf == &h->tcws || buf == &h->plan_dev) drop_graphs(h);
   if (*buf) {
     cudaDeviceSynchronize();
     cudaFree(*buf);
@@ -179,20 +185,10 @@ inline int list_pitch(int kmax) { return (kmax + 3) / 4 * 4; }
 // Gram tile, so the strip height and the tile step are those of the largest L, every
 // unit is one tile long and carries all B series (pad[0] = B), and the first series
 // (smallest L, most trajectories) defines the units' column ranges.
-void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, int tiles,
-                int group_opt, bool shared, int part_lo, int part_hi,
-                const std::vector<int>& pstrip, int egroups, int band_tiles, TcPlan& p,
-                int tile_cols = kTileCols) {
-  p.units.clear();
-  p.col_off.clear();
-  p.slot_lo.clear();
-  const int K = pstrip.empty() ? 1 : (int)pstrip.size() - 1;  // phases
-  auto phase_of = [&](int s) {
-    int q = 0;
-    while (q + 1 < K && s < pstrip[q + 1]) ++q;
-    return q;
-  };
-  std::vector<std::vector<WorkUnit>> mainq(K), bandq(K);  // units of each phase
+//
+// plan_series: the series table and the sizes of everything but the unit list.
+void plan_series(const HostSeries* sd, int B, int sym, int cols_opt, int tiles, bool shared,
+                 int egroups, TcPlan& p, int tile_cols = kTileCols) {
   int row_base = 0, out_base = 0, strip_base = 0;
   long long part_base = 0, col_base = 0;
   p.kmax = 0;
@@ -224,8 +220,50 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
     si.out_base = out_base;
     si.slots = slots;
     si.strip_base = strip_base;
+    si.cols = cols;
+    si.unit_base = 0;
     si.part_base = part_base;
     si.col_base = col_base;
+    if (!shared || b == B - 1) row_base += N;
+    out_base += M;
+    strip_base += strips;
+    part_base += (long long)M * slots;
+    if (sym)  // strip s: the columns from strip s + 1 on
+      col_base += (long long)(strips - 1) * M - (long long)R * ((long long)strips * (strips - 1) / 2);
+    p.kmax = std::max(p.kmax, k);
+    p.Lmax = std::max(p.Lmax, L);
+  }
+  p.sym = sym;
+  p.shared = shared;
+  p.egroups = egroups;
+  p.rows = row_base;
+  p.out_rows = out_base;
+  p.strips = strip_base;
+  p.part_lists = part_base;
+  p.col_lists = col_base;
+}
+
+// Output columns that a band of band_tiles tiles adds on either side of a strip's rows.
+int band_side(int band_tiles) { return (band_tiles * kTileCols - kTileRows) / 2; }
+
+void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, int tiles,
+                int group_opt, bool shared, int part_lo, int part_hi,
+                const std::vector<int>& pstrip, int egroups, int band_tiles, TcPlan& p) {
+  p.units.clear();
+  p.col_off.clear();
+  p.slot_lo.clear();
+  plan_series(sd, B, sym, cols_opt, tiles, shared, egroups, p);
+  const int K = pstrip.empty() ? 1 : (int)pstrip.size() - 1;  // phases
+  auto phase_of = [&](int s) {
+    int q = 0;
+    while (q + 1 < K && s < pstrip[q + 1]) ++q;
+    return q;
+  };
+  std::vector<std::vector<WorkUnit>> mainq(K), bandq(K);  // units of each phase
+  for (int b = 0; b < B; ++b) {
+    const SeriesInfo& si = p.table.s[b];
+    const int M = si.M, R = si.rows_out, cols = si.cols, slots = si.slots;
+    const int strips = (M + R - 1) / R;
     long long off = 0;
     for (int s = 0; s < strips; ++s) {
       p.col_off.push_back(off);
@@ -250,26 +288,12 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
       }
       // band: band_tiles tiles of columns (band_tiles kTileCols - (L-1) outputs) centred on
       // the strip's rows
-      const int bw = std::max(0, (band_tiles * kTileCols - (Lg - 1) - R) / 2);
+      const int bw = band_side(band_tiles);
+      int emax = 0;
+      for (int q = 0; q < nser; ++q) emax = std::max(emax, sd[b + q].e);
       for (int s = std::max(0, part_lo); s < std::min(strips, part_hi); ++s) {
-        const int T0 = s * R;
-        int jlo = std::max(0, T0 - bw);
-        int jhi = std::min(M, T0 + R + bw);
-        // an exclusion zone that leaves the centred band few candidates: the columns
-        // beside the zone instead (those after it, or before it where they are more)
-        int emax = 0;
-        for (int q = 0; q < nser; ++q) emax = std::max(emax, sd[b + q].e);
-        const int width = 2 * bw + R;
-        if (emax > width / 4) {
-          const int64_t after = (int64_t)T0 + R + emax, before = (int64_t)T0 - emax;
-          if (after + width <= M || M - after >= before) {
-            jlo = (int)std::min<int64_t>(after, M);
-            jhi = (int)std::min<int64_t>(after + width, M);
-          } else {
-            jhi = (int)std::max<int64_t>(before, 0);
-            jlo = std::max(0, jhi - width);
-          }
-        }
+        int jlo, jhi;
+        band_columns(M, R, s, bw, emax, &jlo, &jhi);
         // a phase's band units stay clear of the days still being copied (a band only
         // seeds bounds, from whatever candidates it holds)
         const int q = phase_of(s);
@@ -277,18 +301,8 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
         if (jlo < jhi) bandq[q].push_back(WorkUnit{b, s, jlo, jhi, 0, {nser, 0, 0}});
       }
     }
-    if (!shared || b == B - 1) row_base += N;
-    out_base += M;
-    strip_base += strips;
-    part_base += (long long)M * slots;
-    col_base += off;
-    p.kmax = std::max(p.kmax, k);
-    p.Lmax = std::max(p.Lmax, L);
   }
   p.pstrip = pstrip;
-  p.sym = sym;
-  p.shared = shared;
-  p.egroups = egroups;
   p.pu.assign(1, 0);
   for (int q = 0; q < K; ++q) {
     p.units.insert(p.units.end(), mainq[q].begin(), mainq[q].end());
@@ -301,10 +315,6 @@ void build_plan(const HostSeries* sd, int B, int64_t D, int sym, int cols_opt, i
     p.pb.push_back((int)p.units.size());
   }
   p.nband = (int)p.units.size() - p.nunits;
-  p.rows = row_base;
-  p.out_rows = out_base;
-  p.part_lists = part_base;
-  p.col_lists = col_base;
 }
 
 // The main units of CTA pairs from those of single CTAs: within a phase's strips (or a
@@ -335,7 +345,7 @@ traknn_status check_handle(traknn_handle h) {
 
 std::vector<int64_t> shape_key(const HostSeries* sd, int B, int64_t D, const traknn_ctx* h) {
   std::vector<int64_t> key = {D, h->sym, h->unit_cols, (int64_t)h->precision, h->center, B,
-                              h->seg_k, h->group_strips, h->l2_keep_a, h->col_chunks};
+                              h->seg_k, h->group_strips, h->l2_keep_a};
   for (int b = 0; b < B; ++b) {
     key.push_back(sd[b].N);
     key.push_back(sd[b].L);
@@ -362,12 +372,16 @@ struct TcBuffers {
   unsigned int* col_mask;
   int* counter;
   float* pscore;  // [out_rows] scores of partial lists (split series), not returned
+  WorkUnit* units;     // FP32 path: the work list (the tensor-core path's is in plan_dev)
+  long long* col_off;
+  int* slot_lo;
   int Dp;
   size_t total;
 };
 
-TcBuffers tc_layout(const TcPlan& p, int64_t D, bool fp32, char* base) {
+TcBuffers tc_layout(const TcPlan& p, int64_t D, char* base) {
   TcBuffers b;
+  const bool fp32 = p.fp32;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     off = align_up(off, 256);
@@ -397,8 +411,22 @@ TcBuffers tc_layout(const TcPlan& p, int64_t D, bool fp32, char* base) {
       take((size_t)p.out_rows * p.mask_words * sizeof(unsigned int)));
   b.counter = reinterpret_cast<int*>(take(256));
   b.pscore = reinterpret_cast<float*>(take((size_t)p.out_rows * sizeof(float)));
+  const size_t listed = fp32 ? p.strips : 0;
+  b.units = reinterpret_cast<WorkUnit*>(
+      take((fp32 ? (size_t)p.nunits + p.nband : 0) * sizeof(WorkUnit)));
+  b.col_off = reinterpret_cast<long long*>(take(listed * sizeof(long long)));
+  b.slot_lo = reinterpret_cast<int*>(take(listed * sizeof(int)));
   b.total = off;
   return b;
+}
+
+void set_pointers(const HostSeries* sd, int B, TcPlan& p) {
+  for (int b = 0; b < B; ++b) {
+    p.table.s[b].X = sd[b].X;
+    p.table.s[b].idx = sd[b].idx;
+    p.table.s[b].dist = sd[b].dist;
+    p.table.s[b].score = sd[b].score;
+  }
 }
 
 // Make h->plan the plan for these series (built and uploaded when the shape changes)
@@ -434,13 +462,12 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   }
   const int Dk = tc_groups((int)D * emb) * 64;
   const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2048 : 2304) * (shared ? B : 1);
-  const bool fp32 = h->precision == TRAKNN_PREC_FP32;  // (its kernel has two groups)
   const int egroups =
-      fp32 || (h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k &&
-               (Lmax == 1 || Dk <= line || (!shared && tiles_all < 2.0 * h->sm_count)))
+      h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k &&
+              (Lmax == 1 || Dk <= line || (!shared && tiles_all < 2.0 * h->sm_count))
           ? 2
           : 1;
-  const bool pair = !fp32 && egroups == 1 && h->sm_count >= 2;
+  const bool pair = egroups == 1 && h->sm_count >= 2;
   key.push_back(egroups);
   // Band pre-pass width in tiles per strip. Short operand rows: four tiles, two where the
   // whole call has fewer Gram tiles than the GPU SMs, so that the band lasts as long as its
@@ -450,37 +477,12 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   // one tile while its 64 groups of columns still resolve k (k <= 20; N = 10,957, D = 3,726, k
   // = 10 1 / 2 / 4 tiles 1,180 / 1,209 / 1,293 us, four lengths 1,865 / 1,952; D = 512, N =
   // 1,826 139 / 155 / 199), two for larger k (the last case with k = 40: 220 / 203 / 234).
-  // FP32: a band column costs as much as a main one; 1 / 2 / 8 tiles: D = 32, N = 27,394
-  // 2,023 / 1,938 / 1,996 us, N = 4,000 190 / 181 / 233; D = 512, N = 1,826 310 / 410 / 983;
-  // D = 3,726, N = 10,957 11.2 / 12.0 / 16.5 ms
-  const int band_tiles = fp32 ? (D <= 64 ? 2 : 1)
-                         : Dk <= 768 ? (tiles_all < h->sm_count ? 2 : 4)
-                                     : (kmax <= 20 ? 1 : 2);
+  const int band_tiles = Dk <= 768 ? (tiles_all < h->sm_count ? 2 : 4) : (kmax <= 20 ? 1 : 2);
   key.push_back(band_tiles);
   TcPlan& p = h->plan;
   if (p.key != key) {
-    // the column chunks of the FP32 option: that many units per strip
-    int cols = h->unit_cols, tile_cols = kTileCols;
-    p.band = true;
-    if (fp32) {
-      int64_t M = 1, half_tiles = 0;
-      const int Rmin = kTileRows - (Lmax - 1);
-      for (int b = 0; b < (shared ? 1 : B); ++b) {
-        const int64_t Mb = sd[b].N - sd[b].L + 1;
-        M = std::max(M, Mb);
-        for (int64_t t = 0; t < Mb; t += Rmin) half_tiles += (Mb - t + Rmin - 1) / Rmin;
-      }
-      cols = h->col_chunks > 0 ? (int)((M + h->col_chunks - 1) / h->col_chunks) : 0;
-      // A short FP32 call is as long as its units: half tiles (128 x 128) while they do not
-      // go round the SMs twice, and no band before them where they run all at once and a
-      // half tile's products (128 cycles per grid point) outlast the scan of an unbounded
-      // one (N = 300, D = 16 92 us with it, 137 without; N = 1,500, D = 5,000 about 2 x 0.6
-      // ms with it).
-      if (half_tiles <= 2 * h->sm_count) tile_cols = kTileCols / 2;
-      p.band = half_tiles > h->sm_count || D <= 256;
-    }
-    build_plan(sd, B, D, fp32 ? 1 : h->sym, cols, tile_cols < kTileCols ? 1 : tiles, group,
-               shared, part_lo, part_hi, pstrip, egroups, band_tiles, p, tile_cols);
+    build_plan(sd, B, D, h->sym, h->unit_cols, tiles, group, shared, part_lo, part_hi, pstrip,
+               egroups, band_tiles, p);
     p.key.clear();  // until the new list is on the device
     p.emb = emb;
     p.part_lo = part_lo;
@@ -502,15 +504,9 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     p.key = key;
     drop_graphs(h);  // graphs captured the previous work list
   }
-  for (int b = 0; b < B; ++b) {
-    p.table.s[b].X = sd[b].X;
-    p.table.s[b].idx = sd[b].idx;
-    p.table.s[b].dist = sd[b].dist;
-    p.table.s[b].score = sd[b].score;
-  }
-  const TcBuffers probe = tc_layout(p, D, h->precision == TRAKNN_PREC_FP32, nullptr);
-  TRY_ST(ensure_buffer(h, &h->tcws, &h->tcws_bytes, probe.total));
-  *out = tc_layout(p, D, h->precision == TRAKNN_PREC_FP32, static_cast<char*>(h->tcws));
+  set_pointers(sd, B, p);
+  TRY_ST(ensure_buffer(h, &h->tcws, &h->tcws_bytes, tc_layout(p, D, nullptr).total));
+  *out = tc_layout(p, D, static_cast<char*>(h->tcws));
   for (int b = 0; b < B; ++b)  // partial lists: their scores go to the workspace
     if (!p.table.s[b].score) p.table.s[b].score = out->pscore + p.table.s[b].out_base;
   return TRAKNN_OK;
@@ -538,9 +534,8 @@ float band_error_margin(int Dp) {
   return (float)(2.0 * u + u * u + 2.1 * Dp * std::ldexp(1.0, -23) + std::ldexp(1.0, -19));
 }
 
-// Kernel arguments of a call on the handle's plan (the whole work list).
-void fused_args(const traknn_ctx* h, const TcBuffers& b, TcArgs* pa, TcWork* pw) {
-  const TcPlan& p = h->plan;
+// Kernel arguments of a call on plan p (the whole work list).
+void fused_args(const traknn_ctx* h, const TcPlan& p, const TcBuffers& b, TcArgs* pa, TcWork* pw) {
   const size_t ub = align_up(p.units.size() * sizeof(WorkUnit), 256);
   const size_t cb = align_up(p.col_off.size() * sizeof(long long), 256);
   const char* pd = static_cast<const char*>(h->plan_dev);
@@ -572,11 +567,11 @@ void fused_args(const traknn_ctx* h, const TcBuffers& b, TcArgs* pa, TcWork* pw)
   a.band_margin = 0.f;
 
   TcWork& w = *pw;
-  w.units = reinterpret_cast<const WorkUnit*>(pd);
+  w.units = p.fp32 ? b.units : reinterpret_cast<const WorkUnit*>(pd);
   w.nunits = p.nunits;
   w.kstride = list_pitch(p.kmax);
-  w.col_off = reinterpret_cast<const long long*>(pd + ub);
-  w.slot_lo = reinterpret_cast<const int*>(pd + ub + cb);
+  w.col_off = p.fp32 ? b.col_off : reinterpret_cast<const long long*>(pd + ub);
+  w.slot_lo = p.fp32 ? b.slot_lo : reinterpret_cast<const int*>(pd + ub + cb);
   w.sym = p.sym;
   w.col_rec = b.col_rec;
   w.col_ints = p.col_lists * col_pitch(w.kstride);
@@ -593,8 +588,8 @@ void fused_args(const traknn_ctx* h, const TcBuffers& b, TcArgs* pa, TcWork* pw)
 
 // One fused launch: `nu` units from unit u0, unit counter `ctr`; `band`: the pre-pass that
 // only seeds bounds.
-traknn_status launch_units(traknn_ctx* h, const TcBuffers& b, const TcArgs& a, const TcWork& w,
-                           int u0, int nu, int ctr, bool band, cudaStream_t s) {
+traknn_status launch_units(traknn_ctx* h, const TcPlan& p, const TcBuffers& b, const TcArgs& a,
+                           const TcWork& w, int u0, int nu, int ctr, bool band, cudaStream_t s) {
   if (nu <= 0) return TRAKNN_OK;
   TcWork x = w;
   x.units = w.units + u0;
@@ -605,15 +600,15 @@ traknn_status launch_units(traknn_ctx* h, const TcBuffers& b, const TcArgs& a, c
   if (band) {
     x.sym = 0;
     x.write_lists = 0;
-    if (band_single_product(h, h->plan, b.Dp)) {
+    if (band_single_product(h, p, b.Dp)) {
       ax.corr_neg = 1;
       ax.band_margin = band_error_margin(b.Dp);
       split = false;
     }
   }
   ++h->launches;
-  const SeriesTable& sr = h->plan.table;
-  if (h->precision == TRAKNN_PREC_FP32)
+  const SeriesTable& sr = p.table;
+  if (p.fp32)
     TRY_CUDA(launch_fused_fp32(static_cast<const float*>(b.hi), ax, x, sr, h->sm_count, s));
   else
     TRY_CUDA(launch_fused_tc(b.hi, b.lo, split, ax, x, sr, h->sm_count, s));
@@ -621,18 +616,15 @@ traknn_status launch_units(traknn_ctx* h, const TcBuffers& b, const TcArgs& a, c
 }
 
 // Whether the operand preparation also writes the window sums: its rows are trajectories.
-bool windows_in_prep(const traknn_ctx* h) {
-  const SeriesTable& sr = h->plan.table;
-  return h->precision != TRAKNN_PREC_FP32 && sr.n == 1 && sr.s[0].L == 1 &&
-         h->plan.rows == h->plan.out_rows;
+bool windows_in_prep(const TcPlan& p) {
+  return !p.fp32 && p.table.n == 1 && p.table.s[0].L == 1 && p.rows == p.out_rows;
 }
 
 // Means, operand rows [lo, hi) and window sums of the trajectory rows [lo, ohi), whose bounds
 // and masks are cleared; `counters` > 0 also clears that many unit counters, and computes
 // the means first.
-traknn_status enqueue_prep(traknn_ctx* h, const TcBuffers& b, int64_t D, int lo, int hi, int ohi,
-                           int counters, cudaStream_t s) {
-  const TcPlan& p = h->plan;
+traknn_status enqueue_prep(traknn_ctx* h, const TcPlan& p, const TcBuffers& b, int64_t D, int lo,
+                           int hi, int ohi, int counters, cudaStream_t s) {
   const SeriesTable& sr = p.table;
   const float* sw = h->weights ? b.sw : nullptr;
   if (counters > 0)
@@ -640,8 +632,14 @@ traknn_status enqueue_prep(traknn_ctx* h, const TcBuffers& b, int64_t D, int lo,
                                     h->center != 0, s));
   const ClearArgs clear{b.thr,      b.shared_min, p.out_rows, min_slots(p.kmax),
                         b.col_mask, p.mask_words, b.counter,  counters};
-  const bool rows_are_windows = windows_in_prep(h);
-  if (h->precision == TRAKNN_PREC_FP32)
+  const bool rows_are_windows = windows_in_prep(p);
+  UnitList list = p.list;
+  if (p.fp32) {
+    list.units = b.units;
+    list.col_off = b.col_off;
+    list.slot_lo = b.slot_lo;
+  }
+  if (p.fp32)
     TRY_CUDA(launch_prep_fp32_series(sr, p.rows, (int)D, b.Dp, b.mu, sw,
                                      static_cast<float*>(b.hi), b.norms, s));
   else
@@ -649,29 +647,28 @@ traknn_status enqueue_prep(traknn_ctx* h, const TcBuffers& b, int64_t D, int lo,
                                       h->precision == TRAKNN_PREC_SPLIT_BF16, b.mu, sw, b.hi, b.lo,
                                       b.norms, b.cval, rows_are_windows ? b.W : nullptr, clear, s,
                                       lo));
-  if (!rows_are_windows) TRY_CUDA(launch_window_series(sr, ohi, b.norms, b.W, clear, s, lo));
+  if (!rows_are_windows) TRY_CUDA(launch_window_series(sr, ohi, b.norms, b.W, clear, s, lo, list));
   h->launches += (counters > 0 ? 1 : 0) + (hi > lo ? 1 : 0) +
                  (ohi > lo && !rows_are_windows ? 1 : 0);
   return TRAKNN_OK;
 }
 
 // The launch sequence of one call (also what a graph captures).
-traknn_status enqueue_tc(traknn_ctx* h, const TcBuffers& b, int64_t D,
+traknn_status enqueue_tc(traknn_ctx* h, const TcPlan& p, const TcBuffers& b, int64_t D,
                          cudaStream_t s, bool record_events) {
-  const TcPlan& p = h->plan;
   const SeriesTable& sr = p.table;
   TcArgs a;
   TcWork w;
-  fused_args(h, b, &a, &w);
-  TRY_ST(enqueue_prep(h, b, D, 0, p.rows, p.out_rows, 2, s));
+  fused_args(h, p, b, &a, &w);
+  TRY_ST(enqueue_prep(h, p, b, D, 0, p.rows, p.out_rows, 2, s));
   const int slot = h->ev_head;
   if (record_events) TRY_CUDA(cudaEventRecord(h->ev_start[slot], s));
   // threshold pre-pass over the band units (stored after the main units), then the rest
-  if (p.band) TRY_ST(launch_units(h, b, a, w, p.nunits, p.nband, 1, true, s));
+  if (p.band) TRY_ST(launch_units(h, p, b, a, w, p.nunits, p.nband, 1, true, s));
   if (a.pair)
-    TRY_ST(launch_units(h, b, a, w, p.pp[0], p.pp[1] - p.pp[0], 0, false, s));
+    TRY_ST(launch_units(h, p, b, a, w, p.pp[0], p.pp[1] - p.pp[0], 0, false, s));
   else
-    TRY_ST(launch_units(h, b, a, w, 0, p.nunits, 0, false, s));
+    TRY_ST(launch_units(h, p, b, a, w, 0, p.nunits, 0, false, s));
   if (record_events) {
     TRY_CUDA(cudaEventRecord(h->ev_stop[slot], s));
     h->ev_head = (h->ev_head + 1) % traknn_ctx::kRing;
@@ -725,7 +722,7 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
   const int K = (int)p.pstrip.size() - 1;
   TcArgs a;
   TcWork w;
-  fused_args(h, b, &a, &w);
+  fused_args(h, p, b, &a, &w);
   for (int q = 0; q < K; ++q) {
     const int lo = p.pstrip[q + 1] * R;                      // first day (and row) of phase q
     const int hi = q == 0 ? p.rows : p.pstrip[q] * R;        // rows prepared by phase q
@@ -733,10 +730,10 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
     TRY_CUDA(cudaStreamWaitEvent(s, in[q], 0));
     // window sums of rows [lo, ohi) read day norms up to ohi + L - 2: prepared now or
     // by an earlier phase
-    TRY_ST(enqueue_prep(h, b, D, lo, hi, ohi, q == 0 ? 2 * K : 0, s));
-    TRY_ST(launch_units(h, b, a, w, p.pb[q], p.pb[q + 1] - p.pb[q], 2 * q + 1, true, s));
+    TRY_ST(enqueue_prep(h, p, b, D, lo, hi, ohi, q == 0 ? 2 * K : 0, s));
+    TRY_ST(launch_units(h, p, b, a, w, p.pb[q], p.pb[q + 1] - p.pb[q], 2 * q + 1, true, s));
     const std::vector<int>& m = a.pair ? p.pp : p.pu;
-    TRY_ST(launch_units(h, b, a, w, m[q], m[q + 1] - m[q], 2 * q, false, s));
+    TRY_ST(launch_units(h, p, b, a, w, m[q], m[q + 1] - m[q], 2 * q, false, s));
   }
   TRY_CUDA(launch_merge_tc(a, w, sr, s));
   h->launches += 1;
@@ -794,9 +791,9 @@ traknn_status pick_shape(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     for (int cand_t : {4, 8, 16}) {
       TcBuffers buf;
       TRY_ST(prepare_tc(h, sd, B, D, cand_t, false, 1, s, &buf, 0, INT_MAX, {}, cand_g));
-      TRY_ST(enqueue_tc(h, buf, D, s, false));  // warm-up
+      TRY_ST(enqueue_tc(h, h->plan, buf, D, s, false));  // warm-up
       TRY_CUDA(cudaEventRecord(e0, s));
-      TRY_ST(enqueue_tc(h, buf, D, s, false));
+      TRY_ST(enqueue_tc(h, h->plan, buf, D, s, false));
       TRY_CUDA(cudaEventRecord(e1, s));
       TRY_CUDA(cudaEventSynchronize(e1));
       float ms = 0.f;
@@ -894,25 +891,19 @@ int unit_tiles(const HostSeries* sd, int B, int64_t D, int emb, int tiles) {
 traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
                      bool graph, bool shared = false, int emb = 1, int part_lo = 0,
                      int part_hi = INT_MAX) {
-  if (h->precision != TRAKNN_PREC_FP32 && !tc_available()) return TRAKNN_ERR_UNSUPPORTED;
+  if (!tc_available()) return TRAKNN_ERR_UNSUPPORTED;
   int tiles = 8, group = 0;
   const bool whole = part_lo == 0 && part_hi == INT_MAX;
-  const bool tune = h->autotune && h->precision != TRAKNN_PREC_FP32;  // (tensor cores only)
-  if (tune && !shared && emb == 1 && whole) TRY_ST(pick_shape(h, sd, B, D, s, &tiles, &group));
-  if (!tune && !shared) {
+  if (!shared && emb == 1 && whole) TRY_ST(pick_shape(h, sd, B, D, s, &tiles, &group));
+  if (!h->autotune && !shared) {
     default_shape(h, sd, B, D, emb, part_lo, part_hi, &tiles, &group);
-    if (h->precision != TRAKNN_PREC_FP32) tiles = unit_tiles(sd, B, D, emb, tiles);
+    tiles = unit_tiles(sd, B, D, emb, tiles);
   }
-  // FP32: a tile's contraction takes so long that the units must be short for the CTAs to
-  // end together, except at few grid points. 1 / 2 / 4 / 8 tiles: D = 3,726, N = 27,394 60.5 /
-  // 60.3 / 60.8 / 62.7 ms, N = 10,957 10.8 / 11.2 / 12.0 / 12.8; D = 200, N = 10,957 1,056 /
-  // 1,069 / 1,117 / 1,155 us; D = 32, N = 27,394 2,163 / 2,023 / 1,979 / 1,968
-  if (h->precision == TRAKNN_PREC_FP32 && D > 64) tiles = tiles >= 8 ? 2 : 1;
   TcBuffers buf;
   TRY_ST(prepare_tc(h, sd, B, D, tiles, shared, emb, s, &buf, part_lo, part_hi, {}, group));
   h->last_tiles = tiles;
   h->last_group = group > 0 ? group : (h->group_strips > 0 ? h->group_strips : 19);
-  if (!graph) return enqueue_tc(h, buf, D, s, h->profile != 0);
+  if (!graph) return enqueue_tc(h, h->plan, buf, D, s, h->profile != 0);
 
   std::vector<int64_t> key = h->plan.key;
   for (int b = 0; b < B; ++b) {
@@ -928,17 +919,17 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   for (auto& g : h->graphs)
     if (g.key == key) {
       TRY_CUDA(cudaGraphLaunch(g.exec, s));
-      h->launches += 5 - (windows_in_prep(h) ? 1 : 0) +
+      h->launches += 5 - (windows_in_prep(h->plan) ? 1 : 0) +
                      (h->plan.band && h->plan.nband > 0 ? 1 : 0);
       return TRAKNN_OK;
     }
   if (!h->cap_stream) TRY_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   // The first call's results come from plain launches (kernel attributes, first-use costs);
   // its sequence is captured for later calls while they run.
-  TRY_ST(enqueue_tc(h, buf, D, s, false));
+  TRY_ST(enqueue_tc(h, h->plan, buf, D, s, false));
   const int64_t l0 = h->launches;
   TRY_CUDA(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-  const traknn_status st = enqueue_tc(h, buf, D, h->cap_stream, false);
+  const traknn_status st = enqueue_tc(h, h->plan, buf, D, h->cap_stream, false);
   cudaGraph_t g = nullptr;
   const cudaError_t ce = cudaStreamEndCapture(h->cap_stream, &g);
   if (st != TRAKNN_OK) {
@@ -977,8 +968,8 @@ traknn_status run_fp32_both(traknn_ctx* h, const HostSeries& sd, int64_t D, cuda
   const int M = (int)(sd.N - sd.L + 1);
   const Schedule sch = make_schedule(M, sd.L, sd.k, sd.e, h->sm_count, h->col_chunks);
   const Fp32Layout lay = make_layout(sd.N, D, sch);
-  TRY_ST(ensure_buffer(h, &h->tcws, &h->tcws_bytes, lay.total));
-  char* ws = static_cast<char*>(h->tcws);
+  TRY_ST(ensure_buffer(h, &h->fpws, &h->fpws_bytes, lay.total));
+  char* ws = static_cast<char*>(h->fpws);
   float* mu = reinterpret_cast<float*>(ws + lay.mu);
   float* sw = reinterpret_cast<float*>(ws + lay.partial);
   double* norms = reinterpret_cast<double*>(ws + lay.norms);
@@ -1018,13 +1009,68 @@ traknn_status run_fp32_both(traknn_ctx* h, const HostSeries& sd, int64_t D, cuda
   return TRAKNN_OK;
 }
 
-// Forward pass on the CUDA cores: the upper triangle over the shared work plan (one launch
-// sequence for all series), or each series on both triangles. The column-side lists grow
+// The plan of an FP32 call on the upper triangle: tables and sizes of the work list that the
+// window kernel writes.
+void fp32_plan(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, bool shared,
+               TcPlan& p) {
+  int Lmax = 1, emax = 0;
+  for (int b = 0; b < B; ++b) {
+    Lmax = std::max(Lmax, sd[b].L);
+    emax = std::max(emax, sd[b].e);
+  }
+  int64_t M = 1, half_tiles = 0;
+  for (int b = 0; b < (shared ? 1 : B); ++b) {
+    const int64_t Mb = sd[b].N - sd[b].L + 1, R = kTileRows - (Lmax - 1), n = (Mb + R - 1) / R;
+    M = std::max(M, Mb);
+    half_tiles += n * (n + 1) / 2;
+  }
+  // A tile's contraction takes so long that the units must be short for the CTAs to end
+  // together, except at few grid points. 1 / 2 / 4 / 8 tiles: D = 3,726, N = 27,394 60.5 /
+  // 60.3 / 60.8 / 62.7 ms, N = 10,957 10.8 / 11.2 / 12.0 / 12.8; D = 200, N = 10,957 1,056 /
+  // 1,069 / 1,117 / 1,155 us; D = 32, N = 27,394 2,163 / 2,023 / 1,979 / 1,968
+  int tiles = 8, group = 0;
+  if (!shared) default_shape(h, sd, B, D, 1, 0, INT_MAX, &tiles, &group);
+  if (D > 64) tiles = tiles >= 8 ? 2 : 1;
+  // A short call is as long as its units: half tiles (128 x 128) while they do not go round
+  // the SMs twice, and no band before them where they run all at once and a half tile's
+  // products (128 cycles per grid point) outlast the scan of an unbounded one (N = 300, D =
+  // 16 92 us with it, 137 without; N = 1,500, D = 5,000 about 2 x 0.6 ms with it).
+  const bool half = half_tiles <= 2 * h->sm_count;
+  p.band = half_tiles > h->sm_count || D <= 256;
+  // a band column costs as much as a main one; 1 / 2 / 8 tiles: D = 32, N = 27,394 2,023 /
+  // 1,938 / 1,996 us, N = 4,000 190 / 181 / 233; D = 512, N = 1,826 310 / 410 / 983; D =
+  // 3,726, N = 10,957 11.2 / 12.0 / 16.5 ms
+  const int band_tiles = D <= 64 ? 2 : 1;
+  // the column chunks of the option: that many units per strip
+  const int cols = h->col_chunks > 0 ? (int)((M + h->col_chunks - 1) / h->col_chunks) : 0;
+  plan_series(sd, B, 1, cols, half ? 1 : tiles, shared, 2, p, half ? kTileCols / 2 : kTileCols);
+  p.fp32 = true;
+  p.list = UnitList{};
+  p.list.strips = p.strips;
+  p.list.group = group > 0 ? group : h->group_strips > 0 ? h->group_strips : 19;
+  p.list.nser = shared ? B : 1;
+  p.list.emax = emax;
+  p.list.egroups = p.egroups;
+  p.nunits = p.nband = 0;
+  for (int b = 0; b < (shared ? 1 : B); ++b) {
+    SeriesInfo& si = p.table.s[b];
+    si.unit_base = p.nunits;
+    const UnitOrder o = unit_order(si, p.list.group);
+    p.nunits += o.after(-1, 0, 1);
+    p.nband += o.strips();
+  }
+  p.list.bw = band_side(band_tiles);
+  p.list.nmain = p.nunits;
+}
+
+// Forward pass on the CUDA cores: the upper triangle (one launch sequence for all series), or
+// each series on both triangles. The column-side lists grow
 // with M^2 (0.7 KB per row and 1,024 rows at k = 20), both triangles need row lists only:
 // calls whose lists would take more than 32 GB (M > 215,000 at k = 20) or that find no
 // memory for them go series by series and, if it is one series, to both triangles. Plain
-// launches, batched calls too (no captured graph): they can be captured by the caller, and
-// calls on new buffers cost no more than others.
+// launches on a workspace of their own, batched calls too (no captured graph, no work list
+// kept on the host): calls of any shape are asynchronous once the workspace has its size, can
+// be captured by the caller, and leave the tensor-core path's plan and graphs alone.
 traknn_status run_fp32(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
                        bool shared = false) {
   double lists = 0.0;
@@ -1034,7 +1080,13 @@ traknn_status run_fp32(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cu
   }
   if (B == 1 && fp32_short(sd->N - sd->L + 1, D, sd->k)) return run_fp32_both(h, *sd, D, s);
   if (lists <= 32e9) {
-    const traknn_status st = run_tc(h, sd, B, D, s, false, shared);
+    TcPlan& p = h->fplan;
+    fp32_plan(h, sd, B, D, shared, p);
+    set_pointers(sd, B, p);
+    const traknn_status st =
+        ensure_buffer(h, &h->fpws, &h->fpws_bytes, tc_layout(p, D, nullptr).total);
+    if (st == TRAKNN_OK)
+      return enqueue_tc(h, p, tc_layout(p, D, static_cast<char*>(h->fpws)), D, s, h->profile != 0);
     if (st != TRAKNN_ERR_ALLOC) return st;
   }
   if (B == 1) return run_fp32_both(h, *sd, D, s);
@@ -1110,6 +1162,7 @@ traknn_status traknn_destroy(traknn_handle h) {
   for (cudaEvent_t ev : h->ev_in)
     if (ev) cudaEventDestroy(ev);
   if (h->tcws) cudaFree(h->tcws);
+  if (h->fpws) cudaFree(h->fpws);
   if (h->io) cudaFree(h->io);
   if (h->adj) cudaFree(h->adj);
   if (h->plan_dev) cudaFree(h->plan_dev);

@@ -73,3 +73,64 @@ def test_fp32_batched_calls_can_be_captured(tk):
     _captured(hd, lambda: tk.knn_scores_batched(series, **kw))
     assert all(_equal(o, r) for o, r in zip(outs, ref))
     hd.close()
+
+
+def _asynchronous(call):
+    """Whether `call` returns while work enqueued before it still runs."""
+    import torch
+    torch.cuda.synchronize()
+    torch.cuda._sleep(int(1e9))  # about half a second
+    ev = torch.cuda.Event()
+    ev.record()
+    call()
+    running = not ev.query()
+    torch.cuda.synchronize()
+    return running
+
+
+def test_fp32_calls_of_changing_shapes_are_asynchronous(tk):
+    hd = tk.Handle()
+    kw = dict(precision="fp32", handle=hd)
+    calls = [(_integers(N, D, 5, seed=N), L, k) for N, D, L, k in
+             [(4000, 300, 5, 20), (2000, 300, 3, 10), (3001, 40, 1, 33), (1500, 290, 17, 5)]]
+    ref = [tk.knn_scores(X, L, k, **kw) for X, L, k in calls]
+    outs = [_outs(X.shape[0] - L + 1, k) for X, L, k in calls]
+    for (X, L, k), o, r in zip(calls, outs, ref):
+        assert _asynchronous(lambda: tk.knn_scores(X, L, k, out=o, **kw))
+        assert hd.sync_status() == 0 and _equal(o, r)
+    hd.close()
+
+
+def test_fp32_calls_of_new_shapes_and_many_series_can_be_captured(tk):
+    big = _integers(3000, 100, 5, seed=2)
+    hd = tk.Handle()
+    kw = dict(precision="fp32", handle=hd)
+    tk.knn_scores(big, 3, 30, **kw)  # sizes the workspace
+    X = _integers(1700, 60, 5, seed=3)
+    ref = tk.knn_scores(X, 4, 12, precision="fp32")
+    out = _outs(1697, 12)
+    _captured(hd, lambda: tk.knn_scores(X, 4, 12, out=out, **kw))
+    assert _equal(out, ref)
+    # more series than one launch sequence takes
+    Xs = [_integers(60 + b, 60, 5, seed=b) for b in range(70)]
+    ref = [tk.knn_scores(x, 2, 3, precision="fp32") for x in Xs]
+    outs = [_outs(59 + b, 3) for b in range(70)]
+    series = [(x, 2, 3, 1) for x in Xs]
+    _captured(hd, lambda: tk.knn_scores_batched(series, outs=outs, **kw))
+    assert all(_equal(o, r) for o, r in zip(outs, ref))
+    hd.close()
+
+
+def test_fp32_calls_keep_the_graphs_of_batched_calls(tk):
+    hd = tk.Handle()
+    series = [(_integers(1500, 40, 5, seed=b), 3, 7, 2) for b in range(3)]
+    outs = [_outs(1498, 7) for _ in range(3)]
+
+    def batched():
+        tk.knn_scores_batched(series, handle=hd, outs=outs)
+
+    batched()
+    tk.knn_scores(series[0][0], 3, 7, precision="fp32", handle=hd)
+    assert _asynchronous(batched)  # a first call would capture, and wait
+    assert hd.sync_status() == 0
+    hd.close()
