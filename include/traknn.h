@@ -63,7 +63,7 @@ typedef enum {
  * scores are accumulated in FP64 in every mode. */
 typedef enum {
   TRAKNN_PREC_FP32 = 0,       /* CUDA-core FP32 FMA Gram, upper triangle (both triangles for the
-                                 shortest series and where the column-side lists would exceed
+                                 shortest series and where the candidate lists would exceed
                                  32 GB or find no memory) */
   TRAKNN_PREC_SPLIT_BF16 = 1, /* tensor cores: x = hi + lo (two BF16), G = hi.hi + hi.lo + lo.hi, FP32 accumulate */
   TRAKNN_PREC_BF16 = 2        /* tensor cores: single BF16 product, FP32 accumulate (lower accuracy) */
@@ -194,7 +194,7 @@ typedef struct {
  * calls with the same shapes, pointers and options (the handle keeps one graph
  * per such signature, the 16 most recent; a change of shape or a larger workspace
  * drops them; evicting the oldest synchronises `stream` once). With
- * TRAKNN_PREC_FP32 it is a sequence of plain launches, and series whose column-side
+ * TRAKNN_PREC_FP32 it is a sequence of plain launches, and series whose candidate
  * lists would together take more than 32 GB run one after another. Each series is
  * checked as traknn_check_problem would check it; the first failing series' status
  * is returned before anything is enqueued. */
@@ -210,7 +210,7 @@ traknn_status traknn_knn_scores_batched(traknn_handle handle, const traknn_serie
  * outputs equal those of traknn_knn_scores on it alone except that, as in that call,
  * D(t,j) may be evaluated from either operand order: distances agree to a few ulp
  * and neighbour sets may differ only at near ties. With TRAKNN_PREC_FP32 settings
- * whose column-side lists would together take more than 32 GB run one after another.
+ * whose candidate lists would together take more than 32 GB run one after another.
  * 1 <= nset <= 64; each entry is checked as
  * traknn_check_problem would check it; entries with another X or N are refused
  * (TRAKNN_ERR_INVALID_ARG). */

@@ -145,6 +145,8 @@ void drop_graphs(traknn_ctx* h) {
   h->graphs.clear();
 }
 
+size_t buffer_bytes(size_t need) { return align_up(need + need / 8, 1 << 20); }
+
 // Grow a library buffer. Captured graphs refer to the old ones of the tensor-core path, so
 // they go too.
 traknn_status ensure_buffer(traknn_ctx* h, void** buf, size_t* have, size_t need) {
@@ -156,7 +158,7 @@ traknn_status ensure_buffer(traknn_ctx* h, void** buf, size_t* have, size_t need
     *buf = nullptr;
     *have = 0;
   }
-  size_t bytes = align_up(need + need / 8, 1 << 20);
+  const size_t bytes = buffer_bytes(need);
   if (cudaMalloc(buf, bytes) != cudaSuccess) {
     cudaGetLastError();
     *buf = nullptr;
@@ -164,6 +166,20 @@ traknn_status ensure_buffer(traknn_ctx* h, void** buf, size_t* have, size_t need
   }
   *have = bytes;
   return TRAKNN_OK;
+}
+
+// Whether a buffer that holds `have` bytes can be given `need`: asked by calls that have
+// another, smaller way to run, which then neither free a buffer nor wait for the device.
+// (Nothing can be allocated while `s` is captured.)
+bool has_room(size_t have, size_t need, cudaStream_t s) {
+  if (have >= need) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  size_t left = 0, total = 0;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) cudaGetLastError();
+  if (cs != cudaStreamCaptureStatusNone) return false;
+  if (cudaMemGetInfo(&left, &total) == cudaSuccess) return left + have >= buffer_bytes(need);
+  cudaGetLastError();
+  return true;
 }
 
 static_assert(sizeof(WorkUnit) == 32, "work unit layout");
@@ -353,6 +369,15 @@ std::vector<int64_t> shape_key(const HostSeries* sd, int B, int64_t D, const tra
     key.push_back(sd[b].e);
   }
   return key;
+}
+
+// Bytes of a call's candidate lists: row side, column side.
+constexpr double kMaxListBytes = 32e9;  // of calls that have another way to run
+double row_list_bytes(const TcPlan& p) {
+  return (double)p.part_lists * (8.0 * list_cap(list_pitch(p.kmax), p.part_lists) + 4.0);
+}
+double col_list_bytes(const TcPlan& p) {
+  return (double)p.col_lists * col_pitch(list_pitch(p.kmax)) * 4.0;
 }
 
 // Device pointers of the tensor-core workspace for plan `p`.
@@ -1010,8 +1035,8 @@ traknn_status run_fp32_both(traknn_ctx* h, const HostSeries& sd, int64_t D, cuda
 }
 
 // The plan of an FP32 call on the upper triangle: tables and sizes of the work list that the
-// window kernel writes.
-void fp32_plan(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, bool shared,
+// window kernel writes. False if its candidate lists would take more than kMaxListBytes.
+bool fp32_plan(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, bool shared,
                TcPlan& p) {
   int Lmax = 1, emax = 0;
   for (int b = 0; b < B; ++b) {
@@ -1043,15 +1068,24 @@ void fp32_plan(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, bool
   const int band_tiles = D <= 64 ? 2 : 1;
   // the column chunks of the option: that many units per strip
   const int cols = h->col_chunks > 0 ? (int)((M + h->col_chunks - 1) / h->col_chunks) : 0;
-  plan_series(sd, B, 1, cols, half ? 1 : tiles, shared, 2, p, half ? kTileCols / 2 : kTileCols);
+  // Longer units while the row-side lists take more than 8 GB, or more than 1 GB where both
+  // sides' would not stay within kMaxListBytes (more than 60,000 days).
+  for (;; tiles *= 2) {
+    plan_series(sd, B, 1, cols, half ? 1 : tiles, shared, 2, p, half ? kTileCols / 2 : kTileCols);
+    const double rows = row_list_bytes(p);
+    if (half || shared || cols > 0 || tiles >= 1024 || rows <= 1e9 ||
+        (rows <= 8e9 && rows + col_list_bytes(p) <= kMaxListBytes))
+      break;
+  }
   p.fp32 = true;
+  p.nunits = p.nband = 0;
+  if (row_list_bytes(p) + col_list_bytes(p) > kMaxListBytes) return false;
   p.list = UnitList{};
   p.list.strips = p.strips;
   p.list.group = group > 0 ? group : h->group_strips > 0 ? h->group_strips : 19;
   p.list.nser = shared ? B : 1;
   p.list.emax = emax;
   p.list.egroups = p.egroups;
-  p.nunits = p.nband = 0;
   for (int b = 0; b < (shared ? 1 : B); ++b) {
     SeriesInfo& si = p.table.s[b];
     si.unit_base = p.nunits;
@@ -1061,30 +1095,26 @@ void fp32_plan(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, bool
   }
   p.list.bw = band_side(band_tiles);
   p.list.nmain = p.nunits;
+  return true;
 }
 
 // Forward pass on the CUDA cores: the upper triangle (one launch sequence for all series), or
-// each series on both triangles. The column-side lists grow
-// with M^2 (0.7 KB per row and 1,024 rows at k = 20), both triangles need row lists only:
-// calls whose lists would take more than 32 GB (M > 215,000 at k = 20) or that find no
-// memory for them go series by series and, if it is one series, to both triangles. Plain
-// launches on a workspace of their own, batched calls too (no captured graph, no work list
-// kept on the host): calls of any shape are asynchronous once the workspace has its size, can
-// be captured by the caller, and leave the tensor-core path's plan and graphs alone.
+// each series on both triangles. The column-side lists grow with M^2 (0.7 KB per row and
+// 1,024 rows at k = 20), both triangles need row lists only: calls whose lists would take
+// more than 32 GB (M > 213,000 at k = 20) or that find no memory for them go series by series
+// and, if it is one series, to both triangles. Plain launches on a workspace of their own,
+// batched calls too (no captured graph, no work list kept on the host): calls of any shape are
+// asynchronous once the workspace has its size, can be captured by the caller, and leave the
+// tensor-core path's plan and graphs alone.
 traknn_status run_fp32(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
                        bool shared = false) {
-  double lists = 0.0;
-  for (int b = 0; b < B; ++b) {
-    const double M = (double)(sd[b].N - sd[b].L + 1);
-    lists += M * M / (2.0 * (kTileRows - (sd[b].L - 1))) * col_pitch(list_pitch(sd[b].k)) * 4.0;
-  }
   if (B == 1 && fp32_short(sd->N - sd->L + 1, D, sd->k)) return run_fp32_both(h, *sd, D, s);
-  if (lists <= 32e9) {
-    TcPlan& p = h->fplan;
-    fp32_plan(h, sd, B, D, shared, p);
+  TcPlan& p = h->fplan;
+  if (fp32_plan(h, sd, B, D, shared, p)) {
     set_pointers(sd, B, p);
-    const traknn_status st =
-        ensure_buffer(h, &h->fpws, &h->fpws_bytes, tc_layout(p, D, nullptr).total);
+    const size_t need = tc_layout(p, D, nullptr).total;
+    traknn_status st = TRAKNN_ERR_ALLOC;
+    if (has_room(h->fpws_bytes, need, s)) st = ensure_buffer(h, &h->fpws, &h->fpws_bytes, need);
     if (st == TRAKNN_OK)
       return enqueue_tc(h, p, tc_layout(p, D, static_cast<char*>(h->fpws)), D, s, h->profile != 0);
     if (st != TRAKNN_ERR_ALLOC) return st;

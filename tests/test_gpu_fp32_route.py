@@ -134,3 +134,55 @@ def test_fp32_calls_keep_the_graphs_of_batched_calls(tk):
     assert _asynchronous(batched)  # a first call would capture, and wait
     assert hd.sync_status() == 0
     hd.close()
+
+
+def _fill_device(leave):
+    """All of the device's free memory but `leave` bytes."""
+    import torch
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    return torch.empty(max(0, free - leave), dtype=torch.uint8, device="cuda")
+
+
+def test_fp32_calls_without_room_for_lists_stay_asynchronous(tk):
+    """About 1 GB of lists and 0.5 GB left: both triangles, without freeing the workspace and
+    asking for the memory again on every call."""
+    import torch
+    X = _integers(27394, 32, 40, seed=4)
+    ref = tk.knn_scores(X, 5, 20, precision="fp32", center=False)
+    out = _outs(27390, 20)
+    hd = tk.Handle()
+    kw = dict(precision="fp32", center=False, handle=hd)
+    torch.cuda.synchronize()
+    fill = _fill_device(500 << 20)
+    try:
+        tk.knn_scores(X, 5, 20, out=out, **kw)
+        assert hd.sync_status() == 0 and _equal(out, ref)
+        assert _asynchronous(lambda: tk.knn_scores(X, 5, 20, out=out, **kw))
+        assert hd.sync_status() == 0 and _equal(out, ref)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+        hd.close()
+
+
+def test_fp32_lists_stay_within_their_bound(tk):
+    """150,000 days: 45 GB of row-side lists with units of two tiles."""
+    import torch
+    N, k, e = 150000, 20, 3
+    X = _integers(N, 70, 100, seed=5)
+    hd = tk.Handle()
+    out = _outs(N, k)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    tk.knn_scores(X, 1, k, e, precision="fp32", center=False, handle=hd, out=out)
+    assert hd.sync_status() == 0
+    assert before - torch.cuda.mem_get_info()[0] <= 1.125 * 32e9 + 1e9
+    Xi = X.cpu().numpy().astype(np.int64)
+    for t in (0, 1, N // 2, N - 1, 127, 128, 77777):
+        d = ((Xi - Xi[t]) ** 2).sum(axis=1)
+        d[max(0, t - e):t + e + 1] = np.iinfo(np.int64).max
+        order = np.argsort(d, kind="stable")[:k]
+        assert np.array_equal(out[0][t].cpu().numpy(), order)
+        assert np.array_equal(out[1][t].cpu().numpy(), d[order].astype(np.float32))
+    hd.close()
