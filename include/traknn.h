@@ -193,7 +193,8 @@ typedef struct {
  * precision it is captured as a CUDA graph on first use and replayed on later
  * calls with the same shapes, pointers and options (the handle keeps one graph
  * per such signature, the 16 most recent; a change of shape or a larger workspace
- * drops them; evicting the oldest synchronises `stream` once). With
+ * drops them, once more than 16 shapes are in use; evicting the oldest synchronises
+ * `stream` once). With
  * TRAKNN_PREC_FP32 it is a sequence of plain launches, and series whose candidate
  * lists would together take more than 32 GB run one after another. Each series is
  * checked as traknn_check_problem would check it; the first failing series' status
@@ -209,8 +210,9 @@ traknn_status traknn_knn_scores_batched(traknn_handle handle, const traknn_serie
  * that of one setting when the contraction dominates (large D). Each setting's
  * outputs equal those of traknn_knn_scores on it alone except that, as in that call,
  * D(t,j) may be evaluated from either operand order: distances agree to a few ulp
- * and neighbour sets may differ only at near ties. With TRAKNN_PREC_FP32 settings
- * whose candidate lists would together take more than 32 GB run one after another.
+ * and neighbour sets may differ only at near ties. Settings whose
+ * candidate lists would together take more than 32 GB, or find no memory, run in
+ * several sweeps (with TRAKNN_PREC_FP32 one after another).
  * 1 <= nset <= 64; each entry is checked as
  * traknn_check_problem would check it; entries with another X or N are refused
  * (TRAKNN_ERR_INVALID_ARG). */

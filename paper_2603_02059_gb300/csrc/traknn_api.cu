@@ -61,7 +61,16 @@ struct TcPlan {
   UnitList list;
 };
 
+// A tensor-core plan and its work list on the device.
+struct PlanSlot {
+  TcPlan plan;
+  void* dev = nullptr;  // units, col_off, slot_lo
+  size_t bytes = 0;
+  uint64_t used = 0;    // when it was last taken
+};
+
 constexpr size_t kMaxGraphs = 16;  // captured launch sequences kept per handle
+constexpr int kMaxPlans = 16;      // plans kept per handle (a call may take several in turn)
 constexpr int kMaxPhases = 8;      // phases of a host-buffer call
 
 struct GraphEntry {
@@ -109,9 +118,10 @@ struct traknn_ctx {
   int64_t weights_D = 0;
   int stats = 0;
   unsigned long long* stats_dev = nullptr;
-  TcPlan plan, fplan;        // tensor-core plan; the FP32 call's (rebuilt by every call)
-  void* plan_dev = nullptr;  // units, col_off, slot_lo of `plan`
-  size_t plan_dev_bytes = 0;
+  TcPlan fplan;  // the FP32 call's (rebuilt by every call)
+  PlanSlot plans[kMaxPlans];
+  PlanSlot* cur = plans;  // the tensor-core call's
+  uint64_t plan_clock = 0;
   // shape key -> (tiles per unit, strips side by side) chosen by the autotuner
   std::vector<std::pair<std::vector<int64_t>, std::pair<int, int>>> tuned;
   int last_tiles = 0, last_group = 0;  // work-unit shape of the last tensor-core call
@@ -151,7 +161,7 @@ size_t buffer_bytes(size_t need) { return align_up(need + need / 8, 1 << 20); }
 // they go too.
 traknn_status ensure_buffer(traknn_ctx* h, void** buf, size_t* have, size_t need) {
   if (*have >= need) return TRAKNN_OK;
-  if (buf == &h->tcws || buf == &h->plan_dev) drop_graphs(h);
+  if (*buf && buf != &h->fpws && buf != &h->io && buf != &h->adj) drop_graphs(h);
   if (*buf) {
     cudaDeviceSynchronize();
     cudaFree(*buf);
@@ -397,7 +407,7 @@ struct TcBuffers {
   unsigned int* col_mask;
   int* counter;
   float* pscore;  // [out_rows] scores of partial lists (split series), not returned
-  WorkUnit* units;     // FP32 path: the work list (the tensor-core path's is in plan_dev)
+  WorkUnit* units;     // the work list: in the workspace (FP32 path) or in the plan's slot
   long long* col_off;
   int* slot_lo;
   int Dp;
@@ -454,8 +464,24 @@ void set_pointers(const HostSeries* sd, int B, TcPlan& p) {
   }
 }
 
-// Make h->plan the plan for these series (built and uploaded when the shape changes)
-// and size the workspace. Must not run during a stream capture.
+// Epilogue groups of a tensor-core call (see prepare_tc).
+int epilogue_groups(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, bool shared,
+                    int emb, double tiles_all) {
+  int Lmax = 1, kmax = 1;
+  for (int b = 0; b < B; ++b) {
+    Lmax = std::max(Lmax, sd[b].L);
+    kmax = std::max(kmax, sd[b].k);
+  }
+  const int Dk = tc_groups((int)D * emb) * 64;
+  const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2048 : 2304) * (shared ? B : 1);
+  return h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k &&
+                 (Lmax == 1 || Dk <= line || (!shared && tiles_all < 2.0 * h->sm_count))
+             ? 2
+             : 1;
+}
+
+// Make h->cur the plan for these series (built and uploaded when no slot holds it) and size
+// the workspace. Must not run during a stream capture unless the plan is held.
 traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, int tiles,
                          bool shared, int emb, cudaStream_t s, TcBuffers* out,
                          int part_lo = 0, int part_hi = INT_MAX,
@@ -477,21 +503,15 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   // 5): split-BF16 D = 990 453 / 611 us, 1,476 552 / 639, 2,200 746 / 677 (L = 10, k = 20 829 /
   // 834), 3,726 1,291 / 997; BF16 D = 1,800 559 / 577, 2,800 787 / 714; D = 3,726, N = 1,826
   // 230 / 240, 3,000 313 / 342, 4,500 368 / 371, 6,500 538 / 498.
-  int Lmax = 1, kmax = 1;
+  int kmax = 1;
   double tiles_all = 0.0;  // Gram tiles of the call
   for (int b = 0; b < B; ++b) {
-    Lmax = std::max(Lmax, sd[b].L);
     kmax = std::max(kmax, sd[b].k);
     const double M = (double)(sd[b].N - sd[b].L + 1);
     tiles_all += M * M / ((h->sym ? 2.0 : 1.0) * kTileRows * kTileCols);
   }
   const int Dk = tc_groups((int)D * emb) * 64;
-  const int line = (h->precision == TRAKNN_PREC_SPLIT_BF16 ? 2048 : 2304) * (shared ? B : 1);
-  const int egroups =
-      h->epi_groups != 1 && kmax <= 32 && Dk <= h->seg_k &&
-              (Lmax == 1 || Dk <= line || (!shared && tiles_all < 2.0 * h->sm_count))
-          ? 2
-          : 1;
+  const int egroups = epilogue_groups(h, sd, B, D, shared, emb, tiles_all);
   const bool pair = egroups == 1 && h->sm_count >= 2;
   key.push_back(egroups);
   // Band pre-pass width in tiles per strip. Short operand rows: four tiles, two where the
@@ -504,7 +524,18 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   // 1,826 139 / 155 / 199), two for larger k (the last case with k = 40: 220 / 203 / 234).
   const int band_tiles = Dk <= 768 ? (tiles_all < h->sm_count ? 2 : 4) : (kmax <= 20 ? 1 : 2);
   key.push_back(band_tiles);
-  TcPlan& p = h->plan;
+  // the slot that holds the plan, or else the one unused longest
+  PlanSlot* sl = h->plans;
+  for (PlanSlot& c : h->plans) {
+    if (c.plan.key == key) {
+      sl = &c;
+      break;
+    }
+    if (c.used < sl->used) sl = &c;
+  }
+  sl->used = ++h->plan_clock;
+  h->cur = sl;
+  TcPlan& p = sl->plan;
   if (p.key != key) {
     build_plan(sd, B, D, h->sym, h->unit_cols, tiles, group, shared, part_lo, part_hi, pstrip,
                egroups, band_tiles, p);
@@ -518,8 +549,9 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     const size_t cb = align_up(p.col_off.size() * sizeof(long long), 256);
     const size_t sb = align_up(p.slot_lo.size() * sizeof(int), 256);
     TRY_CUDA(cudaStreamSynchronize(s));  // earlier work may still read the old list
-    TRY_ST(ensure_buffer(h, &h->plan_dev, &h->plan_dev_bytes, ub + cb + sb));
-    char* pd = static_cast<char*>(h->plan_dev);
+    if (sl->dev) drop_graphs(h);         // graphs captured it
+    TRY_ST(ensure_buffer(h, &sl->dev, &sl->bytes, ub + cb + sb));
+    char* pd = static_cast<char*>(sl->dev);
     TRY_CUDA(cudaMemcpy(pd, p.units.data(), p.units.size() * sizeof(WorkUnit),
                         cudaMemcpyHostToDevice));
     TRY_CUDA(cudaMemcpy(pd + ub, p.col_off.data(), p.col_off.size() * sizeof(long long),
@@ -527,11 +559,16 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     TRY_CUDA(cudaMemcpy(pd + ub + cb, p.slot_lo.data(), p.slot_lo.size() * sizeof(int),
                         cudaMemcpyHostToDevice));
     p.key = key;
-    drop_graphs(h);  // graphs captured the previous work list
   }
   set_pointers(sd, B, p);
   TRY_ST(ensure_buffer(h, &h->tcws, &h->tcws_bytes, tc_layout(p, D, nullptr).total));
   *out = tc_layout(p, D, static_cast<char*>(h->tcws));
+  char* pd = static_cast<char*>(sl->dev);
+  out->units = reinterpret_cast<WorkUnit*>(pd);
+  pd += align_up(p.units.size() * sizeof(WorkUnit), 256);
+  out->col_off = reinterpret_cast<long long*>(pd);
+  pd += align_up(p.col_off.size() * sizeof(long long), 256);
+  out->slot_lo = reinterpret_cast<int*>(pd);
   for (int b = 0; b < B; ++b)  // partial lists: their scores go to the workspace
     if (!p.table.s[b].score) p.table.s[b].score = out->pscore + p.table.s[b].out_base;
   return TRAKNN_OK;
@@ -561,10 +598,6 @@ float band_error_margin(int Dp) {
 
 // Kernel arguments of a call on plan p (the whole work list).
 void fused_args(const traknn_ctx* h, const TcPlan& p, const TcBuffers& b, TcArgs* pa, TcWork* pw) {
-  const size_t ub = align_up(p.units.size() * sizeof(WorkUnit), 256);
-  const size_t cb = align_up(p.col_off.size() * sizeof(long long), 256);
-  const char* pd = static_cast<const char*>(h->plan_dev);
-
   TcArgs& a = *pa;
   a.Dp = b.Dp;
   a.rows = p.rows;
@@ -592,11 +625,11 @@ void fused_args(const traknn_ctx* h, const TcPlan& p, const TcBuffers& b, TcArgs
   a.band_margin = 0.f;
 
   TcWork& w = *pw;
-  w.units = p.fp32 ? b.units : reinterpret_cast<const WorkUnit*>(pd);
+  w.units = b.units;
   w.nunits = p.nunits;
   w.kstride = list_pitch(p.kmax);
-  w.col_off = p.fp32 ? b.col_off : reinterpret_cast<const long long*>(pd + ub);
-  w.slot_lo = p.fp32 ? b.slot_lo : reinterpret_cast<const int*>(pd + ub + cb);
+  w.col_off = b.col_off;
+  w.slot_lo = b.slot_lo;
   w.sym = p.sym;
   w.col_rec = b.col_rec;
   w.col_ints = p.col_lists * col_pitch(w.kstride);
@@ -740,7 +773,7 @@ std::vector<int> phase_plan(int strips, int R, int64_t N) {
 // sequence; only the order of the work units differs.
 traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cudaStream_t s,
                                 const cudaEvent_t* in) {
-  const TcPlan& p = h->plan;
+  const TcPlan& p = h->cur->plan;
   const SeriesTable& sr = p.table;
   const SeriesInfo& si = sr.s[0];
   const int R = kTileRows - (si.L - 1);
@@ -816,9 +849,9 @@ traknn_status pick_shape(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
     for (int cand_t : {4, 8, 16}) {
       TcBuffers buf;
       TRY_ST(prepare_tc(h, sd, B, D, cand_t, false, 1, s, &buf, 0, INT_MAX, {}, cand_g));
-      TRY_ST(enqueue_tc(h, h->plan, buf, D, s, false));  // warm-up
+      TRY_ST(enqueue_tc(h, h->cur->plan, buf, D, s, false));  // warm-up
       TRY_CUDA(cudaEventRecord(e0, s));
-      TRY_ST(enqueue_tc(h, h->plan, buf, D, s, false));
+      TRY_ST(enqueue_tc(h, h->cur->plan, buf, D, s, false));
       TRY_CUDA(cudaEventRecord(e1, s));
       TRY_CUDA(cudaEventSynchronize(e1));
       float ms = 0.f;
@@ -928,9 +961,9 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   TRY_ST(prepare_tc(h, sd, B, D, tiles, shared, emb, s, &buf, part_lo, part_hi, {}, group));
   h->last_tiles = tiles;
   h->last_group = group > 0 ? group : (h->group_strips > 0 ? h->group_strips : 19);
-  if (!graph) return enqueue_tc(h, h->plan, buf, D, s, h->profile != 0);
+  if (!graph) return enqueue_tc(h, h->cur->plan, buf, D, s, h->profile != 0);
 
-  std::vector<int64_t> key = h->plan.key;
+  std::vector<int64_t> key = h->cur->plan.key;
   for (int b = 0; b < B; ++b) {
     key.push_back((int64_t)reinterpret_cast<uintptr_t>(sd[b].X));
     key.push_back((int64_t)reinterpret_cast<uintptr_t>(sd[b].idx));
@@ -944,17 +977,17 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   for (auto& g : h->graphs)
     if (g.key == key) {
       TRY_CUDA(cudaGraphLaunch(g.exec, s));
-      h->launches += 5 - (windows_in_prep(h->plan) ? 1 : 0) +
-                     (h->plan.band && h->plan.nband > 0 ? 1 : 0);
+      h->launches += 5 - (windows_in_prep(h->cur->plan) ? 1 : 0) +
+                     (h->cur->plan.band && h->cur->plan.nband > 0 ? 1 : 0);
       return TRAKNN_OK;
     }
   if (!h->cap_stream) TRY_CUDA(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   // The first call's results come from plain launches (kernel attributes, first-use costs);
   // its sequence is captured for later calls while they run.
-  TRY_ST(enqueue_tc(h, h->plan, buf, D, s, false));
+  TRY_ST(enqueue_tc(h, h->cur->plan, buf, D, s, false));
   const int64_t l0 = h->launches;
   TRY_CUDA(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-  const traknn_status st = enqueue_tc(h, h->plan, buf, D, h->cap_stream, false);
+  const traknn_status st = enqueue_tc(h, h->cur->plan, buf, D, h->cap_stream, false);
   cudaGraph_t g = nullptr;
   const cudaError_t ce = cudaStreamEndCapture(h->cap_stream, &g);
   if (st != TRAKNN_OK) {
@@ -976,6 +1009,23 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   h->graphs.push_back(GraphEntry{key, exec});
   TRY_CUDA(cudaStreamSynchronize(s));
   return TRAKNN_OK;
+}
+
+// Several settings of one record in one sweep, or, where their candidate lists (whose units are
+// one tile long whatever their number: 3.8 GB a setting at 75 years, k = 20) would take more
+// than kMaxListBytes or find no memory, in two sweeps of half of them, and so on; a single
+// setting then takes the units of a call of its own. The sweeps' plans are all kept.
+traknn_status run_multi(traknn_ctx* h, const HostSeries* sd, int n, int64_t D, cudaStream_t s) {
+  thread_local TcPlan p;
+  plan_series(sd, n, h->sym, 0, 1, true, epilogue_groups(h, sd, n, D, true, 1, 0.0), p);
+  if (row_list_bytes(p) + col_list_bytes(p) <= kMaxListBytes &&
+      has_room(h->tcws_bytes, tc_layout(p, D, nullptr).total, s)) {
+    const traknn_status st = run_tc(h, sd, n, D, s, false, true);
+    if (st != TRAKNN_ERR_ALLOC) return st;
+  }
+  if (n == 1) return run_tc(h, sd, 1, D, s, false);
+  TRY_ST(run_multi(h, sd, n / 2, D, s));
+  return run_multi(h, sd + n / 2, n - n / 2, D, s);
 }
 
 // FP32 calls on both triangles: the shortest ones, and those whose column-side lists would
@@ -1195,7 +1245,8 @@ traknn_status traknn_destroy(traknn_handle h) {
   if (h->fpws) cudaFree(h->fpws);
   if (h->io) cudaFree(h->io);
   if (h->adj) cudaFree(h->adj);
-  if (h->plan_dev) cudaFree(h->plan_dev);
+  for (PlanSlot& c : h->plans)
+    if (c.dev) cudaFree(c.dev);
   if (h->stats_dev) cudaFree(h->stats_dev);
   if (h->err) cudaFree(h->err);
   for (int i = 0; i < traknn_ctx::kRing; ++i) {
@@ -1337,7 +1388,7 @@ traknn_status traknn_knn_scores_multi(traknn_handle h, const traknn_series* sett
   std::stable_sort(sd.begin(), sd.end(),
                    [](const HostSeries& x, const HostSeries& y) { return x.L < y.L; });
   if (h->precision == TRAKNN_PREC_FP32) return run_fp32(h, sd.data(), nset, D, s, true);
-  return run_tc(h, sd.data(), nset, D, s, false, true);
+  return run_multi(h, sd.data(), nset, D, s);
 }
 
 traknn_status traknn_partition(int64_t M, int L, int nparts, int part, int64_t* row_lo,
