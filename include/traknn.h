@@ -95,9 +95,11 @@ typedef enum {
   TRAKNN_OPT_AUTOTUNE = 9,           /* tensor-core paths: 1 times every work-unit shape of
                                         {4, 8, 16} Gram tiles per unit x {10, 19, 38} row strips
                                         run side by side (the strips only while
-                                        TRAKNN_OPT_GROUP_STRIPS is 0) on the first call of each
-                                        problem shape and keeps the fastest (ignored while
-                                        TRAKNN_OPT_UNIT_COLS is set; default 0) */
+                                        TRAKNN_OPT_GROUP_STRIPS is 0), and the default one-tile
+                                        shape of operand rows of more than 768 K entries or k >
+                                        32, on the first call of each problem shape and keeps
+                                        the fastest (ignored while TRAKNN_OPT_UNIT_COLS is set;
+                                        default 0) */
   TRAKNN_OPT_SEGMENT_K = 10,         /* tensor-core paths: the tensor cores accumulate at most this
                                         many grid points (a multiple of 32) of a Gram entry before
                                         the partial sum is added in FP32 to the entry's running

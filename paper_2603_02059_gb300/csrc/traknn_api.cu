@@ -821,55 +821,6 @@ traknn_status validate_series(const HostSeries* sd, int B, int64_t D) {
   return TRAKNN_OK;
 }
 
-// Work-unit shape for this batch: Gram tiles per unit and row strips whose units run
-// side by side (sharing operand tiles in L2). With tuning on (and neither set by an
-// option) every pair of {4, 8, 16} tiles and {10, 19, 38} strips is timed once after a
-// warm-up launch and the fastest is kept per shape; else 8 tiles and the default
-// grouping (19 strips, or the option's value).
-traknn_status pick_shape(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
-                         int* tiles, int* group) {
-  *tiles = 8;
-  *group = 0;
-  if (!h->autotune || h->unit_cols > 0) return TRAKNN_OK;
-  const std::vector<int64_t> key = shape_key(sd, B, D, h);
-  for (auto& t : h->tuned)
-    if (t.first == key) {
-      *tiles = t.second.first;
-      *group = t.second.second;
-      return TRAKNN_OK;
-    }
-  cudaEvent_t e0, e1;
-  TRY_CUDA(cudaEventCreate(&e0));
-  TRY_CUDA(cudaEventCreate(&e1));
-  float best = 1e30f;
-  int best_t = 8, best_g = 0;
-  const std::vector<int> groups = h->group_strips > 0 ? std::vector<int>{h->group_strips}
-                                                      : std::vector<int>{10, 19, 38};
-  for (int cand_g : groups)
-    for (int cand_t : {4, 8, 16}) {
-      TcBuffers buf;
-      TRY_ST(prepare_tc(h, sd, B, D, cand_t, false, 1, s, &buf, 0, INT_MAX, {}, cand_g));
-      TRY_ST(enqueue_tc(h, h->cur->plan, buf, D, s, false));  // warm-up
-      TRY_CUDA(cudaEventRecord(e0, s));
-      TRY_ST(enqueue_tc(h, h->cur->plan, buf, D, s, false));
-      TRY_CUDA(cudaEventRecord(e1, s));
-      TRY_CUDA(cudaEventSynchronize(e1));
-      float ms = 0.f;
-      TRY_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-      if (ms < best) {
-        best = ms;
-        best_t = cand_t;
-        best_g = cand_g;
-      }
-    }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  h->tuned.emplace_back(key, std::make_pair(best_t, best_g));
-  *tiles = best_t;
-  *group = best_g;
-  return TRAKNN_OK;
-}
-
 // Work-unit shape when neither the autotuner nor an option sets it: Gram tiles per
 // unit and row strips side by side (0 = the planner's default). Shorter units let the
 // persistent CTAs run out of work together and keep more of a series' operand tiles in
@@ -915,6 +866,26 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   while (*tiles > 2 && *tiles * Dp > 65536) *tiles /= 2;
 }
 
+// Row-side lists of one epilogue group with units of t tiles.
+double unit_lists(const HostSeries* sd, int B, int t) {
+  double n = 0.0;
+  for (int b = 0; b < B; ++b) {
+    const double M = (double)(sd[b].N - sd[b].L + 1);
+    n += M * std::ceil(M / (t * kTileCols - (sd[b].L - 1)));
+  }
+  return n;
+}
+
+// Units of `tiles` tiles, or longer ones where the lists would take more than 16 GB at their
+// least capacity (hundreds of thousands of days).
+int fit_tiles(const HostSeries* sd, int B, int tiles) {
+  int kmax = 1;
+  for (int b = 0; b < B; ++b) kmax = std::max(kmax, sd[b].k);
+  while (tiles < 1024 && 2.0 * unit_lists(sd, B, tiles) * (list_pitch(kmax) + 44) * 8.0 > 16e9)
+    tiles *= 2;
+  return tiles;
+}
+
 // The unit length a forward call takes: one Gram tile for operand rows of more than 768 K
 // entries, or k > 32 (pairs of CTAs: D = 32, N = 27,394, k = 64 1 / 2 / 4 / 16 tiles 2,238 /
 // 2,301 / 2,353 / 2,609 us), whatever default_shape says. Issued at its full rate the
@@ -928,21 +899,78 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
 int unit_tiles(const HostSeries* sd, int B, int64_t D, int emb, int tiles) {
   int kmax = 1;
   for (int b = 0; b < B; ++b) kmax = std::max(kmax, sd[b].k);
-  auto lists = [&](int t) {
-    double n = 0.0;
-    for (int b = 0; b < B; ++b) {
-      const double M = (double)(sd[b].N - sd[b].L + 1);
-      n += M * std::ceil(M / (t * kTileCols - (sd[b].L - 1)));
-    }
-    return n;
-  };
+  auto lists = [&](int t) { return unit_lists(sd, B, t); };
   if (tc_groups((int)D * emb) * 64 > 768 || kmax > 32)
     for (int t = 1; t < tiles; t *= 2)
       if (lists(t) <= 4e6) return t;
-  // (hundreds of thousands of days: at most 16 GB of lists of the least capacity)
-  while (tiles < 1024 && 2.0 * lists(tiles) * (list_pitch(kmax) + 44) * 8.0 > 16e9) tiles *= 2;
-  return tiles;
+  return fit_tiles(sd, B, tiles);
 }
+
+// Work-unit shapes (Gram tiles per unit, row strips whose units run side by side, sharing
+// operand tiles in L2; 0 strips: the planner's default) that the autotuner times: every pair
+// of {4, 8, 16} tiles (longer where the lists would be too many) and {10, 19, 38} strips (or
+// the option's), and for long operand rows or k > 32 first the shape of a call without the
+// option, whose one-tile units none of those has.
+std::vector<std::pair<int, int>> tune_shapes(const traknn_ctx* h, const HostSeries* sd, int B,
+                                             int64_t D) {
+  std::vector<std::pair<int, int>> v;
+  int kmax = 1;
+  for (int b = 0; b < B; ++b) kmax = std::max(kmax, sd[b].k);
+  if (tc_groups((int)D) * 64 > 768 || kmax > 32) {
+    int tiles = 8, group = 0;
+    default_shape(h, sd, B, D, 1, 0, INT_MAX, &tiles, &group);
+    v.emplace_back(unit_tiles(sd, B, D, 1, tiles), group);
+  }
+  const std::vector<int> groups = h->group_strips > 0 ? std::vector<int>{h->group_strips}
+                                                      : std::vector<int>{10, 19, 38};
+  for (int g : groups)
+    for (int t : {4, 8, 16}) {
+      const std::pair<int, int> shape(fit_tiles(sd, B, t), g);
+      if (std::find(v.begin(), v.end(), shape) == v.end()) v.push_back(shape);
+    }
+  return v;
+}
+
+// The autotuner's shape for this batch: each of tune_shapes is timed once after a warm-up
+// launch, and the fastest is kept per shape of the call.
+traknn_status pick_shape(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cudaStream_t s,
+                         int* tiles, int* group) {
+  const std::vector<int64_t> key = shape_key(sd, B, D, h);
+  for (auto& t : h->tuned)
+    if (t.first == key) {
+      *tiles = t.second.first;
+      *group = t.second.second;
+      return TRAKNN_OK;
+    }
+  cudaEvent_t e0, e1;
+  TRY_CUDA(cudaEventCreate(&e0));
+  TRY_CUDA(cudaEventCreate(&e1));
+  float best = 1e30f;
+  int best_t = 8, best_g = 0;
+  for (const auto& shape : tune_shapes(h, sd, B, D)) {
+    TcBuffers buf;
+    TRY_ST(prepare_tc(h, sd, B, D, shape.first, false, 1, s, &buf, 0, INT_MAX, {}, shape.second));
+    TRY_ST(enqueue_tc(h, h->cur->plan, buf, D, s, false));  // warm-up
+    TRY_CUDA(cudaEventRecord(e0, s));
+    TRY_ST(enqueue_tc(h, h->cur->plan, buf, D, s, false));
+    TRY_CUDA(cudaEventRecord(e1, s));
+    TRY_CUDA(cudaEventSynchronize(e1));
+    float ms = 0.f;
+    TRY_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+    if (ms < best) {
+      best = ms;
+      best_t = shape.first;
+      best_g = shape.second;
+    }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  h->tuned.emplace_back(key, std::make_pair(best_t, best_g));
+  *tiles = best_t;
+  *group = best_g;
+  return TRAKNN_OK;
+}
+
 
 // Forward pass of B series on the tensor cores. With `graph` set the launch
 // sequence is captured once per (shape, pointers, options) and replayed.
@@ -952,8 +980,9 @@ traknn_status run_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, cuda
   if (!tc_available()) return TRAKNN_ERR_UNSUPPORTED;
   int tiles = 8, group = 0;
   const bool whole = part_lo == 0 && part_hi == INT_MAX;
-  if (!shared && emb == 1 && whole) TRY_ST(pick_shape(h, sd, B, D, s, &tiles, &group));
-  if (!h->autotune && !shared) {
+  if (h->autotune && h->unit_cols <= 0 && !shared && emb == 1 && whole) {
+    TRY_ST(pick_shape(h, sd, B, D, s, &tiles, &group));
+  } else if (!shared) {
     default_shape(h, sd, B, D, emb, part_lo, part_hi, &tiles, &group);
     tiles = unit_tiles(sd, B, D, emb, tiles);
   }

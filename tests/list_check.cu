@@ -2,7 +2,9 @@
 // tests/test_list_host.py like plan_check.cu: the closed form that the window kernel writes
 // it from (main_unit, UnitOrder, band_columns) against the list that build_plan makes for
 // the same call, entry by entry: single, batched and several-settings calls, half tiles and
-// several tiles a unit, column chunks, strips side by side from one to all.
+// several tiles a unit, column chunks, strips side by side from one to all. And the
+// tensor-core path's rules around its list: the pairs' units against the single CTAs', the
+// shapes that the autotuner times, and the unit length of long records.
 #include "../paper_2603_02059_gb300/csrc/traknn_api.cu"
 
 #include <cstdio>
@@ -93,9 +95,73 @@ void check(int64_t N, int64_t D, int L, int e, int B, bool shared, int group, in
   }
 }
 
+void check_pairs(int64_t N, int L, int part_lo, int part_hi, const std::vector<int>& pstrip) {
+  const HostSeries sd{nullptr, N, L, 5, L - 1, nullptr, nullptr, nullptr};
+  static TcPlan p;
+  build_plan(&sd, 1, 100, 1, 0, 1, 19, false, part_lo, part_hi, pstrip, 1, 2, p);
+  p.part_lo = part_lo;
+  p.part_hi = part_hi;
+  pair_units(p);
+  const int K = (int)p.pu.size() - 1, R = p.table.s[0].rows_out;
+  bool ok = (int)p.pp.size() == K + 1;
+  for (int q = 0; ok && q < K; ++q) {
+    // (strip, range) of a phase's pairs, both members, against the single units
+    std::vector<std::pair<int, int>> want, got;
+    for (int u = p.pu[q]; u < p.pu[q + 1]; ++u) want.emplace_back(p.units[u].strip, p.units[u].slot);
+    for (int u = p.pp[q]; u < p.pp[q + 1]; ++u)
+      for (int r = 0; r <= p.units[u].pad[1]; ++r) {
+        const WorkUnit& w = p.units[u];  // (the second strip may start beyond the range)
+        if (r == 0 || std::max(w.jlo, (w.strip + r) * R) < w.jhi)
+          got.emplace_back(w.strip + r, w.slot);
+      }
+    std::sort(want.begin(), want.end());
+    std::sort(got.begin(), got.end());
+    ok = ok && want == got;
+  }
+  if (!ok) {
+    std::printf("FAIL pairs N=%lld L=%d part %d %d\n", (long long)N, L, part_lo, part_hi);
+    ++g_fail;
+  }
+}
+
+void check_tuning(int64_t N, int64_t D, int k, int group_opt) {
+  static traknn_ctx h;
+  h.sm_count = 152;
+  h.group_strips = group_opt;
+  const HostSeries sd{nullptr, N, 5, k, 4, nullptr, nullptr, nullptr};
+  int tiles = 8, group = 0;
+  default_shape(&h, &sd, 1, D, 1, 0, INT_MAX, &tiles, &group);
+  tiles = unit_tiles(&sd, 1, D, 1, tiles);
+  const auto v = tune_shapes(&h, &sd, 1, D);
+  const bool one_tile = D > 756 || k > 32;  // the default's units, which the others exceed
+  bool ok = !one_tile || v[0] == std::make_pair(tiles, group);
+  for (const auto& s : v) {
+    const double lists = (double)(N - 4) * std::ceil((N - 4) / (s.first * 256.0 - 4));
+    ok = ok && 2.0 * lists * ((k + 3) / 4 * 4 + 44) * 8.0 <= 16e9;
+  }
+  ok = ok && (N > 100000 || v.size() == (group_opt ? 3u : 9u) + one_tile);
+  if (!ok) {
+    std::printf("FAIL tuning N=%lld D=%lld k=%d\n", (long long)N, (long long)D, k);
+    ++g_fail;
+  }
+}
+
 }  // namespace
 
 int main() {
+  for (int64_t N : {130, 300, 1100, 5000, 27394})
+    for (int L : {1, 5, 17}) {
+      const int R = kTileRows - (L - 1), strips = (int)((N - L + R) / R);
+      check_pairs(N, L, 0, INT_MAX, {});
+      check_pairs(N, L, strips / 3, strips / 2 + 1, {});
+      const std::vector<int> ps = phase_plan(strips, R, N);
+      if (!ps.empty()) check_pairs(N, L, 0, INT_MAX, ps);
+    }
+  for (int64_t N : {500, 10957, 27394, 300000})
+    for (int64_t D : {32, 3726})
+      for (int k : {10, 64})
+        for (int g : {0, 12}) check_tuning(N, D, k, g);
+
   for (int64_t N : {20, 129, 300, 1100, 2501, 5000, 27394})
     for (int64_t D : {16, 200, 3726})
       for (int L : {1, 5, 15})
