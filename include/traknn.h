@@ -89,8 +89,9 @@ typedef enum {
                                         units of one Gram tile of 256 columns for operand rows
                                         of more than 768 K entries or k > 32, else 1 to 16 tiles
                                         by the Gram tiles per SM of an average series of the
-                                        call; longer where the call's candidate lists would take
-                                        many GB (the results are the same) */
+                                        call; longer, whatever is set, where the call's row-side
+                                        candidate lists would take more than 16 GB (the results
+                                        are the same) */
   TRAKNN_OPT_STATS = 8,              /* 1: count kernel events (read with traknn_stats_read) */
   TRAKNN_OPT_AUTOTUNE = 9,           /* tensor-core paths: 1 times every work-unit shape of
                                         {4, 8, 16} Gram tiles per unit x {10, 19, 38} row strips

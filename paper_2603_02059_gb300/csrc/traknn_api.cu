@@ -480,6 +480,34 @@ int epilogue_groups(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D,
              : 1;
 }
 
+// Row-side lists of one epilogue group with units of t tiles (t = 0: of `cols` columns).
+double unit_lists(const HostSeries* sd, int B, int t, int cols = 0) {
+  double n = 0.0;
+  for (int b = 0; b < B; ++b) {
+    const double M = (double)(sd[b].N - sd[b].L + 1);
+    n += M * std::ceil(M / (t > 0 ? t * kTileCols - (sd[b].L - 1) : cols));
+  }
+  return n;
+}
+// Whether that many lists take more than 16 GB at their least capacity (hundreds of thousands
+// of days, or very short units).
+bool too_many_lists(const HostSeries* sd, int B, double lists) {
+  int kmax = 1;
+  for (int b = 0; b < B; ++b) kmax = std::max(kmax, sd[b].k);
+  return 2.0 * lists * (list_pitch(kmax) + 44) * 8.0 > 16e9;
+}
+// Units of `tiles` tiles or of `cols` columns (the option's), or longer ones where their lists
+// would be too many.
+int fit_tiles(const HostSeries* sd, int B, int tiles) {
+  while (tiles < 1024 && too_many_lists(sd, B, unit_lists(sd, B, tiles))) tiles *= 2;
+  return tiles;
+}
+int fit_cols(const HostSeries* sd, int B, int cols) {
+  while (cols > 0 && cols < (1 << 24) && too_many_lists(sd, B, unit_lists(sd, B, 0, cols)))
+    cols *= 2;
+  return cols;
+}
+
 // Make h->cur the plan for these series (built and uploaded when no slot holds it) and size
 // the workspace. Must not run during a stream capture unless the plan is held.
 traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, int tiles,
@@ -537,7 +565,7 @@ traknn_status prepare_tc(traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   h->cur = sl;
   TcPlan& p = sl->plan;
   if (p.key != key) {
-    build_plan(sd, B, D, h->sym, h->unit_cols, tiles, group, shared, part_lo, part_hi, pstrip,
+    build_plan(sd, B, D, h->sym, fit_cols(sd, B, h->unit_cols), tiles, group, shared, part_lo, part_hi, pstrip,
                egroups, band_tiles, p);
     p.key.clear();  // until the new list is on the device
     p.emb = emb;
@@ -864,26 +892,6 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
   }
   *tiles = per_sm >= 64.0 ? 8 : per_sm >= 16.0 ? 4 : all >= 8.0 ? 2 : 1;
   while (*tiles > 2 && *tiles * Dp > 65536) *tiles /= 2;
-}
-
-// Row-side lists of one epilogue group with units of t tiles.
-double unit_lists(const HostSeries* sd, int B, int t) {
-  double n = 0.0;
-  for (int b = 0; b < B; ++b) {
-    const double M = (double)(sd[b].N - sd[b].L + 1);
-    n += M * std::ceil(M / (t * kTileCols - (sd[b].L - 1)));
-  }
-  return n;
-}
-
-// Units of `tiles` tiles, or longer ones where the lists would take more than 16 GB at their
-// least capacity (hundreds of thousands of days).
-int fit_tiles(const HostSeries* sd, int B, int tiles) {
-  int kmax = 1;
-  for (int b = 0; b < B; ++b) kmax = std::max(kmax, sd[b].k);
-  while (tiles < 1024 && 2.0 * unit_lists(sd, B, tiles) * (list_pitch(kmax) + 44) * 8.0 > 16e9)
-    tiles *= 2;
-  return tiles;
 }
 
 // The unit length a forward call takes: one Gram tile for operand rows of more than 768 K

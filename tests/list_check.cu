@@ -4,7 +4,7 @@
 // the same call, entry by entry: single, batched and several-settings calls, half tiles and
 // several tiles a unit, column chunks, strips side by side from one to all. And the
 // tensor-core path's rules around its list: the pairs' units against the single CTAs', the
-// shapes that the autotuner times, and the unit length of long records.
+// shapes that the autotuner times, and the unit lengths of the option.
 #include "../paper_2603_02059_gb300/csrc/traknn_api.cu"
 
 #include <cstdio>
@@ -124,6 +124,18 @@ void check_pairs(int64_t N, int L, int part_lo, int part_hi, const std::vector<i
   }
 }
 
+void check_unit_cols(int64_t N, int k, int cols) {
+  const HostSeries sd{nullptr, N, 5, k, 4, nullptr, nullptr, nullptr};
+  const int got = fit_cols(&sd, 1, cols);
+  const double M = (double)(N - 4);
+  auto bytes = [&](double c) { return 2.0 * M * std::ceil(M / c) * ((k + 3) / 4 * 4 + 44) * 8.0; };
+  // the option's length where its lists fit, else the first doubling that makes them
+  if (bytes(got) > 16e9 || (got > cols && bytes(got / 2) <= 16e9)) {
+    std::printf("FAIL unit_cols N=%lld k=%d %d -> %d\n", (long long)N, k, cols, got);
+    ++g_fail;
+  }
+}
+
 void check_tuning(int64_t N, int64_t D, int k, int group_opt) {
   static traknn_ctx h;
   h.sm_count = 152;
@@ -157,6 +169,8 @@ int main() {
       const std::vector<int> ps = phase_plan(strips, R, N);
       if (!ps.empty()) check_pairs(N, L, 0, INT_MAX, ps);
     }
+  for (int64_t N : {500, 27394, 200000, 1000000})
+    for (int cols : {1, 256, 5000}) check_unit_cols(N, 20, cols), check_unit_cols(N, 64, cols);
   for (int64_t N : {500, 10957, 27394, 300000})
     for (int64_t D : {32, 3726})
       for (int k : {10, 64})
