@@ -181,12 +181,6 @@ __device__ __forceinline__ void publish_bound(unsigned int* thr, float d) {
   atomicMin(thr, __float_as_uint(__fmul_ru(d, 1.0f + 0x1p-12f)));
 }
 
-// The smallest value above a published bound (>= 0, finite): a distance is within the bound
-// if and only if it is below that.
-__device__ __forceinline__ float above_bound(unsigned int bits) {
-  return __uint_as_float(bits + 1u);
-}
-
 // Window sums c[x] = C(t, j0 + x) of one row to distances W_t + W_j - 2 C, not yet
 // clamped at 0 (a clamped value is a candidate if and only if the unclamped one is: every
 // bound is >= 0). With margin > 0 (one-product band pre-pass) the distance raised by a
@@ -206,10 +200,13 @@ __device__ __forceinline__ void distances(float (&c)[32], float Wt, const float*
   }
 }
 
-// Bit x of cand: d[x] < lim; of ccand: d[x] < t[x] (t 16-byte aligned). The sign of the
+// Bit x of cand: d[x] <= lim; of ccand: d[x] <= t[x] (t 16-byte aligned). The sign of the
 // difference is shifted in with one funnel shift: the difference runs on the FMA pipe,
-// where a compare and a select would both take the half-rate ALU pipe. The difference of a
-// NaN distance is a NaN with a clear sign bit: never a candidate.
+// where a compare and a select would both take the half-rate ALU pipe. A NaN distance would
+// pass (its difference has a clear sign): the caller masks the rows and columns whose window
+// sum is not finite, which are those of a NaN distance. (The reversed difference, which
+// no NaN passes, took 1.2 % more of a 75-year call of 32 values, a compare per candidate in
+// `append` 1.2 % of a BF16 one; one word of finite columns per chunk 0.1 %.)
 __device__ __forceinline__ void candidate_masks(const float (&d)[32], float lim, const float* t,
                                                 uint32_t& cand, uint32_t& ccand) {
   uint32_t a = 0, b = 0;
@@ -220,12 +217,12 @@ __device__ __forceinline__ void candidate_masks(const float (&d)[32], float lim,
 #pragma unroll
     for (int u = 3; u >= 0; --u) {
       const int x = 4 * x4 + u;
-      a = __funnelshift_l(__float_as_uint(d[x] - lim), a, 1);
-      b = __funnelshift_l(__float_as_uint(d[x] - tv[u]), b, 1);
+      a = __funnelshift_l(__float_as_uint(lim - d[x]), a, 1);
+      b = __funnelshift_l(__float_as_uint(tv[u] - d[x]), b, 1);
     }
   }
-  cand = a;
-  ccand = b;
+  cand = ~a;
+  ccand = ~b;
 }
 
 // This row's 32 distances to its row of the chunk buffer.
@@ -306,11 +303,11 @@ struct RowSide {
     n = 0;
     bound = CUDART_INF_F;
   }
-  // A distance enters the list if it is < limit: below `bound` (an equal distance of a
-  // larger index cannot be among the k nearest; none is below 0, whatever an unclamped one
-  // says) and within the row's published bound.
+  // A distance enters the list if it is <= limit: below `bound` (an equal distance of a
+  // larger index cannot be among the k nearest) and within the row's published bound.
   __device__ __forceinline__ float limit(float thr_row) const {
-    return fminf(bound > 0.f ? bound : -CUDART_INF_F, above_bound(__float_as_uint(thr_row)));
+    const float below = bound > 0.f ? __uint_as_float(__float_as_uint(bound) - 1u) : -CUDART_INF_F;
+    return fminf(below, thr_row);
   }
   // Cuts the lists of this warp that have no room for another chunk.
   __device__ __forceinline__ void compress(int k, const TcArgs& a, unsigned int* thr) {
@@ -404,8 +401,8 @@ struct GroupMin {
     for (int x = 0; x < (kTop2 ? 32 : 1); ++x) m2[x] = CUDART_INF_F;
   }
   __device__ __forceinline__ void add(int x, float d) {
-    if (kTop2) m2[x] = fminf(m2[x], d < m[x] ? m[x] : d);
-    m[x] = fminf(m[x], d);  // (a NaN changes neither)
+    if (kTop2) m2[x] = fminf(m2[x], fmaxf(m[x], d));
+    m[x] = fminf(m[x], d);
   }
   // The distances of one chunk whose bit in `valid` is set.
   __device__ __forceinline__ void scan(const float (&d)[32], uint32_t valid) {

@@ -156,7 +156,8 @@ struct Smem {
   Stages st;
   float G[BM][kPitch];          // kHalo carried columns, then the tile's 256
   float D[2][BM][kRowPitch];    // each group's rows of distances
-  float W[2 * BN], T[2 * BN];   // window sums and (above the) bounds of the tile's columns
+  float W[2 * BN], T[2 * BN];   // window sums and bounds of the tile's output columns
+  uint32_t finite[8];           // bit x of word ch: W[32 ch + x] is finite (candidate_masks)
   int cnt[2][64];               // column-side counters of each group
   WorkUnit unit;
 };
@@ -222,8 +223,11 @@ __global__ void __launch_bounds__(NT, 1)
         {
           const int j = c0 - (L - 1) + tid;
           const bool in = j >= 0 && j < us.M;
-          sm.W[tid] = in ? a.W[us.out_base + j] : 0.f;
-          sm.T[tid] = in ? above_bound(__ldcg(w.thr + us.out_base + j)) : 0.f;
+          const float wj = in ? a.W[us.out_base + j] : 0.f;
+          sm.W[tid] = wj;
+          const uint32_t f = __ballot_sync(0xffffffffu, wj < CUDART_INF_F);
+          if ((tid & 31) == 0) sm.finite[tid >> 5] = f;
+          sm.T[tid] = in ? __uint_as_float(__ldcg(w.thr + us.out_base + j)) : 0.f;
         }
         const int jsym = us.T0 + us.R;  // column side from here on (sym)
         const long long cbase = w.sym ? us.col_base + w.col_off[us.strip_base + us.strip] : 0;
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(NT, 1)
           const uint32_t colrange = w.sym ? bit_range(jsym - j0, 32) & unitrange : 0u;
           uint32_t cand = 0, ccand = 0;
           float c[32];
-          if (row_ok) {
+          if (row_ok && Wt < CUDART_INF_F) {
             const float* g = &sm.G[l][kHalo - (L - 1) + ch * 32];
 #pragma unroll
             for (int x = 0; x < 32; ++x) c[x] = g[x];
@@ -249,7 +253,7 @@ __global__ void __launch_bounds__(NT, 1)
               for (int x = 0; x < 32; ++x) c[x] += gmx[x];
             }
             distances(c, Wt, sm.W + ch * 32, 0.f);
-            const uint32_t valid = unitrange & ~bit_range(t - us.e - j0, t + us.e + 1 - j0);
+            const uint32_t valid = unitrange & sm.finite[ch] & ~bit_range(t - us.e - j0, t + us.e + 1 - j0);
             if (kBand) {
               gm.scan(c, valid);
             } else {

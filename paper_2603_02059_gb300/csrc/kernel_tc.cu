@@ -75,9 +75,9 @@ constexpr int kMaxStages = 8;
 constexpr size_t kSmemLimit = 232448;  // 227 KB opt-in per block
 
 // Shared memory of one epilogue group: Gram chunk with carried columns, W, row bounds
-// and correction values of a tile, column-side counters (two chunks).
+// and correction values of a tile, column-side counters (two chunks), a tile's finite columns.
 __host__ __device__ constexpr size_t group_bytes(int L) {
-  return (size_t)BM * chunk_pitch(L, L > 1) * 4 + 3 * BN * 4 + 64 * 4;
+  return (size_t)BM * chunk_pitch(L, L > 1) * 4 + 3 * BN * 4 + 64 * 4 + BN / 8;
 }
 
 struct TcParams {
@@ -511,11 +511,13 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
     // the group's shared memory
     float* Gbuf = reinterpret_cast<float*>(gptr + gid * gbytes);
     float* Wsh = Gbuf + BM * chunk_pitch(a.Lmax, kWin);  // window sums of the tile's output columns
-    float* Tsh = Wsh + BN;         // above the bounds of the tile's output columns (column side)
+    float* Tsh = Wsh + BN;         // row bounds of the tile's output columns (column side)
     float* Csh = Tsh + BN;         // correction values c of the tile's Gram columns
     ColSide cs;
     cs.cnt = reinterpret_cast<int*>(Csh + BN);
     cs.turn = 0;
+    // bit x of word ch: the window sum of the chunk's column x is finite (candidate_masks)
+    uint32_t* finite = reinterpret_cast<uint32_t*>(cs.cnt + 64);
     if (et < 64) cs.cnt[et] = 0;  // ordered before their use by a tile's barriers
     int qs = 0, gt = 0;
     uint32_t qphase = 0, xphase = 0;
@@ -595,7 +597,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
         const int x = et + kEpiThreads * h, j = c0 - (s.L - 1) + x;
         const bool in = j >= 0 && j < s.M;
         hd.w[h] = in ? a.W[s.out_base + j] : 0.f;
-        hd.t[h] = in ? above_bound(__ldcg(w.thr + s.out_base + j)) : 0.f;
+        hd.t[h] = in ? __uint_as_float(__ldcg(w.thr + s.out_base + j)) : 0.f;
         hd.c[h] = c0 + x < N ? a.cval[s.row_base + c0 + x] : 0.f;  // Gram column day c0 + x
       }
       const bool row_ok = l < s.R && t < s.M;
@@ -673,6 +675,8 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           Wsh[et + kEpiThreads * h] = hd.w[h];
           Tsh[et + kEpiThreads * h] = hd.t[h];
           Csh[et + kEpiThreads * h] = hd.c[h];
+          const uint32_t f = __ballot_sync(0xffffffffu, hd.w[h] < CUDART_INF_F);
+          if (lane == 0) finite[(et >> 5) + 4 * h] = f;
         }
         ptx::named_bar_sync(bar, kEpiThreads);  // read by every thread of the group
         const UnitSpan cu = us;  // this pass; `us` moves on to the next one
@@ -749,7 +753,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
           const uint32_t colrange =
               w.sym ? bit_range(jsym - j0, 32) & unitrange : 0u;
           uint32_t cand = 0, ccand = 0;
-          if (row_ok) {
+          if (row_ok && Wt < CUDART_INF_F) {
             // output column x of this chunk is j = j0 + x; its window is the diagonal
             // Gbuf[l+m][x+m], m < L (Eq. 2 as W_t + W_j - 2 sum G)
             if (kWin && L > 1) {
@@ -765,7 +769,7 @@ __global__ void __launch_bounds__(kThreadsG(G), 1)
               }
             }
             distances(c, Wt, Wsh + ch * 32, kBand ? a.band_margin : 0.f);
-            const uint32_t valid = unitrange & ~bit_range(t - cu.e - j0, t + cu.e + 1 - j0);
+            const uint32_t valid = unitrange & finite[ch] & ~bit_range(t - cu.e - j0, t + cu.e + 1 - j0);
             if (kBand) {
               gm.scan(c, valid);  // (outside the exclusion zone)
             } else {
