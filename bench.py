@@ -140,8 +140,11 @@ def kernel_traffic():
     try:
         with open(p) as f:
             txt = f.read()
-        with open(os.path.join(ROOT, "paper_2603_02059_gb300", "csrc", "kernel_tc.cu"), "rb") as f:
-            digest = hashlib.sha256(f.read()).hexdigest()[:16]
+        src = hashlib.sha256()
+        for name in ("kernel_tc.cu", "epilogue.cuh"):
+            with open(os.path.join(ROOT, "paper_2603_02059_gb300", "csrc", name), "rb") as f:
+                src.update(f.read())
+        digest = src.hexdigest()[:16]
     except OSError:
         return None
     m_b = re.search(r"^traffic_bytes_per_step:\s*(\d+)", txt, re.M)

@@ -159,9 +159,9 @@ __device__ __forceinline__ bool unit_span(const WorkUnit& wu, const SeriesInfo* 
 // its current bound to an unsorted list of its own in global memory (one 8-byte store; no
 // lane waits for another); bounds come from minima over groups of columns, and a warp cuts a
 // list to its smallest entries only when it runs full; the merge kernel selects the exact
-// k nearest from all lists. What bounds this part is the instruction count per candidate: at 75 years of 32
-// values, L = 5, k = 20 (about 340 row and 250 column candidates per row) the former
-// sorted register list took a 20-step bubble of compares and selects per candidate.
+// k nearest from all lists. What bounds this part is the instruction count per candidate: at
+// 75 years of 32 values, L = 5, k = 20 (about 340 row and 250 column candidates per row) the
+// former sorted register list took a 20-step bubble of compares and selects per candidate.
 
 // Bits [lo, hi) of a 32-bit word (empty when hi <= lo).
 __device__ __forceinline__ uint32_t bit_range(int lo, int hi) {

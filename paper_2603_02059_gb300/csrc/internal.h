@@ -194,7 +194,7 @@ struct WorkUnit {
                // (units of CTA pairs): 1 if strip + 1 belongs to the unit too
 };
 
-// The same work list in closed form (upper triangle): the units of strips [g group,
+// The work list of a call on the upper triangle in closed form (upper triangle): the units of strips [g group,
 // (g+1) group) by column range and then by strip, for the groups g from the last to the first.
 struct UnitOrder {
   int M, R, cols, group;
@@ -270,7 +270,8 @@ struct TcWork {
   int sym;                  // 1: upper triangle + column side
   // Column-side candidate lists, one record of col_pitch() ints per list:
   // [n, unused, row_0, dist_0, row_1, dist_1, ...] (distances as FP32 bit patterns,
-  // entries in row order or, for a full list, the k best), 16-byte aligned, so that
+  // entries in the order their places were handed out or, for an overfull list, the k best
+  // in row order), 16-byte aligned, so that
   // one 16-byte load gives the count and the first entry.
   int32_t* col_rec;
   long long col_ints;       // ints of col_rec (index checks of the debug build)
@@ -363,7 +364,7 @@ enum : int {
   kStatEpiStage = 10,      // TMEM read-out and staging of a chunk
   kStatEpiBar1 = 11,       // barrier after staging (waits for the slowest thread)
   kStatEpiScan = 12,       // row-side scan and emissions, to the barrier after them
-  kStatEpiCol = 13,        // column-side lists (and dense recomputation)
+  kStatEpiCol = 13,        // lists: append, column records, cuts
   kStatEpiCycles = 14,     // epilogue first thread from start to end
   kStatCount = 15
 };

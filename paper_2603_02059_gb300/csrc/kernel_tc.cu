@@ -38,8 +38,8 @@
 // per-row bounds) are handed out dynamically; a unit may serve several series that
 // share its Gram tiles (several trajectory lengths of one record).
 // Every wait is bounded (globaltimer); a wait that runs out records a timeout
-// in the status word, the CTA drains its own copies and MMAs, frees TMEM and
-// returns.
+// in the status word, the CTA (with the other one of its pair) drains its copies and
+// MMAs, frees TMEM and returns.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <math_constants.h>

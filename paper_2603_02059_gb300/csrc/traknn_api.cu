@@ -772,7 +772,8 @@ traknn_status enqueue_tc(traknn_ctx* h, const TcPlan& p, const TcBuffers& b, int
 // last ones) is in. Phase 0 holds at least the days the centring mean reads. With the
 // upper triangle the work a fraction F of the days unlocks is F^2 of the call, and it
 // is concentrated in few strips with few units each, so every phase ends with a tail
-// of idle SMs: a few large phases overlap the copy better than many small ones.
+// of idle SMs: a few large phases overlapped the copy better than many small ones when units
+// were eight tiles long (with one-tile units only the boundary's place was measured again).
 // Empty when the series is too short to split.
 constexpr double kPhaseDays[] = {0.45};
 std::vector<int> phase_plan(int strips, int R, int64_t N) {
@@ -828,7 +829,12 @@ traknn_status enqueue_tc_phased(traknn_ctx* h, const TcBuffers& b, int64_t D, cu
 
 // Trajectory-embedded operands for a single-series tensor-core call: automatic for
 // small grids, where the fixed per-chunk cost of the epilogue (staging, window sums)
-// and not the contraction decides the time, so L times the Gram work costs little.
+// and not the contraction decides the time, so L times the Gram work costs little. The line
+// was drawn when calls with windows ran one epilogue group. Now that they run two, windows
+// win from about L D = 700 on (embedded / windows, us: N = 27,394, L = 5, D = 32 843 / 1,346,
+// 64 919 / 1,361, 128 1,344 / 1,372, 300 2,443 / 1,421; N = 10,957, D = 512, L = 3 534 / 361;
+// N = 1,826 152 / 131; N = 365, D = 64, L = 3 93 / 101): it stands until it is moved for all
+// that depends on it (results of the two forms differ in rounding).
 constexpr int64_t kEmbedAutoMaxLD = 1536;    // automatic: L * D at most this
 constexpr int64_t kEmbedMaxLD = 1 << 20;     // forced: L * D at most this
 bool use_embedding(const traknn_ctx* h, int64_t D, int L) {
@@ -862,16 +868,11 @@ traknn_status validate_series(const HostSeries* sd, int B, int64_t D) {
 // 497 / 455 / 440 / 451 / 471; D = 640, N = 18,000 915 / 826 / 816 / 843 / 854; N = 27,394
 // times alike from 4 to 16.
 //
-// Otherwise eight tiles from 64 Gram tiles per SM (the 75-year series has 78), four from
-// 16, two below (L = 5, D = 3,726: N = 10,957 1.31 -> 1.21 ms with two; N = 13,697 1.87
-// -> 1.83 ms and N = 20,546 3.84 -> 3.72 ms with four; at N = 27,394 the three lengths
-// time alike; 64 series of 3,650 to 27,394 days in one call: four tiles 1.04x faster than
-// eight), and one where the whole call has fewer than 8 (D = 3,726: N = 1,826 351 ->
-// 300 us, N = 4,500 499 -> 435, N = 6,500 656 -> 589). Long operand rows make every tile
-// long too, so a unit also holds at most 65,536 K entries x tiles (Dp x tiles), two tiles
-// at least: at the 0.25-degree grid (Dp = 59,072, N = 27,394, L = 5) 8 / 4 / 2 tiles took
-// 106.0-108.8 / 99.8-100.7 / 98.9-99.9 ms, while at Dp = 3,840 eight tiles stay within the
-// cap; between the two the cap is a choice.
+// Longer operand rows: a bound for unit_tiles, which takes one tile unless that makes more
+// than 4 M lists (one series of more than 32,000 days); then eight tiles from 64 Gram tiles
+// per SM, four from 16, two below and one where the whole call has fewer than 8, and at most
+// 65,536 K entries x tiles (Dp x tiles) a unit, two tiles at least. (Lines drawn by an earlier
+// kernel, whose units were that long by default.)
 void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, int emb,
                    int part_lo, int part_hi, int* tiles, int* group) {
   double t = 0.0;  // Gram tiles of the call
@@ -896,14 +897,13 @@ void default_shape(const traknn_ctx* h, const HostSeries* sd, int B, int64_t D, 
 
 // The unit length a forward call takes: one Gram tile for operand rows of more than 768 K
 // entries, or k > 32 (pairs of CTAs: D = 32, N = 27,394, k = 64 1 / 2 / 4 / 16 tiles 2,238 /
-// 2,301 / 2,353 / 2,609 us), whatever default_shape says. Issued at its full rate the
-// contraction no longer hides what the longer units cost at the end of a launch and in L2, and
-// lists and bounds
-// that live for one tile cost little: 1 / 2 / 4 / 8 tiles, N = 27,394, D = 3,726, L = 5, k =
-// 20 4,949 / 5,062 / 5,905 / 5,945 us (the last two before the MMAs were issued by an
-// elected lane), N = 10,957 997 / 1,029, D = 58,101 91.9 / 94.4 ms, D = 990, N = 10,957 452 /
-// 473 us. Longer again while the call's row-side lists (one per row and unit) number more
-// than 4 M (4 GB).
+// 2,301 / 2,353 / 2,609 us), whatever default_shape says. The contraction, issued at its full
+// rate, does not hide what longer units cost at the end of a launch and in L2, and lists and
+// bounds that live for one tile cost little: 1 / 2 / 4 / 8 tiles, D = 3,726, L = 5, N = 27,394,
+// k = 20 4,979 / 5,229 / 5,342 / 5,598 us (5,537 / 5,527 / 5,581 / 5,693 repeated without a
+// pause, when the power limit sets the clock), N = 10,957, k = 10 988 / 1,000 / 1,087 / 1,120;
+// 1 / 2: D = 58,101 91.9 / 94.4 ms, D = 990, N = 10,957 452 / 473 us. Longer again while the
+// call's row-side lists (one per row and unit) number more than 4 M (4 GB).
 int unit_tiles(const HostSeries* sd, int B, int64_t D, int emb, int tiles) {
   int kmax = 1;
   for (int b = 0; b < B; ++b) kmax = std::max(kmax, sd[b].k);
@@ -1065,14 +1065,13 @@ traknn_status run_multi(traknn_ctx* h, const HostSeries* sd, int n, int64_t D, c
   return run_multi(h, sd + n / 2, n - n / 2, D, s);
 }
 
-// FP32 calls on both triangles: the shortest ones, and those whose column-side lists would
+// FP32 calls on both triangles: the shortest ones, and those whose candidate lists would
 // not fit (run_fp32). Short calls: one tile per CTA, no band and no column side,
 // five launches. Its scan inserts into sorted lists in shared memory, about k steps per
 // candidate, so it pays up to a product of rows and neighbours, the more the longer a tile's
-// products take. Both triangles / upper triangle (us, L = 5): D = 16, N = 300 k = 5 48 / 64, k =
-// 20 86 / 70, N = 800 k = 5 74 / 81; D = 256, N = 300 k = 5 70 / 126, k = 20 106 / 133, N = 500
-// k = 20 134 / 143, N = 800 k = 5 95 / 137, k = 20 175 / 149, N = 1,200 k = 5 140 / 143; D =
-// 800, N = 1,200 k = 5 237 / 210.
+// products take. Both triangles / upper triangle (us, single calls, L = 5): D = 16, N = 300
+// k = 5 77 / 91, N = 800 k = 5 100 / 104; D = 256, N = 300 k = 5 96 / 164, k = 20 131 / 162,
+// N = 500 k = 20 160 / 171, N = 800 k = 5 119 / 163.
 bool fp32_short(int64_t M, int64_t D, int k) {
   return M <= 1024 && M * k <= (D >= 200 ? 10000 : 4500);
 }
