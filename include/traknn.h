@@ -195,10 +195,9 @@ typedef struct {
  * Up to 64 series run in one persistent launch sequence. With a tensor-core
  * precision it is captured as a CUDA graph on first use and replayed on later
  * calls with the same shapes, pointers and options (the handle keeps one graph
- * per such signature, the 16 most recent; a change of shape or a larger workspace
- * drops them, once more than 16 shapes are in use; evicting the oldest synchronises
- * `stream` once). With
- * TRAKNN_PREC_FP32 it is a sequence of plain launches, and series whose candidate
+ * per such signature, the 16 most recent; a larger workspace, or a new problem shape
+ * once 16 shapes are in use, drops them; evicting the oldest synchronises `stream`
+ * once). With TRAKNN_PREC_FP32 it is a sequence of plain launches, and series whose candidate
  * lists would together take more than 32 GB run one after another. Each series is
  * checked as traknn_check_problem would check it; the first failing series' status
  * is returned before anything is enqueued. */
